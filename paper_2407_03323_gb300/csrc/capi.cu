@@ -66,8 +66,8 @@ void free_all(mot_ctx* c) {
         c->eps = c->chi = c->cg_diag = c->tab = nullptr;
         c->vfac = nullptr;
         c->tab_l0 = nullptr;
-        c->active = c->nmask = c->tiles = nullptr;
-        c->diag32 = nullptr;
+        c->active = c->nmask = c->tiles = c->halo = nullptr;
+        c->diag32 = c->diag_lo = nullptr;
         c->h64.ghat = nullptr; c->h64.level_spec = nullptr;
         c->h32.ghat = nullptr; c->h32.level_spec = nullptr;
         c->shared_src->n_shared -= 1;
@@ -79,16 +79,20 @@ void free_all(mot_ctx* c) {
     for (int k = 0; k < 8; ++k) mot::fft_free_axis(c->lev_fft[k]);
     mot::history_free<double>(c);
     mot::history_free<float>(c);
-    double* dptrs[] = {c->eps, c->chi, c->cg_diag, c->J, c->rhs, c->cg_r,
+    double* dptrs[] = {c->eps, c->chi, c->cg_diag, c->J, c->rhs, c->b_ring, c->fit, c->fit_part,
                        c->cg_q, c->red, c->norms, c->outbuf, c->tab, c->Estage};
     for (double* p : dptrs) cudaFree(p);
     cudaFree(c->tab_l0);
     cudaFree(c->dstatus);
     cudaFree(c->cg32);
-    cudaFree(c->cg_df);
+    cudaFree(c->xb_ring);
+    cudaFree(c->b_lo);
+    cudaFree(c->cg_xl);
+    cudaFree(c->diag_lo);
     cudaFree(c->active);
     cudaFree(c->nmask);
     cudaFree(c->tiles);
+    cudaFree(c->halo);
     cudaFree(c->diag32);
     cudaFree(c->vfac);
     cudaFree(c->probe_tab);
@@ -115,11 +119,55 @@ void reset_state(mot_ctx* c, cudaStream_t s) {
     MOT_CUDA_TRY(cudaMemsetAsync(c->J, 0, sizeof(double) * 3 * c->M * c->jring, s));
     if (c->precision == MOT_FP64) mot::history_reset<double>(c, s);
     else mot::history_reset<float>(c, s);
+    MOT_CUDA_TRY(cudaMemsetAsync(c->fit, 0, sizeof(double) * mot::kFitWords, s));
+    c->fit_steps = 0;
     c->n_done = 0;
     c->E_count = 0;
     c->peak_norm = 0.0;
     c->last_norm = 0.0;
     c->fail_step = 0;
+}
+
+// march-state buffers of the solve (geometry and launch shape set before); inner vectors of
+// inactive voxels stay zero (neighbours read them)
+void solve_alloc(mot_ctx* c) {
+    const long long M = c->M;
+    const size_t slots = mot::kFitVectors + 1;
+    MOT_CUDA_TRY(cudaMalloc(&c->J, sizeof(double) * 3 * M * c->jring));
+    MOT_CUDA_TRY(cudaMalloc(&c->rhs, sizeof(double) * 3 * M));
+    MOT_CUDA_TRY(cudaMalloc(&c->cg_q, sizeof(double) * 3 * M));
+    MOT_CUDA_TRY(cudaMalloc(&c->cg32, sizeof(float) * 16 * M));
+    MOT_CUDA_TRY(cudaMemset(c->cg32, 0, sizeof(float) * 16 * M));
+    if (c->precision == MOT_FP64) {
+        MOT_CUDA_TRY(cudaMalloc(&c->b_ring, sizeof(double) * 3 * M * slots));
+    } else {
+        MOT_CUDA_TRY(cudaMalloc(&c->xb_ring, sizeof(float2) * 3 * M * slots));
+        MOT_CUDA_TRY(cudaMalloc(&c->b_lo, sizeof(float) * 3 * M));
+        MOT_CUDA_TRY(cudaMalloc(&c->cg_xl, sizeof(float) * 4 * M));
+        MOT_CUDA_TRY(cudaMemset(c->cg_xl, 0, sizeof(float) * 4 * M));
+    }
+    MOT_CUDA_TRY(cudaMalloc(&c->fit, sizeof(double) * mot::kFitWords));
+    MOT_CUDA_TRY(cudaMalloc(&c->fit_part, sizeof(double) * mot::kFitSums * c->epi_blocks));
+    MOT_CUDA_TRY(cudaMalloc(&c->red, sizeof(double) * 3 * std::max(c->cg_blocks, 1)));
+    MOT_CUDA_TRY(cudaMalloc(&c->dstatus, sizeof(int) * mot::kStatusWords));
+    MOT_CUDA_TRY(cudaMemset(c->dstatus, 0, sizeof(int) * mot::kStatusWords));
+}
+
+// origins (x | y << 10 | z << 20) of the tiles of TX x TY x TZ voxels with chi > 0 somewhere
+std::vector<int> active_tiles(const mot_ctx* c, const std::vector<double>& chi, int TX, int TY,
+                              int TZ) {
+    std::vector<int> tl;
+    for (int z0 = 0; z0 < c->W; z0 += TZ)
+        for (int y0 = 0; y0 < c->V; y0 += TY)
+            for (int x0 = 0; x0 < c->U; x0 += TX) {
+                bool any = false;
+                for (int z = z0; z < std::min(z0 + TZ, c->W) && !any; ++z)
+                    for (int y = y0; y < std::min(y0 + TY, c->V) && !any; ++y)
+                        for (int x = x0; x < std::min(x0 + TX, c->U) && !any; ++x)
+                            any = chi[((long long)z * c->V + y) * c->U + x] > 0.0;
+                if (any) tl.push_back(x0 | (y0 << 10) | (z0 << 20));
+            }
+    return tl;
 }
 
 void history_for(mot_ctx* c, int n, cudaStream_t s, cudaEvent_t* ev = nullptr) {
@@ -259,13 +307,7 @@ mot_status mot_create_padded(const int grid[3], const double h[3], double dt,
             else mot::level_spectra<float>(c);
         }
         // marching state
-        c->jring = std::max(n_taps, 4) + 1;
-        MOT_CUDA_TRY(cudaMalloc(&c->J, sizeof(double) * 3 * M * c->jring));
-        MOT_CUDA_TRY(cudaMalloc(&c->rhs, sizeof(double) * 3 * M));
-        MOT_CUDA_TRY(cudaMalloc(&c->cg_r, sizeof(double) * 3 * M));
-        MOT_CUDA_TRY(cudaMalloc(&c->cg_q, sizeof(double) * 3 * M));
-        MOT_CUDA_TRY(cudaMalloc(&c->cg32, sizeof(float) * 16 * M));
-        MOT_CUDA_TRY(cudaMemset(c->cg32, 0, sizeof(float) * 16 * M));
+        c->jring = std::max({n_taps, 4, mot::kFitVectors}) + 1;
         {
             std::vector<int> act, nm;
             for (long long m = 0; m < M; ++m) {
@@ -293,23 +335,10 @@ mot_status mot_create_padded(const int grid[3], const double h[3], double dt,
                 MOT_CUDA_TRY(cudaMemcpy(c->nmask, nm.data(), sizeof(int) * c->nact,
                                         cudaMemcpyHostToDevice));
             }
-            {   // 8^3 tiles that hold at least one active voxel
-                std::vector<int> tl;
-                for (int z0 = 0; z0 < c->W; z0 += 8)
-                    for (int y0 = 0; y0 < c->V; y0 += 8)
-                        for (int x0 = 0; x0 < c->U; x0 += 8) {
-                            bool any = false;
-                            for (int z = z0; z < std::min(z0 + 8, c->W) && !any; ++z)
-                                for (int y = y0; y < std::min(y0 + 8, c->V) && !any; ++y)
-                                    for (int x = x0; x < std::min(x0 + 8, c->U) && !any; ++x)
-                                        any = chi[((long long)z * c->V + y) * c->U + x] > 0.0;
-                            if (any) tl.push_back(x0 | (y0 << 10) | (z0 << 20));
-                        }
-                c->ntiles = (int)tl.size();
-                // one block per tile at most: the tiled passes give a block one tile at
-                // a time, so further blocks would only wait at the grid barriers (and
-                // keep SMs from concurrent solves of other contexts)
-                c->cg_blocks = std::min(c->cg_blocks, std::max(c->ntiles, 1));
+            {
+                const std::vector<int> big = active_tiles(c, chi, 8, 8, 8);
+                const std::vector<int> small = active_tiles(c, chi, 8, 4, 4);
+                const std::vector<int>& tl = mot::solve_shape(c, big, small);
                 MOT_CUDA_TRY(cudaMalloc(&c->tiles, sizeof(int) * std::max<size_t>(tl.size(), 1)));
                 if (!tl.empty())
                     MOT_CUDA_TRY(cudaMemcpy(c->tiles, tl.data(), sizeof(int) * tl.size(),
@@ -328,21 +357,17 @@ mot_status mot_create_padded(const int grid[3], const double h[3], double dt,
             MOT_CUDA_TRY(cudaMalloc(&c->vfac, sizeof(double) * 4 * M));
             MOT_CUDA_TRY(cudaMemcpy(c->diag32, d32.data(), sizeof(float) * M, cudaMemcpyHostToDevice));
             if (precision == MOT_FP32_HISTORY) {
-                // float-pair state of the double-float residual; entries of inactive
-                // voxels stay zero (neighbours read them)
-                MOT_CUDA_TRY(cudaMalloc(&c->cg_df, sizeof(float) * 17 * M));
-                MOT_CUDA_TRY(cudaMemset(c->cg_df, 0, sizeof(float) * 16 * M));
                 std::vector<float> dlo(M);
                 for (long long m = 0; m < M; ++m) dlo[m] = (float)(dg[m] - (double)d32[m]);
-                MOT_CUDA_TRY(cudaMemcpy(c->cg_df + 16 * M, dlo.data(), sizeof(float) * M,
+                MOT_CUDA_TRY(cudaMalloc(&c->diag_lo, sizeof(float) * M));
+                MOT_CUDA_TRY(cudaMemcpy(c->diag_lo, dlo.data(), sizeof(float) * M,
                                         cudaMemcpyHostToDevice));
             }
             MOT_CUDA_TRY(cudaMemcpy(c->vfac, vf.data(), sizeof(double) * 4 * M, cudaMemcpyHostToDevice));
         }
-        MOT_CUDA_TRY(cudaMalloc(&c->red, sizeof(double) * 3 * std::max(c->cg_blocks, 1)));
+        mot::solve_halo_lists(c);
         if (c->nact) mot::chebyshev_setup(c);
-        MOT_CUDA_TRY(cudaMalloc(&c->dstatus, sizeof(int) * mot::kStatusWords));
-        MOT_CUDA_TRY(cudaMemset(c->dstatus, 0, sizeof(int) * mot::kStatusWords));
+        solve_alloc(c);
         MOT_CUDA_TRY(cudaMalloc(&c->pw_tab, sizeof(double) * mot::kPwTable));
         reset_state(c, c->stream);
         MOT_CUDA_TRY(cudaStreamSynchronize(c->stream));
@@ -386,9 +411,11 @@ mot_status mot_create_shared(mot_ctx* src, mot_ctx** out) {
     c->tol = src->tol; c->max_iter = src->max_iter; c->growth = src->growth;
     c->jring = src->jring; c->hring = src->hring;
     c->eps = src->eps; c->chi = src->chi; c->cg_diag = src->cg_diag;
-    c->active = src->active; c->nmask = src->nmask; c->tiles = src->tiles;
+    c->active = src->active; c->nmask = src->nmask; c->tiles = src->tiles; c->halo = src->halo;
     c->ntiles = src->ntiles; c->nact = src->nact;
-    c->diag32 = src->diag32; c->vfac = src->vfac;
+    c->diag32 = src->diag32; c->diag_lo = src->diag_lo; c->vfac = src->vfac;
+    c->cg_tile = src->cg_tile; c->cg_resident = src->cg_resident; c->cg_split = src->cg_split;
+    c->epi_blocks = src->epi_blocks; c->epi_threads = src->epi_threads;
     c->cheb_lmin = src->cheb_lmin; c->cheb_lmax = src->cheb_lmax; c->cheb_n = src->cheb_n;
     c->cheb_log_rate = src->cheb_log_rate; c->cheb_inv_theta = src->cheb_inv_theta;
     for (int k = 0; k < 64; ++k) { c->cheb_c1[k] = src->cheb_c1[k]; c->cheb_c2[k] = src->cheb_c2[k]; }
@@ -407,26 +434,11 @@ mot_status mot_create_shared(mot_ctx* src, mot_ctx** out) {
     c->device = src->device;
     c->shared_src = src;
     src->n_shared += 1;
-    const long long M = c->M;
     mot_status st = guarded(c, [&] {
         MOT_CUDA_TRY(cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking));
         if (c->precision == MOT_FP64) mot::history_alloc_shared<double>(c, src);
         else mot::history_alloc_shared<float>(c, src);
-        MOT_CUDA_TRY(cudaMalloc(&c->J, sizeof(double) * 3 * M * c->jring));
-        MOT_CUDA_TRY(cudaMalloc(&c->rhs, sizeof(double) * 3 * M));
-        MOT_CUDA_TRY(cudaMalloc(&c->cg_r, sizeof(double) * 3 * M));
-        MOT_CUDA_TRY(cudaMalloc(&c->cg_q, sizeof(double) * 3 * M));
-        MOT_CUDA_TRY(cudaMalloc(&c->cg32, sizeof(float) * 16 * M));
-        MOT_CUDA_TRY(cudaMemset(c->cg32, 0, sizeof(float) * 16 * M));
-        if (src->cg_df) {
-            MOT_CUDA_TRY(cudaMalloc(&c->cg_df, sizeof(float) * 17 * M));
-            MOT_CUDA_TRY(cudaMemset(c->cg_df, 0, sizeof(float) * 16 * M));
-            MOT_CUDA_TRY(cudaMemcpy(c->cg_df + 16 * M, src->cg_df + 16 * M, sizeof(float) * M,
-                                    cudaMemcpyDeviceToDevice));
-        }
-        MOT_CUDA_TRY(cudaMalloc(&c->red, sizeof(double) * 3 * std::max(c->cg_blocks, 1)));
-        MOT_CUDA_TRY(cudaMalloc(&c->dstatus, sizeof(int) * mot::kStatusWords));
-        MOT_CUDA_TRY(cudaMemset(c->dstatus, 0, sizeof(int) * mot::kStatusWords));
+        solve_alloc(c);
         MOT_CUDA_TRY(cudaMalloc(&c->pw_tab, sizeof(double) * mot::kPwTable));
         reset_state(c, c->stream);
         MOT_CUDA_TRY(cudaStreamSynchronize(c->stream));

@@ -95,15 +95,28 @@ struct mot_ctx {
     double* chi = nullptr;
     double* cg_diag = nullptr;   // (T(0)/eps + delta_0)/chi on active voxels, 0 elsewhere
     double* J = nullptr;         // spatial J ring [jring][3][M] (SoA per slot)
-    double* rhs = nullptr;       // [3][M]
-    double* cg_r = nullptr;
-    float* cg_df = nullptr;      // FP32-history: x, b as float pairs ([4][M] float4), diag low parts [M]
-    double* cg_q = nullptr;
+    double* rhs = nullptr;       // [3][M] adjoint: right-hand side on vacuum voxels
+    double* cg_q = nullptr;      // [3][M] adjoint: lambda on vacuum voxels
     float* cg32 = nullptr;       // FP32 inner CG vectors r, p, q, e ([4][M] float4)
+    // start of the solve (solve.cu): right-hand sides of the last steps and the fit
+    double* b_ring = nullptr;    // FP64: [kFitVectors + 1][3][M]
+    float* xb_ring = nullptr;    // FP32-history: (x, b) float2, [kFitVectors + 1][3][M]
+    float* b_lo = nullptr;       //   low part of b_n [3][M]
+    float* cg_xl = nullptr;      //   low part of x, [M] float4 (later refinements)
+    float* diag_lo = nullptr;    //   low part of cg_diag [M]
+    double* fit = nullptr;       // fit state (kFitWords)
+    double* fit_part = nullptr;  // epilogue's partial sums
+    int fit_steps = 0;           // steps solved since the march state was reset
+    int epi_blocks = 1, epi_threads = 256;
+    unsigned solve_seq = 0;      // solve launches (numbers their neighbour exchanges)
     int* active = nullptr;       // voxels with chi > 0
     int* nmask = nullptr;        // per active voxel: in-grid neighbours (27 bits)
-    int* tiles = nullptr;        // 8^3 tiles holding active voxels (packed origins)
+    int* tiles = nullptr;        // solve tiles holding active voxels (packed origins)
     int ntiles = 0;
+    int cg_tile = 0;             // tile shape (0: 8^3, 1: 8 x 4 x 4)
+    bool cg_resident = false;    // one tile per block, kept in registers
+    int* halo = nullptr;         //   halo voxels of every tile
+    bool cg_split = false;       // FP64 residual by components
     float* diag32 = nullptr;     // FP32 copy of cg_diag
     double* vfac = nullptr;      // [4][M]: 0.5/eps, 1/chi (0 if chi = 0), 1/(0.5/eps + d0), chi
     long long nact = 0;
@@ -114,8 +127,8 @@ struct mot_ctx {
     float cheb_c1[64] = {0}, cheb_c2[64] = {0};
     double* red = nullptr;       // reduction scratch
     int* dstatus = nullptr;      // [0] cg iterations of last step, [1] flags, [2] first bad
-                                 // step, [3] total iterations, [4..6] the solve kernel's
-                                 // grid barrier (arrivals, generation, abort)
+                                 // step, [3] total iterations, [4..7] the solve kernel's
+                                 // grid barrier (arrivals, -, abort, finished blocks)
     long long bar_budget = 0;    // longest barrier wait of the solve kernel, SM clock cycles
     double* norms = nullptr;     // per-step ||J_n||^2 of the current call
     int norms_cap = 0;
@@ -208,6 +221,9 @@ namespace mot {
 constexpr int WIN = 8;  // lag window per octant offset of the interaction table
 constexpr int kPwTable = 1 << 16;   // nodes of the plane-wave table of one call
 constexpr int kStatusWords = 8;     // device status words of a context (dstatus)
+constexpr int kFitVectors = 6;      // earlier right-hand sides that the solve's start fits
+constexpr int kFitWords = 72;       // doubles of the device fit state
+constexpr int kFitSums = kFitVectors + 2;   // partial sums of the epilogue per block
 constexpr double kBarrierBudgetS = 2.0;   // longest wait at a grid barrier of the solve
 
 // quadrature.cu
@@ -243,6 +259,9 @@ template <typename R> void level_spectra(mot_ctx* c);
 // solve.cu
 void solve_step(mot_ctx* c, int n, const double* En, double* norm2_out, cudaStream_t s);
 void stencil_setup(mot_ctx* c);
+const std::vector<int>& solve_shape(mot_ctx* c, const std::vector<int>& big,
+                                    const std::vector<int>& small);
+void solve_halo_lists(mot_ctx* c);
 void chebyshev_setup(mot_ctx* c);
 void write_aos(mot_ctx* c, int n, double* out_dev, cudaStream_t s);
 void read_aos(mot_ctx* c, const double* in_dev, double* slot, cudaStream_t s);

@@ -46,55 +46,205 @@ __device__ __forceinline__ long long jslot(int s0, int l, int jring, long long s
     return (long long)sl * stride;
 }
 
+// ---------------------------------------------------------------- start of the solve
+// The solve of step n starts from x0 = sum_{i=1}^{F} c_i x_{n-i}, the coefficients being
+// the least-squares fit of the previous right-hand side by the F before it,
+//     min || b_{n-1} - sum_i c_i b_{n-1-i} ||,        A x_{n-i} = b_{n-i},
+// applied one step later.  The right-hand sides of a band-limited march change
+// smoothly, so the fit of one step serves the next (start residual 1.7 times that of the
+// fit of b_n itself), and nothing of the fit is on the step's critical path: the epilogue
+// of step n forms the dot products <b_n, b_{n-i}> while it holds the values, and one block
+// of the solve kernel sums them, updates the Gram matrix of the ring and solves the F x F
+// system while the others iterate.  F = 6: relative start residual 3e-6 on the eps_r = 12
+// sphere in a pulse that rises smoothly from rest, 1e-4 .. 1e-3 within 100 steps of an
+// abrupt onset, against 7e-3 .. 3e-2 for the quadratic extrapolation (4 vectors: 30 and 5
+// times more, 12: 2 times less).
+// The extrapolation remains where there is nothing to fit: fewer than four solved steps
+// since the march state was reset, or a fit that leaves more than kFitPoor.
+constexpr int kFit = mot::kFitVectors;
+constexpr int kSlots = kFit + 1;           // ring of right-hand sides
+constexpr int kSums = kFit + 2;            // <b,b>, <b,b_{n-i}>, |x|^2 off the active set
+constexpr double kFitPoor = 0.05;          // largest ||b - fit||^2 / ||b||^2 that is used
+constexpr double kFitPivot = 1e-13;        // relative pivot below which a vector is dropped
+
+struct FitRecord {
+    double c[kFit];
+    double scale;      // a power of two near 1 / rms(b) (0: none yet)
+    int use;           // 0: quadratic extrapolation
+    int pad;
+};
+struct FitState {      // device, zeroed with the march state
+    FitRecord rec[2];                  // step n reads rec[n & 1]; its solve writes the other
+    double gram[kSlots * kSlots];      // <b_i, b_j> by ring slot
+};
+static_assert(sizeof(FitState) <= sizeof(double) * mot::kFitWords, "fit state size");
+
+// b ring slot of step n - i, s0 = n mod kSlots
+__device__ __forceinline__ int fslot(int s0, int i) {
+    const int sl = s0 - i;
+    return sl < 0 ? sl + kSlots : sl;
+}
+
 // per-voxel factors precomputed at setup (no FP64 divisions in the step):
 //   f[0][m] = T(1)/eps_m = 0.5/eps_m, f[1][m] = 1/chi_m (0 if chi_m = 0),
 //   f[2][m] = 1/(T(0)/eps_m + delta_0) (used where chi_m = 0), f[3][m] = chi_m
+struct EpiArgs {
+    long long M;
+    const double* f;
+    const double* En;      // AoS excitation (forward; may be null) or dO/dJ (adjoint)
+    const void* hist;      // (G * J)_hist, SoA
+    double* Jring;
+    int s0, jring;
+    Taps tp;
+    int n, bs, nv;         // step, its ring slot, valid (x, b) pairs before it
+    double* b64;           // FP64: right-hand side ring [kSlots][3][M]
+    float2* xb;            // FP32-history: (x, b) ring [kSlots][3][M], b its high part
+    float* bl;             //   low part of b_n [3][M]
+    float4* x0;            //   x0 for the neighbours' reads
+    double* rhs;           // adjoint: rhs on vacuum voxels (k_adj_vacuum)
+    const FitState* fit;
+    double* part;          // [kSums][gridDim]
+};
+
 // One thread per voxel, its three components: the AoS excitation row and the four
-// factors are read once and coalesced (a thread per component would read E with a
-// stride of three and every factor three times).  All loads come before the stores
-// (the new slot Jn lies in the same ring the loads read from, so loads placed after a
-// store could not be moved ahead of it), and the FIR terms of lags 1..3 reuse them.
-template <typename R>
-__global__ void k_epilogue(long long M, const double* __restrict__ f, const double* __restrict__ En,
-                           const R* __restrict__ hist, double* __restrict__ Jring, int s0,
-                           int jring, Taps tp, double* __restrict__ b) {
-    const long long m = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= M) return;
-    const long long st = 3 * M;
-    const double f0 = f[m], ichi = f[M + m], f2 = f[2 * M + m], chi = f[3 * M + m];
-    const double* r1 = Jring + jslot(s0, 1, jring, st);
-    const double* r2 = Jring + jslot(s0, 2, jring, st);
-    const double* r3 = Jring + jslot(s0, 3, jring, st);
-    double* Jn = Jring + jslot(s0, 0, jring, st);
-    double e[3], j1[3], j2[3], j3[3], P[3];
+// factors are read once and coalesced.  All loads of a component come before its stores
+// (the new slot Jn lies in the same ring the loads read from).  ADJ: the adjoint march
+// (see below).  FP32-history keeps x and b of earlier steps as floats: they only shape the
+// start and the fit; the residual of the start that is stored is formed in float pairs.
+template <typename R, bool ADJ>
+__global__ void __launch_bounds__(NT) k_epilogue(const __grid_constant__ EpiArgs a) {
+    constexpr bool DF = std::is_same<R, float>::value;
+    typedef typename std::conditional<DF, float, double>::type D;   // dot products
+    const long long M = a.M, st = 3 * M;
+    const R* hist = static_cast<const R*>(a.hist);
+    const FitRecord& rec = a.fit->rec[a.n & 1];
+    const bool use = rec.use != 0;
+    double c[kFit];
+    float cf[kFit];
 #pragma unroll
-    for (int beta = 0; beta < 3; ++beta) {
-        const long long i = beta * M + m;
-        e[beta] = En ? En[m * 3 + beta] : 0.0;
-        j1[beta] = r1[i];
-        j2[beta] = r2[i];
-        j3[beta] = r3[i];
-        P[beta] = f0 * j1[beta] - chi * (double)hist[i];
+    for (int i = 0; i < kFit; ++i) {
+        c[i] = use ? rec.c[i] : (i == 0 ? 3.0 : i == 1 ? -3.0 : i == 2 ? 1.0 : 0.0);
+        cf[i] = (float)c[i];
     }
+    const double sc = rec.scale == 0.0 ? 1.0 : rec.scale;
+    const float scf = (float)sc;
+    double bb = 0.0, xin = 0.0;
+    D dots[kFit];
 #pragma unroll
-    for (int beta = 0; beta < 3; ++beta) {
-        const long long i = beta * M + m;
-        for (int l = 1; l < tp.n; ++l) {
-            const double jl = l == 1 ? j1[beta] : l == 2 ? j2[beta] : l == 3 ? j3[beta]
-                                                  : Jring[jslot(s0, l, jring, st) + i];
-            P[beta] += tp.d[l] * jl;
+    for (int i = 0; i < kFit; ++i) dots[i] = 0;
+    for (long long m = (long long)blockIdx.x * blockDim.x + threadIdx.x; m < M;
+         m += (long long)gridDim.x * blockDim.x) {
+        const double f0 = a.f[m], ichi = a.f[M + m], f2 = a.f[2 * M + m], chi = a.f[3 * M + m];
+        const bool active = ichi > 0.0;
+        const double* r1 = a.Jring + jslot(a.s0, 1, a.jring, st);
+        double* Jn = a.Jring + jslot(a.s0, 0, a.jring, st);
+        double e[3], j1[3], P[3], x0[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const long long i = k * M + m;
+            e[k] = a.En ? a.En[m * 3 + k] : 0.0;
+            j1[k] = r1[i];
+            P[k] = ADJ ? f0 * j1[k] - (double)hist[i] : f0 * j1[k] - chi * (double)hist[i];
+        }
+        for (int l = 1; l < a.tp.n; ++l) {
+            const double* rl = a.Jring + jslot(a.s0, l, a.jring, st);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) P[k] += a.tp.d[l] * (l == 1 ? j1[k] : rl[k * M + m]);
+        }
+        if (!active) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const double rhs = e[k] - P[k];
+                if (ADJ) {
+                    // the solve's iterate must vanish off the active set; vacuum voxels
+                    // get their lambda after the solve (k_adj_post), when mu is known
+                    a.rhs[k * M + m] = rhs;
+                    Jn[k * M + m] = 0.0;
+                } else {
+                    const double x = rhs * f2;
+                    Jn[k * M + m] = x;
+                    xin += x * x;
+                }
+            }
+            continue;
+        }
+        double b[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            b[k] = ADJ ? e[k] - P[k] : (e[k] - P[k]) * ichi;
+            bb += b[k] * b[k];
+        }
+        if constexpr (DF) {
+            float bh[3], xs[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                bh[k] = (float)b[k];
+                a.bl[k * M + m] = (float)(b[k] - (double)bh[k]);
+            }
+#pragma unroll
+            for (int i = 0; i < kFit; ++i) {
+                if (i >= a.nv) break;
+                const float2* v = a.xb + (long long)fslot(a.bs, i + 1) * st + m;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const float2 w = v[k * M];
+                    xs[k] += cf[i] * w.x;
+                    dots[i] += (bh[k] * scf) * (w.y * scf);
+                }
+            }
+            if (!use) {   // quadratic extrapolation from the FP64 ring
+                const double* r2 = a.Jring + jslot(a.s0, 2, a.jring, st);
+                const double* r3 = a.Jring + jslot(a.s0, 3, a.jring, st);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    x0[k] = 3.0 * j1[k] - 3.0 * r2[k * M + m] + r3[k * M + m];
+                    xs[k] = (float)(ADJ ? chi * x0[k] : x0[k]);
+                }
+            }
+            float2* v0 = a.xb + (long long)a.bs * st + m;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) v0[k * M] = make_float2(xs[k], bh[k]);
+            a.x0[m] = make_float4(xs[0], xs[1], xs[2], 0.f);
+        } else {
+#pragma unroll
+            for (int i = 0; i < kFit; ++i) {
+                if (i >= (use ? a.nv : 3)) break;
+                const double* rx = a.Jring + jslot(a.s0, i + 1, a.jring, st);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) x0[k] += c[i] * (i == 0 ? j1[k] : rx[k * M + m]);
+            }
+#pragma unroll
+            for (int i = 0; i < kFit; ++i) {
+                if (i >= a.nv) break;
+                const double* rb = a.b64 + (long long)fslot(a.bs, i + 1) * st;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) dots[i] += b[k] * rb[k * M + m];
+            }
+            double* b0 = a.b64 + (long long)a.bs * st;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                b0[k * M + m] = b[k];
+                Jn[k * M + m] = ADJ ? chi * x0[k] : x0[k];
+            }
         }
     }
+    // block sums: every thread leaves its kSums values in shared memory, then one warp per
+    // value adds them (an FP64 addition costs 16 cycles of an SM for each warp, so the
+    // shuffles run on one partial per lane instead of on every thread's)
+    __shared__ double red[kSums][NT + 1];
+    red[0][threadIdx.x] = bb;
 #pragma unroll
-    for (int beta = 0; beta < 3; ++beta) {
-        const long long i = beta * M + m;
-        const double rhs = e[beta] - P[beta];
-        if (ichi > 0.0) {
-            b[i] = rhs * ichi;
-            Jn[i] = 3.0 * j1[beta] - 3.0 * j2[beta] + j3[beta];   // quadratic extrapolation as CG start
-        } else {
-            b[i] = 0.0;
-            Jn[i] = rhs * f2;
+    for (int i = 0; i < kFit; ++i) red[1 + i][threadIdx.x] = (double)dots[i];
+    red[kSums - 1][threadIdx.x] = xin;
+    __syncthreads();
+    const int nw = blockDim.x >> 5;
+    for (int q = threadIdx.x >> 5; q < kSums; q += nw) {
+        double v = 0.0;
+        for (int t = threadIdx.x & 31; t < (int)blockDim.x; t += 32) v += red[q][t];
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if ((threadIdx.x & 31) == 0) {
+            if (DF && q >= 1 && q <= kFit) v = v / sc / sc;
+            a.part[(long long)q * gridDim.x + blockIdx.x] = v;
         }
     }
 }
@@ -106,26 +256,25 @@ struct CGArgs {
     const int* nmask;     // per active voxel: bit e set if neighbour e (0..26) is in the grid
     long long nact;
     int U, V, W;
-    const int* tiles;     // origins (x | y << 10 | z << 20) of the 8^3 tiles with active voxels
+    const int* tiles;     // origins (x | y << 10 | z << 20) of the tiles with active voxels
     int ntiles;
+    const int* halo;      // resident tiles: halo voxels (k_halo_list)
+    int nw;               // worker blocks; block nw sums the dot products and fits
     double* x;            // J_n slot (in/out), SoA [3][M]
-    const double* b;      // rhs / chi, SoA
+    const double* b;      // FP64: rhs / chi, SoA (this step's ring slot)
     const float* diag32;  // A's diagonal (T(0)/eps + delta_0)/chi, FP32 copy
     const double* diag;
-    const double* chi;    // chi_m: a voxel is active (in act) iff chi_m > 0
-    double* r64;          // FP64 residual, SoA
     float4* r;            // FP32 inner vectors, one float4 (x, y, z, 0) per voxel
     float4* p;
     float4* q;
     float4* e;
-    // double-float residual state (FP32-history): x and b as float pairs hi + lo, and
-    // the low parts of the diagonal (its high parts are diag32)
-    float4* xh;
-    float4* xl;
-    float4* bh;
-    float4* bl;
+    // FP32-history: (x, b) of this step, SoA; low parts of b; the low parts of the diagonal
+    // (its high parts are diag32); low parts of x in later refinements
+    float2* xb;
+    const float* bl;
     const float* diag_lo;
-    double* red;          // [3][gridDim]
+    float4* xl;
+    double* red;          // [3][nw]
     double tol2;          // outer tolerance^2 (relative to ||b||^2)
     float inv_theta;      // Chebyshev: 1 / theta, theta = (lmin + lmax) / 2
     int n_cheb;           // most Chebyshev iterations per refinement (<= MAXCHEB)
@@ -136,9 +285,14 @@ struct CGArgs {
     int max_outer;
     int step;             // time index n (for the status record)
     int* status;          // [0] inner its, [1] flags, [2] first bad step, [3] total its
-    unsigned* bar;        // grid barrier: [0] arrivals, [1] generation, [2] abort
+    unsigned* bar;        // grid barrier: [0] arrivals, [2] abort, [3] finished blocks
     long long bar_budget; // longest wait at one barrier, SM clock cycles
     double* norm2;        // ||x||^2 output
+    FitState* fit;
+    const double* part;   // epilogue's partial sums [kSums][nepi]
+    int nepi;
+    int bs, nv;           // ring slot of b_n, valid pairs before it
+    unsigned seq;         // first sequence number of this launch's exchanges
 };
 
 __constant__ float c_st32[27 * 6];   // FP32 copy of c_stencil
@@ -186,6 +340,18 @@ __device__ __forceinline__ void stencil_pairs(const R* __restrict__ S, V&& load,
 
 constexpr int kAllNeighbours = (1 << 27) - 1;
 
+// f(std::integral_constant<int, E>) for the 13 pairs E = 14 .. 26
+template <int B, int E> struct UnrollPairs {
+    template <typename F> __device__ __forceinline__ static void run(F&& f) {
+        f(std::integral_constant<int, B>());
+        UnrollPairs<B + 1, E>::run(f);
+    }
+};
+template <int E> struct UnrollPairs<E, E> {
+    template <typename F> __device__ __forceinline__ static void run(F&&) {}
+};
+typedef UnrollPairs<14, 27> Unroll13;
+
 // (A x)_m in FP64 for an active voxel: centre + 13 symmetric pairs
 __device__ __forceinline__ void applyA64(const CGArgs& a, const double* __restrict__ x, int m,
                                          int mask, double o[3]) {
@@ -227,26 +393,30 @@ __device__ __forceinline__ void df_msub(float sh, float sl, float xh, float xl, 
     oh = s;
     ol = __fadd_rn(ol, __fsub_rn(e, pe));
 }
-// (sh, sl) += (vh, vl)
-__device__ __forceinline__ void df_add(float& sh, float& sl, float vh, float vl) {
-    float s, e;
-    df_two_sum(sh, vh, s, e);
-    sh = s;
-    sl = __fadd_rn(sl, __fadd_rn(vl, e));
-}
 __device__ __forceinline__ void df_split(double v, float& h, float& l) {
     h = (float)v;
     l = (float)(v - (double)h);
 }
 
-// pair EP, 26 - EP in double-float (same zero pattern as stencil_pair)
-template <int EP, bool FULL, typename V>
-__device__ __forceinline__ void stencil_pair_df(V&& load, int mask, float* oh, float* ol) {
+// pair EP, 26 - EP in double-float (same zero pattern as stencil_pair).  load(e, vh, vl)
+// gives the x pair of neighbour e (zero outside the grid); PAIR = false: x is a float (the
+// start), its low part zero
+template <int EP, bool PAIR, typename V>
+__device__ __forceinline__ void stencil_pair_df(V&& load, float* oh, float* ol) {
     constexpr int EM = 26 - EP;
     constexpr int ex = EP % 3 - 1, ey = (EP / 3) % 3 - 1, ez = EP / 9 - 1;
-    float sh[3] = {0.f, 0.f, 0.f}, sl[3] = {0.f, 0.f, 0.f};
-    if (FULL || (mask & (1 << EP))) load(std::integral_constant<int, EP>(), sh, sl);
-    if (FULL || (mask & (1 << EM))) load(std::integral_constant<int, EM>(), sh, sl);
+    float sh[3], sl[3];
+    float4 ah, al, bh, bl;
+    load(std::integral_constant<int, EP>(), ah, al);
+    load(std::integral_constant<int, EM>(), bh, bl);
+    df_two_sum(ah.x, bh.x, sh[0], sl[0]);
+    df_two_sum(ah.y, bh.y, sh[1], sl[1]);
+    df_two_sum(ah.z, bh.z, sh[2], sl[2]);
+    if constexpr (PAIR) {
+        sl[0] = __fadd_rn(sl[0], __fadd_rn(al.x, bl.x));
+        sl[1] = __fadd_rn(sl[1], __fadd_rn(al.y, bl.y));
+        sl[2] = __fadd_rn(sl[2], __fadd_rn(al.z, bl.z));
+    }
     const float* H = c_st32 + EP * 6;
     const float* L = c_stl + EP * 6;
     df_msub(H[0], L[0], sh[0], sl[0], oh[0], ol[0]);
@@ -266,58 +436,79 @@ __device__ __forceinline__ void stencil_pair_df(V&& load, int mask, float* oh, f
     }
 }
 
-template <bool FULL, typename V>
-__device__ __forceinline__ void stencil_pairs_df(V&& load, int mask, float* oh, float* ol) {
-    stencil_pair_df<14, FULL>(load, mask, oh, ol);
-    stencil_pair_df<15, FULL>(load, mask, oh, ol);
-    stencil_pair_df<16, FULL>(load, mask, oh, ol);
-    stencil_pair_df<17, FULL>(load, mask, oh, ol);
-    stencil_pair_df<18, FULL>(load, mask, oh, ol);
-    stencil_pair_df<19, FULL>(load, mask, oh, ol);
-    stencil_pair_df<20, FULL>(load, mask, oh, ol);
-    stencil_pair_df<21, FULL>(load, mask, oh, ol);
-    stencil_pair_df<22, FULL>(load, mask, oh, ol);
-    stencil_pair_df<23, FULL>(load, mask, oh, ol);
-    stencil_pair_df<24, FULL>(load, mask, oh, ol);
-    stencil_pair_df<25, FULL>(load, mask, oh, ol);
-    stencil_pair_df<26, FULL>(load, mask, oh, ol);
-}
-
-// r = b - A x at an active voxel in double-float, rounded to FP32.  ch, cl: the voxel's
-// x pair; dh, dl: its diagonal; bh, bl: its b pair; load(e, sh, sl) adds the x pair of
-// neighbour e (compile-time index) to (sh, sl).
-template <bool FULL, typename V>
-__device__ __forceinline__ float4 residual_df_at(float4 ch, float4 cl, float dh, float dl,
-                                                 float4 bh, float4 bl, V&& load, int mask) {
+// r = b - A x at an active voxel in double-float, rounded to FP32.  dh, dl: its diagonal;
+// bh, bl: its b pair
+template <bool PAIR, typename V>
+__device__ __forceinline__ float4 residual_df_at(float dh, float dl, const float* bh,
+                                                 const float* bl, V&& load) {
     float oh[3] = {0.f, 0.f, 0.f}, ol[3] = {0.f, 0.f, 0.f};   // o = A x
     const float* H0 = c_st32 + 13 * 6;
     const float* L0 = c_stl + 13 * 6;
     // centre block: (d - G_0(0)) x; G_0(0) is diagonal (parity)
-    df_msub(-dh, -dl, ch.x, cl.x, oh[0], ol[0]);
-    df_msub(-dh, -dl, ch.y, cl.y, oh[1], ol[1]);
-    df_msub(-dh, -dl, ch.z, cl.z, oh[2], ol[2]);
-    df_msub(H0[0], L0[0], ch.x, cl.x, oh[0], ol[0]);
-    df_msub(H0[1], L0[1], ch.y, cl.y, oh[1], ol[1]);
-    df_msub(H0[2], L0[2], ch.z, cl.z, oh[2], ol[2]);
-    // o = (d - G_0(0)) x - sum_pairs G_0(e) (x_e + x_-e) = A x
-    stencil_pairs_df<FULL>(load, mask, oh, ol);
-    float r[3];
-    const float bhv[3] = {bh.x, bh.y, bh.z}, blv[3] = {bl.x, bl.y, bl.z};
+    float4 c4, cl4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    load(std::integral_constant<int, 13>(), c4, cl4);
+    const float ch[3] = {c4.x, c4.y, c4.z};
+    const float cl[3] = {PAIR ? cl4.x : 0.f, PAIR ? cl4.y : 0.f, PAIR ? cl4.z : 0.f};
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
+    for (int k = 0; k < 3; ++k) {
+        df_msub(-dh, -dl, ch[k], cl[k], oh[k], ol[k]);
+        df_msub(H0[k], L0[k], ch[k], cl[k], oh[k], ol[k]);
+    }
+    // o = (d - G_0(0)) x - sum_pairs G_0(e) (x_e + x_-e) = A x
+    stencil_pair_df<14, PAIR>(load, oh, ol);
+    stencil_pair_df<15, PAIR>(load, oh, ol);
+    stencil_pair_df<16, PAIR>(load, oh, ol);
+    stencil_pair_df<17, PAIR>(load, oh, ol);
+    stencil_pair_df<18, PAIR>(load, oh, ol);
+    stencil_pair_df<19, PAIR>(load, oh, ol);
+    stencil_pair_df<20, PAIR>(load, oh, ol);
+    stencil_pair_df<21, PAIR>(load, oh, ol);
+    stencil_pair_df<22, PAIR>(load, oh, ol);
+    stencil_pair_df<23, PAIR>(load, oh, ol);
+    stencil_pair_df<24, PAIR>(load, oh, ol);
+    stencil_pair_df<25, PAIR>(load, oh, ol);
+    stencil_pair_df<26, PAIR>(load, oh, ol);
+    float r[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
         float s, e;
-        df_two_sum(bhv[c], -oh[c], s, e);
-        r[c] = __fadd_rn(s, __fadd_rn(__fsub_rn(blv[c], ol[c]), e));
+        df_two_sum(bh[k], -oh[k], s, e);
+        r[k] = __fadd_rn(s, __fadd_rn(__fsub_rn(bl[k], ol[k]), e));
     }
     return make_float4(r[0], r[1], r[2], 0.f);
 }
 
-// One Chebyshev pass on 8^3 tiles: d_k (with a one-voxel halo, zero outside the grid)
-// is staged in shared memory, then every active voxel of the tile updates
+// ---------------------------------------------------------------- tiles
+// The FP32 passes run on tiles of the grid.  A pass stages the tile of d_k with a
+// one-voxel halo (zero outside the grid) in shared memory, then every active voxel updates
 //   e += d_k, r -= A d_k, d_{k+1} = c1 d_k + c2 r.
 // Inactive voxels (diag = 0) hold zeros in every vector and are skipped.
-constexpr int TT = 8;
-constexpr int TH = TT + 2;
+// Two shapes (mot::solve_tiles chooses): 8 x 8 x 8 with 256 threads where the grid has
+// enough tiles to fill the GPU, and 8 x 4 x 4 with one voxel a thread for the small grids,
+// where a block has at most one tile: it then keeps e, r, the diagonal and its own d in
+// registers for the whole solve and a pass only fetches the halo.
+template <int X, int Y, int Z, int THREADS> struct TileShape {
+    static constexpr int TX = X, TY = Y, TZ = Z, NTH = THREADS;
+    static constexpr int HX = X + 2, HY = Y + 2, HZ = Z + 2, HALO = HX * HY * HZ;
+    static constexpr int VPT = X * Y * Z / THREADS;      // voxels per thread
+    static_assert(VPT * THREADS == X * Y * Z, "tile voxels per thread");
+    __device__ static void local(int q, int& lx, int& ly, int& lz) {
+        lx = q % TX; ly = (q / TX) % TY; lz = q / (TX * TY);
+    }
+    __device__ static int hidx(int lx, int ly, int lz) { return ((lz + 1) * HY + ly + 1) * HX + lx + 1; }
+    template <int E> __device__ static constexpr int off() {
+        return ((E / 9 - 1) * HY + ((E / 3) % 3 - 1)) * HX + (E % 3 - 1);
+    }
+};
+typedef TileShape<8, 8, 8, 256> BigTile;
+typedef TileShape<8, 4, 4, 128> SmallTile;
+
+__device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
 // asynchronous 16-byte global -> shared copy; zero-fills the destination when !valid
 __device__ __forceinline__ void cp_async16(void* dst, const void* src, bool valid) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
@@ -334,158 +525,349 @@ __device__ __forceinline__ void cp_async_wait0() {   // every group landed
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
 }
 
-// halo (TH^3, zero outside the grid) of d around the tile with origin `org`
-__device__ __forceinline__ void load_halo(const CGArgs& a, const float4* __restrict__ dk,
+// halo (zero outside the grid) of v around the tile with origin `org`
+template <class T>
+__device__ __forceinline__ void load_halo(const CGArgs& a, const float4* __restrict__ v,
                                           float4* buf, int org) {
     const long long UV = (long long)a.U * a.V;
     const int x0 = org & 1023, y0 = (org >> 10) & 1023, z0 = org >> 20;
-    for (int h = threadIdx.x; h < TH * TH * TH; h += blockDim.x) {
-        const int hx = h % TH, hy = (h / TH) % TH, hz = h / (TH * TH);
+    for (int h = threadIdx.x; h < T::HALO; h += T::NTH) {
+        const int hx = h % T::HX, hy = (h / T::HX) % T::HY, hz = h / (T::HX * T::HY);
         const int x = x0 + hx - 1, y = y0 + hy - 1, z = z0 + hz - 1;
         const bool in = x >= 0 && x < a.U && y >= 0 && y < a.V && z >= 0 && z < a.W;
-        cp_async16(&buf[h], in ? dk + ((long long)z * UV + (long long)y * a.U + x) : dk, in);
+        cp_async16(&buf[h], in ? v + ((long long)z * UV + (long long)y * a.U + x) : v, in);
     }
 }
 
-// One Chebyshev iteration over the tiles of this block: r -= A d_k, e += d_k (e = d_0
-// on the first iteration, so e needs no clearing), d_{k+1} = c1 d_k + c2 r.  The halo of the next tile is copied into the other shared
-// buffer while the current one is computed, and each thread loads its voxels' own
-// e, r and diagonal before waiting for the halo.
-constexpr int kVoxPerThread = TT * TT * TT / NT;
-static_assert(kVoxPerThread * NT == TT * TT * TT, "tile voxels per thread");
+// A d at halo position hc of a staged tile, for a voxel of diagonal dg
+template <class T>
+__device__ __forceinline__ void apply32(const float4* sb, int hc, float dg, float4& c, float& o0,
+                                        float& o1, float& o2) {
+    const float* S0 = c_st32 + 13 * 6;
+    c = sb[hc];
+    o0 = (dg - S0[0]) * c.x;
+    o1 = (dg - S0[1]) * c.y;
+    o2 = (dg - S0[2]) * c.z;
+    auto load = [&](auto e, float& sx, float& sy, float& sz) {
+        const float4 v = sb[hc + T::template off<decltype(e)::value>()];
+        sx += v.x;
+        sy += v.y;
+        sz += v.z;
+    };
+    stencil_pairs<true>(c_st32, load, 0, o0, o1, o2);
+}
+
+// voxel index of thread slot v of the tile at org, -1 if outside the grid
+template <class T>
+__device__ __forceinline__ long long tile_voxel(const CGArgs& a, int org, int v) {
+    int lx, ly, lz;
+    T::local(threadIdx.x + v * T::NTH, lx, ly, lz);
+    const int x = (org & 1023) + lx, y = ((org >> 10) & 1023) + ly, z = (org >> 20) + lz;
+    if (x >= a.U || y >= a.V || z >= a.W) return -1;
+    return ((long long)z * a.V + y) * a.U + x;
+}
+
+// One Chebyshev iteration over the tiles of this block with all vectors in memory (e = d_0
+// on the first iteration, so e needs no clearing).  The halo of the next tile is copied
+// into the other shared buffer while the current one is computed, and each thread loads
+// its voxels' own e, r and diagonal before waiting for the halo.  LAST: adds |r|^2.
+template <class T>
 __device__ __forceinline__ void cheb_pass_tiled(const CGArgs& a, const float4* __restrict__ dk,
                                                 float4* __restrict__ dn, float c1, float c2,
-                                                bool first, float4 (*sd)[TH * TH * TH]) {
-    const long long UV = (long long)a.U * a.V;
+                                                bool first, bool last, float4 (*sd)[T::HALO],
+                                                double& rr_p) {
     int tile = blockIdx.x;
-    if (tile < a.ntiles) load_halo(a, dk, sd[0], a.tiles[tile]);
+    if (tile < a.ntiles) load_halo<T>(a, dk, sd[0], a.tiles[tile]);
     cp_async_commit();
-    for (int it = 0; tile < a.ntiles; ++it, tile += gridDim.x) {
-        const int next = tile + gridDim.x;
-        if (next < a.ntiles) load_halo(a, dk, sd[(it + 1) & 1], a.tiles[next]);
+    for (int it = 0; tile < a.ntiles; ++it, tile += a.nw) {
+        const int next = tile + a.nw;
+        if (next < a.ntiles) load_halo<T>(a, dk, sd[(it + 1) & 1], a.tiles[next]);
         cp_async_commit();
         const int org = a.tiles[tile];
-        const int x0 = org & 1023, y0 = (org >> 10) & 1023, z0 = org >> 20;
-        long long mv[kVoxPerThread];
-        float dgv[kVoxPerThread];
-        float4 ev[kVoxPerThread], rv[kVoxPerThread];
+        long long mv[T::VPT];
+        float dgv[T::VPT];
+        float4 ev[T::VPT], rv[T::VPT];
 #pragma unroll
-        for (int v = 0; v < kVoxPerThread; ++v) {
-            const int q = threadIdx.x + v * NT;
-            const int lx = q % TT, ly = (q / TT) % TT, lz = q / (TT * TT);
-            const int x = x0 + lx, y = y0 + ly, z = z0 + lz;
+        for (int v = 0; v < T::VPT; ++v) {
+            const long long m = tile_voxel<T>(a, org, v);
             mv[v] = -1;
-            dgv[v] = 0.f;
-            if (x < a.U && y < a.V && z < a.W) {
-                const long long m = (long long)z * UV + (long long)y * a.U + x;
-                dgv[v] = a.diag32[m];
-                if (dgv[v] != 0.f) {
-                    mv[v] = m;
-                    ev[v] = first ? make_float4(0.f, 0.f, 0.f, 0.f) : a.e[m];
-                    rv[v] = a.r[m];
-                }
+            dgv[v] = m >= 0 ? a.diag32[m] : 0.f;
+            if (dgv[v] != 0.f) {
+                mv[v] = m;
+                ev[v] = first ? make_float4(0.f, 0.f, 0.f, 0.f) : a.e[m];
+                rv[v] = a.r[m];
             }
         }
         cp_async_wait1();
         __syncthreads();
         const float4* sb = sd[it & 1];
 #pragma unroll
-        for (int v = 0; v < kVoxPerThread; ++v) {
+        for (int v = 0; v < T::VPT; ++v) {
             if (mv[v] < 0) continue;
-            const int q = threadIdx.x + v * NT;
-            const int lx = q % TT, ly = (q / TT) % TT, lz = q / (TT * TT);
-            const int hc = ((lz + 1) * TH + (ly + 1)) * TH + (lx + 1);
-            const float dg = dgv[v];
-            const float* S0 = c_st32 + 13 * 6;
-            const float4 c = sb[hc];
-            float o0 = (dg - S0[0]) * c.x, o1 = (dg - S0[1]) * c.y, o2 = (dg - S0[2]) * c.z;
-            auto load = [&](auto e, float& sx, float& sy, float& sz) {
-                constexpr int E = decltype(e)::value;
-                constexpr int off = ((E / 9 - 1) * TH + ((E / 3) % 3 - 1)) * TH + (E % 3 - 1);
-                const float4 v = sb[hc + off];
-                sx += v.x;
-                sy += v.y;
-                sz += v.z;
-            };
-            stencil_pairs<true>(c_st32, load, 0, o0, o1, o2);
+            int lx, ly, lz;
+            T::local(threadIdx.x + v * T::NTH, lx, ly, lz);
+            float4 c;
+            float o0, o1, o2;
+            apply32<T>(sb, T::hidx(lx, ly, lz), dgv[v], c, o0, o1, o2);
             float4 e = ev[v], r = rv[v];
             e.x += c.x; e.y += c.y; e.z += c.z;
             r.x -= o0; r.y -= o1; r.z -= o2;
             const long long m = mv[v];
             a.e[m] = e;
             a.r[m] = r;
+            if (last) rr_p += (double)r.x * r.x + (double)r.y * r.y + (double)r.z * r.z;
             dn[m] = make_float4(c1 * c.x + c2 * r.x, c1 * c.y + c2 * r.y, c1 * c.z + c2 * r.z, 0.f);
         }
         __syncthreads();
     }
 }
 
-// Double-float residual pass on the 8^3 tiles (FP32-history): the two halves of the
-// shared halo buffer hold the hi and lo parts of x around the tile (zero outside the
-// grid and on inactive voxels, so no neighbour mask is needed).  Writes r (rounded to
-// FP32) and the first Chebyshev direction d_0 = r / theta on active voxels and adds
-// |r|^2 (and, on the first pass, |b|^2 in FP64) to the thread's partial sums.
-__device__ __forceinline__ void residual_df_tiled(const CGArgs& a, float4 (*sd)[TH * TH * TH],
-                                                  double& rr_p, double& bb_p, bool first) {
-    const long long UV = (long long)a.U * a.V;
-    const long long M = a.M;
-    for (int tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x) {
-        const int org = a.tiles[tile];
-        load_halo(a, a.xh, sd[0], org);
-        load_halo(a, a.xl, sd[1], org);
-        cp_async_commit();
-        const int x0 = org & 1023, y0 = (org >> 10) & 1023, z0 = org >> 20;
-        long long mv[kVoxPerThread];
-        float dhv[kVoxPerThread], dlv[kVoxPerThread];
-        float4 bhv[kVoxPerThread], blv[kVoxPerThread];
+// A block's one tile, resident for the whole solve: each thread's e, r, d and diagonal in
+// registers, the tile of d_k in shared memory.  Neighbouring blocks exchange d through
+// global memory without a grid barrier: a voxel's d is one 16-byte word whose fourth lane
+// is the sequence number of its iteration, stored and loaded as a unit, and a block waits
+// for exactly the words of its halo (bounded, like the grid barrier).  An iteration then
+// costs one store-to-load trip through L2 instead of fence, counter, poll and halo load.
+// d_k lives in p for even and q for odd k; a block overwrites d_k with d_{k+2} only after
+// it has seen d_{k+1} of its neighbours, which they store after reading d_k.
+template <class T> struct Resident {
+    static constexpr int SHELL = T::HALO - T::TX * T::TY * T::TZ;
+    static constexpr int HPT = (SHELL + T::NTH - 1) / T::NTH;   // halo voxels per thread
+    int m[T::VPT];           // voxel index, -1: none or inactive
+    float dg[T::VPT];
+    float4 e[T::VPT], r[T::VPT], d[T::VPT];
+    int hm[HPT], hs[HPT];    // halo voxels: index (-1: none, stays zero) and shared position
+    // position h of the shell of the HX x HY x HZ box: two z faces, then the rings between
+    __device__ static void shell(int h, int& hx, int& hy, int& hz) {
+        constexpr int FACE = T::HX * T::HY, RING = FACE - T::TX * T::TY;
+        if (h < 2 * FACE) {
+            hz = h < FACE ? 0 : T::HZ - 1;
+            hx = (h % FACE) % T::HX;
+            hy = (h % FACE) / T::HX;
+        } else {
+            const int k = h - 2 * FACE, q = k % RING;
+            hz = 1 + k / RING;
+            if (q < 2 * T::HX) { hy = q < T::HX ? 0 : T::HY - 1; hx = q % T::HX; }
+            else { hy = 1 + (q - 2 * T::HX) / 2; hx = ((q - 2 * T::HX) & 1) ? T::HX - 1 : 0; }
+        }
+    }
+};
+
+template <class T>
+__device__ __forceinline__ void resident_init(const CGArgs& a, Resident<T>& t, float4 (*sd)[T::HALO]) {
+    typedef Resident<T> RT;
 #pragma unroll
-        for (int v = 0; v < kVoxPerThread; ++v) {
-            const int q = threadIdx.x + v * NT;
-            const int x = x0 + q % TT, y = y0 + (q / TT) % TT, z = z0 + q / (TT * TT);
+    for (int v = 0; v < T::VPT; ++v) {
+        t.m[v] = -1;
+        t.dg[v] = 0.f;
+    }
+#pragma unroll
+    for (int i = 0; i < RT::HPT; ++i) t.hm[i] = t.hs[i] = -1;
+    if ((int)blockIdx.x >= a.ntiles) return;
+    const int org = a.tiles[blockIdx.x];
+#pragma unroll
+    for (int v = 0; v < T::VPT; ++v) {
+        const long long m = tile_voxel<T>(a, org, v);
+        t.dg[v] = m >= 0 ? a.diag32[m] : 0.f;
+        if (t.dg[v] != 0.f) t.m[v] = (int)m;
+    }
+#pragma unroll
+    for (int i = 0; i < RT::HPT; ++i) {
+        const int h = threadIdx.x + i * T::NTH;
+        if (h >= RT::SHELL) continue;
+        int hx, hy, hz;
+        RT::shell(h, hx, hy, hz);
+        t.hs[i] = (hz * T::HY + hy) * T::HX + hx;
+        t.hm[i] = a.halo[(long long)blockIdx.x * (RT::HPT * T::NTH) + h];
+        sd[0][t.hs[i]] = sd[1][t.hs[i]] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+}
+
+// halo list of every tile (setup): the voxel of each shell position, -1 where the tile does
+// not need it: outside the grid, inactive, or with no active voxel of the tile next to it.
+// The last condition makes the waits mutual (a block waits only for words of blocks that
+// wait for its own), which is what keeps a word from being overwritten while it is awaited.
+template <class T>
+__global__ void k_halo_list(const int* __restrict__ tiles, const float* __restrict__ diag32, int U,
+                            int V, int W, int* __restrict__ halo) {
+    typedef Resident<T> RT;
+    const int org = tiles[blockIdx.x];
+    const int x0 = org & 1023, y0 = (org >> 10) & 1023, z0 = org >> 20;
+    for (int h = threadIdx.x; h < RT::HPT * T::NTH; h += blockDim.x) {
+        int found = -1;
+        if (h < RT::SHELL) {
+            int hx, hy, hz;
+            RT::shell(h, hx, hy, hz);
+            const int x = x0 + hx - 1, y = y0 + hy - 1, z = z0 + hz - 1;
+            const long long m = ((long long)z * V + y) * U + x;
+            if (x >= 0 && x < U && y >= 0 && y < V && z >= 0 && z < W && diag32[m] != 0.f)
+                for (int e = 0; e < 27; ++e) {
+                    const int nx = x + e % 3 - 1, ny = y + (e / 3) % 3 - 1, nz = z + e / 9 - 1;
+                    if (nx < x0 || nx >= min(x0 + T::TX, U) || ny < y0 || ny >= min(y0 + T::TY, V) ||
+                        nz < z0 || nz >= min(z0 + T::TZ, W))
+                        continue;
+                    if (diag32[((long long)nz * V + ny) * U + nx] != 0.f) found = (int)m;
+                }
+        }
+        halo[(long long)blockIdx.x * (RT::HPT * T::NTH) + h] = found;
+    }
+}
+
+// 16-byte loads and stores that are single-copy atomic (data and sequence number together)
+__device__ __forceinline__ float4 ld_word(const float4* p) {
+    unsigned long long lo, hi;
+    asm volatile("{\n.reg .b128 t;\nld.relaxed.gpu.global.b128 t, [%2];\nmov.b128 {%0, %1}, t;\n}"
+                 : "=l"(lo), "=l"(hi) : "l"(p) : "memory");
+    return make_float4(__uint_as_float((unsigned)lo), __uint_as_float((unsigned)(lo >> 32)),
+                       __uint_as_float((unsigned)hi), __uint_as_float((unsigned)(hi >> 32)));
+}
+__device__ __forceinline__ void st_word(float4* p, float4 v) {
+    const unsigned long long lo = (unsigned long long)__float_as_uint(v.x) |
+                                  ((unsigned long long)__float_as_uint(v.y) << 32);
+    const unsigned long long hi = (unsigned long long)__float_as_uint(v.z) |
+                                  ((unsigned long long)__float_as_uint(v.w) << 32);
+    asm volatile("{\n.reg .b128 t;\nmov.b128 t, {%1, %2};\nst.relaxed.gpu.global.b128 [%0], t;\n}"
+                 ::"l"(p), "l"(lo), "l"(hi) : "memory");
+}
+
+// a wait that ran out of its budget: abort word and timeout flag, as grid_barrier
+__device__ __forceinline__ void wait_failed(const CGArgs& a) {
+    atomicExch(a.bar + 2, 1u);
+    atomicOr(a.status + 1, 4);
+    atomicCAS(a.status + 2, 0, a.step);
+}
+
+// One iteration on the resident tile; k = 0 starts from r (complete in memory, d_0 = r /
+// theta), later ones wait for the words tagged `seq`.  Returns false on a timed-out wait.
+template <class T>
+__device__ __forceinline__ bool cheb_pass_resident(const CGArgs& a, int k, unsigned seq, bool last,
+                                                   float4 (*sd)[T::HALO], Resident<T>& t,
+                                                   double& rr_p) {
+    typedef Resident<T> RT;
+    if ((int)blockIdx.x >= a.ntiles) return true;
+    const float4* dk = (k & 1) ? a.q : a.p;
+    float4* dn = (k & 1) ? a.p : a.q;
+    float4* sb = sd[k & 1];
+    int ok = 1;
+#pragma unroll
+    for (int v = 0; v < T::VPT; ++v) {
+        int lx, ly, lz;
+        T::local(threadIdx.x + v * T::NTH, lx, ly, lz);
+        sb[T::hidx(lx, ly, lz)] = t.m[v] >= 0 ? t.d[v] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    float4 h[RT::HPT];
+    if (k == 0) {
+#pragma unroll
+        for (int i = 0; i < RT::HPT; ++i)
+            if (t.hm[i] >= 0) {
+                h[i] = __ldcg(a.r + t.hm[i]);
+                h[i].x *= a.inv_theta; h[i].y *= a.inv_theta; h[i].z *= a.inv_theta;
+            }
+    } else {
+#pragma unroll
+        for (int i = 0; i < RT::HPT; ++i)
+            if (t.hm[i] >= 0) h[i] = ld_word(dk + t.hm[i]);
+#pragma unroll
+        for (int i = 0; i < RT::HPT; ++i) {
+            if (t.hm[i] < 0 || __float_as_uint(h[i].w) == seq) continue;
+            const long long t0 = clock64();
+            for (int spin = 1;; ++spin) {
+                h[i] = ld_word(dk + t.hm[i]);
+                if (__float_as_uint(h[i].w) == seq) break;
+                if ((spin & 255) != 0) continue;
+                if (ld_acquire_gpu(a.bar + 2) != 0u) { ok = 0; break; }
+                if (clock64() - t0 > a.bar_budget) { wait_failed(a); ok = 0; break; }
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < RT::HPT; ++i)
+        if (t.hm[i] >= 0) sb[t.hs[i]] = h[i];
+    if (!__syncthreads_and(ok)) return false;
+#pragma unroll
+    for (int v = 0; v < T::VPT; ++v) {
+        if (t.m[v] < 0) continue;
+        int lx, ly, lz;
+        T::local(threadIdx.x + v * T::NTH, lx, ly, lz);
+        float4 c;
+        float o0, o1, o2;
+        apply32<T>(sb, T::hidx(lx, ly, lz), t.dg[v], c, o0, o1, o2);
+        float4 &e = t.e[v], &r = t.r[v];
+        e.x += c.x; e.y += c.y; e.z += c.z;
+        r.x -= o0; r.y -= o1; r.z -= o2;
+        if (last) {
+            rr_p += (double)r.x * r.x + (double)r.y * r.y + (double)r.z * r.z;
+        } else {
+            const float c1 = a.c1[k], c2 = a.c2[k];
+            t.d[v] = make_float4(c1 * c.x + c2 * r.x, c1 * c.y + c2 * r.y, c1 * c.z + c2 * r.z,
+                                 __uint_as_float(seq + 1u));
+            st_word(dn + t.m[v], t.d[v]);
+        }
+    }
+    return true;
+}
+
+// Double-float residual pass on the tiles (FP32-history): q holds x (its high part with
+// PAIR, the low part in xl), zero on inactive voxels.  Writes r scaled by sc and (not RES)
+// the first Chebyshev direction d_0 = r / theta on active voxels and adds |r|^2 (unscaled) and, on
+// the first pass, |b|^2 to the thread's partial sums.
+template <class T, bool PAIR, bool RES>
+__device__ __forceinline__ void residual_df_tiled(const CGArgs& a, float4 (*sd)[T::HALO], float sc,
+                                                  double& rr_p, double& bb_p, bool first) {
+    const long long M = a.M;
+    for (int tile = blockIdx.x; tile < a.ntiles; tile += a.nw) {
+        const int org = a.tiles[tile];
+        load_halo<T>(a, a.q, sd[0], org);
+        if (PAIR) load_halo<T>(a, a.xl, sd[1], org);
+        cp_async_commit();
+        long long mv[T::VPT];
+        float dhv[T::VPT], dlv[T::VPT], bh[T::VPT][3], bl[T::VPT][3];
+#pragma unroll
+        for (int v = 0; v < T::VPT; ++v) {
+            const long long m = tile_voxel<T>(a, org, v);
             mv[v] = -1;
-            if (x < a.U && y < a.V && z < a.W) {
-                const long long m = (long long)z * UV + (long long)y * a.U + x;
-                dhv[v] = a.diag32[m];
-                if (dhv[v] != 0.f) {
-                    mv[v] = m;
-                    dlv[v] = a.diag_lo[m];
-                    bhv[v] = a.bh[m];
-                    blv[v] = a.bl[m];
-                    if (first) {
-                        const double b0 = a.b[m], b1 = a.b[M + m], b2 = a.b[2 * M + m];
-                        bb_p += b0 * b0 + b1 * b1 + b2 * b2;
-                    }
+            dhv[v] = m >= 0 ? a.diag32[m] : 0.f;
+            if (dhv[v] != 0.f) {
+                mv[v] = m;
+                dlv[v] = a.diag_lo[m];
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    bh[v][k] = a.xb[k * M + m].y;
+                    bl[v][k] = a.bl[k * M + m];
                 }
             }
         }
         cp_async_wait0();
         __syncthreads();
 #pragma unroll
-        for (int v = 0; v < kVoxPerThread; ++v) {
+        for (int v = 0; v < T::VPT; ++v) {
             if (mv[v] < 0) continue;
-            const int q = threadIdx.x + v * NT;
-            const int hc = ((q / (TT * TT) + 1) * TH + ((q / TT) % TT + 1)) * TH + (q % TT + 1);
-            auto load = [&](auto e, float* sh, float* sl) {
-                constexpr int E = decltype(e)::value;
-                constexpr int off = ((E / 9 - 1) * TH + ((E / 3) % 3 - 1)) * TH + (E % 3 - 1);
-                const float4 vh = sd[0][hc + off], vl = sd[1][hc + off];
-                df_add(sh[0], sl[0], vh.x, vl.x);
-                df_add(sh[1], sl[1], vh.y, vl.y);
-                df_add(sh[2], sl[2], vh.z, vl.z);
+            int lx, ly, lz;
+            T::local(threadIdx.x + v * T::NTH, lx, ly, lz);
+            const int hc = T::hidx(lx, ly, lz);
+            auto load = [&](auto e, float4& vh, float4& vl) {
+                constexpr int o = T::template off<decltype(e)::value>();
+                vh = sd[0][hc + o];
+                if constexpr (PAIR) vl = sd[1][hc + o];
             };
-            const float4 r = residual_df_at<true>(sd[0][hc], sd[1][hc], dhv[v], dlv[v], bhv[v],
-                                                  blv[v], load, 0);
+            float4 r = residual_df_at<PAIR>(dhv[v], dlv[v], bh[v], bl[v], load);
             rr_p += (double)r.x * r.x + (double)r.y * r.y + (double)r.z * r.z;
+            if (first)
+                bb_p += (double)bh[v][0] * bh[v][0] + (double)bh[v][1] * bh[v][1] +
+                        (double)bh[v][2] * bh[v][2];
+            r = make_float4(r.x * sc, r.y * sc, r.z * sc, 0.f);
             a.r[mv[v]] = r;
-            a.p[mv[v]] = make_float4(r.x * a.inv_theta, r.y * a.inv_theta, r.z * a.inv_theta, 0.f);
+            if (!RES)
+                a.p[mv[v]] = make_float4(r.x * a.inv_theta, r.y * a.inv_theta, r.z * a.inv_theta, 0.f);
         }
         __syncthreads();
     }
 }
 
 // block-wide sum of two values; result valid in every thread
+template <int NTH>
 __device__ __forceinline__ void block_sum2(double& a, double& b) {
-    __shared__ double sh[2][NT / 32];
+    __shared__ double sh[2][NTH / 32];
     for (int o = 16; o > 0; o >>= 1) {
         a += __shfl_down_sync(0xffffffffu, a, o);
         b += __shfl_down_sync(0xffffffffu, b, o);
@@ -494,18 +876,14 @@ __device__ __forceinline__ void block_sum2(double& a, double& b) {
     __syncthreads();
     if (lane == 0) { sh[0][wid] = a; sh[1][wid] = b; }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double s0 = 0.0, s1 = 0.0;
-        for (int k = 0; k < NT / 32; ++k) { s0 += sh[0][k]; s1 += sh[1][k]; }
-        sh[0][0] = s0;
-        sh[1][0] = s1;
-    }
-    __syncthreads();
-    a = sh[0][0];
-    b = sh[1][0];
+    double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+    for (int k = 0; k < NTH / 32; ++k) { s0 += sh[0][k]; s1 += sh[1][k]; }
+    a = s0;
+    b = s1;
 }
 
-// sum of the per-block partials, computed by warp 0 (fixed order: identical in every
+// sum of nb per-block partials, computed by warp 0 (fixed order: identical in every
 // block) and broadcast through shared memory
 __device__ __forceinline__ double grid_total(const double* red, int nb) {
     __shared__ double s_tot;
@@ -530,52 +908,39 @@ __device__ __forceinline__ double grid_total(const double* red, int nb) {
 }
 
 // Grid-wide barrier of a cooperative launch (every block resident) with a bounded wait.
-// After a block-level barrier, thread 0 of each block publishes the block's writes
-// (fence), arrives on a counter and, unless it is the last to arrive, waits for the
-// generation word to change; the last block resets the counter and advances the
-// generation.  A wait longer than `budget` SM clock cycles (a block that never
-// arrives) sets the abort word and the timeout flag (4) in status[1] with the step in
-// status[2]; blocks that see the abort word leave at once.  Returns false when the
-// caller must return: the kernel ends without touching the solution any further.
-__device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
-    unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_release_gpu(unsigned* p, unsigned v) {
-    asm volatile("st.release.gpu.global.u32 [%0], %1;\n" ::"l"(p), "r"(v) : "memory");
-}
-__device__ bool grid_barrier(unsigned* bar, long long budget, int* status, int step) {
-    __shared__ int s_ok;
+// Each block's thread 0 publishes the block's writes, arrives on a counter that only
+// grows, and waits until the arrivals of this barrier are complete (n per barrier): one
+// round trip to the counter after the last arrival.  The words are zero at launch: the
+// last block to finish a kernel resets the counter (barrier_done).  A wait longer than
+// `budget` SM clock cycles (a block that never arrives) sets the abort word and the
+// timeout flag (4) in status[1] with the step in status[2]; blocks that see the abort word
+// leave at once.  Returns false when the caller must return: the kernel ends without
+// touching the solution any further.
+__device__ bool grid_barrier(unsigned* bar, unsigned n, unsigned& target, long long budget,
+                             int* status, int step) {
+    int ok = 1;
+    target += n;
     __syncthreads();
     if (threadIdx.x == 0) {
-        int ok = ld_acquire_gpu(bar + 2) == 0;
-        if (ok) {
-            const unsigned gen = ld_acquire_gpu(bar + 1);
-            __threadfence();
-            if (atomicAdd(bar, 1u) == gridDim.x - 1) {
-                bar[0] = 0u;
-                st_release_gpu(bar + 1, gen + 1u);
-            } else {
-                const long long t0 = clock64();
-                while (ld_acquire_gpu(bar + 1) == gen) {
-                    if (ld_acquire_gpu(bar + 2) != 0u) { ok = 0; break; }
-                    if (clock64() - t0 > budget) {
-                        atomicExch(bar + 2, 1u);
-                        atomicOr(status + 1, 4);
-                        atomicCAS(status + 2, 0, step);
-                        ok = 0;
-                        break;
-                    }
-                    __nanosleep(32);
+        __threadfence();
+        atomicAdd(bar, 1u);
+        if ((int)(ld_acquire_gpu(bar) - target) < 0) {
+            const long long t0 = clock64();
+            for (int spin = 1; (int)(ld_acquire_gpu(bar) - target) < 0; ++spin) {
+                if ((spin & 63) != 0) continue;
+                if (ld_acquire_gpu(bar + 2) != 0u) { ok = 0; break; }
+                if (clock64() - t0 > budget) {
+                    atomicExch(bar + 2, 1u);
+                    atomicOr(status + 1, 4);
+                    atomicCAS(status + 2, 0, step);
+                    ok = 0;
+                    break;
                 }
             }
-            __threadfence();
         }
-        s_ok = ok;
+        __threadfence();
     }
-    __syncthreads();
-    return s_ok != 0;
+    return __syncthreads_and(ok) != 0;
 }
 
 // for i = t0, t0 + gs, ... < n: U indices per round, ld(i) for all of them before
@@ -596,239 +961,369 @@ __device__ __forceinline__ void grid_loop(long long t0, long long n, long long g
 
 // Check of the barrier's bounded wait: every block passes `rounds` barriers, except the
 // block `absent` (>= 0), which returns at once; the others' wait then runs out.
-// w[1] flags, w[2] the round of a timeout, w[4..6] the barrier, w[7] blocks that
+// w[1] flags, w[2] the round of a timeout, w[4..7] the barrier, w[8] blocks that
 // passed every round.
 __global__ void __launch_bounds__(NT) k_barrier_check(int* w, long long budget, int rounds,
                                                       int absent) {
     if ((int)blockIdx.x == absent) return;
+    unsigned target = 0;
     for (int r = 1; r <= rounds; ++r)
-        if (!grid_barrier(reinterpret_cast<unsigned*>(w + 4), budget, w, r)) return;
-    if (threadIdx.x == 0) atomicAdd(w + 7, 1);
+        if (!grid_barrier(reinterpret_cast<unsigned*>(w + 4), gridDim.x, target, budget, w, r))
+            return;
+    if (threadIdx.x == 0) atomicAdd(w + 8, 1);
 }
 
-// Mixed-precision iterative refinement: FP64 residual r = b - A x, FP32 conjugate
-// gradients for A e = r / ||r|| to a relative ~1e-5, x += ||r|| e; repeat until the
-// FP64 residual meets tol ||b||.  All blocks take identical decisions because every
-// block sums the same per-block partials in the same order.  DF: the residual is
-// evaluated in double-float arithmetic on float-pair copies of x and b (FP32-history
-// mode); x is split at entry, corrected in pairs and merged back to FP64 at exit.
-template <bool DF>
-__global__ void __launch_bounds__(NT, 3) k_cg(const __grid_constant__ CGArgs a) {
-    auto gsync = [&] { return grid_barrier(a.bar, a.bar_budget, a.status, a.step); };
-    __shared__ float4 sd[2][TH * TH * TH];        // tile halos of the tiled passes
+// The least-squares fit of b_n by b_{n-1} .. b_{n-nv} (one block): sums the epilogue's
+// partial dot products in a fixed order, updates the Gram matrix of the ring and solves
+// the normal equations by a Cholesky factorisation in ring order, newest first (a vector
+// whose remainder after the newer ones is below kFitPivot of its square is left out).
+// The matrix is scaled to unit diagonal.  Lane i of warp 0 holds row i.
+__device__ void fit_block(const CGArgs& a) {
+    __shared__ double t[kSums];
+    const int lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
+    for (int q = threadIdx.x >> 5; q < kSums - 1; q += nwarp) {
+        const double* p = a.part + (long long)q * a.nepi;
+        double v = 0.0;
+        for (int k = lane; k < a.nepi; k += 32) v += p[k];
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if (lane == 0) t[q] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    double* gram = a.fit->gram;
+    const int s0 = a.bs, si = fslot(s0, min(lane, kFit - 1) + 1);
+    const bool row = lane < kFit && lane < a.nv;
+    double A[kFit], L[kFit], rs[kFit];
+    const double bb = t[0];
+    const double dii = row ? gram[si * kSlots + si] : 0.0;
+    const double s = row && dii > 0.0 && dii < 1e300 ? rsqrt(dii) : 0.0;
+#pragma unroll
+    for (int j = 0; j < kFit; ++j) {
+        A[j] = row && j < a.nv ? gram[si * kSlots + fslot(s0, j + 1)] : 0.0;
+        A[j] *= s * __shfl_sync(0xffffffffu, s, j);
+    }
+    double g = row ? t[1 + lane] * s : 0.0, y = 0.0, yy = 0.0;
+#pragma unroll
+    for (int j = 0; j < kFit; ++j) {
+        const double v = __shfl_sync(0xffffffffu, A[j], j);
+        rs[j] = v > kFitPivot ? rsqrt(v) : 0.0;
+        L[j] = lane >= j ? A[j] * rs[j] : 0.0;
+#pragma unroll
+        for (int k = j + 1; k < kFit; ++k) A[k] -= L[j] * __shfl_sync(0xffffffffu, L[j], k);
+        const double yj = __shfl_sync(0xffffffffu, g, j) * rs[j];
+        if (lane == j) y = yj;
+        g -= L[j] * yj;
+        yy += yj * yj;
+    }
+    double c = 0.0;
+#pragma unroll
+    for (int j = kFit - 1; j >= 0; --j) {
+        const double cj = __shfl_sync(0xffffffffu, y, j) * rs[j];
+        if (lane == j) c = cj * s;
+#pragma unroll
+        for (int k = 0; k < j; ++k) {
+            const double ljk = __shfl_sync(0xffffffffu, L[k], j);
+            if (lane == k) y -= ljk * cj;
+        }
+    }
+    double mag = fabs(c);
+    for (int o = 4; o > 0; o >>= 1) mag = fmax(mag, __shfl_xor_sync(0xffffffffu, mag, o));
+    FitRecord& rec = a.fit->rec[(a.step + 1) & 1];
+    if (lane < kFit) rec.c[lane] = c;
+    if (lane == 0) {
+        // a poor or degenerate fit (also NaN anywhere in it) falls back to extrapolation
+        rec.use = a.nv >= 3 && bb > 0.0 && bb - yy <= kFitPoor * bb && mag < 1e4;
+        int e = 0;
+        if (bb > 0.0 && bb < 1e300) frexp(sqrt(bb / (3.0 * (double)a.nact)), &e);
+        rec.scale = ldexp(1.0, max(-120, min(120, -e)));
+        gram[s0 * kSlots + s0] = bb;
+    }
+    if (row) {
+        gram[s0 * kSlots + si] = t[1 + lane];
+        gram[si * kSlots + s0] = t[1 + lane];
+    }
+}
+
+// r = b - A x in FP64 at the active voxels, scaled by sc and rounded to FP32, with (not RES)
+// d_0 = r / theta; adds |r|^2 (and |b|^2 on the first pass) to the thread's sums.
+// Where there are fewer active voxels than lanes on the GPU (SPLIT), a warp takes one
+// component of its 32 voxels: the pass is bound by the FP64 chain of a voxel, and three
+// warps on three sub-partitions run a third of it each.  Warps are dealt to the blocks in
+// turn, so that few voxels spread over many SMs.
+template <int C>
+__device__ __forceinline__ double applyA64_row(const CGArgs& a, const double* __restrict__ x, int m,
+                                               int mask) {
     const long long M = a.M;
-    const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long gs = (long long)gridDim.x * blockDim.x;
-    const int nb = gridDim.x;
+    constexpr int C1 = C == 0 ? 1 : 0, C2 = C == 2 ? 1 : 2;      // the other two components
+    constexpr int K1 = C == 2 ? 4 : 3;                           // coupling (C, C1)
+    constexpr int K2 = C == 0 ? 4 : 5;                           // coupling (C, C2)
+    double o = (a.diag[m] - c_stencil[13 * 6 + C]) * x[C * M + m];
+    double o1 = 0.0;
+    Unroll13::run([&](auto ec) {
+        constexpr int E = decltype(ec)::value;
+        constexpr int d[3] = {E % 3 - 1, (E / 3) % 3 - 1, E / 9 - 1};
+        const bool inp = mask & (1 << E), inm = mask & (1 << (26 - E));
+        const long long mp = m + a.noff[E], mm = m + a.noff[26 - E];
+        o -= c_stencil[E * 6 + C] * ((inp ? x[C * M + mp] : 0.0) + (inm ? x[C * M + mm] : 0.0));
+        if constexpr (d[C] != 0 && d[C1] != 0)
+            o1 -= c_stencil[E * 6 + K1] * ((inp ? x[C1 * M + mp] : 0.0) + (inm ? x[C1 * M + mm] : 0.0));
+        if constexpr (d[C] != 0 && d[C2] != 0)
+            o1 -= c_stencil[E * 6 + K2] * ((inp ? x[C2 * M + mp] : 0.0) + (inm ? x[C2 * M + mm] : 0.0));
+    });
+    return o + o1;
+}
+
+template <bool SPLIT, bool RES>
+__device__ __forceinline__ void residual64(const CGArgs& a, double sc, double& rr_p, double& bb_p,
+                                           bool first) {
+    const long long M = a.M;
+    const int lane = threadIdx.x & 31;
+    const long long warp = (long long)(threadIdx.x >> 5) * a.nw + blockIdx.x;
+    const long long warps = (long long)(blockDim.x >> 5) * a.nw;
+    if constexpr (SPLIT) {
+        const long long groups = (a.nact + 31) / 32;
+        float* rf = reinterpret_cast<float*>(a.r);
+        float* pf = reinterpret_cast<float*>(a.p);
+        for (long long w = warp; w < 3 * groups; w += warps) {
+            const int c = (int)(w / groups);
+            const long long i = (w % groups) * 32 + lane;
+            if (i >= a.nact) continue;
+            const int m = a.act[i], mask = a.nmask[i];
+            double o;
+            if (c == 0) o = applyA64_row<0>(a, a.x, m, mask);
+            else if (c == 1) o = applyA64_row<1>(a, a.x, m, mask);
+            else o = applyA64_row<2>(a, a.x, m, mask);
+            const double b = a.b[c * M + m], r = b - o;
+            if (first) bb_p += b * b;
+            rr_p += r * r;
+            const float rs = (float)(r * sc);
+            rf[4LL * m + c] = rs;
+            if (!RES) pf[4LL * m + c] = rs * a.inv_theta;
+        }
+    } else {
+        for (long long i = warp * 32 + lane; i < a.nact; i += warps * 32) {
+            const int m = a.act[i];
+            double o[3], r[3];
+            applyA64(a, a.x, m, a.nmask[i], o);
+            float4 rs = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const double b = a.b[k * M + m];
+                r[k] = b - o[k];
+                if (first) bb_p += b * b;
+                rr_p += r[k] * r[k];
+            }
+            rs.x = (float)(r[0] * sc);
+            rs.y = (float)(r[1] * sc);
+            rs.z = (float)(r[2] * sc);
+            a.r[m] = rs;
+            if (!RES)
+                a.p[m] = make_float4(rs.x * a.inv_theta, rs.y * a.inv_theta, rs.z * a.inv_theta, 0.f);
+        }
+    }
+}
+
+// Mixed-precision iterative refinement from x0: residual r = b - A x (FP64, or
+// double-float in FP32-history mode, DF), FP32 Chebyshev iterations for A e = r, x += e.
+// One fused pass and one grid barrier per iteration (apply to d_k, update e, r, d_{k+1}; d
+// is double-buffered because neighbours read d_k during the pass).  The iteration's own
+// residual (r is carried, r -= A d_k in FP32) differs from that of x + e by a few FP32
+// roundings of the *start* residual, so once it is below the tolerance with kDrift of the
+// start residual added, the step is done without forming b - A x again; otherwise the next
+// refinement starts from a new true residual.  All blocks take identical decisions because
+// every block sums the same per-block partials in the same order.
+//   RES: a block has at most one tile (see Resident; no grid barrier in the iteration).
+//   SPLIT: FP64 residual by components (see residual64).
+constexpr double kDrift = 1e-6;
+
+template <bool DF, class T, bool RES, bool SPLIT>
+__global__ void __launch_bounds__(T::NTH, RES ? 4 : 3) k_cg(const __grid_constant__ CGArgs a) {
+    __shared__ __align__(16) float4 sd[2][T::HALO];      // tile halos of the passes
+    if ((int)blockIdx.x == a.nw) {       // the fit for the next step, beside the solve
+        fit_block(a);
+        return;
+    }
+    unsigned target = 0, seq = a.seq;
+    auto gsync = [&] {
+        return grid_barrier(a.bar, a.nw, target, a.bar_budget, a.status, a.step);
+    };
+    const long long M = a.M;
+    const long long t0 = (long long)blockIdx.x * T::NTH + threadIdx.x;
+    const long long gs = (long long)a.nw * T::NTH;
+    const int nb = a.nw;
     double* red0 = a.red;
     double* red1 = a.red + nb;
-    double bb = 0.0, rr = 0.0;
+    double* red2 = a.red + 2 * nb;
+    Resident<T> res;
+    if constexpr (RES) resident_init<T>(a, res, sd);
+    double bb = 0.0, rr = 0.0, xx = 0.0;
     int its = 0, outer = 0;
-    bool first = true, converged = false, zeroed = false, nonfinite = false;
-    // grid-stride loops over the active voxels (or all voxels) take four indices per
-    // thread per round and issue all their loads before the first store, so that a
-    // thread has several independent memory requests in flight
-    struct XB { int m; double x0, x1, x2, b0, b1, b2; };
-    struct RF { int m; float4 r; };
-    struct RD { int m; double r0, r1, r2; };
-    struct EHL { int m; float4 e, h, l; };
-    struct EX3 { int m; float4 e; double x0, x1, x2; };
-    struct X3 { bool pair; double x0, x1, x2; };
-    if (DF) {
-        grid_loop<1>(t0, a.nact, gs,
-            [&](long long i) {
-                XB v;
-                v.m = a.act[i];
-                v.x0 = a.x[v.m]; v.x1 = a.x[M + v.m]; v.x2 = a.x[2 * M + v.m];
-                v.b0 = a.b[v.m]; v.b1 = a.b[M + v.m]; v.b2 = a.b[2 * M + v.m];
-                return v;
-            },
-            [&](long long, const XB& v) {
-                float4 h, l;
-                df_split(v.x0, h.x, l.x);
-                df_split(v.x1, h.y, l.y);
-                df_split(v.x2, h.z, l.z);
-                h.w = l.w = 0.f;
-                a.xh[v.m] = h;
-                a.xl[v.m] = l;
-                df_split(v.b0, h.x, l.x);
-                df_split(v.b1, h.y, l.y);
-                df_split(v.b2, h.z, l.z);
-                a.bh[v.m] = h;
-                a.bl[v.m] = l;
-            });
-        if (!gsync()) return;
-    }
-    while (true) {
-        // ---- residual (FP64, or double-float rounded to FP32 with d_0 = r / theta)
-        double rr_p = 0.0, bb_p = 0.0;
-        if (DF) residual_df_tiled(a, sd, rr_p, bb_p, first);
-        for (long long i = t0; !DF && i < a.nact; i += gs) {
-            const int m = a.act[i];
-            if (first) {
-                const double b0 = a.b[m], b1 = a.b[M + m], b2 = a.b[2 * M + m];
-                bb_p += b0 * b0 + b1 * b1 + b2 * b2;
-            }
-            {
-                double o[3];
-                applyA64(a, a.x, m, a.nmask[i], o);
-                const double r0 = a.b[m] - o[0], r1 = a.b[M + m] - o[1], r2 = a.b[2 * M + m] - o[2];
-                rr_p += r0 * r0 + r1 * r1 + r2 * r2;
-                a.r64[m] = r0;
-                a.r64[M + m] = r1;
-                a.r64[2 * M + m] = r2;
-            }
+    bool first = true, converged = false, nonfinite = false, zero = false;
+    bool stored = false;     // x (with its norm in xx) is in a.x; else DF's start is in xb only
+    double sc = a.fit->rec[a.step & 1].scale;
+    if (sc == 0.0) sc = 1.0;
+    // f(voxel, its correction e) over the block's share of the active voxels
+    auto each = [&](auto&& f) {
+        if constexpr (RES) {
+#pragma unroll
+            for (int v = 0; v < T::VPT; ++v)
+                if (res.m[v] >= 0) f(res.m[v], res.e[v]);
+        } else {
+            struct ME { int m; float4 e; };
+            grid_loop<4>(t0, a.nact, gs,
+                [&](long long i) {
+                    ME v;
+                    v.m = a.act[i];
+                    v.e = a.e[v.m];
+                    return v;
+                },
+                [&](long long, const ME& v) { f(v.m, v.e); });
         }
-        block_sum2(rr_p, bb_p);
-        if (threadIdx.x == 0) { red0[blockIdx.x] = rr_p; red1[blockIdx.x] = bb_p; }
+    };
+    while (true) {
+        // ---- residual, scaled by sc
+        double rr_p = 0.0, bb_p = 0.0;
+        if constexpr (DF) {
+            if (stored) residual_df_tiled<T, true, RES>(a, sd, (float)sc, rr_p, bb_p, first);
+            else residual_df_tiled<T, false, RES>(a, sd, (float)sc, rr_p, bb_p, first);
+        } else {
+            residual64<SPLIT, RES>(a, sc, rr_p, bb_p, first);
+        }
+        block_sum2<T::NTH>(rr_p, bb_p);
+        if (threadIdx.x == 0) {
+            red0[blockIdx.x] = rr_p;
+            if (first) red1[blockIdx.x] = bb_p;
+        }
         if (!gsync()) return;
         rr = grid_total(red0, nb);
         if (first) bb = grid_total(red1, nb);
-        first = false;
-        // red0 / red1 are written next after at least one more barrier (the next
-        // residual follows the Chebyshev passes; the final norm follows the merge or
-        // its own barrier), so no barrier is needed here for their readers
-        if (!(rr <= 1e300) || !(bb <= 1e300)) {
-            // NaN or Inf in the right-hand side (or the start): no iteration can help;
-            // J_n is returned as NaN so that the monitor and the caller see it
-            const double qnan = __longlong_as_double(0x7ff8000000000000LL);
-            for (long long i = t0; i < a.nact; i += gs) {
-                const int m = a.act[i];
-                a.x[m] = qnan; a.x[M + m] = qnan; a.x[2 * M + m] = qnan;
-            }
-            nonfinite = true;
-            break;
-        }
-        if (bb == 0.0) {
-            for (long long i = t0; i < a.nact; i += gs) {
-                const int m = a.act[i];
-                a.x[m] = 0.0; a.x[M + m] = 0.0; a.x[2 * M + m] = 0.0;
-            }
-            rr = 0.0;
-            converged = zeroed = true;
-            break;
-        }
+        if (!(rr <= 1e300) || !(bb <= 1e300)) { nonfinite = true; break; }
+        if (bb == 0.0) { zero = converged = true; break; }
         if (rr <= a.tol2 * bb) { converged = true; break; }
-        if (outer >= a.max_outer || its >= a.max_iter) break;
-        // ---- FP32 Chebyshev iteration for A e = r (r holds the FP32 residual).
-        // One fused pass per iteration (apply to d_k, update e, r, d_{k+1}) and one grid
-        // barrier; d is double-buffered because neighbours read d_k during the pass.
-        // iterations for the reduction still needed (with a factor 10 of margin), never
-        // asking for more than FP32 can deliver in one refinement (5e-6)
-        const double need = fmax(0.1 * sqrt(a.tol2 * bb / rr), 5e-6);
-        const int n_it = min(a.n_cheb, max(3, (int)ceil(log(0.5 * need) / a.log_rate)));
-        // The double-float residual is already an FP32 vector with d_0 beside it; it is
-        // iterated as it is unless its norm is far from 1 (FP32 range).  Otherwise (and
-        // always for the FP64 residual) r is first scaled to unit norm in FP64, so that
-        // a tiny residual cannot underflow in FP32, and e is scaled back by ||r||.
-        const bool scaled = !DF || !(rr >= 1e-40 && rr <= 1e40);
-        const double sc = scaled ? 1.0 / sqrt(rr) : 1.0;
-        if (scaled) {
-            const float sc32 = (float)sc;
-            if constexpr (DF) {
-                grid_loop<4>(t0, a.nact, gs,
-                    [&](long long i) { const int m = a.act[i]; return RF{m, a.r[m]}; },
-                    [&](long long, const RF& v) {
-                        const float4 rv = make_float4(v.r.x * sc32, v.r.y * sc32, v.r.z * sc32, 0.f);
-                        a.r[v.m] = rv;
-                        a.p[v.m] = make_float4(rv.x * a.inv_theta, rv.y * a.inv_theta,
-                                               rv.z * a.inv_theta, 0.f);
-                    });
-            } else {
-                grid_loop<4>(t0, a.nact, gs,
-                    [&](long long i) {
-                        const int m = a.act[i];
-                        return RD{m, a.r64[m], a.r64[M + m], a.r64[2 * M + m]};
-                    },
-                    [&](long long, const RD& v) {
-                        const float4 rv = make_float4((float)(v.r0 * sc), (float)(v.r1 * sc),
-                                                      (float)(v.r2 * sc), 0.f);
-                        a.r[v.m] = rv;
-                        a.p[v.m] = make_float4(rv.x * a.inv_theta, rv.y * a.inv_theta,
-                                               rv.z * a.inv_theta, 0.f);
-                    });
-            }
+        if (first && rr > bb) {
+            // a start worse than none (an abrupt change of the excitation): from zero
+            each([&](long long m, const float4&) {
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    if (DF) a.xb[k * M + m].x = 0.f;
+                    else a.x[k * M + m] = 0.0;
+                }
+                if (DF) a.q[m] = make_float4(0.f, 0.f, 0.f, 0.f);
+            });
+            first = false;
             if (!gsync()) return;
+            continue;
         }
-        float4* dk = a.p;
-        float4* dn = a.q;
-        for (int k = 0; k < n_it; ++k) {
-            cheb_pass_tiled(a, dk, dn, a.c1[k], a.c2[k], k == 0, sd);
-            if (!gsync()) return;
-            float4* t = dk; dk = dn; dn = t;
+        first = false;
+        if (outer >= a.max_outer || its >= a.max_iter) break;
+        if (!(rr * sc * sc >= 1e-24 && rr * sc * sc <= 1e24)) {
+            // the scale of the previous step does not bring this residual into FP32's range
+            sc = 1.0 / sqrt(rr);
+            if (!gsync()) return;        // every block has read the partial sums
+            continue;
+        }
+        // ---- Chebyshev: iterations for the reduction still needed, never asking for more
+        // than FP32 can deliver in one refinement (5e-6).  FP64 aims a factor 10 below the
+        // tolerance (the march's error is then the history's rounding, 1e-14 on the 8^3
+        // cube, not the solve's 2e-13); the FP32 history's own error is far above its
+        // tolerance already
+        const double back = 1.0 / sc, goal = sqrt(a.tol2 * bb), have = sqrt(rr);
+        const double need = fmax((DF ? 0.8 : 0.1) * (goal - kDrift * have) / have, 5e-6);
+        const int n_it = min(a.n_cheb, max(2, (int)ceil(log(0.5 * need) / a.log_rate)));
+        rr_p = 0.0;
+        if constexpr (RES) {
+#pragma unroll
+            for (int v = 0; v < T::VPT; ++v) {
+                res.e[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (res.m[v] < 0) continue;
+                const float4 r = __ldcg(a.r + res.m[v]);
+                res.r[v] = r;
+                res.d[v] = make_float4(r.x * a.inv_theta, r.y * a.inv_theta, r.z * a.inv_theta, 0.f);
+            }
+            for (int k = 0; k < n_it; ++k)
+                if (!cheb_pass_resident<T>(a, k, seq + k, k == n_it - 1, sd, res, rr_p)) return;
+            seq += n_it;
+        } else {
+            float4* dk = a.p;
+            float4* dn = a.q;
+            for (int k = 0; k < n_it; ++k) {
+                cheb_pass_tiled<T>(a, dk, dn, a.c1[k], a.c2[k], k == 0, k == n_it - 1, sd, rr_p);
+                if (!gsync()) return;
+                float4* tmp = dk; dk = dn; dn = tmp;
+            }
         }
         its += n_it;
-        // ---- correction x += (1 / sc) e (FP64, or in float pairs)
-        const double back = 1.0 / sc;
-        float bkh, bkl;
-        df_split(back, bkh, bkl);
-        if constexpr (DF) {
-            grid_loop<1>(t0, a.nact, gs,
-                [&](long long i) {
-                    const int m = a.act[i];
-                    return EHL{m, a.e[m], a.xh[m], a.xl[m]};
-                },
-                [&](long long, const EHL& v) {
-                    const float ec[3] = {v.e.x, v.e.y, v.e.z};
-                    float hc[3] = {v.h.x, v.h.y, v.h.z}, lc[3] = {v.l.x, v.l.y, v.l.z};
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) {
-                        const float p = __fmul_rn(bkh, ec[c]);
-                        const float pe = __fmaf_rn(bkh, ec[c], -p) + __fmul_rn(bkl, ec[c]);
-                        df_add(hc[c], lc[c], p, pe);
-                    }
-                    a.xh[v.m] = make_float4(hc[0], hc[1], hc[2], 0.f);
-                    a.xl[v.m] = make_float4(lc[0], lc[1], lc[2], 0.f);
-                });
-        } else {
-            grid_loop<4>(t0, a.nact, gs,
-                [&](long long i) {
-                    const int m = a.act[i];
-                    return EX3{m, a.e[m], a.x[m], a.x[M + m], a.x[2 * M + m]};
-                },
-                [&](long long, const EX3& v) {
-                    a.x[v.m] = v.x0 + back * (double)v.e.x;
-                    a.x[M + v.m] = v.x1 + back * (double)v.e.y;
-                    a.x[2 * M + v.m] = v.x2 + back * (double)v.e.z;
-                });
-        }
-        if (!gsync()) return;
         ++outer;
-    }
-    // norm of the solution (all voxels, active and not).  In the double-float mode the
-    // same pass merges x = hi + lo back to FP64 at the active voxels (their pairs were
-    // last written before the final residual's barrier; a voxel's x is read and
-    // written by its own thread only); elsewhere x is read as it is, and x written by
-    // other blocks without a barrier since (zeroed or non-finite start) needs one
-    const bool merge = DF && !zeroed && !nonfinite;
-    if ((zeroed || nonfinite) && !gsync()) return;
-    double xx = 0.0, dummy = 0.0;
-    grid_loop<4>(t0, M, gs,
-        [&](long long m) {
-            X3 v;
-            v.pair = merge && a.chi[m] > 0.0;
-            if (v.pair) {
-                const float4 h = a.xh[m], l = a.xl[m];
-                v.x0 = (double)h.x + (double)l.x;
-                v.x1 = (double)h.y + (double)l.y;
-                v.x2 = (double)h.z + (double)l.z;
-            } else {
-                v.x0 = a.x[m]; v.x1 = a.x[M + m]; v.x2 = a.x[2 * M + m];
+        // ---- x += e / sc (DF: the float start becomes an FP64 x) and its norm
+        xx = 0.0;
+        each([&](long long m, const float4& e) {
+            const float ec[3] = {e.x, e.y, e.z};
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                double x = DF && !stored ? (double)a.xb[k * M + m].x : a.x[k * M + m];
+                x += back * (double)ec[k];
+                a.x[k * M + m] = x;
+                if (DF) a.xb[k * M + m].x = (float)x;
+                xx += x * x;
             }
-            return v;
-        },
-        [&](long long m, const X3& v) {
-            if (v.pair) { a.x[m] = v.x0; a.x[M + m] = v.x1; a.x[2 * M + m] = v.x2; }
-            xx += v.x0 * v.x0 + v.x1 * v.x1 + v.x2 * v.x2;
         });
-    block_sum2(xx, dummy);
-    // the third partial-sum array: nothing in this launch has read it, so no barrier
-    // is needed before the write (red0 may still be read for the last residual norm)
-    double* red2 = a.red + 2 * nb;
-    if (threadIdx.x == 0) red2[blockIdx.x] = xx;
-    if (!gsync()) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        const double nx = grid_total(red2, nb);
+        stored = true;
+        block_sum2<T::NTH>(rr_p, xx);
+        if (threadIdx.x == 0) red1[blockIdx.x] = rr_p;
+        if (!gsync()) return;
+        const double left = sqrt(grid_total(red1, nb)) * back;
+        if (left + kDrift * have <= goal) { converged = true; break; }
+        if (!(left <= 1e300)) { nonfinite = true; break; }
+        // ---- not there yet: a new residual (DF: of x as float pairs)
+        sc = 1.0 / left;
+        if constexpr (DF) {
+            each([&](long long m, const float4&) {
+                float4 h, l;
+                df_split(a.x[m], h.x, l.x);
+                df_split(a.x[M + m], h.y, l.y);
+                df_split(a.x[2 * M + m], h.z, l.z);
+                h.w = l.w = 0.f;
+                a.q[m] = h;
+                a.xl[m] = l;
+            });
+            if (!gsync()) return;
+        }
+    }
+    // ---- an x not stored yet, and its norm.  NaN or Inf in the right-hand side or the
+    // start: no iteration can help; J_n is returned as NaN so that the monitor and the
+    // caller see it
+    if (!stored || nonfinite) {
+        double dummy = 0.0;
+        xx = 0.0;
+        each([&](long long m, const float4&) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                double x = DF && !stored ? (double)a.xb[k * M + m].x : a.x[k * M + m];
+                if (zero) x = 0.0;
+                if (nonfinite) x = __longlong_as_double(0x7ff8000000000000LL);
+                a.x[k * M + m] = x;
+                if (DF) a.xb[k * M + m].x = (float)x;
+                xx += x * x;
+            }
+        });
+        block_sum2<T::NTH>(xx, dummy);
+    }
+    // the last block to finish adds up the norm (fixed order) and leaves the barrier words
+    // zero for the next launch: every other block has passed its last barrier
+    __shared__ int s_last;
+    if (threadIdx.x == 0) {
+        red2[blockIdx.x] = xx;
+        __threadfence();
+        s_last = atomicAdd(a.bar + 3, 1u) == (unsigned)(nb - 1);
+        __threadfence();
+    }
+    __syncthreads();
+    if (!s_last) return;
+    const double nx = grid_total(red2, nb) +
+                      grid_total(a.part + (long long)(kSums - 1) * a.nepi, a.nepi);
+    if (threadIdx.x == 0) {
+        a.bar[0] = 0u;
+        a.bar[3] = 0u;
         *a.norm2 = nx;
         a.status[0] = its;
         int flag = 0;
@@ -862,31 +1357,8 @@ __global__ void k_from_aos(const double* __restrict__ in, long long M, double* _
 // In adjoint time tau = N + 1 - n the ring holds lambda.  With mu = chi lambda,
 //   Z_0^T lambda_n = g_n - sum_{l>=1} Z_l^T lambda_{n+l},
 //   Z_l^T lambda = (T(l)/eps + delta_l) lambda - G_l * (chi lambda)      (G_l^T = G_l),
-// and Z_0^T lambda = A mu with the same symmetric A as the forward solve.
-template <typename R>
-__global__ void k_epilogue_adj(long long M, const double* __restrict__ f,
-                               const double* __restrict__ g, const R* __restrict__ hist,
-                               double* __restrict__ Lring, int s0, int jring, Taps tp,
-                               double* __restrict__ b) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= 3 * M) return;
-    const long long m = i % M;
-    const int beta = (int)(i / M);
-    const long long st = 3 * M;
-    const double l1 = Lring[jslot(s0, 1, jring, st) + i];
-    const double l2 = Lring[jslot(s0, 2, jring, st) + i];
-    const double l3 = Lring[jslot(s0, 3, jring, st) + i];
-    double P = f[m] * l1 - (double)hist[i];
-    for (int l = 1; l < tp.n; ++l) P += tp.d[l] * Lring[jslot(s0, l, jring, st) + i];
-    const double rhs = g[m * 3 + beta] - P;
-    double* Ln = Lring + jslot(s0, 0, jring, st);
-    const double chi = f[3 * M + m];
-    b[i] = rhs;                                        // A mu = rhs on active voxels
-    // the solve's iterate must vanish off the active set; vacuum voxels get their
-    // lambda after the solve (k_adj_post), when mu is known
-    Ln[i] = chi > 0.0 ? chi * (3.0 * l1 - 3.0 * l2 + l3) : 0.0;
-}
-
+// and Z_0^T lambda = A mu with the same symmetric A as the forward solve (k_epilogue with
+// ADJ: b = rhs on active voxels, the start in terms of mu).
 // lambda = mu / chi on active voxels; on vacuum voxels (chi = 0) the row of Z_0^T reads
 // (T(0) + delta_0) lambda_m - (G_0 * mu)_m = rhs_m, so lambda_m = (rhs_m + (G_0 * mu)_m)
 // / (T(0) + delta_0).  Gradient accumulation on active voxels:
@@ -982,7 +1454,7 @@ __global__ void k_dot(const double* __restrict__ x, const double* __restrict__ y
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)
         s += x[i] * y[i];
-    block_sum2(s, d);
+    block_sum2<NT>(s, d);
     if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
@@ -1060,14 +1532,6 @@ void stencil_setup(mot_ctx* c) {
                 noff[(ez + 1) * 9 + (ey + 1) * 3 + (ex + 1)] = ex + c->U * (ey + c->V * ez);
     for (int e = 0; e < 27; ++e) c->noff[e] = noff[e];
     if (c->n_taps > MAXTAPS) throw MotError{MOT_ERR_ARG, "at most 64 FIR taps are supported"};
-    int per_sm = 0;
-    if (c->precision == MOT_FP64)
-        MOT_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cg<false>, NT, 0));
-    else
-        MOT_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cg<true>, NT, 0));
-    if (per_sm < 1) throw MotError{MOT_ERR_CUDA, "CG kernel cannot be made resident"};
-    const long long need = (c->M + NT - 1) / NT;
-    c->cg_blocks = (int)std::min<long long>((long long)per_sm * c->nsm, std::max<long long>(need, 1));
     int khz = 0;
     MOT_CUDA_TRY(cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, c->device));
     c->bar_budget = (long long)(kBarrierBudgetS * 1e3 * std::max(khz, 1000000));
@@ -1200,14 +1664,39 @@ void chebyshev_setup(mot_ctx* c) {
     }
 }
 
-template <typename R>
+namespace {
+
+int fit_slot(int n) { return n % kSlots; }
+
+// pairs (x, b) of the steps before the one being launched
+int fit_pairs(const mot_ctx* c) { return std::min(c->fit_steps, kFit); }
+
+template <typename R, bool ADJ>
 void epilogue(mot_ctx* c, int n, const double* En, cudaStream_t s) {
-    const long long tot = c->M;
-    k_epilogue<R><<<(int)((tot + NT - 1) / NT), NT, 0, s>>>(
-        c->M, c->vfac, En, hbuf<R>(c).hist_spatial, c->J, (int)slot_index(n, c->jring), c->jring,
-        taps_of(c), c->rhs);
+    EpiArgs a;
+    a.M = c->M;
+    a.f = c->vfac;
+    a.En = En;
+    a.hist = hbuf<R>(c).hist_spatial;
+    a.Jring = c->J;
+    a.s0 = (int)slot_index(n, c->jring);
+    a.jring = c->jring;
+    a.tp = taps_of(c);
+    a.n = n;
+    a.bs = fit_slot(n);
+    a.nv = fit_pairs(c);
+    a.b64 = c->b_ring;
+    a.xb = reinterpret_cast<float2*>(c->xb_ring);
+    a.bl = c->b_lo;
+    a.x0 = reinterpret_cast<float4*>(c->cg32) + 2 * c->M;
+    a.rhs = c->rhs;
+    a.fit = reinterpret_cast<const FitState*>(c->fit);
+    a.part = c->fit_part;
+    k_epilogue<R, ADJ><<<c->epi_blocks, c->epi_threads, 0, s>>>(a);
     MOT_LAUNCH_CHECK();
 }
+
+}  // namespace
 
 CGArgs make_cg_args(mot_ctx* c, int n, double* norm2_out) {
     CGArgs a;
@@ -1219,26 +1708,22 @@ CGArgs make_cg_args(mot_ctx* c, int n, double* norm2_out) {
     a.U = c->U; a.V = c->V; a.W = c->W;
     a.tiles = c->tiles;
     a.ntiles = c->ntiles;
+    a.halo = c->halo;
+    a.nw = c->cg_blocks;
     a.x = c->J + slot_index(n, c->jring) * 3 * c->M;
-    a.b = c->rhs;
+    a.bs = fit_slot(n);
+    a.nv = fit_pairs(c);
+    a.b = c->b_ring ? c->b_ring + (long long)a.bs * 3 * c->M : nullptr;
+    a.xb = c->xb_ring ? reinterpret_cast<float2*>(c->xb_ring) + (long long)a.bs * 3 * c->M : nullptr;
+    a.bl = c->b_lo;
     a.diag32 = c->diag32;
     a.diag = c->cg_diag;
-    a.chi = c->chi;
-    a.r64 = c->cg_r;
+    a.diag_lo = c->diag_lo;
     a.r = reinterpret_cast<float4*>(c->cg32);
     a.p = a.r + c->M;
     a.q = a.r + 2 * c->M;
     a.e = a.r + 3 * c->M;
-    a.xh = a.xl = a.bh = a.bl = nullptr;
-    a.diag_lo = nullptr;
-    if (c->cg_df) {
-        float4* d4 = reinterpret_cast<float4*>(c->cg_df);
-        a.xh = d4;
-        a.xl = d4 + c->M;
-        a.bh = d4 + 2 * c->M;
-        a.bl = d4 + 3 * c->M;
-        a.diag_lo = c->cg_df + 16 * c->M;
-    }
+    a.xl = c->cg_xl ? reinterpret_cast<float4*>(c->cg_xl) : nullptr;
     a.red = c->red;
     a.tol2 = c->tol * c->tol;
     a.inv_theta = c->cheb_inv_theta;
@@ -1255,18 +1740,90 @@ CGArgs make_cg_args(mot_ctx* c, int n, double* norm2_out) {
     a.bar = reinterpret_cast<unsigned*>(c->dstatus + 4);
     a.bar_budget = c->bar_budget;
     a.norm2 = norm2_out;
+    a.fit = reinterpret_cast<FitState*>(c->fit);
+    a.part = c->fit_part;
+    a.nepi = c->epi_blocks;
+    // every active voxel's words in p and q are rewritten by each launch, so numbers that
+    // only have to differ from those of the launch before may wrap
+    a.seq = ++c->solve_seq * 1024u;
     return a;
 }
 
+namespace {
+
+// kernel variant of a context's solve and its block size
+struct SolveKernel { void* fn; int threads; };
+SolveKernel solve_kernel(int precision, int tile, bool resident, bool split) {
+    const bool df = precision != MOT_FP64;
+    if (tile == 0) {
+        if (df) return {(void*)k_cg<true, BigTile, false, false>, BigTile::NTH};
+        return {(void*)k_cg<false, BigTile, false, false>, BigTile::NTH};
+    }
+    if (df) return {resident ? (void*)k_cg<true, SmallTile, true, false>
+                             : (void*)k_cg<true, SmallTile, false, false>, SmallTile::NTH};
+    if (split) return {resident ? (void*)k_cg<false, SmallTile, true, true>
+                                : (void*)k_cg<false, SmallTile, false, true>, SmallTile::NTH};
+    return {resident ? (void*)k_cg<false, SmallTile, true, false>
+                     : (void*)k_cg<false, SmallTile, false, false>, SmallTile::NTH};
+}
+
+}  // namespace
+
 void launch_cg(mot_ctx* c, void** args, cudaStream_t s) {
-    void* k = c->precision == MOT_FP64 ? (void*)k_cg<false> : (void*)k_cg<true>;
-    MOT_CUDA_TRY(cudaLaunchCooperativeKernel(k, c->cg_blocks, NT, args, 0, s));
+    const SolveKernel k = solve_kernel(c->precision, c->cg_tile, c->cg_resident, c->cg_split);
+    MOT_CUDA_TRY(cudaLaunchCooperativeKernel(k.fn, c->cg_blocks + 1, k.threads, args, 0, s));
+    ++c->fit_steps;
+}
+
+// Shape of the solve on this geometry: tile lists of both shapes are given; sets the tile
+// (0: 8^3, 1: 8 x 4 x 4), the worker blocks and the epilogue's launch, and returns the
+// chosen list.
+const std::vector<int>& solve_shape(mot_ctx* c, const std::vector<int>& big,
+                                    const std::vector<int>& small) {
+    // The 8^3 tile loads less halo per voxel (2.0 against 2.8) but a pass on it takes a
+    // block about 4 us; with fewer than two such tiles per SM the small tile is faster
+    c->cg_tile = (int)big.size() >= 2 * c->nsm ? 0 : 1;
+    const std::vector<int>& tl = c->cg_tile ? small : big;
+    c->ntiles = (int)tl.size();
+    c->cg_split = c->precision == MOT_FP64 && c->cg_tile && c->nact <= 128LL * c->nsm;
+    int per_sm = 0;
+    SolveKernel k = solve_kernel(c->precision, c->cg_tile, true, c->cg_split);
+    MOT_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.fn, k.threads, 0));
+    c->cg_resident = c->cg_tile == 1 && c->ntiles + 1 <= per_sm * c->nsm;
+    if (!c->cg_resident) {
+        k = solve_kernel(c->precision, c->cg_tile, false, c->cg_split);
+        MOT_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.fn, k.threads, 0));
+    }
+    if (per_sm < 1) throw MotError{MOT_ERR_CUDA, "CG kernel cannot be made resident"};
+    // one block per tile at most: the tiled passes give a block one tile at a time, so
+    // further blocks would only wait at the grid barriers (and keep SMs from concurrent
+    // solves of other contexts).  The component-split FP64 residual has work for more:
+    // a block for every four warps of it, up to one per SM.
+    int want = std::max(c->ntiles, 1);
+    if (c->cg_split)
+        want = std::max(want, std::min(c->nsm, (int)(3 * ((c->nact + 31) / 32) + 3) / 4));
+    c->cg_blocks = std::max(1, std::min(per_sm * c->nsm - 1, want));
+    // epilogue: small blocks on small grids (its FP64 terms are bound by the SMs in use)
+    c->epi_threads = c->M <= 64LL * c->nsm ? 64 : NT;
+    c->epi_blocks = (int)std::min<long long>((c->M + c->epi_threads - 1) / c->epi_threads,
+                                             8LL * c->nsm);
+    return tl;
+}
+
+// halo lists of the resident tiles (tiles and diag32 on the device)
+void solve_halo_lists(mot_ctx* c) {
+    if (!c->cg_resident || !c->ntiles) return;
+    typedef Resident<SmallTile> RT;
+    MOT_CUDA_TRY(cudaMalloc(&c->halo, sizeof(int) * RT::HPT * SmallTile::NTH * (size_t)c->ntiles));
+    k_halo_list<SmallTile><<<c->ntiles, SmallTile::NTH, 0, c->stream>>>(c->tiles, c->diag32, c->U,
+                                                                        c->V, c->W, c->halo);
+    MOT_LAUNCH_CHECK();
 }
 
 // rhs + CG for step n; ||J_n||^2 into norm2_out (device), J_n in ring slot n
 void solve_step(mot_ctx* c, int n, const double* En, double* norm2_out, cudaStream_t s) {
-    if (c->precision == MOT_FP64) epilogue<double>(c, n, En, s);
-    else epilogue<float>(c, n, En, s);
+    if (c->precision == MOT_FP64) epilogue<double, false>(c, n, En, s);
+    else epilogue<float, false>(c, n, En, s);
     CGArgs a = make_cg_args(c, n, norm2_out);
     void* args[] = {&a};
     launch_cg(c, args, s);
@@ -1295,15 +1852,9 @@ void history_out(mot_ctx* c, int n, double* out_dev, cudaStream_t s) {
 void adjoint_step(mot_ctx* c, int tau, int n, const double* g_aos, const double* J_aos,
                   int j_first, double* grad_chi, double* lam_out, double* norm2_out,
                   cudaStream_t s) {
-    const long long tot = 3 * c->M;
     const int s0 = (int)slot_index(tau, c->jring);
-    if (c->precision == MOT_FP64)
-        k_epilogue_adj<double><<<(int)((tot + NT - 1) / NT), NT, 0, s>>>(
-            c->M, c->vfac, g_aos, c->h64.hist_spatial, c->J, s0, c->jring, taps_of(c), c->rhs);
-    else
-        k_epilogue_adj<float><<<(int)((tot + NT - 1) / NT), NT, 0, s>>>(
-            c->M, c->vfac, g_aos, c->h32.hist_spatial, c->J, s0, c->jring, taps_of(c), c->rhs);
-    MOT_LAUNCH_CHECK();
+    if (c->precision == MOT_FP64) epilogue<double, true>(c, tau, g_aos, s);
+    else epilogue<float, true>(c, tau, g_aos, s);
     CGArgs a = make_cg_args(c, tau, norm2_out);
     void* args[] = {&a};
     launch_cg(c, args, s);
@@ -1343,14 +1894,14 @@ extern "C" mot_status mot_barrier_check(int n_blocks, int rounds, int absent, do
     }
     if (n_blocks < 1 || n_blocks > per_sm * nsm) return MOT_ERR_ARG;   // must be co-resident
     int* w = nullptr;
-    if (cudaMalloc(&w, sizeof(int) * 8) != cudaSuccess) {
+    if (cudaMalloc(&w, sizeof(int) * 9) != cudaSuccess) {
         cudaGetLastError();
         return MOT_ERR_OOM;
     }
     long long budget = (long long)(budget_s * 1e3 * std::max(khz, 1000000));
     void* args[] = {&w, &budget, &rounds, &absent};
-    int h[8] = {0};
-    cudaError_t e = cudaMemset(w, 0, sizeof(int) * 8);
+    int h[9] = {0};
+    cudaError_t e = cudaMemset(w, 0, sizeof(int) * 9);
     if (e == cudaSuccess)
         e = cudaLaunchCooperativeKernel((void*)k_barrier_check, n_blocks, NT, args, 0, nullptr);
     if (e == cudaSuccess) e = cudaMemcpy(h, w, sizeof h, cudaMemcpyDeviceToHost);
@@ -1359,7 +1910,7 @@ extern "C" mot_status mot_barrier_check(int n_blocks, int rounds, int absent, do
         cudaGetLastError();
         return MOT_ERR_CUDA;
     }
-    *passed = h[7];
+    *passed = h[8];
     *timeout_round = h[2];
     return (h[1] & 4) ? MOT_ERR_TIMEOUT : MOT_OK;
 }
