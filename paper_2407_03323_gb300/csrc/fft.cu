@@ -338,9 +338,24 @@ struct MidArgs {
     int n_o2;                 // outer index o = comp * n_o2 + o2
     long long in_c, in_o, in_a;    // strides: component, outer, axis (in elements)
     long long out_c, out_o, out_a;
-    int Hu;                   // contiguous extent tiled by TB
+    int Hu;                   // contiguous extent
     int dir;
 };
+
+// Line L of a strided pass: its element offsets in the input and output; false past the
+// last line.  Lines are numbered through (component, outer, ku), and a CTA takes
+// consecutive ones: runs cut at each row of Hu = P/2 + 1 would leave much of the last run
+// of every row idle (Hu = 33: 1 of 32 lines).
+__device__ __forceinline__ bool mid_line(const MidArgs& a, long long L, long long& src,
+                                         long long& dst) {
+    const long long o = L / a.Hu;
+    const int ku = (int)(L - o * a.Hu);
+    const int comp = (int)(o / a.n_o2), o2 = (int)(o - (long long)comp * a.n_o2);
+    const bool live = comp < 3;
+    src = live ? comp * a.in_c + o2 * a.in_o + ku : 0;
+    dst = live ? comp * a.out_c + o2 * a.out_o + ku : 0;
+    return live;
+}
 
 template <typename R>
 __global__ void __launch_bounds__(NT) k_mid(const typename CT<R>::c* __restrict__ in,
@@ -355,25 +370,24 @@ __global__ void __launch_bounds__(NT) k_mid(const typename CT<R>::c* __restrict_
     C* b0 = stw + tw_entries<C>(rl.P);
     C* b1 = b0 + rl.P * ld;
     const int P = rl.P;
-    const int ntile = (a.Hu + TB - 1) / TB;
-    const long long o = blockIdx.x / ntile;
-    const int ku0 = (int)(blockIdx.x % ntile) * TB;
-    const long long comp = o / a.n_o2, o2 = o % a.n_o2;
-    const C* src = in + comp * a.in_c + o2 * a.in_o + ku0;
-    C* dst = out + comp * a.out_c + o2 * a.out_o + ku0;
+    // a thread's line t is the same in every round (blockDim is a multiple of TB)
+    const int t = threadIdx.x % TB;
+    long long src_off, dst_off;
+    const bool live = mid_line(a, (long long)blockIdx.x * TB + t, src_off, dst_off);
+    const C* src = in + src_off;
+    C* dst = out + dst_off;
     load_tw(stw, tw, P);
     for (int it = threadIdx.x; it < P * TB; it += blockDim.x) {
-        const int j = it / TB, t = it % TB;
-        const bool ok = j < a.n_in && ku0 + t < a.Hu;
-        cp_async_c(&b0[j * ld + t], ok ? src + j * a.in_a + t : src, ok);
+        const int j = it / TB;
+        const bool ok = live && j < a.n_in;
+        cp_async_c(&b0[j * ld + t], ok ? src + j * a.in_a : in, ok);
     }
     cp_async_commit_wait();
     __syncthreads();
     C* res = fft_tile<C, TB>(b0, b1, P, rl.r, rl.n, ld, stw, a.dir);
-    for (int it = threadIdx.x; it < a.n_out * TB; it += blockDim.x) {
-        const int j = it / TB, t = it % TB;
-        if (ku0 + t < a.Hu) dst[j * a.out_a + t] = res[j * ld + t];
-    }
+    if (!live) return;
+    for (int j = threadIdx.x / TB; j < a.n_out; j += blockDim.x / TB)
+        dst[j * a.out_a] = res[j * ld + t];
 }
 
 // ------------------------------------------------------------------ strided passes, four-step
@@ -393,14 +407,11 @@ k_mid4s(const typename CT<R>::c* __restrict__ in, typename CT<R>::c* __restrict_
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* Y = reinterpret_cast<C*>(smem_raw);          // [P1][P2][NL]
     C* stw = Y + P * NL;                            // roots exp(-2 pi i k / P) (tw_entries)
-    const int ntile = (a.Hu + NL - 1) / NL;
-    const long long o = blockIdx.x / ntile;
-    const int ku0 = (int)(blockIdx.x % ntile) * NL;
-    const long long comp = o / a.n_o2, o2 = o % a.n_o2;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const bool live = ku0 + lane < a.Hu;
-    const C* src = in + comp * a.in_c + o2 * a.in_o + ku0 + lane;
-    C* dst = out + comp * a.out_c + o2 * a.out_o + ku0 + lane;
+    long long src_off, dst_off;
+    const bool live = mid_line(a, (long long)blockIdx.x * NL + lane, src_off, dst_off);
+    const C* src = in + src_off;
+    C* dst = out + dst_off;
     for (int i = threadIdx.x; i < tw_entries<C>(P); i += blockDim.x) stw[i] = tw[i];
     __syncthreads();
     if (warp < P1) {
@@ -492,8 +503,8 @@ template <typename R>
 void mid_pass(const typename CT<R>::c* in, typename CT<R>::c* out, const AxisFFT& ax,
               const MidArgs& a, cudaStream_t s) {
     const int P = ax.P;
-    const long long lines = 3LL * a.n_o2;
-    const int nb32 = (int)(lines * ((a.Hu + 31) / 32));
+    const long long lines = 3LL * a.n_o2 * a.Hu;
+    const int nb32 = (int)((lines + 31) / 32);
     switch (P) {
         case 64: launch_mid4s<R, 8, 8>(in, out, table<R>(ax), a, nb32, s); return;
         case 96: launch_mid4s<R, 8, 12>(in, out, table<R>(ax), a, nb32, s); return;
@@ -503,7 +514,7 @@ void mid_pass(const typename CT<R>::c* in, typename CT<R>::c* out, const AxisFFT
     constexpr int TB = Tile<R>::TB;
     const size_t sm = smem_bytes<R>(P);
     set_smem(k_mid<R>, sm);
-    k_mid<R><<<(int)(lines * ((a.Hu + TB - 1) / TB)), NT, sm, s>>>(in, out, table<R>(ax),
+    k_mid<R><<<(int)((lines + TB - 1) / TB), NT, sm, s>>>(in, out, table<R>(ax),
                                                                     radix_list(ax), a);
     MOT_LAUNCH_CHECK();
 }

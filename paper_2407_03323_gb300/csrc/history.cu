@@ -567,6 +567,26 @@ __device__ __forceinline__ void fft_dit_reg(C* x, const C* __restrict__ tw, int 
     DitCross<C, Q, T, 1, DIR>::run(x, tw, t);
 }
 
+// Octant bin o and its mirror m (bit 0: kv, bit 1: kw): whether it exists, the signs'
+// flags and its rfft bin.  Blocks take consecutive octant bins across rfft rows: rows of
+// Hu = P/2 + 1 bins cut into runs of 16 or 32 would leave up to half of the lanes idle
+// (Hu = 33: 1 of the last run's 16 or 32), and every lane costs FP64 issue slots.
+template <typename R>
+__device__ __forceinline__ void mirror_bin(const FarArgs<R>& a, long long o, int m, bool& fv,
+                                           bool& fw, bool& live, long long& row) {
+    fv = (m & 1) != 0;
+    fw = (m & 2) != 0;
+    live = o < a.noct;
+    row = 0;
+    if (!live) return;
+    const int ku = (int)(o % a.Hu), kv_o = (int)((o / a.Hu) % a.Hv),
+              kw_o = (int)(o / ((long long)a.Hu * a.Hv));
+    const bool mv = kv_o > 0 && 2 * kv_o < a.Pv, mw = kw_o > 0 && 2 * kw_o < a.Pw;
+    live = (!fv || mv) && (!fw || mw);
+    const int kv = fv ? a.Pv - kv_o : kv_o, kw = fw ? a.Pw - kw_o : kw_o;
+    row = ((long long)kw * a.Pv + kv) * a.Hu + ku;
+}
+
 template <typename R, int Q, int T> struct FarRegSmem {
     typedef typename CT<R>::c C;
     static constexpr int P = Q * T, S = P / 2, NB = 32 / T;
@@ -593,25 +613,16 @@ __global__ void __launch_bounds__(96) k_far_reg(FarArgs<R> a) {
     SM& sm = *reinterpret_cast<SM*>(smem_raw);
     const int comp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int t = lane / NB, line = lane % NB;
-    const int ut = blockIdx.x % a.ntile;
-    const int rest = blockIdx.x / a.ntile;
-    const int mirror = rest & 3;
-    const int orow = rest >> 2;
-    const int kv_o = orow % a.Hv, kw_o = orow / a.Hv;
-    const bool fv = (mirror & 1) != 0, fw = (mirror & 2) != 0;
-    const bool mv = kv_o > 0 && 2 * kv_o < a.Pv;
-    const bool mw = kw_o > 0 && 2 * kw_o < a.Pw;
-    if ((fv && !mv) || (fw && !mw)) return;
-    const int kv = fv ? a.Pv - kv_o : kv_o;
-    const int kw = fw ? a.Pw - kw_o : kw_o;
-    const int ku0 = ut * NB;
-    const int nlive = min(NB, a.Hu - ku0);
-    const bool live = line < nlive;
-    const long long row = ((long long)kw * a.Pv + kv) * a.Hu + ku0 + line;
-    const long long obase = ((long long)kw_o * a.Hv + kv_o) * a.Hu + ku0;
+    const int mirror = blockIdx.x & 3;
+    const long long o0 = (long long)(blockIdx.x >> 2) * NB;   // first octant bin of the block
+    bool fv, fw, live;
+    long long row;
+    mirror_bin(a, o0 + line, mirror, fv, fw, live, row);
+    if (!__syncthreads_or(live)) return;
     for (int i = threadIdx.x; i < (S + 1) * 6 * NB; i += blockDim.x) {
         const int l = i % NB;
-        if (l < nlive) cp_async_c(&sm.H[0][0][0] + i, a.H + (long long)(i / NB) * a.noct + obase + l);
+        if (o0 + l < a.noct)
+            cp_async_c(&sm.H[0][0][0] + i, a.H + (long long)(i / NB) * a.noct + o0 + l);
     }
     const int tfirst = max(1, a.n0 - a.lmax);
     for (int i = threadIdx.x; i < P; i += blockDim.x) {
@@ -678,8 +689,7 @@ void far_launch_reg(mot_ctx* c, FarArgs<R>& a, cudaStream_t s) {
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SM)));
     MOT_CUDA_TRY(cudaFuncSetAttribute(k_far_reg<R, Q, T>,
                                       cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-    a.ntile = (c->Hu + SM::NB - 1) / SM::NB;
-    const long long blocks = (long long)c->Hw * c->Hv * 4 * a.ntile;
+    const long long blocks = 4 * ((c->noct + SM::NB - 1) / SM::NB);
     k_far_reg<R, Q, T><<<(int)blocks, 96, sizeof(SM), s>>>(a);
     MOT_LAUNCH_CHECK();
 }
@@ -730,25 +740,17 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k_far_4s(FarArgs<
     extern __shared__ __align__(16) unsigned char smem_raw[];
     typename F::Smem& sm = *reinterpret_cast<typename F::Smem*>(smem_raw);
     const int tid = threadIdx.x;
-    const int ut = blockIdx.x % a.ntile;
-    const int rest = blockIdx.x / a.ntile;
-    const int mirror = rest & 3;
-    const int orow = rest >> 2;
-    const int kv_o = orow % a.Hv, kw_o = orow / a.Hv;
-    const bool fv = (mirror & 1) != 0, fw = (mirror & 2) != 0;
-    const bool mv = kv_o > 0 && 2 * kv_o < a.Pv;
-    const bool mw = kw_o > 0 && 2 * kw_o < a.Pw;
-    if ((fv && !mv) || (fw && !mw)) return;
-    const int kv = fv ? a.Pv - kv_o : kv_o;
-    const int kw = fw ? a.Pw - kw_o : kw_o;
-    const int ku0 = ut * NB;
-    const int nlive = min(NB, a.Hu - ku0);
-    const long long row0 = ((long long)kw * a.Pv + kv) * a.Hu + ku0;
-    const long long obase = ((long long)kw_o * a.Hv + kv_o) * a.Hu + ku0;
+    const int mirror = blockIdx.x & 3;
+    const long long o0 = (long long)(blockIdx.x >> 2) * NB;   // first octant bin of the block
+    const int bin = tid % NB, ct = tid / NB;
+    bool fv, fw, bin_live;
+    long long row;
+    mirror_bin(a, o0 + bin, mirror, fv, fw, bin_live, row);
+    if (!__syncthreads_or(bin_live)) return;
     for (int i = tid; i < (S + 1) * 6 * NB; i += F::NTB) {
         const int l = i % NB, wc = i / NB;      // wc = w * 6 + c
-        if (l < nlive)
-            cp_async_c(&sm.H[wc / 6][(wc % 6) * NB + l], a.H + (long long)wc * a.noct + obase + l);
+        if (o0 + l < a.noct)
+            cp_async_c(&sm.H[wc / 6][(wc % 6) * NB + l], a.H + (long long)wc * a.noct + o0 + l);
     }
     const int tfirst = max(1, a.n0 - a.lmax);
     for (int i = tid; i < P; i += F::NTB) {
@@ -759,10 +761,9 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k_far_4s(FarArgs<
     }
     __syncthreads();
     // ---- phase A
-    const int bin = tid % NB, ct = tid / NB;
     const int t = ct % T, comp = ct / T;
     const bool athr = tid < F::NA;
-    const bool live = athr && bin < nlive;
+    const bool live = athr && bin_live;
     const R sig = comp == 0 ? (R)1 : (comp == 1 ? (fv ? (R)-1 : (R)1) : (fw ? (R)-1 : (R)1));
     C x[Q1];
     if (athr) {
@@ -771,7 +772,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k_far_4s(FarArgs<
             const int slot = sm.in[t + T * n2];
             C v;
             v.x = 0; v.y = 0;
-            if (slot >= 0 && live) v = a.ring[((long long)slot * 3 + comp) * a.nbins + row0 + bin];
+            if (slot >= 0 && live) v = a.ring[((long long)slot * 3 + comp) * a.nbins + row];
             v.x *= sig; v.y *= sig;
             x[n2] = v;
         });
@@ -846,7 +847,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k_far_4s(FarArgs<
         const int pos = t + T * n2;                  // >= S
         C v = x[n2];
         v.x *= scale; v.y *= scale;
-        a.acc[((long long)sm.out[pos - S] * 3 + comp) * a.nbins + row0 + bin] = v;
+        a.acc[((long long)sm.out[pos - S] * 3 + comp) * a.nbins + row] = v;
     });
 }
 
@@ -858,8 +859,7 @@ void far_launch_4s(mot_ctx* c, FarArgs<R>& a, cudaStream_t s) {
                                       sm_bytes));
     MOT_CUDA_TRY(cudaFuncSetAttribute(k_far_4s<R, P>,
                                       cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-    a.ntile = (c->Hu + F::NB - 1) / F::NB;
-    const long long blocks = (long long)c->Hw * c->Hv * 4 * a.ntile;
+    const long long blocks = 4 * ((c->noct + F::NB - 1) / F::NB);
     k_far_4s<R, P><<<(int)blocks, F::NTB, sm_bytes, s>>>(a);
     MOT_LAUNCH_CHECK();
 }
