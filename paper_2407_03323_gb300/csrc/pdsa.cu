@@ -266,26 +266,52 @@ __global__ void k_sum_parts(const double* __restrict__ part, int nb, double* __r
     }
 }
 
-// w -= sum_j h[j] V_j
+// w -= sum_j h[j] V_j; h[nvec - 1] also into *coef, and with `part` the partial sums of
+// the new ||w||^2 (one per block), so that the norm needs no pass of its own
 __global__ void k_sub_combo(double* __restrict__ w, const double* __restrict__ V,
-                            const double* __restrict__ h, int nvec, long long L) {
+                            const double* __restrict__ h, int nvec, long long L,
+                            double* __restrict__ coef, double* __restrict__ part) {
     extern __shared__ double sh[];
+    __shared__ double sm[NT / 32];
     for (int j = threadIdx.x; j < nvec; j += blockDim.x) sh[j] = h[j];
     __syncthreads();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *coef = sh[nvec - 1];
+    double acc = 0.0;
     for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < L;
          r += (long long)gridDim.x * blockDim.x) {
         double s = w[r];
         for (int j = 0; j < nvec; ++j) s = fma(-sh[j], V[(long long)j * L + r], s);
         w[r] = s;
+        acc = fma(s, s, acc);
+    }
+    if (!part) return;
+    acc = warp_sum(acc);
+    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        acc = warp_sum(threadIdx.x < NT / 32 ? sm[threadIdx.x] : 0.0);
+        if (threadIdx.x == 0) part[blockIdx.x] = acc;
     }
 }
 
-// out = w / sqrt(nrm2[0])
-__global__ void k_normalise(const double* __restrict__ w, const double* __restrict__ nrm2,
-                            long long L, double* __restrict__ out) {
+// out = w / ||w|| from the nb partial sums of ||w||^2 (every block adds them up in the same
+// order; block 0 leaves ||w||^2 in *nrm2)
+__global__ void k_normalise(const double* __restrict__ w, const double* __restrict__ part, int nb,
+                            long long L, double* __restrict__ out, double* __restrict__ nrm2) {
+    __shared__ double sm[NT / 32], tot;
+    double s = 0.0;
+    for (int k = threadIdx.x; k < nb; k += blockDim.x) s += part[k];
+    s = warp_sum(s);
+    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        s = warp_sum(threadIdx.x < NT / 32 ? sm[threadIdx.x] : 0.0);
+        if (threadIdx.x == 0) tot = s;
+    }
+    __syncthreads();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *nrm2 = tot;
     const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= L) return;
-    out[r] = w[r] / sqrt(nrm2[0]);
+    if (r < L) out[r] = w[r] / sqrt(tot);
 }
 
 // plain three-term Lanczos, scalars kept on the device:
@@ -636,6 +662,7 @@ mot_status mot_pdsa_lanczos(mot_ctx* c, int n, int flags, int k, unsigned long l
             double* w = sc.get<double>(L);
             double* h = sc.get<double>(k + 2);
             double* part = sc.get<double>((long long)(k + 2) * nb);
+            double* coef = sc.get<double>(3LL * (k + 1));   // per step: two coefficients, ||w||^2
             const size_t shm = sizeof(double) * (k + 1);
             if (shm > 48 * 1024) {   // raise to the opt-in maximum (process-wide attribute)
                 int dev = 0, optin = 0;
@@ -650,32 +677,44 @@ mot_status mot_pdsa_lanczos(mot_ctx* c, int n, int flags, int k, unsigned long l
             }
             k_rand_vec<<<g1, NT, 0, s>>>(seed, c->eps, M, w);
             MOT_LAUNCH_CHECK();
-            dots(c, w, 1, L, w, part, h, s);
-            k_normalise<<<g1, NT, 0, s>>>(w, h, L, V);
+            k_dots<<<dim3(nb, 1), NT, 0, s>>>(w, 1, L, w, part);
             MOT_LAUNCH_CHECK();
-            double hv[2];
-            for (int j = 0; j < k; ++j) {
-                apply(c, V + (long long)j * L, w, s);
-                double a = 0.0;
-                for (int pass = 0; pass < 2; ++pass) {   // w -= V_{0..j} (V_{0..j}^T w), twice
-                    dots(c, V, j + 1, L, w, part, h, s);
-                    MOT_CUDA_TRY(cudaMemcpyAsync(hv, h + j, sizeof(double), cudaMemcpyDeviceToHost, s));
-                    k_sub_combo<<<nb, NT, shm, s>>>(w, V, h, j + 1, L);
+            k_normalise<<<g1, NT, 0, s>>>(w, part, nb, L, V, coef + 3LL * k);
+            MOT_LAUNCH_CHECK();
+            // the scalars of a step stay on the device and are read every BATCH steps (a
+            // host read per orthogonalisation left the GPU idle for a third of a step);
+            // steps queued past an invariant subspace are dropped
+            constexpr int BATCH = 32;
+            std::vector<double> hc(3 * BATCH);
+            bool stop = false;
+            for (int done = 0; done < k && !stop;) {
+                const int cnt = std::min(BATCH, k - done);
+                for (int j = done; j < done + cnt; ++j) {
+                    apply(c, V + (long long)j * L, w, s);
+                    for (int pass = 0; pass < 2; ++pass) {   // w -= V_{0..j} (V_{0..j}^T w), twice
+                        dots(c, V, j + 1, L, w, part, h, s);
+                        k_sub_combo<<<nb, NT, shm, s>>>(w, V, h, j + 1, L, coef + 3LL * j + pass,
+                                                        pass ? part : nullptr);
+                        MOT_LAUNCH_CHECK();
+                    }
+                    k_normalise<<<g1, NT, 0, s>>>(w, part, nb, L, V + (long long)(j + 1) * L,
+                                                  coef + 3LL * j + 2);
                     MOT_LAUNCH_CHECK();
-                    MOT_CUDA_TRY(cudaStreamSynchronize(s));
-                    a += hv[0];
                 }
-                dots(c, w, 1, L, w, part, h + k + 1, s);
-                MOT_CUDA_TRY(cudaMemcpyAsync(hv + 1, h + k + 1, sizeof(double), cudaMemcpyDeviceToHost, s));
+                MOT_CUDA_TRY(cudaMemcpyAsync(hc.data(), coef + 3LL * done, sizeof(double) * 3 * cnt,
+                                             cudaMemcpyDeviceToHost, s));
                 MOT_CUDA_TRY(cudaStreamSynchronize(s));
-                const double b = sqrt(std::max(hv[1], 0.0));
-                alpha.push_back(a);
-                tnorm = std::max(tnorm, fabs(a) + b + (beta.empty() ? 0.0 : beta.back()));
-                last_beta = b;
-                if (j + 1 == k || b <= 1e-13 * tnorm) break;    // k steps or an invariant subspace
-                beta.push_back(b);
-                k_normalise<<<g1, NT, 0, s>>>(w, h + k + 1, L, V + (long long)(j + 1) * L);
-                MOT_LAUNCH_CHECK();
+                for (int t = 0; t < cnt && !stop; ++t) {
+                    const double a = hc[3 * t] + hc[3 * t + 1];
+                    const double b = sqrt(std::max(hc[3 * t + 2], 0.0));
+                    alpha.push_back(a);
+                    tnorm = std::max(tnorm, fabs(a) + b + (beta.empty() ? 0.0 : beta.back()));
+                    last_beta = b;
+                    // k steps or an invariant subspace
+                    if ((int)alpha.size() == k || b <= 1e-13 * tnorm) stop = true;
+                    else beta.push_back(b);
+                }
+                done += cnt;
             }
         } else {
             // plain three-term recurrence: four vectors; alpha_j, beta_j^2 stay on the
