@@ -1155,7 +1155,10 @@ __global__ void __launch_bounds__(T::NTH, RES ? 4 : 3) k_cg(const __grid_constan
     double* red1 = a.red + nb;
     double* red2 = a.red + 2 * nb;
     Resident<T> res;
-    if constexpr (RES) resident_init<T>(a, res, sd);
+    if constexpr (RES) {
+        resident_init<T>(a, res, sd);
+        __syncthreads();     // its zeros, before a residual pass copies halos over them
+    }
     double bb = 0.0, rr = 0.0, xx = 0.0;
     int its = 0, outer = 0;
     bool first = true, converged = false, nonfinite = false, zero = false;

@@ -98,3 +98,23 @@ def test_solution_satisfies_its_equation(mot, grid, kind, precision, tol):
             b = (E[i] - P) * np.where(chi > 0, 1.0 / np.where(chi > 0, chi, 1.0), 0.0)[:, None]
             r = b - _z0_over_chi(ctx, eps, taps, J[i])
             assert np.linalg.norm(r) <= tol * np.linalg.norm(b), (i, np.linalg.norm(r) / np.linalg.norm(b))
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32_history"])
+@pytest.mark.parametrize("grid,kind", [((5, 6, 40), "cube"), ((20, 21, 23), "holes")])
+def test_repeated_marches_are_bitwise_equal(mot, grid, kind, precision):
+    """Blocks of the solve run unordered between their exchanges; every sum is taken in a
+    fixed order, so a march from rest gives the same bits every time."""
+    W, V, U = grid
+    eps = _shape(kind, W, V, U)
+    rng = np.random.default_rng(5)
+    E = rng.normal(size=(24, eps.size, 3)) * ((eps - 1.0) / eps).reshape(-1)[None, :, None]
+    with mot.Context(eps, wl.fir_taps("fir3", 1e-3), precision=precision, scheme="blocked",
+                     block=4) as ctx:
+        first = None
+        for _ in range(12):
+            ctx.restart(0, None)
+            ctx.set_excitation(E)
+            J = ctx.march(24)
+            first = J if first is None else first
+            assert np.array_equal(J, first)
