@@ -115,10 +115,16 @@ void free_all(mot_ctx* c) {
     if (c->stream) cudaStreamDestroy(c->stream);
 }
 
-void reset_state(mot_ctx* c, cudaStream_t s) {
+// Back to rest.  A march from step 1 reads no spectral ring slot before writing it (lags
+// reach back to step 1 only) and its first step fires every far level, which writes all of
+// the level's accumulators; so the rings (41 GB at 104^3, 7 ms) are cleared only for a
+// replay that starts later (`rings`).
+void reset_state(mot_ctx* c, cudaStream_t s, bool rings = false) {
     MOT_CUDA_TRY(cudaMemsetAsync(c->J, 0, sizeof(double) * 3 * c->M * c->jring, s));
-    if (c->precision == MOT_FP64) mot::history_reset<double>(c, s);
-    else mot::history_reset<float>(c, s);
+    if (rings) {
+        if (c->precision == MOT_FP64) mot::history_reset<double>(c, s);
+        else mot::history_reset<float>(c, s);
+    }
     MOT_CUDA_TRY(cudaMemsetAsync(c->fit, 0, sizeof(double) * mot::kFitWords, s));
     c->fit_steps = 0;
     c->n_done = 0;
@@ -770,7 +776,7 @@ mot_status mot_eval_history(mot_ctx* c, int n_hist, const double* J_hist, double
     }
     return guarded(c, [&] {
         cudaStream_t s = stream ? (cudaStream_t)stream : c->stream;
-        reset_state(c, s);
+        reset_state(c, s, true);
         const long long step = 3 * c->M;
         double* tmp = nullptr;
         MOT_CUDA_TRY(cudaMalloc(&tmp, sizeof(double) * step * (n_hist + 1)));
@@ -835,7 +841,7 @@ mot_status mot_restart(mot_ctx* c, int n0, int n_hist, const double* J_hist, voi
     std::vector<void*> owned;
     mot_status st = guarded(c, [&] {
         cudaStream_t s = stream ? (cudaStream_t)stream : c->stream;
-        reset_state(c, s);
+        reset_state(c, s, n0 > 0);
         const double* Jd = n_hist ? on_device(c, J_hist, n_hist, owned, s) : nullptr;
         const long long step = 3 * c->M;
         // replay the history path over the window: every far-level firing that

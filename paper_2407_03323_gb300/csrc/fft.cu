@@ -590,14 +590,13 @@ bool x_pass_codelet(bool fwd, mot_ctx* c, const double* Jsoa, typename CT<R>::c*
     }
 }
 
+// x and y passes of the forward transform, [3][W][V][U] -> hb.tmp2 [3][W][Pv][Hu]
 template <typename R>
-void fft_forward(mot_ctx* c, const double* Jsoa, typename CT<R>::c* out, cudaStream_t s,
-                 const double* scale) {
-    typedef typename CT<R>::c C;
+void fft_forward_xy(mot_ctx* c, const double* Jsoa, cudaStream_t s, const double* scale) {
     HistoryBuffers<R>& hb = hbuf<R>(c);
     constexpr int TB = Tile<R>::TB;
     const int U = c->U, V = c->V, W = c->W;
-    const int Pu = c->ax[0].P, Pv = c->ax[1].P, Pw = c->ax[2].P, Hu = c->Hu;
+    const int Pu = c->ax[0].P, Pv = c->ax[1].P, Hu = c->Hu;
     // x
     if (!x_pass_codelet<R>(true, c, Jsoa, hb.tmp1, nullptr, scale, s)) {
         const long long npairs = 3LL * W * ((V + 1) / 2);
@@ -617,32 +616,33 @@ void fft_forward(mot_ctx* c, const double* Jsoa, typename CT<R>::c* out, cudaStr
         a.Hu = Hu; a.dir = -1;
         mid_pass<R>(hb.tmp1, hb.tmp2, c->ax[1], a, s);
     }
-    // z: [3][W][Pv][Hu] -> [3][Pw][Pv][Hu]
-    {
-        MidArgs a;
-        a.n_in = W; a.n_out = Pw; a.n_o2 = Pv;
-        a.in_c = (long long)W * Pv * Hu; a.in_o = Hu; a.in_a = (long long)Pv * Hu;
-        a.out_c = (long long)Pw * Pv * Hu; a.out_o = Hu; a.out_a = (long long)Pv * Hu;
-        a.Hu = Hu; a.dir = -1;
-        mid_pass<R>(hb.tmp2, out, c->ax[2], a, s);
-    }
+}
+
+// z pass of the forward transform, hb.tmp2 -> [3][Pw][Pv][Hu]
+template <typename R>
+void fft_forward_z(mot_ctx* c, typename CT<R>::c* out, cudaStream_t s) {
+    const int W = c->W, Pv = c->ax[1].P, Pw = c->ax[2].P, Hu = c->Hu;
+    MidArgs a;
+    a.n_in = W; a.n_out = Pw; a.n_o2 = Pv;
+    a.in_c = (long long)W * Pv * Hu; a.in_o = Hu; a.in_a = (long long)Pv * Hu;
+    a.out_c = (long long)Pw * Pv * Hu; a.out_o = Hu; a.out_a = (long long)Pv * Hu;
+    a.Hu = Hu; a.dir = -1;
+    mid_pass<R>(hbuf<R>(c).tmp2, out, c->ax[2], a, s);
 }
 
 template <typename R>
-void fft_inverse(mot_ctx* c, const typename CT<R>::c* in, R* out, cudaStream_t s) {
+void fft_forward(mot_ctx* c, const double* Jsoa, typename CT<R>::c* out, cudaStream_t s) {
+    fft_forward_xy<R>(c, Jsoa, s, nullptr);
+    fft_forward_z<R>(c, out, s);
+}
+
+// y and x passes of the inverse transform, hb.tmp2 [3][W][Pv][Hu] -> [3][W][V][U]
+template <typename R>
+void fft_inverse_yx(mot_ctx* c, R* out, cudaStream_t s) {
     HistoryBuffers<R>& hb = hbuf<R>(c);
     constexpr int TB = Tile<R>::TB;
     const int U = c->U, V = c->V, W = c->W;
-    const int Pu = c->ax[0].P, Pv = c->ax[1].P, Pw = c->ax[2].P, Hu = c->Hu;
-    // z: [3][Pw][Pv][Hu] -> [3][W][Pv][Hu]
-    {
-        MidArgs a;
-        a.n_in = Pw; a.n_out = W; a.n_o2 = Pv;
-        a.in_c = (long long)Pw * Pv * Hu; a.in_o = Hu; a.in_a = (long long)Pv * Hu;
-        a.out_c = (long long)W * Pv * Hu; a.out_o = Hu; a.out_a = (long long)Pv * Hu;
-        a.Hu = Hu; a.dir = +1;
-        mid_pass<R>(in, hb.tmp2, c->ax[2], a, s);
-    }
+    const int Pu = c->ax[0].P, Pv = c->ax[1].P, Hu = c->Hu;
     // y: [3][W][Pv][Hu] -> [3][W][V][Hu]
     {
         MidArgs a;
@@ -664,8 +664,26 @@ void fft_inverse(mot_ctx* c, const typename CT<R>::c* in, R* out, cudaStream_t s
     }
 }
 
-template void fft_forward<double>(mot_ctx*, const double*, double2*, cudaStream_t, const double*);
-template void fft_forward<float>(mot_ctx*, const double*, float2*, cudaStream_t, const double*);
+template <typename R>
+void fft_inverse(mot_ctx* c, const typename CT<R>::c* in, R* out, cudaStream_t s) {
+    const int W = c->W, Pv = c->ax[1].P, Pw = c->ax[2].P, Hu = c->Hu;
+    // z: [3][Pw][Pv][Hu] -> [3][W][Pv][Hu]
+    MidArgs a;
+    a.n_in = Pw; a.n_out = W; a.n_o2 = Pv;
+    a.in_c = (long long)Pw * Pv * Hu; a.in_o = Hu; a.in_a = (long long)Pv * Hu;
+    a.out_c = (long long)W * Pv * Hu; a.out_o = Hu; a.out_a = (long long)Pv * Hu;
+    a.Hu = Hu; a.dir = +1;
+    mid_pass<R>(in, hbuf<R>(c).tmp2, c->ax[2], a, s);
+    fft_inverse_yx<R>(c, out, s);
+}
+
+template void fft_forward_xy<double>(mot_ctx*, const double*, cudaStream_t, const double*);
+template void fft_forward_xy<float>(mot_ctx*, const double*, cudaStream_t, const double*);
+template void fft_forward_z<double>(mot_ctx*, double2*, cudaStream_t);
+template void fft_forward_z<float>(mot_ctx*, float2*, cudaStream_t);
+template void fft_inverse_yx<double>(mot_ctx*, double*, cudaStream_t);
+template void fft_inverse_yx<float>(mot_ctx*, float*, cudaStream_t);
+template void fft_forward<double>(mot_ctx*, const double*, double2*, cudaStream_t);
 template void fft_inverse<double>(mot_ctx*, const double2*, double*, cudaStream_t);
 template void fft_inverse<float>(mot_ctx*, const float2*, float*, cudaStream_t);
 

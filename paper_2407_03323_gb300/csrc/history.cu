@@ -3,15 +3,11 @@
 //
 // Spectral ring: Jhat_{n'} is kept at slot n' mod hring (hring >= ell), so the
 // forward FFT of each J runs once and is reused by every later step.  The per-bin
-// product is a real symmetric 3x3 matrix times a complex 3-vector.  The stored kernel
-// spectrum covers the octant k_i <= P_i/2; one load serves the four bins
-// (ku, +-kv, +-kw), with the sign of the (a, b) component flipped for every mirrored
-// axis among a, b (the component is odd in k_a and k_b).
-//
-// FP32-history: the spectra, rings and MAC are FP32; each lag's contribution is
-// formed with FP32 FMAs and added into the running sum with an error-free two-sum,
-// so the accumulation over up to ell lags adds no error beyond one rounding of the
-// compensated total.
+// product is a real symmetric 3x3 matrix times a complex 3-vector (zmac.cu, together with
+// the z passes of the transforms).  The stored kernel spectrum covers the octant
+// k_i <= P_i/2; it serves the four bins (ku, +-kv, +-kw), with the sign of the (a, b)
+// component flipped for every mirrored axis among a, b (the component is odd in k_a and
+// k_b).
 // Blocked temporal scheme (Secs. 4-5, MOT_HISTORY_BLOCKED): lags 1..B-1 are multiplied
 // every step as above; the lags [a, a + S) form a level of length S, with a = S for
 // S = B, 2B, 4B, ... and, where the last of these would reach far past ell, a shorter
@@ -40,20 +36,13 @@ namespace {
 
 constexpr int NT = 256;
 
-template <typename R> struct Acc;
-template <> struct Acc<double> {
-    double2 s;
-    __device__ void zero() { s = make_double2(0.0, 0.0); }
-    __device__ void add(double2 v) { s.x += v.x; s.y += v.y; }
-    __device__ double2 get() const { return s; }
-};
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
     s = a + b;
     const float bp = s - a;
     const float ap = s - bp;
     e = (a - ap) + (b - bp);
 }
-template <> struct Acc<float> {
+struct Acc {
     float2 s, c;
     __device__ void zero() { s = make_float2(0.f, 0.f); c = make_float2(0.f, 0.f); }
     __device__ void add(float2 v) {
@@ -70,24 +59,28 @@ struct MacGeom {
 };
 
 // this step's entries of the far levels' accumulator rings ([3][nbins] each)
-template <typename C> struct FarSums {
-    const C* p[8];
+struct FarSums {
+    const float2* p[8];
     int n;
 };
 
-// Phat(k) = scale * sum_{l=1}^{L} Ghat_l(k) Jhat_{n-l}(k) over all rfft bins.
+// The lag products of the FP32-history march on large grids, as a kernel of its own between
+// the z passes: Phat(k) = scale * (far sums + sum_{l=1}^{L} Ghat_l(k) Jhat_{n-l}(k)) over all
+// rfft bins.  It is bound by HBM and needs many warps with their loads in flight (104^3:
+// 0.335 ms, 0.75 of the copy bandwidth, with 40 + 46 us for the z passes around it); the fused
+// kernel of zmac.cu, whose blocks alternate between transforms and products, takes 0.72 ms
+// there and wins where launches count (18^3 bins: 41 against 49 us of a step).
 // A warp covers 8 consecutive octant bins (ku) x 4 mirrors: lane = mirror * 8 + j.
 // The 8 lanes of a mirror read 8 consecutive bins of a ring row; the kernel values of
 // the 8 bins ([lag][octant bin][6], 6 per bin) are one contiguous load shared by the
 // 4 mirror groups.  Ring slots are walked backwards from slot_first = (n-1) mod hring.
-template <typename R>
-__global__ void __launch_bounds__(NT) k_mac(const R* __restrict__ ghat,
-                                            const typename CT<R>::c* __restrict__ ring, int hring,
-                                            int slot_first, int L, MacGeom g, R scale,
-                                            typename CT<R>::c* __restrict__ phat,
-                                            FarSums<typename CT<R>::c> far) {
-    typedef typename CT<R>::c C;
-    typedef typename std::conditional<std::is_same<R, double>::value, double2, float2>::type R2;
+__global__ void __launch_bounds__(NT) k_mac(const float* __restrict__ ghat,
+                                            const float2* __restrict__ ring, int hring,
+                                            int slot_first, int L, MacGeom g, float scale,
+                                            float2* __restrict__ phat, FarSums far) {
+    typedef float R;
+    typedef float2 C;
+    typedef float2 R2;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int mirror = lane >> 3, j = lane & 7;
     const long long o = ((long long)blockIdx.x * (NT / 32) + warp) * 8 + j;
@@ -105,7 +98,7 @@ __global__ void __launch_bounds__(NT) k_mac(const R* __restrict__ ghat,
     const R sxy = fv ? (R)-1 : (R)1;
     const R sxz = fw ? (R)-1 : (R)1;
     const R syz = (fv != fw) ? (R)-1 : (R)1;
-    Acc<R> ax, ay, az;
+    Acc ax, ay, az;
     ax.zero(); ay.zero(); az.zero();
     for (int k = 0; k < far.n; ++k) {   // far-lag contributions of this step
         const C* f = far.p[k];
@@ -293,6 +286,14 @@ MacGeom geom(const mot_ctx* c) {
     return g;
 }
 
+// Whether a step's z passes and lag products run fused (zmac.cu).  FP64 always: it is bound
+// by its multiply-adds either way and saves the passes over memory (24^3 direct: 124 against
+// 200 us).  FP32 on (kv, ku) planes of up to 8 positions per SM (P <= 48), where the launches
+// and not the memory bound the step; at P = 64 both take 57 us, at 210 see k_mac.
+template <typename R> bool fused_z(const mot_ctx* c) {
+    return sizeof(R) == 8 || (long long)c->ax[1].P * c->Hu <= 8LL * c->nsm;
+}
+
 }  // namespace
 
 namespace mot {
@@ -329,7 +330,7 @@ void history_alloc(mot_ctx* c) {
     const long long slot = 3 * c->nbins;
     MOT_CUDA_TRY(cudaMalloc(&hb.jhat_ring, sizeof(C) * slot * c->hring));
     MOT_CUDA_TRY(cudaMalloc(&hb.ghat, sizeof(R) * 6 * c->noct * c->ell));
-    MOT_CUDA_TRY(cudaMalloc(&hb.phat, sizeof(C) * slot));
+    if (!fused_z<R>(c)) MOT_CUDA_TRY(cudaMalloc(&hb.phat, sizeof(C) * slot));
     MOT_CUDA_TRY(cudaMalloc(&hb.tmp1, sizeof(C) * 3LL * c->W * c->V * c->Hu));
     MOT_CUDA_TRY(cudaMalloc(&hb.tmp2, sizeof(C) * 3LL * c->W * c->ax[1].P * c->Hu));
     MOT_CUDA_TRY(cudaMalloc(&hb.hist_spatial, sizeof(R) * 3 * c->M));
@@ -370,7 +371,7 @@ void history_alloc_shared(mot_ctx* c, mot_ctx* src) {
     hb.ghat = sb.ghat;
     hb.level_spec = sb.level_spec;
     MOT_CUDA_TRY(cudaMalloc(&hb.jhat_ring, sizeof(C) * slot * c->hring));
-    MOT_CUDA_TRY(cudaMalloc(&hb.phat, sizeof(C) * slot));
+    if (!fused_z<R>(c)) MOT_CUDA_TRY(cudaMalloc(&hb.phat, sizeof(C) * slot));
     MOT_CUDA_TRY(cudaMalloc(&hb.tmp1, sizeof(C) * 3LL * c->W * c->V * c->Hu));
     MOT_CUDA_TRY(cudaMalloc(&hb.tmp2, sizeof(C) * 3LL * c->W * c->ax[1].P * c->Hu));
     MOT_CUDA_TRY(cudaMalloc(&hb.hist_spatial, sizeof(R) * 3 * c->M));
@@ -1186,34 +1187,49 @@ void history_step(mot_ctx* c, int n, cudaStream_t s, cudaEvent_t* ev) {
     typedef typename CT<R>::c C;
     HistoryBuffers<R>& hb = hbuf<R>(c);
     const long long slot = 3 * c->nbins;
+    const bool blocked = c->scheme == MOT_HISTORY_BLOCKED;
+    const bool fused = fused_z<R>(c);
+    bool fires = false;
+    for (int k = 0; blocked && k < c->nlev; ++k) fires = fires || (n - 1) % c->lev_S[k] == 0;
     if (n >= 2) {
         const double* Jprev = c->J + slot_index(n - 1, c->jring) * 3 * c->M;
-        fft_forward<R>(c, Jprev, hb.jhat_ring + slot_index(n - 1, c->hring) * slot, s,
-                       c->adjoint ? c->chi : nullptr);
-        c->stats.launches += 3;
+        fft_forward_xy<R>(c, Jprev, s, c->adjoint ? c->chi : nullptr);
+        c->stats.launches += 2;
+        if (fires || !fused) {     // a firing reads the spectrum of J_{n-1}
+            fft_forward_z<R>(c, hb.jhat_ring + slot_index(n - 1, c->hring) * slot, s);
+            c->stats.launches += 1;
+        }
     }
     if (ev) MOT_CUDA_TRY(cudaEventRecord(ev[0], s));
-    const bool blocked = c->scheme == MOT_HISTORY_BLOCKED;
     if (blocked)   // each firing level writes its own accumulator ring
         for (int k = c->nlev - 1; k >= 0; --k)
             if ((n - 1) % c->lev_S[k] == 0) far_level<R>(c, k, n, s);
     if (ev) MOT_CUDA_TRY(cudaEventRecord(ev[1], s));
-    const R scale = (R)(1.0 / ((double)c->ax[0].P * c->ax[1].P * c->ax[2].P));
-    const long long nblk = (c->noct + 8 * (NT / 32) - 1) / (8 * (NT / 32));
-    const int L = blocked ? std::min(c->block - 1, c->ell) : c->ell;
-    FarSums<C> far;
-    far.n = blocked ? c->nlev : 0;
-    for (int k = 0; k < far.n; ++k)
-        far.p[k] = hb.acc_ring + (c->lev_acc[k] + slot_index(n, c->lev_S[k])) * slot;
-    k_mac<R><<<(int)nblk, NT, 0, s>>>(hb.ghat, hb.jhat_ring, c->hring,
-                                      (int)slot_index(n - 1, c->hring), L, geom(c), scale,
-                                      hb.phat, far);
-    MOT_LAUNCH_CHECK();
+    // lags 1 .. L; J_n = 0 for n <= 0, so lags beyond n - 1 add nothing
+    const int L = std::min(blocked ? std::min(c->block - 1, c->ell) : c->ell, n - 1);
+    const C* far[8];
+    const int nfar = blocked ? c->nlev : 0;
+    for (int k = 0; k < nfar; ++k)
+        far[k] = hb.acc_ring + (c->lev_acc[k] + slot_index(n, c->lev_S[k])) * slot;
+    if (fused) {
+        zmac<R>(c, n, n >= 2 && !fires, L, far, nfar, s);
+    } else if constexpr (std::is_same<R, float>::value) {
+        FarSums fs;
+        fs.n = nfar;
+        for (int k = 0; k < nfar; ++k) fs.p[k] = far[k];
+        const float scale = (float)(1.0 / ((double)c->ax[0].P * c->ax[1].P * c->ax[2].P));
+        const long long nblk = (c->noct + 8 * (NT / 32) - 1) / (8 * (NT / 32));
+        k_mac<<<(int)nblk, NT, 0, s>>>(hb.ghat, hb.jhat_ring, c->hring,
+                                       (int)slot_index(n - 1, c->hring), L, geom(c), scale,
+                                       hb.phat, fs);
+        MOT_LAUNCH_CHECK();
+    }
     c->stats.launches += 1;
     c->stats.mac_launches += 1;
     if (ev) MOT_CUDA_TRY(cudaEventRecord(ev[2], s));
-    fft_inverse<R>(c, hb.phat, hb.hist_spatial, s);
-    c->stats.launches += 3;
+    if (fused) fft_inverse_yx<R>(c, hb.hist_spatial, s);
+    else fft_inverse<R>(c, hb.phat, hb.hist_spatial, s);
+    c->stats.launches += fused ? 2 : 3;
 }
 
 template void history_alloc<double>(mot_ctx*);

@@ -61,7 +61,7 @@ template <typename R> struct HistoryBuffers {
     typedef typename CT<R>::c C;
     C* jhat_ring = nullptr;      // [slots][3][Pw][Pv][Hu]
     R* ghat = nullptr;           // [lags][6][Hw][Hv][Hu] (lag 1 first)
-    C* phat = nullptr;           // [3][Pw][Pv][Hu]
+    C* phat = nullptr;           // [3][Pw][Pv][Hu] (FP32 large grids)
     C* tmp1 = nullptr;           // FFT intermediates
     C* tmp2 = nullptr;
     R* hist_spatial = nullptr;   // [3][W][V][U]   (G * J history, spatial)
@@ -239,10 +239,18 @@ void spectrum_of_combination(mot_ctx* c, const double* w_host, int n, bool round
 void fft_plan_axis(AxisFFT& a, int P);
 void fft_free_axis(AxisFFT& a);
 template <typename R>
-void fft_forward(mot_ctx* c, const double* Jsoa, typename CT<R>::c* out, cudaStream_t s,
-                 const double* scale = nullptr);
+void fft_forward(mot_ctx* c, const double* Jsoa, typename CT<R>::c* out, cudaStream_t s);
 template <typename R>
 void fft_inverse(mot_ctx* c, const typename CT<R>::c* in, R* out, cudaStream_t s);
+// the parts of them around the z passes; the (kv, ku) planes in between are in hb.tmp2
+template <typename R>
+void fft_forward_xy(mot_ctx* c, const double* Jsoa, cudaStream_t s, const double* scale);
+template <typename R> void fft_forward_z(mot_ctx* c, typename CT<R>::c* out, cudaStream_t s);
+template <typename R> void fft_inverse_yx(mot_ctx* c, R* out, cudaStream_t s);
+// zmac.cu: z transform of J_{n-1} into the ring (fwd), lag products and far sums, inverse z
+template <typename R>
+void zmac(mot_ctx* c, int n, bool fwd, int L, const typename CT<R>::c* const* far, int nfar,
+          cudaStream_t s);
 // history.cu
 // far levels of the blocked scheme for block B and ell (host only): level k covers
 // lags [a[k], a[k] + S[k]); returns the number of levels, or -1 if more than 8 are needed
@@ -250,8 +258,9 @@ int level_plan(int block, int ell, bool fit, int S[8], int a[8]);
 template <typename R> void history_alloc(mot_ctx* c);
 template <typename R> void history_alloc_shared(mot_ctx* c, mot_ctx* src);
 template <typename R> void history_free(mot_ctx* c);
-// ev (optional, 3 events): recorded after the forward FFT, after the far-lag block
-// products and after the near-lag MAC
+// ev (optional, 3 events): recorded after the forward x and y (and, on steps where a level
+// fires, z) passes, after the far-lag block products and after the z passes with the
+// near-lag products
 template <typename R> void history_step(mot_ctx* c, int n, cudaStream_t s,
                                         cudaEvent_t* ev = nullptr);
 template <typename R> void history_reset(mot_ctx* c, cudaStream_t s);

@@ -408,7 +408,7 @@ void ensure_operator(mot_ctx* c, int n, int flags) {
 // y = A_n x, both [3][M] on the device
 void apply(mot_ctx* c, const double* x, double* y, cudaStream_t s) {
     const double scale = 1.0 / ((double)c->ax[0].P * c->ax[1].P * c->ax[2].P);
-    mot::fft_forward<double>(c, x, c->pdsa_xhat, s, nullptr);
+    mot::fft_forward<double>(c, x, c->pdsa_xhat, s);
     k_pdsa_mul<<<nblk(c->nbins, NT), NT, 0, s>>>(c->pdsa_spec, c->pdsa_xhat, c->Hu, c->Hv,
                                                  c->ax[1].P, c->ax[2].P, c->nbins, scale);
     MOT_LAUNCH_CHECK();

@@ -5,9 +5,9 @@
 //   2. Phat(k) = scale * (sum of the far levels' entries + sum_{l=1}^{L} Ghat_l(k) Jhat_{n-l}(k)),
 //      lag 1 from the transform just made;
 //   3. inverse z transform of Phat, of which the W rows the grid needs go back in place.
-// As three kernels the step wrote Jhat and read it back for lag 1, and wrote and read Phat:
-// 3 x 2 passes over [3][Pw][Pv][Hu] that this kernel does not make (at 104^3 in FP32 336 of
-// 2,000 MB), and two launches of about 7 us each, a tenth of a step on grids up to 32^3.
+// As three kernels the step wrote Jhat and read it back for lag 1, wrote and read Phat, and
+// had two more launches.  Used for FP64 and for small FP32 grids (fused_z in history.cu says
+// where the line lies); FP32 on large grids keeps the separate HBM-bound product kernel.
 //
 // A block takes TB consecutive positions of the (kv, ku) plane (contiguous in every array,
 // also across rows) and all three components: 3 TB lines in two shared-memory buffers.  TB
@@ -36,6 +36,10 @@ template <> struct Acc<double> {
     __device__ void zero() { s = make_double2(0.0, 0.0); }
     __device__ void add(double2 v) { s.x += v.x; s.y += v.y; }
     __device__ double2 get() const { return s; }
+    __device__ void merge(int o) {           // add lane ^ o's sum
+        s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+        s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+    }
 };
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
     s = a + b;
@@ -52,6 +56,12 @@ template <> struct Acc<float> {
         two_sum(s.y, v.y, s.y, e); c.y += e;
     }
     __device__ float2 get() const { return make_float2(s.x + c.x, s.y + c.y); }
+    __device__ void merge(int o) {
+        const float cx = __shfl_xor_sync(0xffffffffu, c.x, o), cy = __shfl_xor_sync(0xffffffffu, c.y, o);
+        add(make_float2(__shfl_xor_sync(0xffffffffu, s.x, o), __shfl_xor_sync(0xffffffffu, s.y, o)));
+        c.x += cx;
+        c.y += cy;
+    }
 };
 
 template <typename R> struct ZArgs {
@@ -64,6 +74,7 @@ template <typename R> struct ZArgs {
     int nfar, fwd;        // fwd: make Jhat_{n-1} here (else it is in the ring already)
     int hring, slot1;     // ring slot of J_{n-1}
     int L;                // lags 1 .. L
+    int split;            // lanes that share the lags of a bin (a power of two, <= 8 and hring)
     int W, Pv, Pw, Hu, Hv, Hw;
     int plane;            // Pv * Hu
     long long nbins, noct;
@@ -71,10 +82,22 @@ template <typename R> struct ZArgs {
     RadixList rl;
 };
 
-// o[] += G x for the real symmetric G = (xx, yy, zz, xy, xz, yz)
-template <typename R, typename C>
-__device__ __forceinline__ void add_product(Acc<R>* acc, const R* G, const C& x, const C& y,
-                                            const C& z) {
+// acc += G x for the real symmetric G = (xx, yy, zz, xy, xz, yz).  FP64 chains the 18
+// multiply-adds into the sums (no separate additions: every FP64 instruction holds a
+// sub-partition for 64 cycles); FP32 forms a lag's contribution first, for the two-sum
+__device__ __forceinline__ void add_product(Acc<double>* acc, const double* G, const double2& x,
+                                            const double2& y, const double2& z) {
+    double2 &o0 = acc[0].s, &o1 = acc[1].s, &o2 = acc[2].s;
+    o0.x = fma(G[0], x.x, fma(G[3], y.x, fma(G[4], z.x, o0.x)));
+    o0.y = fma(G[0], x.y, fma(G[3], y.y, fma(G[4], z.y, o0.y)));
+    o1.x = fma(G[3], x.x, fma(G[1], y.x, fma(G[5], z.x, o1.x)));
+    o1.y = fma(G[3], x.y, fma(G[1], y.y, fma(G[5], z.y, o1.y)));
+    o2.x = fma(G[4], x.x, fma(G[5], y.x, fma(G[2], z.x, o2.x)));
+    o2.y = fma(G[4], x.y, fma(G[5], y.y, fma(G[2], z.y, o2.y)));
+}
+__device__ __forceinline__ void add_product(Acc<float>* acc, const float* G, const float2& x,
+                                            const float2& y, const float2& z) {
+    typedef float2 C;
     C ox, oy, oz;
     ox.x = G[0] * x.x + G[3] * y.x + G[4] * z.x;
     ox.y = G[0] * x.y + G[3] * y.y + G[4] * z.y;
@@ -94,10 +117,15 @@ __device__ __forceinline__ void products(const ZArgs<R>& a, const typename CT<R>
     typedef typename CT<R>::c C;
     typedef typename std::conditional<std::is_same<R, double>::value, double2, float2>::type R2;
     constexpr int U = sizeof(R) == 4 ? 3 : 2;    // lags whose loads are issued together
-    for (int it = threadIdx.x; it < a.Hw * TB; it += blockDim.x) {
+    const int g = threadIdx.x & (a.split - 1);     // this lane's share of the lags
+    const int items = a.Hw * TB, per = blockDim.x / a.split;
+    // all lanes make every round, the surplus on the last item (their results are dropped):
+    // the shares are added with full-warp shuffles
+    for (int it0 = 0; it0 < items; it0 += per) {
+        const int it = min(it0 + (int)threadIdx.x / a.split, items - 1);
         const int t = it % TB, kw = it / TB;
-        const int f = f0 + t;
-        if (f >= a.plane) continue;
+        const int f = min(f0 + t, a.plane - 1);
+        const bool keep = it0 + (int)threadIdx.x / a.split < items && f0 + t < a.plane;
         const int kv = f / a.Hu, ku = f - kv * a.Hu;
         const bool fv = 2 * kv > a.Pv;
         const int kvo = fv ? a.Pv - kv : kv;
@@ -112,7 +140,7 @@ __device__ __forceinline__ void products(const ZArgs<R>& a, const typename CT<R>
 #pragma unroll
         for (int c = 0; c < 3; ++c) { acc1[c].zero(); acc2[c].zero(); }
 #pragma unroll 2
-        for (int k = 0; k < a.nfar; ++k) {   // far-lag contributions of this step
+        for (int k = g; k < a.nfar; k += a.split) {   // far-lag contributions of this step
             const C* p = a.far[k];
             C u[3], v[3];
 #pragma unroll
@@ -120,36 +148,39 @@ __device__ __forceinline__ void products(const ZArgs<R>& a, const typename CT<R>
 #pragma unroll
             for (int c = 0; c < 3; ++c) { acc1[c].add(u[c]); acc2[c].add(v[c]); }
         }
-        const R2* gp = reinterpret_cast<const R2*>(a.ghat + o * 6);
-        const long long gstep = a.noct * 3;   // in R2 units per lag
+        const R2* gp = reinterpret_cast<const R2*>(a.ghat + o * 6) + g * (a.noct * 3);
+        const long long gstep = a.noct * 3 * a.split;   // in R2 units per lag of this lane
         const long long stride = 3 * a.nbins;
         auto lag = [&](const R2& g01, const R2& g23, const R2& g45, const C* x, const C* y) {
             const R G[6] = {g01.x, g01.y, g23.x, sv * g23.y, g45.x, sv * g45.y};
             const R H[6] = {G[0], G[1], G[2], G[3], -G[4], -G[5]};
-            add_product<R>(acc1, G, x[0], x[1], x[2]);
-            add_product<R>(acc2, H, y[0], y[1], y[2]);
+            add_product(acc1, G, x[0], x[1], x[2]);
+            add_product(acc2, H, y[0], y[1], y[2]);
         };
-        int slot = a.slot1, l = 1;
-        if (a.fwd && a.L >= 1) {
-            const C* x = X + kw * ld + t;
-            const C* y = X + kw2 * ld + t;
+        int l = 1 + g, slot = a.slot1 - g;
+        if (slot < 0) slot += a.hring;
+        if (a.fwd && l == 1 && a.L >= 1) {
+            const C* x = X + kw * ld + (f - f0);
+            const C* y = X + kw2 * ld + (f - f0);
             const C xs[3] = {x[0], x[TB], x[2 * TB]}, ys[3] = {y[0], y[TB], y[2 * TB]};
             lag(gp[0], gp[1], gp[2], xs, ys);
             gp += gstep;
-            slot = slot == 0 ? a.hring - 1 : slot - 1;
-            l = 2;
+            slot -= a.split;
+            if (slot < 0) slot += a.hring;
+            l += a.split;
         }
-        for (; l <= a.L; l += U) {
-            R2 g[U][3];
+        for (; l <= a.L; l += U * a.split) {
+            R2 gv[U][3];
             C x[U][3], y[U][3];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                if (l + u > a.L) break;
+                if (l + u * a.split > a.L) break;
                 const C* base = a.ring + (long long)slot * stride;
-                slot = slot == 0 ? a.hring - 1 : slot - 1;
+                slot -= a.split;
+                if (slot < 0) slot += a.hring;
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
-                    g[u][c] = gp[c];
+                    gv[u][c] = gp[c];
                     x[u][c] = base[c * a.nbins + bin1];
                     y[u][c] = base[c * a.nbins + bin2];
                 }
@@ -157,10 +188,14 @@ __device__ __forceinline__ void products(const ZArgs<R>& a, const typename CT<R>
             }
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                if (l + u > a.L) break;
-                lag(g[u][0], g[u][1], g[u][2], x[u], y[u]);
+                if (l + u * a.split > a.L) break;
+                lag(gv[u][0], gv[u][1], gv[u][2], x[u], y[u]);
             }
         }
+        for (int o2 = 1; o2 < a.split; o2 <<= 1)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) { acc1[c].merge(o2); acc2[c].merge(o2); }
+        if (!keep || g != 0) continue;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             C v = acc1[c].get();
@@ -301,7 +336,10 @@ void launch(const ZArgs<R>& a, cudaStream_t s) {
         throw MotError{MOT_ERR_ARG, "FFT length too large for one shared-memory tile"};
     MOT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
     MOT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-    const int threads = TB >= 8 ? 256 : 128;
+    // whole rounds of the product step: Hw = P / 2 + 1 is odd, and 33 x 4 pairs on 128 threads
+    // would take a second round for 4 of them (every round holds the FP64 units in full)
+    const int lanes = a.Hw * TB * a.split, rounds = (lanes + 255) / 256;
+    const int threads = ((lanes + rounds - 1) / rounds + 31) / 32 * 32;
     kern<<<(a.plane + TB - 1) / TB, threads, sm, s>>>(a);
     MOT_LAUNCH_CHECK();
 }
@@ -344,13 +382,25 @@ void zmac(mot_ctx* c, int n, bool fwd, int L, const typename CT<R>::c* const* fa
     a.rl.P = c->ax[2].P;
     a.rl.n = c->ax[2].nrad;
     for (int i = 0; i < 16; ++i) a.rl.r[i] = c->ax[2].rad[i];
+    // Lanes that share the lags of a bin: an FP64 instruction holds its sub-partition for 64
+    // cycles whatever its lanes do, so a small grid spreads its products over the GPU
+    // (8^3, 15 lags, 1,296 bin pairs: 35 us without the split)
+    a.split = 1;
+    const long long items = (long long)a.plane * a.Hw;
+    while (sizeof(R) == 8 && a.split < 8 && a.L >= 2 * a.split &&
+           2 * a.split * items <= 32LL * 8 * c->nsm)
+        a.split *= 2;
     // TB = 8 where that gives two blocks per SM at least and two blocks fit an SM's shared
-    // memory; TB = 2 for small planes (16^3: 18 blocks of 8) and long lines
+    // memory (FP64 only: FP32 comes here with small planes); fewer for small planes
+    // (16 x 9: 18 blocks of 8) and long lines
     const bool wide = a.plane >= 16LL * c->nsm && zmac_smem<R>(a.Pw, 8) <= 110 * 1024;
     const bool mid = a.plane >= 4LL * c->nsm && zmac_smem<R>(a.Pw, 4) <= 200 * 1024;
-    if (wide) launch_len<R, 8>(a, s);
-    else if (mid) launch_len<R, 4>(a, s);
-    else launch_len<R, 2>(a, s);
+    if constexpr (sizeof(R) == 8) {
+        if (wide) return launch_len<R, 8>(a, s);
+    }
+    if (mid) launch_len<R, 4>(a, s);
+    else if (a.plane >= 2LL * c->nsm) launch_len<R, 2>(a, s);
+    else launch<R, 1, 1, 1>(a, s);
 }
 
 template void zmac<double>(mot_ctx*, int, bool, int, const double2* const*, int, cudaStream_t);
