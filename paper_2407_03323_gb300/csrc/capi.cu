@@ -154,7 +154,9 @@ void solve_alloc(mot_ctx* c) {
     }
     MOT_CUDA_TRY(cudaMalloc(&c->fit, sizeof(double) * mot::kFitWords));
     MOT_CUDA_TRY(cudaMalloc(&c->fit_part, sizeof(double) * mot::kFitSums * c->epi_blocks));
-    MOT_CUDA_TRY(cudaMalloc(&c->red, sizeof(double) * 3 * std::max(c->cg_blocks, 1)));
+    // [3][blocks] doubles, then (16-byte aligned) [2][blocks] exchange words
+    MOT_CUDA_TRY(cudaMalloc(&c->red, sizeof(double) * (7 * (size_t)c->cg_blocks + 1)));
+    MOT_CUDA_TRY(cudaMemset(c->red, 0, sizeof(double) * (7 * (size_t)c->cg_blocks + 1)));
     MOT_CUDA_TRY(cudaMalloc(&c->dstatus, sizeof(int) * mot::kStatusWords));
     MOT_CUDA_TRY(cudaMemset(c->dstatus, 0, sizeof(int) * mot::kStatusWords));
 }

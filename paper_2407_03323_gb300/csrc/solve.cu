@@ -69,15 +69,19 @@ constexpr double kFitPivot = 1e-13;        // relative pivot below which a vecto
 
 struct FitRecord {
     double c[kFit];
-    double scale;      // a power of two near 1 / rms(b) (0: none yet)
     int use;           // 0: quadratic extrapolation
-    int pad;
+    int e;             // 2^e is near 1 / rms(b)
 };
 struct FitState {      // device, zeroed with the march state
     FitRecord rec[2];                  // step n reads rec[n & 1]; its solve writes the other
     double gram[kSlots * kSlots];      // <b_i, b_j> by ring slot
 };
 static_assert(sizeof(FitState) <= sizeof(double) * mot::kFitWords, "fit state size");
+
+// 2^e, |e| <= 1000 (double) / 120 (float)
+__device__ __forceinline__ double pow2d(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+__device__ __forceinline__ float pow2f(int e) { return __int_as_float((127 + e) << 23); }
+__device__ __forceinline__ bool is_zero(double v) { return (__double_as_longlong(v) << 1) == 0; }
 
 // b ring slot of step n - i, s0 = n mod kSlots
 __device__ __forceinline__ int fslot(int s0, int i) {
@@ -106,11 +110,15 @@ struct EpiArgs {
     double* part;          // [kSums][gridDim]
 };
 
-// One thread per voxel, its three components: the AoS excitation row and the four
-// factors are read once and coalesced.  All loads of a component come before its stores
-// (the new slot Jn lies in the same ring the loads read from).  ADJ: the adjoint march
-// (see below).  FP32-history keeps x and b of earlier steps as floats: they only shape the
-// start and the fit; the residual of the start that is stored is formed in float pairs.
+// One thread per voxel, its three components: the AoS excitation row and the factors are
+// read once and coalesced.  All loads of a voxel come before its stores (the new slot Jn
+// lies in the same ring the loads read from).  ADJ: the adjoint march (see below).
+// Bound by FP64 issue: an FP64 instruction holds its sub-partition for 64 cycles, so the
+// terms are arranged for few of them (b = ((e - g1 j1) - delta_2 j2 ..) / chi + hist: three
+// per component with FIR3), vacuum voxels with nothing but zeros in them take none, there
+// is no division (scales are powers of two), and FP32-history forms its dot products in
+// FP32: it keeps x and b of earlier steps as floats, which only shape the start and the
+// fit; the residual of the start that is stored is formed in float pairs.
 template <typename R, bool ADJ>
 __global__ void __launch_bounds__(NT) k_epilogue(const __grid_constant__ EpiArgs a) {
     constexpr bool DF = std::is_same<R, float>::value;
@@ -119,49 +127,60 @@ __global__ void __launch_bounds__(NT) k_epilogue(const __grid_constant__ EpiArgs
     const R* hist = static_cast<const R*>(a.hist);
     const FitRecord& rec = a.fit->rec[a.n & 1];
     const bool use = rec.use != 0;
-    double c[kFit];
-    float cf[kFit];
+    const float scf = DF ? pow2f(rec.e) : 1.f;
+    D c[kFit];
 #pragma unroll
-    for (int i = 0; i < kFit; ++i) {
-        c[i] = use ? rec.c[i] : (i == 0 ? 3.0 : i == 1 ? -3.0 : i == 2 ? 1.0 : 0.0);
-        cf[i] = (float)c[i];
-    }
-    const double sc = rec.scale == 0.0 ? 1.0 : rec.scale;
-    const float scf = (float)sc;
-    double bb = 0.0, xin = 0.0;
-    D dots[kFit];
+    for (int i = 0; i < kFit; ++i)
+        c[i] = use ? (D)rec.c[i] : (D)(i == 0 ? 3.0 : i == 1 ? -3.0 : i == 2 ? 1.0 : 0.0);
+    const double* r1 = a.Jring + jslot(a.s0, 1, a.jring, st);
+    const double* r2 = a.Jring + jslot(a.s0, 2, a.jring, st);
+    double* Jn = a.Jring + jslot(a.s0, 0, a.jring, st);
+    const double d1 = a.tp.n > 1 ? a.tp.d[1] : 0.0, d2 = a.tp.n > 2 ? a.tp.d[2] : 0.0;
+    double xin = 0.0;
+    D bb = 0, dots[kFit];
 #pragma unroll
     for (int i = 0; i < kFit; ++i) dots[i] = 0;
     for (long long m = (long long)blockIdx.x * blockDim.x + threadIdx.x; m < M;
          m += (long long)gridDim.x * blockDim.x) {
-        const double f0 = a.f[m], ichi = a.f[M + m], f2 = a.f[2 * M + m], chi = a.f[3 * M + m];
-        const bool active = ichi > 0.0;
-        const double* r1 = a.Jring + jslot(a.s0, 1, a.jring, st);
-        double* Jn = a.Jring + jslot(a.s0, 0, a.jring, st);
-        double e[3], j1[3], P[3], x0[3] = {0.0, 0.0, 0.0};
+        const double f0 = a.f[m], ichi = a.f[M + m];
+        const bool active = !is_zero(ichi);
+        double t[3], j1[3], j2[3] = {0.0, 0.0, 0.0};
+        bool zero = true;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             const long long i = k * M + m;
-            e[k] = a.En ? a.En[m * 3 + k] : 0.0;
+            t[k] = a.En ? a.En[m * 3 + k] : 0.0;
             j1[k] = r1[i];
-            P[k] = ADJ ? f0 * j1[k] - (double)hist[i] : f0 * j1[k] - chi * (double)hist[i];
+            if (a.tp.n > 2) j2[k] = r2[i];
+            zero = zero && is_zero(t[k]) && is_zero(j1[k]) && is_zero(j2[k]);
         }
-        for (int l = 1; l < a.tp.n; ++l) {
-            const double* rl = a.Jring + jslot(a.s0, l, a.jring, st);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) P[k] += a.tp.d[l] * (l == 1 ? j1[k] : rl[k * M + m]);
-        }
-        if (!active) {
+        if (!active && zero && a.tp.n <= 3) {      // vacuum at rest
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                const double rhs = e[k] - P[k];
+                if (ADJ) a.rhs[k * M + m] = (double)hist[k * M + m];
+                Jn[k * M + m] = 0.0;
+            }
+            continue;
+        }
+        const double g1 = f0 + d1;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) t[k] -= g1 * j1[k] + d2 * j2[k];
+        for (int l = 3; l < a.tp.n; ++l) {
+            const double* rl = a.Jring + jslot(a.s0, l, a.jring, st);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) t[k] -= a.tp.d[l] * rl[k * M + m];
+        }
+        if (!active) {
+            const double f2 = a.f[2 * M + m];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
                 if (ADJ) {
                     // the solve's iterate must vanish off the active set; vacuum voxels
                     // get their lambda after the solve (k_adj_post), when mu is known
-                    a.rhs[k * M + m] = rhs;
+                    a.rhs[k * M + m] = t[k] + (double)hist[k * M + m];
                     Jn[k * M + m] = 0.0;
                 } else {
-                    const double x = rhs * f2;
+                    const double x = t[k] * f2;     // chi = 0: no field term
                     Jn[k * M + m] = x;
                     xin += x * x;
                 }
@@ -171,8 +190,8 @@ __global__ void __launch_bounds__(NT) k_epilogue(const __grid_constant__ EpiArgs
         double b[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            b[k] = ADJ ? e[k] - P[k] : (e[k] - P[k]) * ichi;
-            bb += b[k] * b[k];
+            const double h = (double)hist[k * M + m];
+            b[k] = ADJ ? t[k] + h : t[k] * ichi + h;
         }
         if constexpr (DF) {
             float bh[3], xs[3] = {0.f, 0.f, 0.f};
@@ -180,6 +199,7 @@ __global__ void __launch_bounds__(NT) k_epilogue(const __grid_constant__ EpiArgs
             for (int k = 0; k < 3; ++k) {
                 bh[k] = (float)b[k];
                 a.bl[k * M + m] = (float)(b[k] - (double)bh[k]);
+                bb += (bh[k] * scf) * (bh[k] * scf);
             }
 #pragma unroll
             for (int i = 0; i < kFit; ++i) {
@@ -188,17 +208,17 @@ __global__ void __launch_bounds__(NT) k_epilogue(const __grid_constant__ EpiArgs
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
                     const float2 w = v[k * M];
-                    xs[k] += cf[i] * w.x;
+                    xs[k] += c[i] * w.x;
                     dots[i] += (bh[k] * scf) * (w.y * scf);
                 }
             }
             if (!use) {   // quadratic extrapolation from the FP64 ring
-                const double* r2 = a.Jring + jslot(a.s0, 2, a.jring, st);
-                const double* r3 = a.Jring + jslot(a.s0, 3, a.jring, st);
+                const double* q2 = a.Jring + jslot(a.s0, 2, a.jring, st);
+                const double* q3 = a.Jring + jslot(a.s0, 3, a.jring, st);
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
-                    x0[k] = 3.0 * j1[k] - 3.0 * r2[k * M + m] + r3[k * M + m];
-                    xs[k] = (float)(ADJ ? chi * x0[k] : x0[k]);
+                    const double x0 = 3.0 * j1[k] - 3.0 * q2[k * M + m] + q3[k * M + m];
+                    xs[k] = (float)(ADJ ? a.f[3 * M + m] * x0 : x0);
                 }
             }
             float2* v0 = a.xb + (long long)a.bs * st + m;
@@ -206,6 +226,7 @@ __global__ void __launch_bounds__(NT) k_epilogue(const __grid_constant__ EpiArgs
             for (int k = 0; k < 3; ++k) v0[k * M] = make_float2(xs[k], bh[k]);
             a.x0[m] = make_float4(xs[0], xs[1], xs[2], 0.f);
         } else {
+            double x0[3] = {0.0, 0.0, 0.0};
 #pragma unroll
             for (int i = 0; i < kFit; ++i) {
                 if (i >= (use ? a.nv : 3)) break;
@@ -221,31 +242,43 @@ __global__ void __launch_bounds__(NT) k_epilogue(const __grid_constant__ EpiArgs
                 for (int k = 0; k < 3; ++k) dots[i] += b[k] * rb[k * M + m];
             }
             double* b0 = a.b64 + (long long)a.bs * st;
+            const double chi = ADJ ? a.f[3 * M + m] : 1.0;
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
+                bb += b[k] * b[k];
                 b0[k * M + m] = b[k];
                 Jn[k * M + m] = ADJ ? chi * x0[k] : x0[k];
             }
         }
     }
-    // block sums: every thread leaves its kSums values in shared memory, then one warp per
-    // value adds them (an FP64 addition costs 16 cycles of an SM for each warp, so the
-    // shuffles run on one partial per lane instead of on every thread's)
-    __shared__ double red[kSums][NT + 1];
+    // block sums: every thread leaves its values in shared memory, then one warp per value
+    // adds them (the shuffles run on one partial per lane instead of on every thread's).
+    // FP32-history partials stay scaled by 4^e (fit_block unscales the totals).
+    __shared__ D red[kFit + 1][NT + 1];
+    __shared__ double redx[NT / 32];
     red[0][threadIdx.x] = bb;
 #pragma unroll
-    for (int i = 0; i < kFit; ++i) red[1 + i][threadIdx.x] = (double)dots[i];
-    red[kSums - 1][threadIdx.x] = xin;
-    __syncthreads();
-    const int nw = blockDim.x >> 5;
-    for (int q = threadIdx.x >> 5; q < kSums; q += nw) {
-        double v = 0.0;
-        for (int t = threadIdx.x & 31; t < (int)blockDim.x; t += 32) v += red[q][t];
+    for (int i = 0; i < kFit; ++i) red[1 + i][threadIdx.x] = dots[i];
+    const bool vac = __syncthreads_or(!is_zero(xin));
+    const int nw = blockDim.x >> 5, lane = threadIdx.x & 31;
+    for (int q = threadIdx.x >> 5; q < kFit + 1; q += nw) {
+        D v = 0;
+        for (int t = lane; t < (int)blockDim.x; t += 32) v += red[q][t];
         for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if ((threadIdx.x & 31) == 0) {
-            if (DF && q >= 1 && q <= kFit) v = v / sc / sc;
-            a.part[(long long)q * gridDim.x + blockIdx.x] = v;
-        }
+        if (lane == 0) a.part[(long long)q * gridDim.x + blockIdx.x] = (double)v;
+    }
+    double* xpart = a.part + (long long)(kSums - 1) * gridDim.x + blockIdx.x;
+    if (!vac) {
+        if (threadIdx.x == 0) *xpart = 0.0;
+        return;
+    }
+    for (int o = 16; o > 0; o >>= 1) xin += __shfl_down_sync(0xffffffffu, xin, o);
+    if (lane == 0) redx[threadIdx.x >> 5] = xin;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double v = 0.0;
+        for (int w = 0; w < nw; ++w) v += redx[w];
+        *xpart = v;
     }
 }
 
@@ -269,16 +302,19 @@ struct CGArgs {
     float4* q;
     float4* e;
     // FP32-history: (x, b) of this step, SoA; low parts of b; the low parts of the diagonal
-    // (its high parts are diag32); low parts of x in later refinements
+    // (its high parts are diag32); the start for the neighbours' reads, and the low parts of
+    // x in later refinements
     float2* xb;
     const float* bl;
     const float* diag_lo;
     float4* xl;
-    double* red;          // [3][nw]
+    double* red;          // [3][nw] FP64 partial sums: norm; wide residual sums
+    float4* red4;         // [2][nw] exchanged partial sums (values, sequence number)
     double tol2;          // outer tolerance^2 (relative to ||b||^2)
+    float tol;
     float inv_theta;      // Chebyshev: 1 / theta, theta = (lmin + lmax) / 2
     int n_cheb;           // most Chebyshev iterations per refinement (<= MAXCHEB)
-    double log_rate;      // log of the Chebyshev convergence rate (< 0)
+    float inv_log2_rate;  // 1 / log2 of the Chebyshev convergence rate (< 0)
     float c1[MAXCHEB];    // d_{k+1} = c1[k] d_k + c2[k] r_{k+1}
     float c2[MAXCHEB];
     int max_iter;         // cap on total inner iterations
@@ -575,7 +611,7 @@ template <class T>
 __device__ __forceinline__ void cheb_pass_tiled(const CGArgs& a, const float4* __restrict__ dk,
                                                 float4* __restrict__ dn, float c1, float c2,
                                                 bool first, bool last, float4 (*sd)[T::HALO],
-                                                double& rr_p) {
+                                                float& rr_p) {
     int tile = blockIdx.x;
     if (tile < a.ntiles) load_halo<T>(a, dk, sd[0], a.tiles[tile]);
     cp_async_commit();
@@ -615,7 +651,7 @@ __device__ __forceinline__ void cheb_pass_tiled(const CGArgs& a, const float4* _
             const long long m = mv[v];
             a.e[m] = e;
             a.r[m] = r;
-            if (last) rr_p += (double)r.x * r.x + (double)r.y * r.y + (double)r.z * r.z;
+            if (last) rr_p += r.x * r.x + r.y * r.y + r.z * r.z;
             dn[m] = make_float4(c1 * c.x + c2 * r.x, c1 * c.y + c2 * r.y, c1 * c.z + c2 * r.z, 0.f);
         }
         __syncthreads();
@@ -737,12 +773,13 @@ __device__ __forceinline__ void wait_failed(const CGArgs& a) {
     atomicCAS(a.status + 2, 0, a.step);
 }
 
-// One iteration on the resident tile; k = 0 starts from r (complete in memory, d_0 = r /
-// theta), later ones wait for the words tagged `seq`.  Returns false on a timed-out wait.
-template <class T>
+// One iteration on the resident tile: waits for the halo words tagged seq + k (with RFIRST
+// the first iteration starts from r instead, complete in memory: d_0 = r / theta).  Returns
+// false on a timed-out wait.
+template <class T, bool RFIRST>
 __device__ __forceinline__ bool cheb_pass_resident(const CGArgs& a, int k, unsigned seq, bool last,
                                                    float4 (*sd)[T::HALO], Resident<T>& t,
-                                                   double& rr_p) {
+                                                   float& rr_p) {
     typedef Resident<T> RT;
     if ((int)blockIdx.x >= a.ntiles) return true;
     const float4* dk = (k & 1) ? a.q : a.p;
@@ -756,7 +793,7 @@ __device__ __forceinline__ bool cheb_pass_resident(const CGArgs& a, int k, unsig
         sb[T::hidx(lx, ly, lz)] = t.m[v] >= 0 ? t.d[v] : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     float4 h[RT::HPT];
-    if (k == 0) {
+    if (RFIRST && k == 0) {
 #pragma unroll
         for (int i = 0; i < RT::HPT; ++i)
             if (t.hm[i] >= 0) {
@@ -796,7 +833,7 @@ __device__ __forceinline__ bool cheb_pass_resident(const CGArgs& a, int k, unsig
         e.x += c.x; e.y += c.y; e.z += c.z;
         r.x -= o0; r.y -= o1; r.z -= o2;
         if (last) {
-            rr_p += (double)r.x * r.x + (double)r.y * r.y + (double)r.z * r.z;
+            rr_p += r.x * r.x + r.y * r.y + r.z * r.z;
         } else {
             const float c1 = a.c1[k], c2 = a.c2[k];
             t.d[v] = make_float4(c1 * c.x + c2 * r.x, c1 * c.y + c2 * r.y, c1 * c.z + c2 * r.z,
@@ -807,17 +844,28 @@ __device__ __forceinline__ bool cheb_pass_resident(const CGArgs& a, int k, unsig
     return true;
 }
 
-// Double-float residual pass on the tiles (FP32-history): q holds x (its high part with
-// PAIR, the low part in xl), zero on inactive voxels.  Writes r scaled by sc and (not RES)
-// the first Chebyshev direction d_0 = r / theta on active voxels and adds |r|^2 (unscaled) and, on
-// the first pass, |b|^2 to the thread's partial sums.
+// Partial sums of a thread: |r|^2 and |b|^2 scaled by 4^e in FP32, or (wide) unscaled in FP64
+struct Sums {
+    float rr, bb;
+    double rrw, bbw;
+    __device__ void add_r(const float* r, bool wide, float sc) {
+        if (wide) rrw += (double)r[0] * r[0] + (double)r[1] * r[1] + (double)r[2] * r[2];
+        rr += (r[0] * sc) * (r[0] * sc) + (r[1] * sc) * (r[1] * sc) + (r[2] * sc) * (r[2] * sc);
+    }
+};
+
+// Double-float residual pass on the tiles (FP32-history): the start is in xl; later (PAIR) x
+// is in q (high) and xl (low); zero on inactive voxels.  Leaves r scaled by sc = 2^e and the
+// first Chebyshev direction d_0 = r / theta of the active voxels: resident tiles keep them
+// and send d_0 out as the words of iteration 0, the others store both.
 template <class T, bool PAIR, bool RES>
 __device__ __forceinline__ void residual_df_tiled(const CGArgs& a, float4 (*sd)[T::HALO], float sc,
-                                                  double& rr_p, double& bb_p, bool first) {
+                                                  bool wide, Sums& sum, Resident<T>& res,
+                                                  unsigned seq) {
     const long long M = a.M;
     for (int tile = blockIdx.x; tile < a.ntiles; tile += a.nw) {
         const int org = a.tiles[tile];
-        load_halo<T>(a, a.q, sd[0], org);
+        load_halo<T>(a, PAIR ? a.q : a.xl, sd[0], org);
         if (PAIR) load_halo<T>(a, a.xl, sd[1], org);
         cp_async_commit();
         long long mv[T::VPT];
@@ -850,15 +898,23 @@ __device__ __forceinline__ void residual_df_tiled(const CGArgs& a, float4 (*sd)[
                 vh = sd[0][hc + o];
                 if constexpr (PAIR) vl = sd[1][hc + o];
             };
-            float4 r = residual_df_at<PAIR>(dhv[v], dlv[v], bh[v], bl[v], load);
-            rr_p += (double)r.x * r.x + (double)r.y * r.y + (double)r.z * r.z;
-            if (first)
-                bb_p += (double)bh[v][0] * bh[v][0] + (double)bh[v][1] * bh[v][1] +
-                        (double)bh[v][2] * bh[v][2];
-            r = make_float4(r.x * sc, r.y * sc, r.z * sc, 0.f);
-            a.r[mv[v]] = r;
-            if (!RES)
-                a.p[mv[v]] = make_float4(r.x * a.inv_theta, r.y * a.inv_theta, r.z * a.inv_theta, 0.f);
+            const float4 r4 = residual_df_at<PAIR>(dhv[v], dlv[v], bh[v], bl[v], load);
+            const float rv[3] = {r4.x, r4.y, r4.z};
+            sum.add_r(rv, wide, sc);
+            const float* h = bh[v];
+            if (wide) sum.bbw += (double)h[0] * h[0] + (double)h[1] * h[1] + (double)h[2] * h[2];
+            sum.bb += (h[0] * sc) * (h[0] * sc) + (h[1] * sc) * (h[1] * sc) + (h[2] * sc) * (h[2] * sc);
+            const float4 r = make_float4(r4.x * sc, r4.y * sc, r4.z * sc, 0.f);
+            const float4 d = make_float4(r.x * a.inv_theta, r.y * a.inv_theta, r.z * a.inv_theta,
+                                         __uint_as_float(seq));
+            if constexpr (RES) {
+                res.r[v] = r;
+                res.d[v] = d;
+                st_word(a.p + mv[v], d);
+            } else {
+                a.r[mv[v]] = r;
+                a.p[mv[v]] = d;
+            }
         }
         __syncthreads();
     }
@@ -905,6 +961,60 @@ __device__ __forceinline__ double grid_total(const double* red, int nb) {
     const double r = s_tot;
     __syncthreads();
     return r;
+}
+
+// Sums over the worker blocks without a grid barrier: a block publishes its two partial
+// sums and a sequence number as one 16-byte word, and every block adds all words in the
+// same order once they carry that number (bounded waits).  Two sets of words alternate: a
+// block publishes to a set again only after it has collected the other, which every block
+// publishes after it has read the first.
+template <int NTH>
+__device__ __forceinline__ void publish(const CGArgs& a, int set, unsigned tag, float v0, float v1) {
+    __shared__ float sh[2][NTH / 32];
+    for (int o = 16; o > 0; o >>= 1) {
+        v0 += __shfl_down_sync(0xffffffffu, v0, o);
+        v1 += __shfl_down_sync(0xffffffffu, v1, o);
+    }
+    if ((threadIdx.x & 31) == 0) { sh[0][threadIdx.x >> 5] = v0; sh[1][threadIdx.x >> 5] = v1; }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        v0 = v1 = 0.f;
+#pragma unroll
+        for (int k = 0; k < NTH / 32; ++k) { v0 += sh[0][k]; v1 += sh[1][k]; }
+        st_word(a.red4 + set * a.nw + blockIdx.x, make_float4(v0, v1, 0.f, __uint_as_float(tag)));
+    }
+}
+template <int NTH>
+__device__ __forceinline__ bool collect(const CGArgs& a, int set, unsigned tag, float& v0, float& v1) {
+    __shared__ float sh[2][NTH / 32];
+    int ok = 1;
+    v0 = v1 = 0.f;
+    for (int b = threadIdx.x; b < a.nw; b += NTH) {
+        const float4* p = a.red4 + set * a.nw + b;
+        float4 w = ld_word(p);
+        if (__float_as_uint(w.w) != tag) {
+            const long long t0 = clock64();
+            for (int spin = 1;; ++spin) {
+                w = ld_word(p);
+                if (__float_as_uint(w.w) == tag) break;
+                if ((spin & 255) != 0) continue;
+                if (ld_acquire_gpu(a.bar + 2) != 0u) { ok = 0; break; }
+                if (clock64() - t0 > a.bar_budget) { wait_failed(a); ok = 0; break; }
+            }
+        }
+        v0 += w.x;
+        v1 += w.y;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        v0 += __shfl_xor_sync(0xffffffffu, v0, o);
+        v1 += __shfl_xor_sync(0xffffffffu, v1, o);
+    }
+    if ((threadIdx.x & 31) == 0) { sh[0][threadIdx.x >> 5] = v0; sh[1][threadIdx.x >> 5] = v1; }
+    if (!__syncthreads_and(ok)) return false;
+    v0 = v1 = 0.f;
+#pragma unroll
+    for (int k = 0; k < NTH / 32; ++k) { v0 += sh[0][k]; v1 += sh[1][k]; }
+    return true;
 }
 
 // Grid-wide barrier of a cooperative launch (every block resident) with a bounded wait.
@@ -978,7 +1088,7 @@ __global__ void __launch_bounds__(NT) k_barrier_check(int* w, long long budget, 
 // the normal equations by a Cholesky factorisation in ring order, newest first (a vector
 // whose remainder after the newer ones is below kFitPivot of its square is left out).
 // The matrix is scaled to unit diagonal.  Lane i of warp 0 holds row i.
-__device__ void fit_block(const CGArgs& a) {
+template <bool DF> __device__ void fit_block(const CGArgs& a) {
     __shared__ double t[kSums];
     const int lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
     for (int q = threadIdx.x >> 5; q < kSums - 1; q += nwarp) {
@@ -986,7 +1096,9 @@ __device__ void fit_block(const CGArgs& a) {
         double v = 0.0;
         for (int k = lane; k < a.nepi; k += 32) v += p[k];
         for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) t[q] = v;
+        // FP32-history sums are scaled by 4^e of this step
+        const double un = DF ? pow2d(-2 * a.fit->rec[a.step & 1].e) : 1.0;
+        if (lane == 0) t[q] = v * un;
     }
     __syncthreads();
     if (threadIdx.x >= 32) return;
@@ -1033,9 +1145,10 @@ __device__ void fit_block(const CGArgs& a) {
     if (lane == 0) {
         // a poor or degenerate fit (also NaN anywhere in it) falls back to extrapolation
         rec.use = a.nv >= 3 && bb > 0.0 && bb - yy <= kFitPoor * bb && mag < 1e4;
-        int e = 0;
-        if (bb > 0.0 && bb < 1e300) frexp(sqrt(bb / (3.0 * (double)a.nact)), &e);
-        rec.scale = ldexp(1.0, max(-120, min(120, -e)));
+        // 2^e near 1 / rms(b), from the exponents alone
+        const double mean = bb / (3.0 * (double)a.nact);
+        const int lim = DF ? 120 : 500, ex = ((__double2hiint(mean) >> 20) & 2047) - 1023;
+        rec.e = mean > 0.0 && ex < 1024 ? max(-lim, min(lim, -(ex >> 1))) : 0;
         gram[s0 * kSlots + s0] = bb;
     }
     if (row) {
@@ -1074,12 +1187,23 @@ __device__ __forceinline__ double applyA64_row(const CGArgs& a, const double* __
 }
 
 template <bool SPLIT, bool RES>
-__device__ __forceinline__ void residual64(const CGArgs& a, double sc, double& rr_p, double& bb_p,
-                                           bool first) {
+__device__ __forceinline__ void residual64(const CGArgs& a, int e, bool first, bool wide, Sums& sum) {
     const long long M = a.M;
+    const double sc = pow2d(e);
     const int lane = threadIdx.x & 31;
     const long long warp = (long long)(threadIdx.x >> 5) * a.nw + blockIdx.x;
     const long long warps = (long long)(blockDim.x >> 5) * a.nw;
+    // one component: sums of the scaled values, r in FP32
+    auto part = [&](double b, double r) {
+        const float rs = (float)(r * sc);
+        sum.rr += rs * rs;
+        if (first) {
+            const float bs = (float)(b * sc);
+            sum.bb += bs * bs;
+        }
+        if (wide) { sum.rrw += r * r; sum.bbw += b * b; }
+        return rs;
+    };
     if constexpr (SPLIT) {
         const long long groups = (a.nact + 31) / 32;
         float* rf = reinterpret_cast<float*>(a.r);
@@ -1093,32 +1217,25 @@ __device__ __forceinline__ void residual64(const CGArgs& a, double sc, double& r
             if (c == 0) o = applyA64_row<0>(a, a.x, m, mask);
             else if (c == 1) o = applyA64_row<1>(a, a.x, m, mask);
             else o = applyA64_row<2>(a, a.x, m, mask);
-            const double b = a.b[c * M + m], r = b - o;
-            if (first) bb_p += b * b;
-            rr_p += r * r;
-            const float rs = (float)(r * sc);
+            const double b = a.b[c * M + m];
+            const float rs = part(b, b - o);
             rf[4LL * m + c] = rs;
             if (!RES) pf[4LL * m + c] = rs * a.inv_theta;
         }
     } else {
         for (long long i = warp * 32 + lane; i < a.nact; i += warps * 32) {
             const int m = a.act[i];
-            double o[3], r[3];
+            double o[3];
             applyA64(a, a.x, m, a.nmask[i], o);
-            float4 rs = make_float4(0.f, 0.f, 0.f, 0.f);
+            float rs[3];
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 const double b = a.b[k * M + m];
-                r[k] = b - o[k];
-                if (first) bb_p += b * b;
-                rr_p += r[k] * r[k];
+                rs[k] = part(b, b - o[k]);
             }
-            rs.x = (float)(r[0] * sc);
-            rs.y = (float)(r[1] * sc);
-            rs.z = (float)(r[2] * sc);
-            a.r[m] = rs;
+            a.r[m] = make_float4(rs[0], rs[1], rs[2], 0.f);
             if (!RES)
-                a.p[m] = make_float4(rs.x * a.inv_theta, rs.y * a.inv_theta, rs.z * a.inv_theta, 0.f);
+                a.p[m] = make_float4(rs[0] * a.inv_theta, rs[1] * a.inv_theta, rs[2] * a.inv_theta, 0.f);
         }
     }
 }
@@ -1132,18 +1249,27 @@ __device__ __forceinline__ void residual64(const CGArgs& a, double sc, double& r
 // start residual added, the step is done without forming b - A x again; otherwise the next
 // refinement starts from a new true residual.  All blocks take identical decisions because
 // every block sums the same per-block partials in the same order.
-//   RES: a block has at most one tile (see Resident; no grid barrier in the iteration).
+//   RES: a block has at most one tile (see Resident; no grid barrier in the iteration).  In
+//     FP32-history the first two iterations run while the sums of the residual are still
+//     on their way: at least three are made anyway, and x is not touched by them.
 //   SPLIT: FP64 residual by components (see residual64).
-constexpr double kDrift = 1e-6;
+// The scalars that steer the iteration are FP32 numbers scaled by powers of two (an FP64
+// square root, logarithm and division for every warp cost 4 to 7 us of a 45 us solve).  Sums
+// that leave FP32's range at the scale of the step before (wide) are formed again in FP64,
+// which gives the new scale.
+constexpr float kDrift = 1e-6f;
+// sequence numbers that a residual and two iterations whose results are dropped may have used
+constexpr unsigned kAborted = 4;
 
 template <bool DF, class T, bool RES, bool SPLIT>
 __global__ void __launch_bounds__(T::NTH, RES ? 4 : 3) k_cg(const __grid_constant__ CGArgs a) {
     __shared__ __align__(16) float4 sd[2][T::HALO];      // tile halos of the passes
     if ((int)blockIdx.x == a.nw) {       // the fit for the next step, beside the solve
-        fit_block(a);
+        fit_block<DF>(a);
         return;
     }
-    unsigned target = 0, seq = a.seq;
+    unsigned target = 0, seq = a.seq, tag = a.seq;
+    int set = 0;
     auto gsync = [&] {
         return grid_barrier(a.bar, a.nw, target, a.bar_budget, a.status, a.step);
     };
@@ -1159,18 +1285,17 @@ __global__ void __launch_bounds__(T::NTH, RES ? 4 : 3) k_cg(const __grid_constan
         resident_init<T>(a, res, sd);
         __syncthreads();     // its zeros, before a residual pass copies halos over them
     }
-    double bb = 0.0, rr = 0.0, xx = 0.0;
-    int its = 0, outer = 0;
-    bool first = true, converged = false, nonfinite = false, zero = false;
-    bool stored = false;     // x (with its norm in xx) is in a.x; else DF's start is in xb only
-    double sc = a.fit->rec[a.step & 1].scale;
-    if (sc == 0.0) sc = 1.0;
+    float bb = 0.f, rr = 0.f;            // scaled by 4^e0 and 4^e
+    int e = a.fit->rec[a.step & 1].e, e0 = e;
+    int its = 0, outer = 0, wides = 0;
+    bool first = true, wide = false, converged = false, nonfinite = false, zero = false;
+    bool stored = false;     // x is in a.x; else DF's start is in xb only
     // f(voxel, its correction e) over the block's share of the active voxels
     auto each = [&](auto&& f) {
         if constexpr (RES) {
 #pragma unroll
             for (int v = 0; v < T::VPT; ++v)
-                if (res.m[v] >= 0) f(res.m[v], res.e[v]);
+                if (res.m[v] >= 0) f(res.m[v], res.e[v], v);
         } else {
             struct ME { int m; float4 e; };
             grid_loop<4>(t0, a.nact, gs,
@@ -1180,107 +1305,139 @@ __global__ void __launch_bounds__(T::NTH, RES ? 4 : 3) k_cg(const __grid_constan
                     v.e = a.e[v.m];
                     return v;
                 },
-                [&](long long, const ME& v) { f(v.m, v.e); });
+                [&](long long, const ME& v) { f(v.m, v.e, 0); });
         }
     };
     while (true) {
-        // ---- residual, scaled by sc
-        double rr_p = 0.0, bb_p = 0.0;
+        // ---- residual, scaled by 2^e
+        Sums sum = {0.f, 0.f, 0.0, 0.0};
         if constexpr (DF) {
-            if (stored) residual_df_tiled<T, true, RES>(a, sd, (float)sc, rr_p, bb_p, first);
-            else residual_df_tiled<T, false, RES>(a, sd, (float)sc, rr_p, bb_p, first);
+            if (stored) residual_df_tiled<T, true, RES>(a, sd, pow2f(e), wide, sum, res, seq);
+            else residual_df_tiled<T, false, RES>(a, sd, pow2f(e), wide, sum, res, seq);
         } else {
-            residual64<SPLIT, RES>(a, sc, rr_p, bb_p, first);
+            residual64<SPLIT, RES>(a, e, first, wide, sum);
         }
-        block_sum2<T::NTH>(rr_p, bb_p);
-        if (threadIdx.x == 0) {
-            red0[blockIdx.x] = rr_p;
-            if (first) red1[blockIdx.x] = bb_p;
+        if (wide) {                      // sums in FP64: the true scale, or none
+            block_sum2<T::NTH>(sum.rrw, sum.bbw);
+            if (threadIdx.x == 0) { red0[blockIdx.x] = sum.rrw; red1[blockIdx.x] = sum.bbw; }
+            if (!gsync()) return;
+            const double rw = grid_total(red0, nb), bw = grid_total(red1, nb);
+            if (!(rw <= 1e300) || !(bw <= 1e300)) { nonfinite = true; break; }
+            if (bw == 0.0) { zero = converged = true; break; }
+            int ex = 0;
+            frexp(sqrt(first ? bw : rw), &ex);
+            e = max(-(DF ? 120 : 500), min(DF ? 120 : 500, -ex));
+            if (first) e0 = e;
+            wide = false;
+            seq += kAborted;
+            if (!gsync()) return;
+            continue;
         }
-        if (!gsync()) return;
-        rr = grid_total(red0, nb);
-        if (first) bb = grid_total(red1, nb);
-        if (!(rr <= 1e300) || !(bb <= 1e300)) { nonfinite = true; break; }
-        if (bb == 0.0) { zero = converged = true; break; }
-        if (rr <= a.tol2 * bb) { converged = true; break; }
-        if (first && rr > bb) {
-            // a start worse than none (an abrupt change of the excitation): from zero
-            each([&](long long m, const float4&) {
+        publish<T::NTH>(a, set, ++tag, sum.rr, sum.bb);
+        float rr_p = 0.f;
+        constexpr bool early = RES && DF;     // iterate while the sums travel
+        bool ran2 = false;
+        if constexpr (RES) {
 #pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    if (DF) a.xb[k * M + m].x = 0.f;
-                    else a.x[k * M + m] = 0.0;
-                }
-                if (DF) a.q[m] = make_float4(0.f, 0.f, 0.f, 0.f);
-            });
-            first = false;
+            for (int v = 0; v < T::VPT; ++v) res.e[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        if (early && !stored) {
+            for (int k = 0; k < 2; ++k)
+                if (!cheb_pass_resident<T, false>(a, k, seq + k, false, sd, res, rr_p)) return;
+            ran2 = true;
+        } else {
+            if (!gsync()) return;        // r complete (with x as pairs: q read by all)
+        }
+        float b_tot;
+        if (!collect<T::NTH>(a, set, tag, rr, b_tot)) return;
+        set ^= 1;
+        if (first) bb = b_tot;
+        const float sb = sqrtf(bb), goal = a.tol * sb * pow2f(max(-120, min(120, e - e0))),
+                    have = sqrtf(rr);
+        // a NaN or Inf in the sums, a vanishing right-hand side or a scale far off
+        const bool off = !(rr <= 1e14f) || (first && !(bb >= 1e-10f && bb <= 1e14f)) ||
+                         (!first && have > goal && rr < 1e-30f);
+        const bool odd = off && ++wides <= 3;      // (the FP64 sums settle it the first time)
+        if (!odd && !(rr <= 1e30f)) { nonfinite = true; break; }
+        if (!odd && have <= goal) { converged = true; break; }
+        if (odd || (first && rr > bb)) {
+            if (!odd) {
+                // a start worse than none (an abrupt change of the excitation): from zero
+                each([&](long long m, const float4&, int) {
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        if (DF) a.xb[k * M + m].x = 0.f;
+                        else a.x[k * M + m] = 0.0;
+                    }
+                    if (DF) a.xl[m] = make_float4(0.f, 0.f, 0.f, 0.f);
+                });
+                first = false;
+            }
+            wide = odd;
+            seq += kAborted;
             if (!gsync()) return;
             continue;
         }
         first = false;
         if (outer >= a.max_outer || its >= a.max_iter) break;
-        if (!(rr * sc * sc >= 1e-24 && rr * sc * sc <= 1e24)) {
-            // the scale of the previous step does not bring this residual into FP32's range
-            sc = 1.0 / sqrt(rr);
-            if (!gsync()) return;        // every block has read the partial sums
-            continue;
-        }
         // ---- Chebyshev: iterations for the reduction still needed, never asking for more
         // than FP32 can deliver in one refinement (5e-6).  FP64 aims a factor 10 below the
         // tolerance (the march's error is then the history's rounding, 1e-14 on the 8^3
         // cube, not the solve's 2e-13); the FP32 history's own error is far above its
         // tolerance already
-        const double back = 1.0 / sc, goal = sqrt(a.tol2 * bb), have = sqrt(rr);
-        const double need = fmax((DF ? 0.8 : 0.1) * (goal - kDrift * have) / have, 5e-6);
-        const int n_it = min(a.n_cheb, max(2, (int)ceil(log(0.5 * need) / a.log_rate)));
-        rr_p = 0.0;
+        const float need = fmaxf((DF ? 0.8f : 0.1f) * (goal - kDrift * have) / have, 5e-6f);
+        const int n_it = min(a.n_cheb, max(3, (int)ceilf(log2f(0.5f * need) * a.inv_log2_rate)));
         if constexpr (RES) {
+            if constexpr (!DF) {
 #pragma unroll
-            for (int v = 0; v < T::VPT; ++v) {
-                res.e[v] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (res.m[v] < 0) continue;
-                const float4 r = __ldcg(a.r + res.m[v]);
-                res.r[v] = r;
-                res.d[v] = make_float4(r.x * a.inv_theta, r.y * a.inv_theta, r.z * a.inv_theta, 0.f);
+                for (int v = 0; v < T::VPT; ++v) {
+                    if (res.m[v] < 0) continue;
+                    const float4 r = __ldcg(a.r + res.m[v]);
+                    res.r[v] = r;
+                    res.d[v] = make_float4(r.x * a.inv_theta, r.y * a.inv_theta, r.z * a.inv_theta, 0.f);
+                }
             }
-            for (int k = 0; k < n_it; ++k)
-                if (!cheb_pass_resident<T>(a, k, seq + k, k == n_it - 1, sd, res, rr_p)) return;
+            for (int k = ran2 ? 2 : 0; k < n_it; ++k)
+                if (!cheb_pass_resident<T, !DF>(a, k, seq + k, k == n_it - 1, sd, res, rr_p)) return;
             seq += n_it;
         } else {
             float4* dk = a.p;
             float4* dn = a.q;
             for (int k = 0; k < n_it; ++k) {
                 cheb_pass_tiled<T>(a, dk, dn, a.c1[k], a.c2[k], k == 0, k == n_it - 1, sd, rr_p);
-                if (!gsync()) return;
+                if (k < n_it - 1 && !gsync()) return;
                 float4* tmp = dk; dk = dn; dn = tmp;
             }
         }
         its += n_it;
         ++outer;
-        // ---- x += e / sc (DF: the float start becomes an FP64 x) and its norm
-        xx = 0.0;
-        each([&](long long m, const float4& e) {
-            const float ec[3] = {e.x, e.y, e.z};
+        publish<T::NTH>(a, set, ++tag, rr_p, 0.f);
+        if (!RES && !gsync()) return;    // the update deals the voxels out by list
+        // ---- x += e / 2^e (DF: the float start becomes an FP64 x)
+        const double back = pow2d(-e);
+        each([&](long long m, const float4& d, int) {
+            const float ec[3] = {d.x, d.y, d.z};
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 double x = DF && !stored ? (double)a.xb[k * M + m].x : a.x[k * M + m];
                 x += back * (double)ec[k];
                 a.x[k * M + m] = x;
                 if (DF) a.xb[k * M + m].x = (float)x;
-                xx += x * x;
             }
         });
         stored = true;
-        block_sum2<T::NTH>(rr_p, xx);
-        if (threadIdx.x == 0) red1[blockIdx.x] = rr_p;
-        if (!gsync()) return;
-        const double left = sqrt(grid_total(red1, nb)) * back;
+        float left, dummy;
+        if (!collect<T::NTH>(a, set, tag, left, dummy)) return;
+        set ^= 1;
+        left = sqrtf(left);
         if (left + kDrift * have <= goal) { converged = true; break; }
-        if (!(left <= 1e300)) { nonfinite = true; break; }
+        if (!(left <= 1e14f)) { nonfinite = true; break; }
         // ---- not there yet: a new residual (DF: of x as float pairs)
-        sc = 1.0 / left;
+        e = max(-(DF ? 120 : 500), min(DF ? 120 : 500,
+                e - (((__float_as_int(fmaxf(left, 1e-37f)) >> 23) & 255) - 127)));
         if constexpr (DF) {
-            each([&](long long m, const float4&) {
+            if (!gsync()) return;        // q: every block is done with its halo words
+            each([&](long long m, const float4&, int) {
                 float4 h, l;
                 df_split(a.x[m], h.x, l.x);
                 df_split(a.x[M + m], h.y, l.y);
@@ -1289,28 +1446,27 @@ __global__ void __launch_bounds__(T::NTH, RES ? 4 : 3) k_cg(const __grid_constan
                 a.q[m] = h;
                 a.xl[m] = l;
             });
-            if (!gsync()) return;
         }
+        if (!gsync()) return;
     }
     // ---- an x not stored yet, and its norm.  NaN or Inf in the right-hand side or the
     // start: no iteration can help; J_n is returned as NaN so that the monitor and the
     // caller see it
-    if (!stored || nonfinite) {
-        double dummy = 0.0;
-        xx = 0.0;
-        each([&](long long m, const float4&) {
+    double xx = 0.0, unused = 0.0;
+    each([&](long long m, const float4&, int) {
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                double x = DF && !stored ? (double)a.xb[k * M + m].x : a.x[k * M + m];
-                if (zero) x = 0.0;
-                if (nonfinite) x = __longlong_as_double(0x7ff8000000000000LL);
+        for (int k = 0; k < 3; ++k) {
+            double x = DF && !stored ? (double)a.xb[k * M + m].x : a.x[k * M + m];
+            if (zero) x = 0.0;
+            if (nonfinite) x = __longlong_as_double(0x7ff8000000000000LL);
+            if (!stored || nonfinite) {
                 a.x[k * M + m] = x;
                 if (DF) a.xb[k * M + m].x = (float)x;
-                xx += x * x;
             }
-        });
-        block_sum2<T::NTH>(xx, dummy);
-    }
+            xx += x * x;
+        }
+    });
+    block_sum2<T::NTH>(xx, unused);
     // the last block to finish adds up the norm (fixed order) and leaves the barrier words
     // zero for the next launch: every other block has passed its last barrier
     __shared__ int s_last;
@@ -1691,7 +1847,7 @@ void epilogue(mot_ctx* c, int n, const double* En, cudaStream_t s) {
     a.b64 = c->b_ring;
     a.xb = reinterpret_cast<float2*>(c->xb_ring);
     a.bl = c->b_lo;
-    a.x0 = reinterpret_cast<float4*>(c->cg32) + 2 * c->M;
+    a.x0 = reinterpret_cast<float4*>(c->cg_xl);
     a.rhs = c->rhs;
     a.fit = reinterpret_cast<const FitState*>(c->fit);
     a.part = c->fit_part;
@@ -1728,10 +1884,12 @@ CGArgs make_cg_args(mot_ctx* c, int n, double* norm2_out) {
     a.e = a.r + 3 * c->M;
     a.xl = c->cg_xl ? reinterpret_cast<float4*>(c->cg_xl) : nullptr;
     a.red = c->red;
+    a.red4 = reinterpret_cast<float4*>(c->red + 3LL * c->cg_blocks + (c->cg_blocks & 1));
     a.tol2 = c->tol * c->tol;
+    a.tol = (float)c->tol;
     a.inv_theta = c->cheb_inv_theta;
     a.n_cheb = c->cheb_n;
-    a.log_rate = c->cheb_log_rate;
+    a.inv_log2_rate = (float)(std::log(2.0) / c->cheb_log_rate);
     for (int k = 0; k < MAXCHEB; ++k) {
         a.c1[k] = k < c->cheb_n ? c->cheb_c1[k] : 0.f;
         a.c2[k] = k < c->cheb_n ? c->cheb_c2[k] : 0.f;
