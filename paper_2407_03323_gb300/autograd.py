@@ -93,7 +93,7 @@ class MarchFunction(torch.autograd.Function):
             g.index_add_(1, fctx.probe_idx, grad_out[lo - 1:hi])
             return g
 
-        adj = Context(fctx.eps, fctx.taps, **fctx.options)
+        adj = ctx.share()      # the forward context's setup (quadrature, spectra) serves both
         try:
             adj.adjoint_begin(N)
             if fctx.J_all is not None:

@@ -139,7 +139,8 @@ __global__ void __launch_bounds__(NT) k_mac(const float* __restrict__ ghat,
 
 // temporal spectra of the level of length S over lags [a, a + S):
 // H(w) = sum_{m=0}^{lmax-a} Ghat_{a+m} exp(-2 pi i w m / (2S)), lmax = min(a + S - 1, ell),
-// w = 0..S (the rest follows by H(2S - w) = conj H(w)); out [w][6][octant bin], one
+// w = 0..S (the rest follows by H(2S - w) = conj H(w)), times 1 / (2S), the normalisation of
+// the firing's transforms (a power of two, so exact); out [w][6][octant bin], one
 // plane per component so that a warp over consecutive bins reads one contiguous run
 template <typename R>
 __global__ void k_level_spec(const R* __restrict__ ghat, long long noct, int S, int a, int lmax,
@@ -161,10 +162,11 @@ __global__ void k_level_spec(const R* __restrict__ ghat, long long noct, int S, 
         }
     }
     C* op = out + (long long)w * 6 * noct + o;
+    const double scale = 1.0 / (2 * S);
     for (int c = 0; c < 6; ++c) {
         C v;
-        v.x = acc[c].x;
-        v.y = acc[c].y;
+        v.x = acc[c].x * scale;
+        v.y = acc[c].y * scale;
         op[c * noct] = v;
     }
 }
@@ -263,18 +265,13 @@ __global__ void __launch_bounds__(NT) k_far(FarArgs<R> a) {
     }
     __syncthreads();
     C* Y = fft_tile<C, L3>(X, other, P, a.rl.r, a.rl.n, ld, stw, +1);
-    const R scale = (R)1 / (R)P;
     for (int it = threadIdx.x; it < a.S * L3; it += blockDim.x) {
         const int j = it / L3, t = it % L3;
         const int comp = t / TB, bb = t % TB;
         if (ku0 + bb >= a.Hu) continue;
         const long long slot = s_out[j];
         C* dst = a.acc + (slot * 3 + comp) * a.nbins + row + bb;
-        const C y = Y[(a.S + j) * ld + t];
-        C v;
-        v.x = y.x * scale;
-        v.y = y.y * scale;
-        *dst = v;
+        *dst = Y[(a.S + j) * ld + t];
     }
 }
 
@@ -588,6 +585,38 @@ __device__ __forceinline__ void mirror_bin(const FarArgs<R>& a, long long o, int
     row = ((long long)kw * a.Pv + kv) * a.Hu + ku;
 }
 
+// y = h0 x0 + h1 x1 + h2 x2, twelve chained multiply-adds
+template <typename C>
+__device__ __forceinline__ C row_product(const C& h0, const C& x0, const C& h1, const C& x1,
+                                         const C& h2, const C& x2) {
+    C o;
+    o.x = h0.x * x0.x;
+    o.y = h0.x * x0.y;
+    o.x = fma(-h0.y, x0.y, o.x);
+    o.y = fma(h0.y, x0.x, o.y);
+    o.x = fma(h1.x, x1.x, o.x);
+    o.y = fma(h1.x, x1.y, o.y);
+    o.x = fma(-h1.y, x1.y, o.x);
+    o.y = fma(h1.y, x1.x, o.y);
+    o.x = fma(h2.x, x2.x, o.x);
+    o.y = fma(h2.x, x2.y, o.y);
+    o.x = fma(-h2.y, x2.y, o.x);
+    o.y = fma(h2.y, x2.x, o.y);
+    return o;
+}
+// v, its sign bits flipped where neg (a multiplication by +-1 would be an FP64 instruction)
+__device__ __forceinline__ double flip(double v, bool neg) {
+    return __hiloint2double(__double2hiint(v) ^ (neg ? 0x80000000 : 0), __double2loint(v));
+}
+__device__ __forceinline__ float flip(float v, bool neg) {
+    return __int_as_float(__float_as_int(v) ^ (neg ? 0x80000000 : 0));
+}
+template <typename C> __device__ __forceinline__ C cflip(C v, bool neg) {
+    v.x = flip(v.x, neg);
+    v.y = flip(v.y, neg);
+    return v;
+}
+
 template <typename R, int Q, int T> struct FarRegSmem {
     typedef typename CT<R>::c C;
     static constexpr int P = Q * T, S = P / 2, NB = 32 / T;
@@ -633,7 +662,7 @@ __global__ void __launch_bounds__(96) k_far_reg(FarArgs<R> a) {
     }
     for (int i = threadIdx.x; i < tw_entries<C>(P); i += blockDim.x) sm.tw[i] = a.tw[i];
     __syncthreads();
-    const R sig = comp == 0 ? (R)1 : (comp == 1 ? (fv ? (R)-1 : (R)1) : (fw ? (R)-1 : (R)1));
+    const bool neg = comp == 1 ? fv : comp == 2 ? fw : false;    // sigma of this component
     C x[Q];
     Unroll<0, Q>::run([&](auto q) {
         constexpr int j = decltype(q)::value;
@@ -643,12 +672,12 @@ __global__ void __launch_bounds__(96) k_far_reg(FarArgs<R> a) {
         if (slot >= 0 && live) v = a.ring[((long long)slot * 3 + comp) * a.nbins + row];
         x[j] = v;
     });
-    fft_dif_reg<C, Q, T, -1>(x, sm.tw, t);
+    // one thread per line: natural order (dft_ct); otherwise bit-reversed
+    if constexpr (T == 1) dft_ct<Q, -1>(x);
+    else fft_dif_reg<C, Q, T, -1>(x, sm.tw, t);
     Unroll<0, Q>::run([&](auto q) {
         constexpr int j = decltype(q)::value;
-        C v = x[j];
-        v.x *= sig; v.y *= sig;
-        sm.X[t * Q + j][comp][line] = v;
+        sm.X[t * Q + j][comp][line] = cflip(x[j], neg);
     });
     cp_async_commit_wait();
     __syncthreads();
@@ -659,27 +688,26 @@ __global__ void __launch_bounds__(96) k_far_reg(FarArgs<R> a) {
     const int brt = bitrev<T>(t);
     Unroll<0, Q>::run([&](auto q) {
         constexpr int j = decltype(q)::value;
-        const int w = bitrev<Q>(j) * T + brt;      // frequency of position t Q + j
+        const int w = T == 1 ? j : bitrev<Q>(j) * T + brt;      // frequency of position t Q + j
         const bool cj = w > S;
         const int ws = cj ? P - w : w;
         C h0 = sm.H[ws][i0][line], h1 = sm.H[ws][i1][line], h2 = sm.H[ws][i2][line];
-        if (cj) { h0.y = -h0.y; h1.y = -h1.y; h2.y = -h2.y; }
+        h0.y = flip(h0.y, cj);
+        h1.y = flip(h1.y, cj);
+        h2.y = flip(h2.y, cj);
         const int pos = t * Q + j;
-        x[j] = cadd(cadd(cmul(h0, sm.X[pos][0][line]), cmul(h1, sm.X[pos][1][line])),
-                    cmul(h2, sm.X[pos][2][line]));
+        x[j] = row_product(h0, sm.X[pos][0][line], h1, sm.X[pos][1][line], h2, sm.X[pos][2][line]);
     });
-    fft_dit_reg<C, Q, T, +1>(x, sm.tw, t);
+    if constexpr (T == 1) dft_ct<Q, +1>(x);
+    else fft_dit_reg<C, Q, T, +1>(x, sm.tw, t);
     if (!live) return;
-    const R scale = sig / (R)P;
     // outputs are the last S positions: threads t >= T/2 hold them
     if (t * Q + Q <= S) return;
     Unroll<0, Q>::run([&](auto q) {
         constexpr int j = decltype(q)::value;
         const int pos = t * Q + j;
         if (pos < S) return;
-        C v = x[j];
-        v.x *= scale; v.y *= scale;
-        a.acc[((long long)sm.out[pos - S] * 3 + comp) * a.nbins + row] = v;
+        a.acc[((long long)sm.out[pos - S] * 3 + comp) * a.nbins + row] = cflip(x[j], neg);
     });
 }
 
@@ -765,7 +793,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k_far_4s(FarArgs<
     const int t = ct % T, comp = ct / T;
     const bool athr = tid < F::NA;
     const bool live = athr && bin_live;
-    const R sig = comp == 0 ? (R)1 : (comp == 1 ? (fv ? (R)-1 : (R)1) : (fw ? (R)-1 : (R)1));
+    const bool neg = comp == 1 ? fv : comp == 2 ? fw : false;    // sigma of this component
     C x[Q1];
     if (athr) {
         Unroll<0, Q1>::run([&](auto q) {
@@ -774,14 +802,13 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k_far_4s(FarArgs<
             C v;
             v.x = 0; v.y = 0;
             if (slot >= 0 && live) v = a.ring[((long long)slot * 3 + comp) * a.nbins + row];
-            v.x *= sig; v.y *= sig;
-            x[n2] = v;
+            x[n2] = cflip(v, neg);
         });
-        fft_dif_reg<C, Q1, 1, -1>(x, sm.tw, 0);      // register j holds k2 = bitrev(j)
+        dft_ct<Q1, -1>(x);
         C* yr = sm.Y[F::row(comp, t, bin)];
         Unroll<0, Q1>::run([&](auto q) {
-            constexpr int j = decltype(q)::value;
-            yr[F::col(bitrev<Q1>(j), tid)] = x[j];
+            constexpr int k2 = decltype(q)::value;
+            yr[F::col(k2, tid)] = x[k2];
         });
     }
     cp_async_commit_wait();
@@ -803,11 +830,11 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k_far_4s(FarArgs<
                 constexpr int tt = decltype(q)::value;
                 v[c][tt] = cmul(sm.Y[F::row(c, tt, b)][F::col(k2, F::athread(c, tt, b))], wt[tt]);
             });
-            fft_dif_reg<C, T, 1, -1>(v[c], sm.tw, 0);   // register j holds k1 = bitrev(j)
+            dft_ct<T, -1>(v[c]);
         });
         Unroll<0, T>::run([&](auto q) {
             constexpr int j = decltype(q)::value;
-            const int w = k2 + Q1 * bitrev<T>(j);
+            const int w = k2 + Q1 * j;
             const bool cj = w > S;
             const int ws = cj ? P - w : w;
             const C* hp = &sm.H[ws][b];
@@ -815,16 +842,16 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k_far_4s(FarArgs<
 #pragma unroll
             for (int cc = 0; cc < 6; ++cc) {
                 h[cc] = hp[cc * NB];
-                if (cj) h[cc].y = -h[cc].y;
+                h[cc].y = flip(h[cc].y, cj);
             }
             const C x0 = v[0][j], x1 = v[1][j], x2 = v[2][j];
-            v[0][j] = cadd(cadd(cmul(h[0], x0), cmul(h[3], x1)), cmul(h[4], x2));
-            v[1][j] = cadd(cadd(cmul(h[3], x0), cmul(h[1], x1)), cmul(h[5], x2));
-            v[2][j] = cadd(cadd(cmul(h[4], x0), cmul(h[5], x1)), cmul(h[2], x2));
+            v[0][j] = row_product(h[0], x0, h[3], x1, h[4], x2);
+            v[1][j] = row_product(h[3], x0, h[1], x1, h[5], x2);
+            v[2][j] = row_product(h[4], x0, h[5], x1, h[2], x2);
         });
         Unroll<0, 3>::run([&](auto cq) {
             constexpr int c = decltype(cq)::value;
-            fft_dit_reg<C, T, 1, +1>(v[c], sm.tw, 0);   // register t holds C_t
+            dft_ct<T, +1>(v[c]);
             Unroll<0, T>::run([&](auto q) {
                 constexpr int tt = decltype(q)::value;
                 C w = wt[tt];
@@ -839,16 +866,13 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k_far_4s(FarArgs<
     const C* yr = sm.Y[F::row(comp, t, bin)];
     Unroll<0, Q1>::run([&](auto q) {
         constexpr int j = decltype(q)::value;
-        x[j] = yr[F::col(bitrev<Q1>(j), tid)];
+        x[j] = yr[F::col(j, tid)];
     });
-    fft_dit_reg<C, Q1, 1, +1>(x, sm.tw, 0);          // register n2 holds y[t + T n2]
-    const R scale = sig / (R)P;
+    dft_ct<Q1, +1>(x);
     Unroll<Q1 / 2, Q1>::run([&](auto q) {
         constexpr int n2 = decltype(q)::value;
         const int pos = t + T * n2;                  // >= S
-        C v = x[n2];
-        v.x *= scale; v.y *= scale;
-        a.acc[((long long)sm.out[pos - S] * 3 + comp) * a.nbins + row] = v;
+        a.acc[((long long)sm.out[pos - S] * 3 + comp) * a.nbins + row] = cflip(x[n2], neg);
     });
 }
 
@@ -1004,14 +1028,13 @@ __global__ void __launch_bounds__(128, P <= 16 ? 4 : 2) k_far_fs(FarArgs<float> 
         float sy, sz;
         mirror_of(m, live, bidx, sy, sz);
         if (!live) return;
-        const float sc = 1.f / (float)P;
         Unroll<Q1 / 2, Q1>::run([&](auto q) {
             constexpr int n2 = decltype(q)::value;
             const int pos = t + T * n2;                      // >= S
             float2* dst = a.acc + (long long)sm.out[pos - S] * 3 * a.nbins + bidx;
-            dst[0] = make_float2(sc * y[0][n2].x, sc * y[0][n2].y);
-            dst[a.nbins] = make_float2(sy * sc * y[1][n2].x, sy * sc * y[1][n2].y);
-            dst[2 * a.nbins] = make_float2(sz * sc * y[2][n2].x, sz * sc * y[2][n2].y);
+            dst[0] = y[0][n2];
+            dst[a.nbins] = make_float2(sy * y[1][n2].x, sy * y[1][n2].y);
+            dst[2 * a.nbins] = make_float2(sz * y[2][n2].x, sz * y[2][n2].y);
         });
     };
     float2 x[3][Q1];

@@ -7,6 +7,9 @@
 //     E^s_p(t_n) = sum_{l>=0} sum_m G_l(r_p - r_m) J_{n-l,m},
 // and the transposed operator, the source of the adjoint march for an objective of E^s,
 //     g_{k,m} = sum_{l>=0} sum_p G_l(r_p - r_m)^T W_{k+l,p}         (G_l^T = G_l).
+// Both are bound by FP64 issue (an FP64 instruction holds its sub-partition for 64 cycles:
+// loads and index arithmetic hide behind it), so the nine multiply-adds of a pair, lag and
+// step are chained into the sums and steps that a pair's lags do not reach are skipped.
 // The elements of every probe-voxel pair are windows of WIN lags from the element
 // quadrature (mot_probe_setup); both products run in FP64 with one thread per voxel
 // and a block of time steps per thread.
@@ -44,8 +47,10 @@ __global__ void __launch_bounds__(PT) k_probe_field(const double* __restrict__ t
     const double* tp = tab + (long long)p * 6 * mot::WIN * M;
     for (long long m = threadIdx.x; m < M; m += PT) {
         const int lo = l0[(long long)p * M + m];
+        if (n0 + TBN <= lo) continue;                    // every J_{n-l} lies before the first
 #pragma unroll
         for (int i = 0; i < mot::WIN; ++i) {
+            if (n0 + TBN <= lo + i) break;
             const double gxx = tp[(0 * mot::WIN + i) * M + m], gyy = tp[(1 * mot::WIN + i) * M + m];
             const double gzz = tp[(2 * mot::WIN + i) * M + m], gxy = tp[(3 * mot::WIN + i) * M + m];
             const double gxz = tp[(4 * mot::WIN + i) * M + m], gyz = tp[(5 * mot::WIN + i) * M + m];
@@ -55,9 +60,9 @@ __global__ void __launch_bounds__(PT) k_probe_field(const double* __restrict__ t
                 if (n < 0 || n0 + k >= N) continue;
                 const double* j = J + ((long long)n * M + m) * 3;
                 const double j0 = j[0], j1 = j[1], j2 = j[2];
-                acc[k][0] += gxx * j0 + gxy * j1 + gxz * j2;
-                acc[k][1] += gxy * j0 + gyy * j1 + gyz * j2;
-                acc[k][2] += gxz * j0 + gyz * j1 + gzz * j2;
+                acc[k][0] = fma(gxx, j0, fma(gxy, j1, fma(gxz, j2, acc[k][0])));
+                acc[k][1] = fma(gxy, j0, fma(gyy, j1, fma(gyz, j2, acc[k][1])));
+                acc[k][2] = fma(gxz, j0, fma(gyz, j1, fma(gzz, j2, acc[k][2])));
             }
         }
     }
@@ -95,8 +100,10 @@ __global__ void __launch_bounds__(PT) k_probe_transpose(const double* __restrict
     for (int p = 0; p < P; ++p) {
         const double* tp = tab + (long long)p * 6 * mot::WIN * M;
         const int lo = l0[(long long)p * M + m];
+        if (k0 + lo >= N) continue;                      // every W_{k+l} lies past the last
 #pragma unroll
         for (int i = 0; i < mot::WIN; ++i) {
+            if (k0 + lo + i >= N) break;
             const double gxx = tp[(0 * mot::WIN + i) * M + m], gyy = tp[(1 * mot::WIN + i) * M + m];
             const double gzz = tp[(2 * mot::WIN + i) * M + m], gxy = tp[(3 * mot::WIN + i) * M + m];
             const double gxz = tp[(4 * mot::WIN + i) * M + m], gyz = tp[(5 * mot::WIN + i) * M + m];
@@ -106,9 +113,9 @@ __global__ void __launch_bounds__(PT) k_probe_transpose(const double* __restrict
                 if (n >= N) continue;
                 const double* w = W + ((long long)n * P + p) * 3;
                 const double w0 = w[0], w1 = w[1], w2 = w[2];
-                acc[k][0] += gxx * w0 + gxy * w1 + gxz * w2;
-                acc[k][1] += gxy * w0 + gyy * w1 + gyz * w2;
-                acc[k][2] += gxz * w0 + gyz * w1 + gzz * w2;
+                acc[k][0] = fma(gxx, w0, fma(gxy, w1, fma(gxz, w2, acc[k][0])));
+                acc[k][1] = fma(gxy, w0, fma(gyy, w1, fma(gyz, w2, acc[k][1])));
+                acc[k][2] = fma(gxz, w0, fma(gyz, w1, fma(gzz, w2, acc[k][2])));
             }
         }
     }
