@@ -50,6 +50,8 @@ __global__ void __launch_bounds__(NT) k_fwd_x(const double* __restrict__ in, int
     const long long npairs = 3LL * W * VP;
     const long long pair0 = (long long)blockIdx.x * TB;
     load_tw(stw, tw, P);
+    pdl_trigger();
+    pdl_wait();
     // load: z = a + i b, zero-padded; batches of kLoadBatch loads in flight per thread
     for (int it0 = threadIdx.x; it0 < TB * P; it0 += kLoadBatch * blockDim.x) {
         double va[kLoadBatch], vb[kLoadBatch];
@@ -124,6 +126,8 @@ __global__ void __launch_bounds__(NT) k_inv_x(const typename CT<R>::c* __restric
     const long long npairs = 3LL * W * VP;
     const long long pair0 = (long long)blockIdx.x * TB;
     load_tw(stw, tw, P);
+    pdl_trigger();
+    pdl_wait();
     for (int it0 = threadIdx.x; it0 < TB * Hu; it0 += kLoadBatch * blockDim.x) {
         C Aq[kLoadBatch], Bq[kLoadBatch];
 #pragma unroll
@@ -240,6 +244,8 @@ __global__ void k_fwd_x4s(const double* __restrict__ in, int U, int V, int W,
     const long long npairs = 3LL * W * VP;
     const long long pair0 = (long long)blockIdx.x * kXL;
     for (int i = threadIdx.x; i < tw_entries<C>(P); i += blockDim.x) stw[i] = tw[i];
+    pdl_trigger();
+    pdl_wait();
     // z = a + i b of the two rows of a pair; positions >= U are the zero padding
     for (int it = threadIdx.x; it < kXL * U; it += blockDim.x) {
         const int t = it / U, j = it % U;
@@ -295,6 +301,8 @@ __global__ void k_inv_x4s(const typename CT<R>::c* __restrict__ in, int U, int V
     const long long npairs = 3LL * W * VP;
     const long long pair0 = (long long)blockIdx.x * kXL;
     for (int i = threadIdx.x; i < tw_entries<C>(P); i += blockDim.x) stw[i] = tw[i];
+    pdl_trigger();
+    pdl_wait();
     // Z[k] = A[k] + i B[k] and Z[P-k] = conj A[k] + i conj B[k] from the two halves
     for (int it = threadIdx.x; it < kXL * Hu; it += blockDim.x) {
         const int t = it / Hu, k = it % Hu;
@@ -377,6 +385,8 @@ __global__ void __launch_bounds__(NT) k_mid(const typename CT<R>::c* __restrict_
     const C* src = in + src_off;
     C* dst = out + dst_off;
     load_tw(stw, tw, P);
+    pdl_trigger();
+    pdl_wait();
     for (int it = threadIdx.x; it < P * TB; it += blockDim.x) {
         const int j = it / TB;
         const bool ok = live && j < a.n_in;
@@ -413,6 +423,8 @@ k_mid4s(const typename CT<R>::c* __restrict__ in, typename CT<R>::c* __restrict_
     const C* src = in + src_off;
     C* dst = out + dst_off;
     for (int i = threadIdx.x; i < tw_entries<C>(P); i += blockDim.x) stw[i] = tw[i];
+    pdl_trigger();
+    pdl_wait();
     __syncthreads();
     if (warp < P1) {
         const int n1 = warp;
@@ -483,16 +495,17 @@ template <typename K> void set_smem(K kern, size_t bytes) {
 
 template <typename R, int P1, int P2>
 void launch_mid4s(const typename CT<R>::c* in, typename CT<R>::c* out,
-                  const typename CT<R>::c* tw, const MidArgs& a, int nblocks, cudaStream_t s) {
+                  const typename CT<R>::c* tw, const MidArgs& a, int nblocks, bool dep,
+                  cudaStream_t s) {
     typedef typename CT<R>::c C;
     const size_t sm = sizeof(C) * ((size_t)P1 * P2 * 32 + (size_t)tw_entries<C>(P1 * P2));
     constexpr int threads = 32 * (P1 > P2 ? P1 : P2);
     if (a.dir < 0) {
         set_smem(k_mid4s<R, P1, P2, -1>, sm);
-        k_mid4s<R, P1, P2, -1><<<nblocks, threads, sm, s>>>(in, out, tw, a);
+        launch_dependent(dep, k_mid4s<R, P1, P2, -1>, nblocks, threads, sm, s, in, out, tw, a);
     } else {
         set_smem(k_mid4s<R, P1, P2, +1>, sm);
-        k_mid4s<R, P1, P2, +1><<<nblocks, threads, sm, s>>>(in, out, tw, a);
+        launch_dependent(dep, k_mid4s<R, P1, P2, +1>, nblocks, threads, sm, s, in, out, tw, a);
     }
     MOT_LAUNCH_CHECK();
 }
@@ -501,20 +514,20 @@ void launch_mid4s(const typename CT<R>::c* in, typename CT<R>::c* out,
 // lengths that have a factor pair below, the generic Stockham tile otherwise
 template <typename R>
 void mid_pass(const typename CT<R>::c* in, typename CT<R>::c* out, const AxisFFT& ax,
-              const MidArgs& a, cudaStream_t s) {
+              const MidArgs& a, bool dep, cudaStream_t s) {
     const int P = ax.P;
     const long long lines = 3LL * a.n_o2 * a.Hu;
     const int nb32 = (int)((lines + 31) / 32);
     switch (P) {
-        case 64: launch_mid4s<R, 8, 8>(in, out, table<R>(ax), a, nb32, s); return;
-        case 96: launch_mid4s<R, 8, 12>(in, out, table<R>(ax), a, nb32, s); return;
-        case 210: launch_mid4s<R, 14, 15>(in, out, table<R>(ax), a, nb32, s); return;
+        case 64: launch_mid4s<R, 8, 8>(in, out, table<R>(ax), a, nb32, dep, s); return;
+        case 96: launch_mid4s<R, 8, 12>(in, out, table<R>(ax), a, nb32, dep, s); return;
+        case 210: launch_mid4s<R, 14, 15>(in, out, table<R>(ax), a, nb32, dep, s); return;
         default: break;
     }
     constexpr int TB = Tile<R>::TB;
     const size_t sm = smem_bytes<R>(P);
     set_smem(k_mid<R>, sm);
-    k_mid<R><<<(int)((lines + TB - 1) / TB), NT, sm, s>>>(in, out, table<R>(ax),
+    launch_dependent(dep, k_mid<R>, (int)((lines + TB - 1) / TB), NT, sm, s, in, out, table<R>(ax),
                                                                     radix_list(ax), a);
     MOT_LAUNCH_CHECK();
 }
@@ -569,11 +582,11 @@ void launch_x4s(bool fwd, mot_ctx* c, const double* Jsoa, typename CT<R>::c* spe
     const int blocks = (int)((npairs + kXL - 1) / kXL);
     if (fwd) {
         set_smem(k_fwd_x4s<R, P1, P2>, sm);
-        k_fwd_x4s<R, P1, P2><<<blocks, threads, sm, s>>>(Jsoa, c->U, c->V, c->W, spec,
+        launch_dependent(mot::dependent_launches(c), k_fwd_x4s<R, P1, P2>, blocks, threads, sm, s, Jsoa, c->U, c->V, c->W, spec,
                                                          table<R>(c->ax[0]), scale);
     } else {
         set_smem(k_inv_x4s<R, P1, P2>, sm);
-        k_inv_x4s<R, P1, P2><<<blocks, threads, sm, s>>>(spec, c->U, c->V, c->W, real,
+        launch_dependent(mot::dependent_launches(c), k_inv_x4s<R, P1, P2>, blocks, threads, sm, s, spec, c->U, c->V, c->W, real,
                                                          table<R>(c->ax[0]));
     }
     MOT_LAUNCH_CHECK();
@@ -602,7 +615,7 @@ void fft_forward_xy(mot_ctx* c, const double* Jsoa, cudaStream_t s, const double
         const long long npairs = 3LL * W * ((V + 1) / 2);
         const size_t sm = smem_bytes<R>(Pu);
         set_smem(k_fwd_x<R>, sm);
-        k_fwd_x<R><<<(int)((npairs + TB - 1) / TB), NT, sm, s>>>(Jsoa, U, V, W, hb.tmp1,
+        launch_dependent(mot::dependent_launches(c), k_fwd_x<R>, (int)((npairs + TB - 1) / TB), NT, sm, s, Jsoa, U, V, W, hb.tmp1,
                                                                  table<R>(c->ax[0]),
                                                                  radix_list(c->ax[0]), scale);
         MOT_LAUNCH_CHECK();
@@ -614,7 +627,7 @@ void fft_forward_xy(mot_ctx* c, const double* Jsoa, cudaStream_t s, const double
         a.in_c = (long long)W * V * Hu; a.in_o = (long long)V * Hu; a.in_a = Hu;
         a.out_c = (long long)W * Pv * Hu; a.out_o = (long long)Pv * Hu; a.out_a = Hu;
         a.Hu = Hu; a.dir = -1;
-        mid_pass<R>(hb.tmp1, hb.tmp2, c->ax[1], a, s);
+        mid_pass<R>(hb.tmp1, hb.tmp2, c->ax[1], a, dependent_launches(c), s);
     }
 }
 
@@ -627,7 +640,7 @@ void fft_forward_z(mot_ctx* c, typename CT<R>::c* out, cudaStream_t s) {
     a.in_c = (long long)W * Pv * Hu; a.in_o = Hu; a.in_a = (long long)Pv * Hu;
     a.out_c = (long long)Pw * Pv * Hu; a.out_o = Hu; a.out_a = (long long)Pv * Hu;
     a.Hu = Hu; a.dir = -1;
-    mid_pass<R>(hbuf<R>(c).tmp2, out, c->ax[2], a, s);
+    mid_pass<R>(hbuf<R>(c).tmp2, out, c->ax[2], a, dependent_launches(c), s);
 }
 
 template <typename R>
@@ -650,14 +663,14 @@ void fft_inverse_yx(mot_ctx* c, R* out, cudaStream_t s) {
         a.in_c = (long long)W * Pv * Hu; a.in_o = (long long)Pv * Hu; a.in_a = Hu;
         a.out_c = (long long)W * V * Hu; a.out_o = (long long)V * Hu; a.out_a = Hu;
         a.Hu = Hu; a.dir = +1;
-        mid_pass<R>(hb.tmp2, hb.tmp1, c->ax[1], a, s);
+        mid_pass<R>(hb.tmp2, hb.tmp1, c->ax[1], a, dependent_launches(c), s);
     }
     // x: c2r
     if (!x_pass_codelet<R>(false, c, nullptr, hb.tmp1, out, nullptr, s)) {
         const long long npairs = 3LL * W * ((V + 1) / 2);
         const size_t sm = smem_bytes<R>(Pu);
         set_smem(k_inv_x<R>, sm);
-        k_inv_x<R><<<(int)((npairs + TB - 1) / TB), NT, sm, s>>>(hb.tmp1, U, V, W, out,
+        launch_dependent(mot::dependent_launches(c), k_inv_x<R>, (int)((npairs + TB - 1) / TB), NT, sm, s, hb.tmp1, U, V, W, out,
                                                                  table<R>(c->ax[0]),
                                                                  radix_list(c->ax[0]));
         MOT_LAUNCH_CHECK();
@@ -673,7 +686,7 @@ void fft_inverse(mot_ctx* c, const typename CT<R>::c* in, R* out, cudaStream_t s
     a.in_c = (long long)Pw * Pv * Hu; a.in_o = Hu; a.in_a = (long long)Pv * Hu;
     a.out_c = (long long)W * Pv * Hu; a.out_o = Hu; a.out_a = (long long)Pv * Hu;
     a.Hu = Hu; a.dir = +1;
-    mid_pass<R>(in, hbuf<R>(c).tmp2, c->ax[2], a, s);
+    mid_pass<R>(in, hbuf<R>(c).tmp2, c->ax[2], a, dependent_launches(c), s);
     fft_inverse_yx<R>(c, out, s);
 }
 

@@ -81,6 +81,8 @@ __global__ void __launch_bounds__(NT) k_mac(const float* __restrict__ ghat,
     typedef float R;
     typedef float2 C;
     typedef float2 R2;
+    pdl_trigger();
+    pdl_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int mirror = lane >> 3, j = lane & 7;
     const long long o = ((long long)blockIdx.x * (NT / 32) + warp) * 8 + j;
@@ -196,6 +198,8 @@ __global__ void __launch_bounds__(NT) k_far(FarArgs<R> a) {
     constexpr int L3 = 3 * TB;
     constexpr int ld = L3 + 1;
     const int P = 2 * a.S;
+    pdl_trigger();
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* stw = reinterpret_cast<C*>(smem_raw);
     C* b0 = stw + tw_entries<C>(P);
@@ -639,6 +643,8 @@ __global__ void __launch_bounds__(96) k_far_reg(FarArgs<R> a) {
     typedef typename CT<R>::c C;
     typedef FarRegSmem<R, Q, T> SM;
     constexpr int P = SM::P, S = SM::S, NB = SM::NB;
+    pdl_trigger();
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SM& sm = *reinterpret_cast<SM*>(smem_raw);
     const int comp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -719,7 +725,7 @@ void far_launch_reg(mot_ctx* c, FarArgs<R>& a, cudaStream_t s) {
     MOT_CUDA_TRY(cudaFuncSetAttribute(k_far_reg<R, Q, T>,
                                       cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     const long long blocks = 4 * ((c->noct + SM::NB - 1) / SM::NB);
-    k_far_reg<R, Q, T><<<(int)blocks, 96, sizeof(SM), s>>>(a);
+    launch_dependent(mot::dependent_launches(c), k_far_reg<R, Q, T>, (int)blocks, 96, sizeof(SM), s, a);
     MOT_LAUNCH_CHECK();
 }
 
@@ -766,6 +772,8 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k_far_4s(FarArgs<
     typedef Far4<R, P> F;
     typedef typename F::C C;
     constexpr int Q1 = F::Q1, T = F::T, NB = F::NB, S = F::S;
+    pdl_trigger();
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     typename F::Smem& sm = *reinterpret_cast<typename F::Smem*>(smem_raw);
     const int tid = threadIdx.x;
@@ -885,7 +893,7 @@ void far_launch_4s(mot_ctx* c, FarArgs<R>& a, cudaStream_t s) {
     MOT_CUDA_TRY(cudaFuncSetAttribute(k_far_4s<R, P>,
                                       cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     const long long blocks = 4 * ((c->noct + F::NB - 1) / F::NB);
-    k_far_4s<R, P><<<(int)blocks, F::NTB, sm_bytes, s>>>(a);
+    launch_dependent(mot::dependent_launches(c), k_far_4s<R, P>, (int)blocks, F::NTB, sm_bytes, s, a);
     MOT_LAUNCH_CHECK();
 }
 
@@ -907,7 +915,7 @@ void far_launch(mot_ctx* c, FarArgs<R>& a, cudaStream_t s) {
     MOT_CUDA_TRY(cudaFuncSetAttribute(k_far<R, TB>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
     MOT_CUDA_TRY(cudaFuncSetAttribute(k_far<R, TB>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     const long long blocks = (long long)c->Hw * c->Hv * 4 * a.ntile;
-    k_far<R, TB><<<(int)blocks, NT, sm, s>>>(a);
+    launch_dependent(mot::dependent_launches(c), k_far<R, TB>, (int)blocks, NT, sm, s, a);
     MOT_LAUNCH_CHECK();
 }
 
@@ -983,6 +991,8 @@ __global__ void __launch_bounds__(128, P <= 16 ? 4 : 2) k_far_fs(FarArgs<float> 
         }
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     }
+    pdl_trigger();
+    pdl_wait();          // the level spectra above are setup constants; the ring is not
     for (int i = tid; i < P; i += F::NTH) {
         const int time = a.w0 + i;
         sm.in[i] = time >= tfirst ? time % a.hring : -1;
@@ -1146,7 +1156,7 @@ void far_launch_fs(mot_ctx* c, FarArgs<float>& a, cudaStream_t s) {
     MOT_CUDA_TRY(cudaFuncSetAttribute(k_far_fs<P>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                       100));
     const long long blocks = (c->noct + F::NB - 1) / F::NB;
-    k_far_fs<P><<<(int)blocks, F::NTH, sm_bytes, s>>>(a);
+    launch_dependent(mot::dependent_launches(c), k_far_fs<P>, (int)blocks, F::NTH, sm_bytes, s, a);
     MOT_LAUNCH_CHECK();
 }
 
@@ -1242,7 +1252,7 @@ void history_step(mot_ctx* c, int n, cudaStream_t s, cudaEvent_t* ev) {
         for (int k = 0; k < nfar; ++k) fs.p[k] = far[k];
         const float scale = (float)(1.0 / ((double)c->ax[0].P * c->ax[1].P * c->ax[2].P));
         const long long nblk = (c->noct + 8 * (NT / 32) - 1) / (8 * (NT / 32));
-        k_mac<<<(int)nblk, NT, 0, s>>>(hb.ghat, hb.jhat_ring, c->hring,
+        launch_dependent(mot::dependent_launches(c), k_mac, (int)nblk, NT, 0, s, hb.ghat, hb.jhat_ring, c->hring,
                                        (int)slot_index(n - 1, c->hring), L, geom(c), scale,
                                        hb.phat, fs);
         MOT_LAUNCH_CHECK();

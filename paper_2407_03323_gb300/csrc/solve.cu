@@ -121,6 +121,8 @@ struct EpiArgs {
 // fit; the residual of the start that is stored is formed in float pairs.
 template <typename R, bool ADJ>
 __global__ void __launch_bounds__(NT) k_epilogue(const __grid_constant__ EpiArgs a) {
+    pdl_trigger();
+    pdl_wait();
     constexpr bool DF = std::is_same<R, float>::value;
     typedef typename std::conditional<DF, float, double>::type D;   // dot products
     const long long M = a.M, st = 3 * M;
@@ -1264,6 +1266,7 @@ constexpr unsigned kAborted = 4;
 template <bool DF, class T, bool RES, bool SPLIT>
 __global__ void __launch_bounds__(T::NTH, RES ? 4 : 3) k_cg(const __grid_constant__ CGArgs a) {
     __shared__ __align__(16) float4 sd[2][T::HALO];      // tile halos of the passes
+    pdl_trigger();                       // (launched as an ordinary, cooperative kernel)
     if ((int)blockIdx.x == a.nw) {       // the fit for the next step, beside the solve
         fit_block<DF>(a);
         return;
@@ -1496,6 +1499,8 @@ __global__ void __launch_bounds__(T::NTH, RES ? 4 : 3) k_cg(const __grid_constan
 
 // SoA slot -> AoS output [m][b]
 __global__ void k_to_aos(const double* __restrict__ x, long long M, double* __restrict__ out) {
+    pdl_trigger();
+    pdl_wait();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= 3 * M) return;
     const long long m = i / 3;
@@ -1851,7 +1856,7 @@ void epilogue(mot_ctx* c, int n, const double* En, cudaStream_t s) {
     a.rhs = c->rhs;
     a.fit = reinterpret_cast<const FitState*>(c->fit);
     a.part = c->fit_part;
-    k_epilogue<R, ADJ><<<c->epi_blocks, c->epi_threads, 0, s>>>(a);
+    launch_dependent(mot::dependent_launches(c), k_epilogue<R, ADJ>, c->epi_blocks, c->epi_threads, 0, s, a);
     MOT_LAUNCH_CHECK();
 }
 
@@ -2032,7 +2037,7 @@ void adjoint_step(mot_ctx* c, int tau, int n, const double* g_aos, const double*
 
 void write_aos(mot_ctx* c, int n, double* out_dev, cudaStream_t s) {
     const long long tot = 3 * c->M;
-    k_to_aos<<<(int)((tot + NT - 1) / NT), NT, 0, s>>>(c->J + slot_index(n, c->jring) * 3 * c->M,
+    launch_dependent(mot::dependent_launches(c), k_to_aos, (int)((tot + NT - 1) / NT), NT, 0, s, c->J + slot_index(n, c->jring) * 3 * c->M,
                                                        c->M, out_dev);
     MOT_LAUNCH_CHECK();
 }

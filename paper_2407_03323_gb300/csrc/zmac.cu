@@ -263,6 +263,8 @@ __global__ void __launch_bounds__(256, 2) k_zmac(const __grid_constant__ ZArgs<R
     C* b1 = b0 + P * ld;
     const int f0 = blockIdx.x * TB;
     load_tw(stw, a.tw, P);
+    pdl_trigger();
+    pdl_wait();
     if (a.fwd) {
         // lines c * TB + t: component c, plane position f0 + t
         const int rows = kFourStep ? a.W : P;      // Stockham reads the zero padding too
@@ -324,7 +326,7 @@ template <typename R> size_t zmac_smem(int P, int TB) {
 }
 
 template <typename R, int TB, int P1, int P2>
-void launch(const ZArgs<R>& a, cudaStream_t s) {
+void launch(mot_ctx* c, const ZArgs<R>& a, cudaStream_t s) {
     const size_t sm = zmac_smem<R>(a.Pw, TB);
     auto kern = k_zmac<R, TB, P1, P2>;
     // the limit is process-wide and Pw varies by context: the device's opt-in maximum,
@@ -340,17 +342,17 @@ void launch(const ZArgs<R>& a, cudaStream_t s) {
     // would take a second round for 4 of them (every round holds the FP64 units in full)
     const int lanes = a.Hw * TB * a.split, rounds = (lanes + 255) / 256;
     const int threads = ((lanes + rounds - 1) / rounds + 31) / 32 * 32;
-    kern<<<(a.plane + TB - 1) / TB, threads, sm, s>>>(a);
+    launch_dependent(mot::dependent_launches(c), kern, (a.plane + TB - 1) / TB, threads, sm, s, a);
     MOT_LAUNCH_CHECK();
 }
 
 template <typename R, int TB>
-void launch_len(const ZArgs<R>& a, cudaStream_t s) {
+void launch_len(mot_ctx* c, const ZArgs<R>& a, cudaStream_t s) {
     switch (a.Pw) {
-        case 64: launch<R, TB, 8, 8>(a, s); break;
-        case 96: launch<R, TB, 8, 12>(a, s); break;
-        case 210: launch<R, TB, 14, 15>(a, s); break;
-        default: launch<R, TB, 1, 1>(a, s);
+        case 64: launch<R, TB, 8, 8>(c, a, s); break;
+        case 96: launch<R, TB, 8, 12>(c, a, s); break;
+        case 210: launch<R, TB, 14, 15>(c, a, s); break;
+        default: launch<R, TB, 1, 1>(c, a, s);
     }
 }
 
@@ -396,11 +398,11 @@ void zmac(mot_ctx* c, int n, bool fwd, int L, const typename CT<R>::c* const* fa
     const bool wide = a.plane >= 16LL * c->nsm && zmac_smem<R>(a.Pw, 8) <= 110 * 1024;
     const bool mid = a.plane >= 4LL * c->nsm && zmac_smem<R>(a.Pw, 4) <= 200 * 1024;
     if constexpr (sizeof(R) == 8) {
-        if (wide) return launch_len<R, 8>(a, s);
+        if (wide) return launch_len<R, 8>(c, a, s);
     }
-    if (mid) launch_len<R, 4>(a, s);
-    else if (a.plane >= 2LL * c->nsm) launch_len<R, 2>(a, s);
-    else launch<R, 1, 1, 1>(a, s);
+    if (mid) launch_len<R, 4>(c, a, s);
+    else if (a.plane >= 2LL * c->nsm) launch_len<R, 2>(c, a, s);
+    else launch<R, 1, 1, 1>(c, a, s);
 }
 
 template void zmac<double>(mot_ctx*, int, bool, int, const double2* const*, int, cudaStream_t);
