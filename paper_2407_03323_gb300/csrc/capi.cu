@@ -344,9 +344,10 @@ mot_status mot_create_padded(const int grid[3], const double h[3], double dt,
                                         cudaMemcpyHostToDevice));
             }
             {
-                const std::vector<int> big = active_tiles(c, chi, 8, 8, 8);
-                const std::vector<int> small = active_tiles(c, chi, 8, 4, 4);
-                const std::vector<int>& tl = mot::solve_shape(c, big, small);
+                const std::vector<int> lists[3] = {active_tiles(c, chi, 8, 4, 4),
+                                                   active_tiles(c, chi, 8, 4, 8),
+                                                   active_tiles(c, chi, 8, 8, 8)};
+                const std::vector<int>& tl = mot::solve_shape(c, lists);
                 MOT_CUDA_TRY(cudaMalloc(&c->tiles, sizeof(int) * std::max<size_t>(tl.size(), 1)));
                 if (!tl.empty())
                     MOT_CUDA_TRY(cudaMemcpy(c->tiles, tl.data(), sizeof(int) * tl.size(),

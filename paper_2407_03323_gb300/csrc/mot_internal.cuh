@@ -143,7 +143,7 @@ struct mot_ctx {
     int* nmask = nullptr;        // per active voxel: in-grid neighbours (27 bits)
     int* tiles = nullptr;        // solve tiles holding active voxels (packed origins)
     int ntiles = 0;
-    int cg_tile = 0;             // tile shape (0: 8^3, 1: 8 x 4 x 4)
+    int cg_tile = 4;             // voxels per thread of the tile: 8x4x4, 8x4x8, 8x8x8
     bool cg_resident = false;    // one tile per block, kept in registers
     int* halo = nullptr;         //   halo voxels of every tile
     bool cg_split = false;       // FP64 residual by components
@@ -300,8 +300,7 @@ template <typename R> void level_spectra(mot_ctx* c);
 // solve.cu
 void solve_step(mot_ctx* c, int n, const double* En, double* norm2_out, cudaStream_t s);
 void stencil_setup(mot_ctx* c);
-const std::vector<int>& solve_shape(mot_ctx* c, const std::vector<int>& big,
-                                    const std::vector<int>& small);
+const std::vector<int>& solve_shape(mot_ctx* c, const std::vector<int> (&tiles)[3]);
 void solve_halo_lists(mot_ctx* c);
 void chebyshev_setup(mot_ctx* c);
 void write_aos(mot_ctx* c, int n, double* out_dev, cudaStream_t s);

@@ -521,25 +521,34 @@ __device__ __forceinline__ float4 residual_df_at(float dh, float dl, const float
 // one-voxel halo (zero outside the grid) in shared memory, then every active voxel updates
 //   e += d_k, r -= A d_k, d_{k+1} = c1 d_k + c2 r.
 // Inactive voxels (diag = 0) hold zeros in every vector and are skipped.
-// Two shapes (mot::solve_tiles chooses): 8 x 8 x 8 with 256 threads where the grid has
-// enough tiles to fill the GPU, and 8 x 4 x 4 with one voxel a thread for the small grids,
-// where a block has at most one tile: it then keeps e, r, the diagonal and its own d in
-// registers for the whole solve and a pass only fetches the halo.
-template <int X, int Y, int Z, int THREADS> struct TileShape {
-    static constexpr int TX = X, TY = Y, TZ = Z, NTH = THREADS;
+// A thread takes VPT voxels next to each other along z, so that the planes of the stencil
+// that they share are read from shared memory once (apply_column).  Tiles of 8 x 4 x 4,
+// 8 x 4 x 8 and 8 x 8 x 8 voxels on 128 threads (VPT = 1, 2, 4): the smallest whose tiles all
+// find a block of their own on the GPU, which then keeps e, r, d and the diagonal in
+// registers for the whole solve and fetches only the halo in a pass; grids with more tiles
+// than that take 8 x 8 x 8 on 256 threads with the vectors in memory (solve_shape).  Solve
+// phase with the 8 x 4 x 4 tile resident or in memory only, and now: 133 x 27 x 21 150 ->
+// 115 us, 48^3 cube 150 -> 109, 56^3 sphere 172 -> 106, 64^3 cube 280 -> 182; in memory, 88^3
+// cube 411 -> 391, sphere 365 -> 321 (three blocks per SM instead of two: 375 and 341).
+template <int X, int Y, int Z, int V> struct TileShape {
+    static constexpr int TX = X, TY = Y, TZ = Z, VPT = V, NTH = X * Y * Z / V;
     static constexpr int HX = X + 2, HY = Y + 2, HZ = Z + 2, HALO = HX * HY * HZ;
-    static constexpr int VPT = X * Y * Z / THREADS;      // voxels per thread
-    static_assert(VPT * THREADS == X * Y * Z, "tile voxels per thread");
-    __device__ static void local(int q, int& lx, int& ly, int& lz) {
-        lx = q % TX; ly = (q / TX) % TY; lz = q / (TX * TY);
+    static_assert(NTH % 32 == 0 && Z % V == 0, "tile shape");
+    // position of the thread's first voxel; voxel v of it lies v further along z
+    __device__ static void local(int& lx, int& ly, int& lz) {
+        lx = threadIdx.x % TX;
+        ly = (threadIdx.x / TX) % TY;
+        lz = threadIdx.x / (TX * TY) * VPT;
     }
     __device__ static int hidx(int lx, int ly, int lz) { return ((lz + 1) * HY + ly + 1) * HX + lx + 1; }
     template <int E> __device__ static constexpr int off() {
         return ((E / 9 - 1) * HY + ((E / 3) % 3 - 1)) * HX + (E % 3 - 1);
     }
 };
-typedef TileShape<8, 8, 8, 256> BigTile;
-typedef TileShape<8, 4, 4, 128> SmallTile;
+typedef TileShape<8, 4, 4, 1> Tile1;
+typedef TileShape<8, 4, 8, 2> Tile2;
+typedef TileShape<8, 8, 8, 4> Tile4;
+typedef TileShape<8, 8, 8, 2> TileMem;   // vectors in memory
 
 __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
     unsigned v;
@@ -577,30 +586,74 @@ __device__ __forceinline__ void load_halo(const CGArgs& a, const float4* __restr
     }
 }
 
-// A d at halo position hc of a staged tile, for a voxel of diagonal dg
+// A d at the thread's VPT voxels (one above the other, the first at halo position hc), for
+// their diagonals dg; c: d itself.  The 27 points of a voxel are three planes of 3 x 3, and a
+// plane's sums serve the voxels below, in and above it.  With the element's parities (even
+// in each offset on the diagonal; (a, b) odd in d_a and d_b) a plane contributes
+//   U  to the voxel in it, E + O to the one below and E - O to the one above:
+// per component the centre, the sums over x+-1, y+-1 and the four corners, the corners'
+// alternating sum (xy), and the x- and y-odd differences (xz, yz, in O).  31 additions and
+// 36 multiply-adds a plane against 39 and 75 for a voxel on its own, and 9 (VPT + 2) / VPT
+// shared loads a voxel instead of 27.
 template <class T>
-__device__ __forceinline__ void apply32(const float4* sb, int hc, float dg, float4& c, float& o0,
-                                        float& o1, float& o2) {
-    const float* S0 = c_st32 + 13 * 6;
-    c = sb[hc];
-    o0 = (dg - S0[0]) * c.x;
-    o1 = (dg - S0[1]) * c.y;
-    o2 = (dg - S0[2]) * c.z;
-    auto load = [&](auto e, float& sx, float& sy, float& sz) {
-        const float4 v = sb[hc + T::template off<decltype(e)::value>()];
-        sx += v.x;
-        sy += v.y;
-        sz += v.z;
-    };
-    stencil_pairs<true>(c_st32, load, 0, o0, o1, o2);
+__device__ __forceinline__ void apply_column(const float4* sb, int hc, const float* dg, float4* c,
+                                             float (*o)[3]) {
+    constexpr int V = T::VPT;
+    const float* G = c_st32;
+    constexpr int C0 = 13 * 6, X1 = 14 * 6, Y1 = 16 * 6, XY = 17 * 6, Z1 = 22 * 6, XZ = 23 * 6,
+                  YZ = 25 * 6, XYZ = 26 * 6;        // (1,0,0), (0,1,0), (1,1,0), (0,0,1), ...
+#pragma unroll
+    for (int v = 0; v < V; ++v) o[v][0] = o[v][1] = o[v][2] = 0.f;
+#pragma unroll
+    for (int p = -1; p <= V; ++p) {
+        const float4* q = sb + hc + p * (T::HX * T::HY);
+        const float4 m0 = q[0], xm = q[-1], xp = q[1], ym = q[-T::HX], yp = q[T::HX];
+        const float4 mm = q[-T::HX - 1], pm = q[-T::HX + 1], mp = q[T::HX - 1], pp = q[T::HX + 1];
+        // corner sums: all, alternating, x-odd, y-odd (first index x)
+        const float ax = pp.x + mp.x, bx = pp.x - mp.x, cx = pm.x + mm.x, dx = pm.x - mm.x;
+        const float ay = pp.y + mp.y, by = pp.y - mp.y, cy = pm.y + mm.y, dy = pm.y - mm.y;
+        const float az = pp.z + mp.z, bz = pp.z - mp.z, cz = pm.z + mm.z, dz = pm.z - mm.z;
+        const float Scx = ax + cx, Ax = bx - dx, Cxx = bx + dx;
+        const float Scy = ay + cy, Ay = by - dy, Cyy = ay - cy;
+        const float Scz = az + cz, Cxz = bz + dz, Cyz = az - cz;
+        const float Sxx = xp.x + xm.x, Syx = yp.x + ym.x, Dxx = xp.x - xm.x;
+        const float Sxy = xp.y + xm.y, Syy = yp.y + ym.y, Dyy = yp.y - ym.y;
+        const float Sxz = xp.z + xm.z, Syz = yp.z + ym.z, Dxz = xp.z - xm.z, Dyz = yp.z - ym.z;
+        const float Ex = G[Z1] * m0.x + G[XZ] * Sxx + G[YZ] * Syx + G[XYZ] * Scx + G[XYZ + 3] * Ay;
+        const float Ey = G[Z1 + 1] * m0.y + G[XZ + 1] * Sxy + G[YZ + 1] * Syy + G[XYZ + 1] * Scy +
+                         G[XYZ + 3] * Ax;
+        const float Ez = G[Z1 + 2] * m0.z + G[XZ + 2] * Sxz + G[YZ + 2] * Syz + G[XYZ + 2] * Scz;
+        const float Ox = G[XZ + 4] * Dxz + G[XYZ + 4] * Cxz;
+        const float Oy = G[YZ + 5] * Dyz + G[XYZ + 5] * Cyz;
+        const float Oz = G[XZ + 4] * Dxx + G[XYZ + 4] * Cxx + G[YZ + 5] * Dyy + G[XYZ + 5] * Cyy;
+        if (p >= 0 && p < V) {
+            c[p] = m0;
+            o[p][0] += (dg[p] - G[C0]) * m0.x;
+            o[p][1] += (dg[p] - G[C0 + 1]) * m0.y;
+            o[p][2] += (dg[p] - G[C0 + 2]) * m0.z;
+            o[p][0] -= G[X1] * Sxx + G[Y1] * Syx + G[XY] * Scx + G[XY + 3] * Ay;
+            o[p][1] -= G[X1 + 1] * Sxy + G[Y1 + 1] * Syy + G[XY + 1] * Scy + G[XY + 3] * Ax;
+            o[p][2] -= G[X1 + 2] * Sxz + G[Y1 + 2] * Syz + G[XY + 2] * Scz;
+        }
+        if (p >= 1) {                 // the voxel below: this plane is at +z of it
+            o[p - 1][0] -= Ex + Ox;
+            o[p - 1][1] -= Ey + Oy;
+            o[p - 1][2] -= Ez + Oz;
+        }
+        if (p + 1 < V) {              // the voxel above
+            o[p + 1][0] -= Ex - Ox;
+            o[p + 1][1] -= Ey - Oy;
+            o[p + 1][2] -= Ez - Oz;
+        }
+    }
 }
 
-// voxel index of thread slot v of the tile at org, -1 if outside the grid
+// voxel index of the thread's voxel v in the tile at org, -1 if outside the grid
 template <class T>
 __device__ __forceinline__ long long tile_voxel(const CGArgs& a, int org, int v) {
     int lx, ly, lz;
-    T::local(threadIdx.x + v * T::NTH, lx, ly, lz);
-    const int x = (org & 1023) + lx, y = ((org >> 10) & 1023) + ly, z = (org >> 20) + lz;
+    T::local(lx, ly, lz);
+    const int x = (org & 1023) + lx, y = ((org >> 10) & 1023) + ly, z = (org >> 20) + lz + v;
     if (x >= a.U || y >= a.V || z >= a.W) return -1;
     return ((long long)z * a.V + y) * a.U + x;
 }
@@ -639,17 +692,18 @@ __device__ __forceinline__ void cheb_pass_tiled(const CGArgs& a, const float4* _
         cp_async_wait1();
         __syncthreads();
         const float4* sb = sd[it & 1];
+        int lx, ly, lz;
+        T::local(lx, ly, lz);
+        float4 cv[T::VPT];
+        float o[T::VPT][3];
+        apply_column<T>(sb, T::hidx(lx, ly, lz), dgv, cv, o);
 #pragma unroll
         for (int v = 0; v < T::VPT; ++v) {
             if (mv[v] < 0) continue;
-            int lx, ly, lz;
-            T::local(threadIdx.x + v * T::NTH, lx, ly, lz);
-            float4 c;
-            float o0, o1, o2;
-            apply32<T>(sb, T::hidx(lx, ly, lz), dgv[v], c, o0, o1, o2);
+            const float4 c = cv[v];
             float4 e = ev[v], r = rv[v];
             e.x += c.x; e.y += c.y; e.z += c.z;
-            r.x -= o0; r.y -= o1; r.z -= o2;
+            r.x -= o[v][0]; r.y -= o[v][1]; r.z -= o[v][2];
             const long long m = mv[v];
             a.e[m] = e;
             a.r[m] = r;
@@ -788,12 +842,11 @@ __device__ __forceinline__ bool cheb_pass_resident(const CGArgs& a, int k, unsig
     float4* dn = (k & 1) ? a.p : a.q;
     float4* sb = sd[k & 1];
     int ok = 1;
+    int lx, ly, lz;
+    T::local(lx, ly, lz);
 #pragma unroll
-    for (int v = 0; v < T::VPT; ++v) {
-        int lx, ly, lz;
-        T::local(threadIdx.x + v * T::NTH, lx, ly, lz);
-        sb[T::hidx(lx, ly, lz)] = t.m[v] >= 0 ? t.d[v] : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
+    for (int v = 0; v < T::VPT; ++v)
+        sb[T::hidx(lx, ly, lz + v)] = t.m[v] >= 0 ? t.d[v] : make_float4(0.f, 0.f, 0.f, 0.f);
     float4 h[RT::HPT];
     if (RFIRST && k == 0) {
 #pragma unroll
@@ -823,17 +876,16 @@ __device__ __forceinline__ bool cheb_pass_resident(const CGArgs& a, int k, unsig
     for (int i = 0; i < RT::HPT; ++i)
         if (t.hm[i] >= 0) sb[t.hs[i]] = h[i];
     if (!__syncthreads_and(ok)) return false;
+    float4 cv[T::VPT];
+    float o[T::VPT][3];
+    apply_column<T>(sb, T::hidx(lx, ly, lz), t.dg, cv, o);
 #pragma unroll
     for (int v = 0; v < T::VPT; ++v) {
         if (t.m[v] < 0) continue;
-        int lx, ly, lz;
-        T::local(threadIdx.x + v * T::NTH, lx, ly, lz);
-        float4 c;
-        float o0, o1, o2;
-        apply32<T>(sb, T::hidx(lx, ly, lz), t.dg[v], c, o0, o1, o2);
+        const float4 c = cv[v];
         float4 &e = t.e[v], &r = t.r[v];
         e.x += c.x; e.y += c.y; e.z += c.z;
-        r.x -= o0; r.y -= o1; r.z -= o2;
+        r.x -= o[v][0]; r.y -= o[v][1]; r.z -= o[v][2];
         if (last) {
             rr_p += r.x * r.x + r.y * r.y + r.z * r.z;
         } else {
@@ -893,8 +945,8 @@ __device__ __forceinline__ void residual_df_tiled(const CGArgs& a, float4 (*sd)[
         for (int v = 0; v < T::VPT; ++v) {
             if (mv[v] < 0) continue;
             int lx, ly, lz;
-            T::local(threadIdx.x + v * T::NTH, lx, ly, lz);
-            const int hc = T::hidx(lx, ly, lz);
+            T::local(lx, ly, lz);
+            const int hc = T::hidx(lx, ly, lz + v);
             auto load = [&](auto e, float4& vh, float4& vl) {
                 constexpr int o = T::template off<decltype(e)::value>();
                 vh = sd[0][hc + o];
@@ -1260,11 +1312,12 @@ __device__ __forceinline__ void residual64(const CGArgs& a, int e, bool first, b
 // that leave FP32's range at the scale of the step before (wide) are formed again in FP64,
 // which gives the new scale.
 constexpr float kDrift = 1e-6f;
+constexpr float kFloor = 1e-6f;
 // sequence numbers that a residual and two iterations whose results are dropped may have used
 constexpr unsigned kAborted = 4;
 
 template <bool DF, class T, bool RES, bool SPLIT>
-__global__ void __launch_bounds__(T::NTH, RES ? 4 : 3) k_cg(const __grid_constant__ CGArgs a) {
+__global__ void __launch_bounds__(T::NTH, RES ? 4 : 2) k_cg(const __grid_constant__ CGArgs a) {
     __shared__ __align__(16) float4 sd[2][T::HALO];      // tile halos of the passes
     pdl_trigger();                       // (launched as an ordinary, cooperative kernel)
     if ((int)blockIdx.x == a.nw) {       // the fit for the next step, beside the solve
@@ -1289,6 +1342,7 @@ __global__ void __launch_bounds__(T::NTH, RES ? 4 : 3) k_cg(const __grid_constan
         __syncthreads();     // its zeros, before a residual pass copies halos over them
     }
     float bb = 0.f, rr = 0.f;            // scaled by 4^e0 and 4^e
+    double xx = 0.0;                     // |x|^2 of the block's share, once x is stored
     int e = a.fit->rec[a.step & 1].e, e0 = e;
     int its = 0, outer = 0, wides = 0;
     bool first = true, wide = false, converged = false, nonfinite = false, zero = false;
@@ -1384,11 +1438,11 @@ __global__ void __launch_bounds__(T::NTH, RES ? 4 : 3) k_cg(const __grid_constan
         first = false;
         if (outer >= a.max_outer || its >= a.max_iter) break;
         // ---- Chebyshev: iterations for the reduction still needed, never asking for more
-        // than FP32 can deliver in one refinement (5e-6).  FP64 aims a factor 10 below the
+        // than FP32 can deliver in one refinement (kFloor).  FP64 aims a factor 10 below the
         // tolerance (the march's error is then the history's rounding, 1e-14 on the 8^3
         // cube, not the solve's 2e-13); the FP32 history's own error is far above its
         // tolerance already
-        const float need = fmaxf((DF ? 0.8f : 0.1f) * (goal - kDrift * have) / have, 5e-6f);
+        const float need = fmaxf((DF ? 0.8f : 0.1f) * (goal - kDrift * have) / have, kFloor);
         const int n_it = min(a.n_cheb, max(3, (int)ceilf(log2f(0.5f * need) * a.inv_log2_rate)));
         if constexpr (RES) {
             if constexpr (!DF) {
@@ -1418,6 +1472,7 @@ __global__ void __launch_bounds__(T::NTH, RES ? 4 : 3) k_cg(const __grid_constan
         if (!RES && !gsync()) return;    // the update deals the voxels out by list
         // ---- x += e / 2^e (DF: the float start becomes an FP64 x)
         const double back = pow2d(-e);
+        xx = 0.0;
         each([&](long long m, const float4& d, int) {
             const float ec[3] = {d.x, d.y, d.z};
 #pragma unroll
@@ -1426,6 +1481,7 @@ __global__ void __launch_bounds__(T::NTH, RES ? 4 : 3) k_cg(const __grid_constan
                 x += back * (double)ec[k];
                 a.x[k * M + m] = x;
                 if (DF) a.xb[k * M + m].x = (float)x;
+                xx += x * x;
             }
         });
         stored = true;
@@ -1455,20 +1511,21 @@ __global__ void __launch_bounds__(T::NTH, RES ? 4 : 3) k_cg(const __grid_constan
     // ---- an x not stored yet, and its norm.  NaN or Inf in the right-hand side or the
     // start: no iteration can help; J_n is returned as NaN so that the monitor and the
     // caller see it
-    double xx = 0.0, unused = 0.0;
-    each([&](long long m, const float4&, int) {
+    double unused = 0.0;
+    if (!stored || nonfinite) {
+        xx = 0.0;
+        each([&](long long m, const float4&, int) {
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            double x = DF && !stored ? (double)a.xb[k * M + m].x : a.x[k * M + m];
-            if (zero) x = 0.0;
-            if (nonfinite) x = __longlong_as_double(0x7ff8000000000000LL);
-            if (!stored || nonfinite) {
+            for (int k = 0; k < 3; ++k) {
+                double x = DF && !stored ? (double)a.xb[k * M + m].x : a.x[k * M + m];
+                if (zero) x = 0.0;
+                if (nonfinite) x = __longlong_as_double(0x7ff8000000000000LL);
                 a.x[k * M + m] = x;
                 if (DF) a.xb[k * M + m].x = (float)x;
+                xx += x * x;
             }
-            xx += x * x;
-        }
-    });
+        });
+    }
     block_sum2<T::NTH>(xx, unused);
     // the last block to finish adds up the norm (fixed order) and leaves the barrier words
     // zero for the next launch: every other block has passed its last barrier
@@ -1814,7 +1871,7 @@ void chebyshev_setup(mot_ctx* c) {
     const double theta = 0.5 * (B + A), delta = 0.5 * (B - A), sigma = theta / delta;
     const double kap = B / A;
     const double rate = (std::sqrt(kap) - 1.0) / (std::sqrt(kap) + 1.0);
-    int nk = (int)std::ceil(std::log(5e-6) / std::log(rate));
+    int nk = (int)std::ceil(std::log(0.5 * kFloor) / std::log(rate));
     nk = std::max(4, std::min(nk, MAXCHEB));
     c->cheb_n = nk;
     c->cheb_log_rate = std::log(rate);
@@ -1919,18 +1976,19 @@ namespace {
 
 // kernel variant of a context's solve and its block size
 struct SolveKernel { void* fn; int threads; };
+template <class T> SolveKernel kernel_of(bool df, bool split) {
+    if (df) return {(void*)k_cg<true, T, true, false>, T::NTH};
+    if (split) return {(void*)k_cg<false, T, true, true>, T::NTH};
+    return {(void*)k_cg<false, T, true, false>, T::NTH};
+}
+// tile 1, 2 or 4 (voxels per thread); vectors in memory only with tile 4
 SolveKernel solve_kernel(int precision, int tile, bool resident, bool split) {
     const bool df = precision != MOT_FP64;
-    if (tile == 0) {
-        if (df) return {(void*)k_cg<true, BigTile, false, false>, BigTile::NTH};
-        return {(void*)k_cg<false, BigTile, false, false>, BigTile::NTH};
-    }
-    if (df) return {resident ? (void*)k_cg<true, SmallTile, true, false>
-                             : (void*)k_cg<true, SmallTile, false, false>, SmallTile::NTH};
-    if (split) return {resident ? (void*)k_cg<false, SmallTile, true, true>
-                                : (void*)k_cg<false, SmallTile, false, true>, SmallTile::NTH};
-    return {resident ? (void*)k_cg<false, SmallTile, true, false>
-                     : (void*)k_cg<false, SmallTile, false, false>, SmallTile::NTH};
+    if (!resident)
+        return {df ? (void*)k_cg<true, TileMem, false, false>
+                   : (void*)k_cg<false, TileMem, false, false>, TileMem::NTH};
+    return tile == 1 ? kernel_of<Tile1>(df, split)
+           : tile == 2 ? kernel_of<Tile2>(df, split) : kernel_of<Tile4>(df, split);
 }
 
 }  // namespace
@@ -1941,49 +1999,62 @@ void launch_cg(mot_ctx* c, void** args, cudaStream_t s) {
     ++c->fit_steps;
 }
 
-// Shape of the solve on this geometry: tile lists of both shapes are given; sets the tile
-// (0: 8^3, 1: 8 x 4 x 4), the worker blocks and the epilogue's launch, and returns the
-// chosen list.
-const std::vector<int>& solve_shape(mot_ctx* c, const std::vector<int>& big,
-                                    const std::vector<int>& small) {
-    // The 8^3 tile loads less halo per voxel (2.0 against 2.8) but a pass on it takes a
-    // block about 4 us; with fewer than two such tiles per SM the small tile is faster
-    c->cg_tile = (int)big.size() >= 2 * c->nsm ? 0 : 1;
-    const std::vector<int>& tl = c->cg_tile ? small : big;
-    c->ntiles = (int)tl.size();
-    c->cg_split = c->precision == MOT_FP64 && c->cg_tile && c->nact <= 128LL * c->nsm;
-    int per_sm = 0;
-    SolveKernel k = solve_kernel(c->precision, c->cg_tile, true, c->cg_split);
-    MOT_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.fn, k.threads, 0));
-    c->cg_resident = c->cg_tile == 1 && c->ntiles + 1 <= per_sm * c->nsm;
+// Shape of the solve on this geometry.  tiles[i]: active tiles of 8 x 4 x 4, 8 x 4 x 8 and
+// 8 x 8 x 8 voxels; sets the tile, the worker blocks and the epilogue's launch, and returns
+// the chosen list.
+const std::vector<int>& solve_shape(mot_ctx* c, const std::vector<int> (&tiles)[3]) {
+    // FP64 residual by components while the voxels' warps are fewer than the GPU's
+    // sub-partitions (an FP64 chain of one voxel is 170 instructions of 64 cycles each)
+    c->cg_split = c->precision == MOT_FP64 && c->nact <= 128LL * c->nsm;
+    int pick = 2, per_sm = 0;
+    c->cg_resident = false;
+    for (int i = 0; i < 3 && !c->cg_resident; ++i) {
+        const SolveKernel k = solve_kernel(c->precision, 1 << i, true, c->cg_split);
+        MOT_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.fn, k.threads, 0));
+        if ((long long)tiles[i].size() + 1 <= (long long)per_sm * c->nsm) {
+            c->cg_resident = true;
+            pick = i;
+        }
+    }
     if (!c->cg_resident) {
-        k = solve_kernel(c->precision, c->cg_tile, false, c->cg_split);
+        c->cg_split = false;
+        const SolveKernel k = solve_kernel(c->precision, 4, false, false);
         MOT_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.fn, k.threads, 0));
     }
     if (per_sm < 1) throw MotError{MOT_ERR_CUDA, "CG kernel cannot be made resident"};
+    c->cg_tile = 1 << pick;
+    c->ntiles = (int)tiles[pick].size();
     // one block per tile at most: the tiled passes give a block one tile at a time, so
-    // further blocks would only wait at the grid barriers (and keep SMs from concurrent
-    // solves of other contexts).  The component-split FP64 residual has work for more:
-    // a block for every four warps of it, up to one per SM.
+    // further blocks would only wait (and keep SMs from concurrent solves of other
+    // contexts).  The component-split FP64 residual has work for more: a block for every
+    // four warps of it, up to two per SM.
     int want = std::max(c->ntiles, 1);
     if (c->cg_split)
-        want = std::max(want, std::min(c->nsm, (int)(3 * ((c->nact + 31) / 32) + 3) / 4));
+        want = std::max(want, std::min(2 * c->nsm, (int)(3 * ((c->nact + 31) / 32) + 3) / 4));
     c->cg_blocks = std::max(1, std::min(per_sm * c->nsm - 1, want));
     // epilogue: small blocks on small grids (its FP64 terms are bound by the SMs in use)
     c->epi_threads = c->M <= 64LL * c->nsm ? 64 : NT;
     c->epi_blocks = (int)std::min<long long>((c->M + c->epi_threads - 1) / c->epi_threads,
                                              8LL * c->nsm);
-    return tl;
+    return tiles[pick];
 }
+
+namespace {
+template <class T> void halo_lists(mot_ctx* c) {
+    typedef Resident<T> RT;
+    MOT_CUDA_TRY(cudaMalloc(&c->halo, sizeof(int) * RT::HPT * T::NTH * (size_t)c->ntiles));
+    k_halo_list<T><<<c->ntiles, T::NTH, 0, c->stream>>>(c->tiles, c->diag32, c->U, c->V, c->W,
+                                                        c->halo);
+    MOT_LAUNCH_CHECK();
+}
+}  // namespace
 
 // halo lists of the resident tiles (tiles and diag32 on the device)
 void solve_halo_lists(mot_ctx* c) {
     if (!c->cg_resident || !c->ntiles) return;
-    typedef Resident<SmallTile> RT;
-    MOT_CUDA_TRY(cudaMalloc(&c->halo, sizeof(int) * RT::HPT * SmallTile::NTH * (size_t)c->ntiles));
-    k_halo_list<SmallTile><<<c->ntiles, SmallTile::NTH, 0, c->stream>>>(c->tiles, c->diag32, c->U,
-                                                                        c->V, c->W, c->halo);
-    MOT_LAUNCH_CHECK();
+    if (c->cg_tile == 1) halo_lists<Tile1>(c);
+    else if (c->cg_tile == 2) halo_lists<Tile2>(c);
+    else halo_lists<Tile4>(c);
 }
 
 // rhs + CG for step n; ||J_n||^2 into norm2_out (device), J_n in ring slot n
