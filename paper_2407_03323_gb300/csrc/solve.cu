@@ -1668,27 +1668,49 @@ __global__ void k_apply64(const __grid_constant__ CGArgs a, const double* __rest
     y[2 * a.M + m] = o[2];
 }
 
-// partial dot products per block
-__global__ void k_dot(const double* __restrict__ x, const double* __restrict__ y, long long n,
-                      double* __restrict__ part) {
+// The setup's Lanczos recurrence with its scalars on the device (sc[2 j] = alpha_j,
+// sc[2 j + 1] = ||w||^2 after step j): partial sums per block, added up by every block of
+// the next kernel in the same order.
+constexpr int kLzBlocks = NT;
+__device__ __forceinline__ double lz_sum(const double* part) {
+    double s = part[threadIdx.x], d = 0.0;      // one partial per thread
+    block_sum2<NT>(s, d);
+    return s;
+}
+__global__ void __launch_bounds__(NT) k_lz_dot(const double* __restrict__ x, const double* __restrict__ y,
+                                               long long n, double* __restrict__ part) {
     double s = 0.0, d = 0.0;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x)
+    for (long long i = (long long)blockIdx.x * NT + threadIdx.x; i < n; i += (long long)gridDim.x * NT)
         s += x[i] * y[i];
     block_sum2<NT>(s, d);
     if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
-
-// w = w - alpha v - beta u
-__global__ void k_axpy2(double* __restrict__ w, const double* __restrict__ v, double alpha,
-                        const double* __restrict__ u, double beta, long long n) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) w[i] -= alpha * v[i] + beta * u[i];
+// w -= alpha v + beta u with alpha = sum(part_in), beta^2 = *b2 (0: none); partial |w|^2
+__global__ void __launch_bounds__(NT) k_lz_step(double* __restrict__ w, const double* __restrict__ v,
+                                                const double* __restrict__ u,
+                                                const double* __restrict__ part_in,
+                                                const double* __restrict__ b2, long long n,
+                                                double* __restrict__ alpha_out,
+                                                double* __restrict__ part) {
+    const double alpha = lz_sum(part_in), beta = b2 ? sqrt(*b2) : 0.0;
+    double s = 0.0, d = 0.0;
+    for (long long i = (long long)blockIdx.x * NT + threadIdx.x; i < n; i += (long long)gridDim.x * NT) {
+        const double r = w[i] - (alpha * v[i] + (b2 ? beta * u[i] : 0.0));
+        w[i] = r;
+        s += r * r;
+    }
+    block_sum2<NT>(s, d);
+    if (threadIdx.x == 0) part[blockIdx.x] = s;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *alpha_out = alpha;
 }
-
-__global__ void k_scale(double* __restrict__ w, double s, long long n) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) w[i] *= s;
+// w /= ||w|| (left alone when it vanished: the host stops there); ||w||^2 out
+__global__ void __launch_bounds__(NT) k_lz_scale(double* __restrict__ w, const double* __restrict__ part_in,
+                                                 long long n, double* __restrict__ b2_out) {
+    const double b2 = lz_sum(part_in);
+    const double f = b2 > 0.0 ? 1.0 / sqrt(b2) : 0.0;
+    for (long long i = (long long)blockIdx.x * NT + threadIdx.x; i < n; i += (long long)gridDim.x * NT)
+        w[i] *= f;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *b2_out = b2;
 }
 
 }  // namespace
@@ -1790,12 +1812,14 @@ double tridiag_eig(const std::vector<double>& al, const std::vector<double>& be,
 // converge; the bound above keeps every mode in (0, a + b)).
 void chebyshev_setup(mot_ctx* c) {
     const long long n3 = 3 * c->M;
-    const int nb = 256;
+    constexpr int kSteps = 40;
     double *v0 = nullptr, *v1 = nullptr, *w = nullptr, *part = nullptr;
     MOT_CUDA_TRY(cudaMalloc(&v0, sizeof(double) * n3));
     MOT_CUDA_TRY(cudaMalloc(&v1, sizeof(double) * n3));
     MOT_CUDA_TRY(cudaMalloc(&w, sizeof(double) * n3));
-    MOT_CUDA_TRY(cudaMalloc(&part, sizeof(double) * nb));
+    // two sets of partial sums, then the scalars of every step (read once at the end)
+    MOT_CUDA_TRY(cudaMalloc(&part, sizeof(double) * (2 * kLzBlocks + 2 * kSteps)));
+    double *pa = part, *pb = part + kLzBlocks, *sc = part + 2 * kLzBlocks;
     std::vector<double> al, be;
     try {
         std::vector<double> h(n3, 0.0), act(c->nact);
@@ -1817,34 +1841,30 @@ void chebyshev_setup(mot_ctx* c) {
         CGArgs a{};
         a.M = c->M; a.act = c->active; a.nmask = c->nmask; a.nact = c->nact; a.diag = c->cg_diag;
         for (int e = 0; e < 27; ++e) a.noff[e] = c->noff[e];
-        auto dot = [&](const double* x, const double* y) {
-            k_dot<<<nb, NT, 0, c->stream>>>(x, y, n3, part);
-            MOT_LAUNCH_CHECK();
-            std::vector<double> hp(nb);
-            MOT_CUDA_TRY(cudaMemcpyAsync(hp.data(), part, sizeof(double) * nb, cudaMemcpyDeviceToHost,
-                                         c->stream));
-            MOT_CUDA_TRY(cudaStreamSynchronize(c->stream));
-            double s = 0.0;
-            for (double x : hp) s += x;
-            return s;
-        };
-        double beta = 0.0;
-        const int blocks = (int)((n3 + NT - 1) / NT);
-        for (int j = 0; j < 40; ++j) {
+        for (int j = 0; j < kSteps; ++j) {
             MOT_CUDA_TRY(cudaMemsetAsync(w, 0, sizeof(double) * n3, c->stream));
             k_apply64<<<(int)((c->nact + NT - 1) / NT), NT, 0, c->stream>>>(a, v1, w);
             MOT_LAUNCH_CHECK();
-            const double alpha = dot(w, v1);
-            k_axpy2<<<blocks, NT, 0, c->stream>>>(w, v1, alpha, v0, beta, n3);
+            k_lz_dot<<<kLzBlocks, NT, 0, c->stream>>>(w, v1, n3, pa);
             MOT_LAUNCH_CHECK();
-            al.push_back(alpha);
-            be.push_back(beta);
-            beta = std::sqrt(std::max(dot(w, w), 0.0));
-            if (!(beta > 1e-14)) break;
-            k_scale<<<blocks, NT, 0, c->stream>>>(w, 1.0 / beta, n3);
+            k_lz_step<<<kLzBlocks, NT, 0, c->stream>>>(w, v1, v0, pa, j ? sc + 2 * j - 1 : nullptr,
+                                                       n3, sc + 2 * j, pb);
+            MOT_LAUNCH_CHECK();
+            k_lz_scale<<<kLzBlocks, NT, 0, c->stream>>>(w, pb, n3, sc + 2 * j + 1);
             MOT_LAUNCH_CHECK();
             std::swap(v0, v1);
             std::swap(v1, w);
+        }
+        std::vector<double> hs(2 * kSteps);
+        MOT_CUDA_TRY(cudaMemcpyAsync(hs.data(), sc, sizeof(double) * 2 * kSteps,
+                                     cudaMemcpyDeviceToHost, c->stream));
+        MOT_CUDA_TRY(cudaStreamSynchronize(c->stream));
+        double beta = 0.0;
+        for (int j = 0; j < kSteps; ++j) {
+            al.push_back(hs[2 * j]);
+            be.push_back(beta);
+            beta = std::sqrt(std::max(hs[2 * j + 1], 0.0));
+            if (!(beta > 1e-14)) break;      // invariant: the steps after it are dropped
         }
     } catch (...) {
         cudaFree(v0); cudaFree(v1); cudaFree(w); cudaFree(part);

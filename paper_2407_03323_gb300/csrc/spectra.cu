@@ -28,12 +28,19 @@ __global__ void trig_table_kernel(int P, int N, int H, double* cosw, double* sin
     sinw[i] = (d == 0 ? 0.0 : 2.0) * s;
 }
 
-__global__ void extract_lag_kernel(const int* __restrict__ tab_l0, const double* __restrict__ tab,
-                                   long long noff, int l, int cc, double* __restrict__ g) {
+// Batches of transforms: slab b = (lag - l_first) * 6 + component, one after the other in
+// every array.  (One launch per lag, component and pass is 900 launches for a 20^3 grid's 36
+// lags, 6.5 of 21 ms of its creation.)
+
+// slab b of g: the octant elements of its lag and component
+__global__ void extract_lags_kernel(const int* __restrict__ tab_l0, const double* __restrict__ tab,
+                                    long long noff, int l_first, int nslab, double* __restrict__ g) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= noff) return;
-    const int idx = l - tab_l0[i];
-    g[i] = (idx >= 0 && idx < mot::WIN) ? tab[(i * 6 + cc) * mot::WIN + idx] : 0.0;
+    if (i >= noff * nslab) return;
+    const int b = (int)(i / noff), cc = b % 6;
+    const long long o = i % noff;
+    const int idx = l_first + b / 6 - tab_l0[o];
+    g[i] = (idx >= 0 && idx < mot::WIN) ? tab[(o * 6 + cc) * mot::WIN + idx] : 0.0;
 }
 
 // g[d] = sum_{l <= n} w[l] G_l(d) for component cc (the lags of the window at d)
@@ -62,48 +69,55 @@ __global__ void accum_kernel(const double* __restrict__ src, long long noct, dou
     dst[i] = fma(w, v, dst[i]);
 }
 
-// out[o2][o1][k] = sum_{d < n} in[o2][o1][d] * w[d][k]         (transform along the fastest axis)
-__global__ void pass_fast(const double* __restrict__ in, int n, long long nrows,
-                          const double* __restrict__ w, int K, double* __restrict__ out) {
+// cosine or sine table of one axis for each component (cc0: component of slab 0)
+struct AxisTables {
+    const double* w[6];
+    int cc0;
+    double sign;       // of the odd components' result (two odd axes: (-i)(-i) = -1)
+};
+// odd axes of component cc (order xx, yy, zz, xy, xz, yz): bit a set if odd along a
+__host__ __device__ constexpr int odd_mask(int cc) { return cc < 3 ? 0 : cc == 3 ? 3 : cc == 4 ? 5 : 6; }
+
+// out[row][k] = sum_{d < n} in[row][d] * w[d][k]       (along the fastest axis; rows per slab)
+__global__ void pass_fast(const double* __restrict__ in, int n, long long rows, int nslab,
+                          AxisTables t, int K, double* __restrict__ out) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nrows * K) return;
+    if (i >= rows * nslab * K) return;
     const long long row = i / K;
     const int k = (int)(i % K);
+    const double* w = t.w[(t.cc0 + (int)(row / rows)) % 6];
     const double* src = in + row * n;
     double acc = 0.0;
     for (int d = 0; d < n; ++d) acc = fma(src[d], w[(long long)d * K + k], acc);
     out[i] = acc;
 }
 
-// out[o][k][f] = sum_{d < n} in[o][d][f] * w[d][k]           (transform along a middle axis)
-__global__ void pass_mid(const double* __restrict__ in, int n, int F, long long nouter,
-                         const double* __restrict__ w, int K, double* __restrict__ out) {
+// out[o][k][f] = sum_{d < n} in[o][d][f] * w[d][k]     (along a middle axis; outer per slab)
+__global__ void pass_mid(const double* __restrict__ in, int n, int F, long long outer, int nslab,
+                         AxisTables t, int K, double* __restrict__ out) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nouter * K * F) return;
+    if (i >= outer * nslab * K * F) return;
     const int f = (int)(i % F);
     const int k = (int)((i / F) % K);
     const long long o = i / ((long long)F * K);
+    const int cc = (t.cc0 + (int)(o / outer)) % 6;
+    const double* w = t.w[cc];
     const double* src = in + o * (long long)n * F + f;
     double acc = 0.0;
     for (int d = 0; d < n; ++d) acc = fma(src[(long long)d * F], w[(long long)d * K + k], acc);
-    out[i] = acc;
+    out[i] = odd_mask(cc) ? t.sign * acc : acc;
 }
 
-// [6][noct] (component-major) -> [noct][6] in the history precision
+// [lags][6][noct] (component-major) -> [lags][noct][6] in the history precision
 template <typename R>
-__global__ void interleave_kernel(const double* __restrict__ src, long long noct,
+__global__ void interleave_kernel(const double* __restrict__ src, long long noct, int lags,
                                   R* __restrict__ dst) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= 6 * noct) return;
-    const long long o = i / 6;
-    const int cc = (int)(i % 6);
-    dst[i] = (R)src[cc * noct + o];
-}
-
-// x[i] *= s (in place)
-__global__ void scale_inplace_kernel(double* x, long long n, double s) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) x[i] *= s;
+    if (i >= 6 * noct * lags) return;
+    const long long l = i / (6 * noct), r = i % (6 * noct);
+    const long long o = r / 6;
+    const int cc = (int)(r % 6);
+    dst[i] = (R)src[(l * 6 + cc) * noct + o];
 }
 
 inline int nblk(long long n, int b) { return (int)((n + b - 1) / b); }
@@ -123,39 +137,42 @@ struct Scratch {
     ~Scratch() { cudaFree(g); cudaFree(t1); cudaFree(t2); }
 };
 
-// odd axes of component cc (order xx, yy, zz, xy, xz, yz): bit a set if odd along a
-const int kOddMask[6] = {0, 0, 0, 3, 5, 6};
+AxisTables axis_tables(const TrigTables& tt, int axis, int cc0, bool last) {
+    AxisTables t;
+    for (int cc = 0; cc < 6; ++cc)
+        t.w[cc] = (odd_mask(cc) >> axis) & 1 ? tt.sinw[axis] : tt.cosw[axis];
+    t.cc0 = cc0;
+    t.sign = last ? -1.0 : 1.0;
+    return t;
+}
 
-// spectrum of the octant kernel sc.g (component cc) into dst [noct]
-void transform_one(mot_ctx* c, const TrigTables& tt, Scratch& sc, int cc, double* dst) {
+// spectra of the nslab octant kernels in sc.g (components cc0, cc0 + 1, .. modulo 6) into
+// dst [nslab][noct]
+void transform(mot_ctx* c, const TrigTables& tt, Scratch& sc, int cc0, int nslab, double* dst) {
     const int U = c->U, V = c->V, W = c->W;
     const int Hu = c->Hu, Hv = c->Hv, Hw = c->Hw;
     cudaStream_t s = c->stream;
-    const int odd = kOddMask[cc];
-    const double* wx = (odd & 1) ? tt.sinw[0] : tt.cosw[0];
-    const double* wy = (odd & 2) ? tt.sinw[1] : tt.cosw[1];
-    const double* wz = (odd & 4) ? tt.sinw[2] : tt.cosw[2];
     // x: [W][V][U] -> [W][V][Hu]
-    pass_fast<<<nblk((long long)W * V * Hu, 256), 256, 0, s>>>(sc.g, U, (long long)W * V, wx, Hu, sc.t1);
+    pass_fast<<<nblk((long long)W * V * Hu * nslab, 256), 256, 0, s>>>(
+        sc.g, U, (long long)W * V, nslab, axis_tables(tt, 0, cc0, false), Hu, sc.t1);
     MOT_LAUNCH_CHECK();
     // y: [W][V][Hu] -> [W][Hv][Hu]
-    pass_mid<<<nblk((long long)W * Hv * Hu, 256), 256, 0, s>>>(sc.t1, V, Hu, W, wy, Hv, sc.t2);
+    pass_mid<<<nblk((long long)W * Hv * Hu * nslab, 256), 256, 0, s>>>(
+        sc.t1, V, Hu, W, nslab, axis_tables(tt, 1, cc0, false), Hv, sc.t2);
     MOT_LAUNCH_CHECK();
     // z: [W][Hv*Hu] -> [Hw][Hv*Hu]
-    pass_mid<<<nblk((long long)Hw * Hv * Hu, 256), 256, 0, s>>>(sc.t2, W, Hv * Hu, 1, wz, Hw, dst);
+    pass_mid<<<nblk((long long)Hw * Hv * Hu * nslab, 256), 256, 0, s>>>(
+        sc.t2, W, Hv * Hu, 1, nslab, axis_tables(tt, 2, cc0, true), Hw, dst);
     MOT_LAUNCH_CHECK();
-    if (odd) {   // two odd axes: (-i)(-i) = -1
-        scale_inplace_kernel<<<nblk(c->noct, 256), 256, 0, s>>>(dst, c->noct, -1.0);
-        MOT_LAUNCH_CHECK();
-    }
 }
 
-void spectrum_one(mot_ctx* c, const TrigTables& tt, Scratch& sc, int l, int cc, double* dst) {
+// spectra of lags l .. l + lags - 1, all components, into dst [lags][6][noct]
+void spectra_of_lags(mot_ctx* c, const TrigTables& tt, Scratch& sc, int l, int lags, double* dst) {
     const long long noff = (long long)c->U * c->V * c->W;
-    extract_lag_kernel<<<nblk(noff, 256), 256, 0, c->stream>>>(c->tab_l0, c->tab, noff, l, cc,
-                                                              sc.g);
+    extract_lags_kernel<<<nblk(noff * 6 * lags, 256), 256, 0, c->stream>>>(
+        c->tab_l0, c->tab, noff, l, 6 * lags, sc.g);
     MOT_LAUNCH_CHECK();
-    transform_one(c, tt, sc, cc, dst);
+    transform(c, tt, sc, 0, 6 * lags, dst);
 }
 
 void make_tables(mot_ctx* c, TrigTables& tt) {
@@ -170,11 +187,18 @@ void make_tables(mot_ctx* c, TrigTables& tt) {
     }
 }
 
-void make_scratch(mot_ctx* c, Scratch& sc) {
+// scratch of `slabs` transforms at a time
+void make_scratch(mot_ctx* c, Scratch& sc, int slabs) {
     const long long noff = (long long)c->U * c->V * c->W;
-    MOT_CUDA_TRY(cudaMalloc(&sc.g, sizeof(double) * noff));
-    MOT_CUDA_TRY(cudaMalloc(&sc.t1, sizeof(double) * (long long)c->W * c->V * c->Hu));
-    MOT_CUDA_TRY(cudaMalloc(&sc.t2, sizeof(double) * (long long)c->W * c->Hv * c->Hu));
+    MOT_CUDA_TRY(cudaMalloc(&sc.g, sizeof(double) * noff * slabs));
+    MOT_CUDA_TRY(cudaMalloc(&sc.t1, sizeof(double) * (long long)c->W * c->V * c->Hu * slabs));
+    MOT_CUDA_TRY(cudaMalloc(&sc.t2, sizeof(double) * (long long)c->W * c->Hv * c->Hu * slabs));
+}
+
+// lags per batch: about a million octant bins, a few tens of MB of scratch (one lag at a
+// time from about 50^3 on, where its passes fill the GPU by themselves)
+int batch_lags(const mot_ctx* c, int lags) {
+    return (int)std::max(1LL, std::min((long long)lags, (1LL << 20) / (6 * c->noct)));
 }
 
 }  // namespace
@@ -185,20 +209,22 @@ namespace mot {
 void compute_spectra(mot_ctx* c) {
     TrigTables tt;
     Scratch sc;
+    const int nb = batch_lags(c, c->ell);
     make_tables(c, tt);
-    make_scratch(c, sc);
+    make_scratch(c, sc, 6 * nb);
     double* tmp = nullptr;
-    MOT_CUDA_TRY(cudaMalloc(&tmp, sizeof(double) * c->noct * 6));
+    MOT_CUDA_TRY(cudaMalloc(&tmp, sizeof(double) * c->noct * 6 * nb));
     try {
-        for (int l = 1; l <= c->ell; ++l) {
-            for (int cc = 0; cc < 6; ++cc) spectrum_one(c, tt, sc, l, cc, tmp + cc * c->noct);
+        for (int l = 1; l <= c->ell; l += nb) {
+            const int m = std::min(nb, c->ell - l + 1);
+            spectra_of_lags(c, tt, sc, l, m, tmp);
             const long long off = (long long)(l - 1) * 6 * c->noct;
             if (c->precision == MOT_FP64)
-                interleave_kernel<double><<<nblk(6 * c->noct, 256), 256, 0, c->stream>>>(
-                    tmp, c->noct, c->h64.ghat + off);
+                interleave_kernel<double><<<nblk(6 * c->noct * m, 256), 256, 0, c->stream>>>(
+                    tmp, c->noct, m, c->h64.ghat + off);
             else
-                interleave_kernel<float><<<nblk(6 * c->noct, 256), 256, 0, c->stream>>>(
-                    tmp, c->noct, c->h32.ghat + off);
+                interleave_kernel<float><<<nblk(6 * c->noct * m, 256), 256, 0, c->stream>>>(
+                    tmp, c->noct, m, c->h32.ghat + off);
             MOT_LAUNCH_CHECK();
         }
         MOT_CUDA_TRY(cudaStreamSynchronize(c->stream));
@@ -213,11 +239,11 @@ void spectrum_of_lag(mot_ctx* c, int l, double* host_out) {
     TrigTables tt;
     Scratch sc;
     make_tables(c, tt);
-    make_scratch(c, sc);
+    make_scratch(c, sc, 6);
     double* tmp = nullptr;
     MOT_CUDA_TRY(cudaMalloc(&tmp, sizeof(double) * c->noct * 6));
     try {
-        for (int cc = 0; cc < 6; ++cc) spectrum_one(c, tt, sc, l, cc, tmp + cc * c->noct);
+        spectra_of_lags(c, tt, sc, l, 1, tmp);
         MOT_CUDA_TRY(cudaMemcpyAsync(host_out, tmp, sizeof(double) * c->noct * 6,
                                      cudaMemcpyDeviceToHost, c->stream));
         MOT_CUDA_TRY(cudaStreamSynchronize(c->stream));
@@ -239,7 +265,7 @@ void spectrum_of_combination(mot_ctx* c, const double* w_host, int n, bool round
     TrigTables tt;
     Scratch sc;
     make_tables(c, tt);
-    make_scratch(c, sc);
+    make_scratch(c, sc, 6);
     double* tmp = nullptr;
     double* w = nullptr;
     const long long noff = (long long)c->U * c->V * c->W;
@@ -252,17 +278,17 @@ void spectrum_of_combination(mot_ctx* c, const double* w_host, int n, bool round
         if (!round32) {
             for (int cc = 0; cc < 6; ++cc) {
                 extract_weighted_kernel<<<nblk(noff, 256), 256, 0, s>>>(c->tab_l0, c->tab, noff,
-                                                                       w, n, cc, sc.g);
+                                                                       w, n, cc, sc.g + cc * noff);
                 MOT_LAUNCH_CHECK();
-                transform_one(c, tt, sc, cc, tmp + cc * c->noct);
             }
-            interleave_kernel<double><<<nblk(6 * c->noct, 256), 256, 0, s>>>(tmp, c->noct, dst);
+            transform(c, tt, sc, 0, 6, tmp);
+            interleave_kernel<double><<<nblk(6 * c->noct, 256), 256, 0, s>>>(tmp, c->noct, 1, dst);
             MOT_LAUNCH_CHECK();
         } else {
             MOT_CUDA_TRY(cudaMemsetAsync(dst, 0, sizeof(double) * 6 * c->noct, s));
             for (int l = 0; l <= n; ++l) {
                 if (w_host[l] == 0.0) continue;
-                for (int cc = 0; cc < 6; ++cc) spectrum_one(c, tt, sc, l, cc, tmp + cc * c->noct);
+                spectra_of_lags(c, tt, sc, l, 1, tmp);
                 accum_kernel<<<nblk(6 * c->noct, 256), 256, 0, s>>>(tmp, c->noct, w_host[l],
                                                                     l >= 1, dst);
                 MOT_LAUNCH_CHECK();
