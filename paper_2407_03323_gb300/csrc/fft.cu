@@ -643,12 +643,6 @@ void fft_forward_z(mot_ctx* c, typename CT<R>::c* out, cudaStream_t s) {
     mid_pass<R>(hbuf<R>(c).tmp2, out, c->ax[2], a, dependent_launches(c), s);
 }
 
-template <typename R>
-void fft_forward(mot_ctx* c, const double* Jsoa, typename CT<R>::c* out, cudaStream_t s) {
-    fft_forward_xy<R>(c, Jsoa, s, nullptr);
-    fft_forward_z<R>(c, out, s);
-}
-
 // y and x passes of the inverse transform, hb.tmp2 [3][W][Pv][Hu] -> [3][W][V][U]
 template <typename R>
 void fft_inverse_yx(mot_ctx* c, R* out, cudaStream_t s) {
@@ -696,8 +690,6 @@ template void fft_forward_z<double>(mot_ctx*, double2*, cudaStream_t);
 template void fft_forward_z<float>(mot_ctx*, float2*, cudaStream_t);
 template void fft_inverse_yx<double>(mot_ctx*, double*, cudaStream_t);
 template void fft_inverse_yx<float>(mot_ctx*, float*, cudaStream_t);
-template void fft_forward<double>(mot_ctx*, const double*, double2*, cudaStream_t);
-template void fft_inverse<double>(mot_ctx*, const double2*, double*, cudaStream_t);
 template void fft_inverse<float>(mot_ctx*, const float2*, float*, cudaStream_t);
 
 }  // namespace mot

@@ -66,40 +66,12 @@ __global__ void k_pdsa_diag(const double* __restrict__ eps, long long M, double 
     a[m] = e > 1.0 ? (aT + beta * e) / (e - 1.0) : 0.0;
 }
 
-// yhat(k) = scale * Khat(k) xhat(k) over all rfft bins, Khat from its octant
-// ([noct][6]: xx yy zz xy xz yz); mirrored v / w bins flip the components odd there
-__global__ void k_pdsa_mul(const double* __restrict__ spec, double2* __restrict__ xh, int Hu,
-                           int Hv, int Pv, int Pw, long long nbins, double scale) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nbins) return;
-    const int ku = (int)(i % Hu);
-    const int kv = (int)((i / Hu) % Pv);
-    const int kw = (int)(i / ((long long)Hu * Pv));
-    const bool fv = kv >= Hv, fw = 2 * kw > Pw;
-    const int ov = fv ? Pv - kv : kv;
-    const int ow = fw ? Pw - kw : kw;
-    const double* g = spec + (((long long)ow * Hv + ov) * Hu + ku) * 6;
-    const double gxx = g[0], gyy = g[1], gzz = g[2];
-    const double gxy = fv ? -g[3] : g[3];
-    const double gxz = fw ? -g[4] : g[4];
-    const double gyz = (fv != fw) ? -g[5] : g[5];
-    const double2 x = xh[i], y = xh[nbins + i], z = xh[2 * nbins + i];
-    double2 ox, oy, oz;
-    ox.x = scale * (gxx * x.x + gxy * y.x + gxz * z.x);
-    ox.y = scale * (gxx * x.y + gxy * y.y + gxz * z.y);
-    oy.x = scale * (gxy * x.x + gyy * y.x + gyz * z.x);
-    oy.y = scale * (gxy * x.y + gyy * y.y + gyz * z.y);
-    oz.x = scale * (gxz * x.x + gyz * y.x + gzz * z.x);
-    oz.y = scale * (gxz * x.y + gyz * y.y + gzz * z.y);
-    xh[i] = ox;
-    xh[nbins + i] = oy;
-    xh[2 * nbins + i] = oz;
-}
-
 // y = a x - conv on active voxels, 0 elsewhere ([3][M])
 __global__ void k_pdsa_combine(const double* __restrict__ a, const double* __restrict__ eps,
                                const double* __restrict__ x, const double* __restrict__ conv,
                                long long M, double* __restrict__ y) {
+    pdl_trigger();
+    pdl_wait();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= 3 * M) return;
     const long long m = i % M;
@@ -226,6 +198,8 @@ __global__ void k_rand_vec(unsigned long long seed, const double* __restrict__ e
 // part[j][block] = partial dot(V_j, w) for j in this block row's DOTV vectors
 __global__ void k_dots(const double* __restrict__ V, int nvec, long long L,
                        const double* __restrict__ w, double* __restrict__ part) {
+    pdl_trigger();
+    pdl_wait();
     __shared__ double sm[DOTV][NT / 32];
     const int j0 = blockIdx.y * DOTV;
     double acc[DOTV];
@@ -253,6 +227,8 @@ __global__ void k_dots(const double* __restrict__ V, int nvec, long long L,
 
 // h[j] = sum of the nb partials of vector j (one block per vector)
 __global__ void k_sum_parts(const double* __restrict__ part, int nb, double* __restrict__ h) {
+    pdl_trigger();
+    pdl_wait();
     __shared__ double sm[NT / 32];
     double s = 0.0;
     for (int k = threadIdx.x; k < nb; k += blockDim.x) s += part[(long long)blockIdx.x * nb + k];
@@ -271,6 +247,8 @@ __global__ void k_sum_parts(const double* __restrict__ part, int nb, double* __r
 __global__ void k_sub_combo(double* __restrict__ w, const double* __restrict__ V,
                             const double* __restrict__ h, int nvec, long long L,
                             double* __restrict__ coef, double* __restrict__ part) {
+    pdl_trigger();
+    pdl_wait();
     extern __shared__ double sh[];
     __shared__ double sm[NT / 32];
     for (int j = threadIdx.x; j < nvec; j += blockDim.x) sh[j] = h[j];
@@ -298,6 +276,8 @@ __global__ void k_sub_combo(double* __restrict__ w, const double* __restrict__ V
 // order; block 0 leaves ||w||^2 in *nrm2)
 __global__ void k_normalise(const double* __restrict__ w, const double* __restrict__ part, int nb,
                             long long L, double* __restrict__ out, double* __restrict__ nrm2) {
+    pdl_trigger();
+    pdl_wait();
     __shared__ double sm[NT / 32], tot;
     double s = 0.0;
     for (int k = threadIdx.x; k < nb; k += blockDim.x) s += part[k];
@@ -320,6 +300,8 @@ __global__ void k_normalise(const double* __restrict__ w, const double* __restri
 __global__ void k_lz_a(double* __restrict__ w, const double* __restrict__ vprev,
                        const double* __restrict__ b2prev, const double* __restrict__ v,
                        long long L, double* __restrict__ part) {
+    pdl_trigger();
+    pdl_wait();
     __shared__ double sm[NT / 32];
     const double bp = b2prev ? sqrt(fmax(*b2prev, 0.0)) : 0.0;
     double acc = 0.0;
@@ -342,6 +324,8 @@ __global__ void k_lz_a(double* __restrict__ w, const double* __restrict__ vprev,
 // w -= alpha v; part[block] = partial ||w||^2
 __global__ void k_lz_b(double* __restrict__ w, const double* __restrict__ alpha,
                        const double* __restrict__ v, long long L, double* __restrict__ part) {
+    pdl_trigger();
+    pdl_wait();
     __shared__ double sm[NT / 32];
     const double a = *alpha;
     double acc = 0.0;
@@ -363,6 +347,8 @@ __global__ void k_lz_b(double* __restrict__ w, const double* __restrict__ alpha,
 // out = w / sqrt(*b2), or 0 when the norm vanished (the host stops there)
 __global__ void k_lz_c(const double* __restrict__ w, const double* __restrict__ b2, long long L,
                        double* __restrict__ out) {
+    pdl_trigger();
+    pdl_wait();
     const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= L) return;
     const double n2 = *b2;
@@ -379,7 +365,6 @@ void ensure_operator(mot_ctx* c, int n, int flags) {
     if (!c->pdsa_spec) {
         MOT_CUDA_TRY(cudaMalloc(&c->pdsa_spec, sizeof(double) * 6 * c->noct));
         MOT_CUDA_TRY(cudaMalloc(&c->pdsa_a, sizeof(double) * M));
-        MOT_CUDA_TRY(cudaMalloc(&c->pdsa_xhat, sizeof(double2) * 3 * c->nbins));
         MOT_CUDA_TRY(cudaMalloc(&c->pdsa_conv, sizeof(double) * 3 * M));
     }
     c->pdsa_n = c->pdsa_flags = -1;
@@ -407,13 +392,11 @@ void ensure_operator(mot_ctx* c, int n, int flags) {
 
 // y = A_n x, both [3][M] on the device
 void apply(mot_ctx* c, const double* x, double* y, cudaStream_t s) {
-    const double scale = 1.0 / ((double)c->ax[0].P * c->ax[1].P * c->ax[2].P);
-    mot::fft_forward<double>(c, x, c->pdsa_xhat, s);
-    k_pdsa_mul<<<nblk(c->nbins, NT), NT, 0, s>>>(c->pdsa_spec, c->pdsa_xhat, c->Hu, c->Hv,
-                                                 c->ax[1].P, c->ax[2].P, c->nbins, scale);
-    MOT_LAUNCH_CHECK();
-    mot::fft_inverse<double>(c, c->pdsa_xhat, c->pdsa_conv, s);
-    k_pdsa_combine<<<nblk(3 * c->M, NT), NT, 0, s>>>(c->pdsa_a, c->eps, x, c->pdsa_conv, c->M, y);
+    mot::fft_forward_xy<double>(c, x, s, nullptr);
+    mot::zproduct(c, c->pdsa_spec, s);
+    mot::fft_inverse_yx<double>(c, c->pdsa_conv, s);
+    launch_dependent(mot::dependent_launches(c), k_pdsa_combine, nblk(3 * c->M, NT), NT, 0, s,
+                     c->pdsa_a, c->eps, x, c->pdsa_conv, c->M, y);
     MOT_LAUNCH_CHECK();
 }
 
@@ -437,9 +420,9 @@ void dots(mot_ctx* c, const double* V, int nvec, long long L, const double* w, d
           double* h, cudaStream_t s) {
     const int nb = grid_rows(c, L);
     dim3 g(nb, (nvec + DOTV - 1) / DOTV);
-    k_dots<<<g, NT, 0, s>>>(V, nvec, L, w, part);
+    launch_dependent(mot::dependent_launches(c), k_dots, g, NT, 0, s, V, nvec, L, w, part);
     MOT_LAUNCH_CHECK();
-    k_sum_parts<<<nvec, NT, 0, s>>>(part, nb, h);
+    launch_dependent(mot::dependent_launches(c), k_sum_parts, nvec, NT, 0, s, part, nb, h);
     MOT_LAUNCH_CHECK();
 }
 
@@ -677,9 +660,9 @@ mot_status mot_pdsa_lanczos(mot_ctx* c, int n, int flags, int k, unsigned long l
             }
             k_rand_vec<<<g1, NT, 0, s>>>(seed, c->eps, M, w);
             MOT_LAUNCH_CHECK();
-            k_dots<<<dim3(nb, 1), NT, 0, s>>>(w, 1, L, w, part);
+            launch_dependent(mot::dependent_launches(c), k_dots, dim3(nb, 1), NT, 0, s, w, 1, L, w, part);
             MOT_LAUNCH_CHECK();
-            k_normalise<<<g1, NT, 0, s>>>(w, part, nb, L, V, coef + 3LL * k);
+            launch_dependent(mot::dependent_launches(c), k_normalise, g1, NT, 0, s, w, part, nb, L, V, coef + 3LL * k);
             MOT_LAUNCH_CHECK();
             // the scalars of a step stay on the device and are read every BATCH steps (a
             // host read per orthogonalisation left the GPU idle for a third of a step);
@@ -693,11 +676,11 @@ mot_status mot_pdsa_lanczos(mot_ctx* c, int n, int flags, int k, unsigned long l
                     apply(c, V + (long long)j * L, w, s);
                     for (int pass = 0; pass < 2; ++pass) {   // w -= V_{0..j} (V_{0..j}^T w), twice
                         dots(c, V, j + 1, L, w, part, h, s);
-                        k_sub_combo<<<nb, NT, shm, s>>>(w, V, h, j + 1, L, coef + 3LL * j + pass,
+                        launch_dependent(mot::dependent_launches(c), k_sub_combo, nb, NT, shm, s, w, V, h, j + 1, L, coef + 3LL * j + pass,
                                                         pass ? part : nullptr);
                         MOT_LAUNCH_CHECK();
                     }
-                    k_normalise<<<g1, NT, 0, s>>>(w, part, nb, L, V + (long long)(j + 1) * L,
+                    launch_dependent(mot::dependent_launches(c), k_normalise, g1, NT, 0, s, w, part, nb, L, V + (long long)(j + 1) * L,
                                                   coef + 3LL * j + 2);
                     MOT_LAUNCH_CHECK();
                 }
@@ -727,7 +710,7 @@ mot_status mot_pdsa_lanczos(mot_ctx* c, int n, int flags, int k, unsigned long l
             k_rand_vec<<<g1, NT, 0, s>>>(seed, c->eps, M, w);
             MOT_LAUNCH_CHECK();
             dots(c, w, 1, L, w, part, b2d + k, s);               // ||w||^2 of the start
-            k_lz_c<<<g1, NT, 0, s>>>(w, b2d + k, L, vbuf[1]);   // v_0
+            launch_dependent(mot::dependent_launches(c), k_lz_c, g1, NT, 0, s, w, b2d + k, L, vbuf[1]);   // v_0
             MOT_LAUNCH_CHECK();
             constexpr int BATCH = 256;
             std::vector<double> ha(BATCH), hb(BATCH);
@@ -741,15 +724,15 @@ mot_status mot_pdsa_lanczos(mot_ctx* c, int n, int flags, int k, unsigned long l
                     double* v = vbuf[(j + 1) % 3];
                     double* vnext = vbuf[(j + 2) % 3];
                     apply(c, v, w, s);
-                    k_lz_a<<<nb, NT, 0, s>>>(w, vprev, j ? b2d + j - 1 : nullptr, v, L, part);
+                    launch_dependent(mot::dependent_launches(c), k_lz_a, nb, NT, 0, s, w, vprev, j ? b2d + j - 1 : nullptr, v, L, part);
                     MOT_LAUNCH_CHECK();
-                    k_sum_parts<<<1, NT, 0, s>>>(part, nb, ad + j);
+                    launch_dependent(mot::dependent_launches(c), k_sum_parts, 1, NT, 0, s, part, nb, ad + j);
                     MOT_LAUNCH_CHECK();
-                    k_lz_b<<<nb, NT, 0, s>>>(w, ad + j, v, L, part);
+                    launch_dependent(mot::dependent_launches(c), k_lz_b, nb, NT, 0, s, w, ad + j, v, L, part);
                     MOT_LAUNCH_CHECK();
-                    k_sum_parts<<<1, NT, 0, s>>>(part, nb, b2d + j);
+                    launch_dependent(mot::dependent_launches(c), k_sum_parts, 1, NT, 0, s, part, nb, b2d + j);
                     MOT_LAUNCH_CHECK();
-                    k_lz_c<<<g1, NT, 0, s>>>(w, b2d + j, L, vnext);
+                    launch_dependent(mot::dependent_launches(c), k_lz_c, g1, NT, 0, s, w, b2d + j, L, vnext);
                     MOT_LAUNCH_CHECK();
                 }
                 MOT_CUDA_TRY(cudaMemcpyAsync(ha.data(), ad + done, sizeof(double) * cnt,

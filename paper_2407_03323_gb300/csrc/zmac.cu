@@ -67,7 +67,7 @@ template <> struct Acc<float> {
 template <typename R> struct ZArgs {
     typedef typename CT<R>::c C;
     C* tmp;               // [3][W][plane]: y-transformed J_{n-1} in, z-inverted Phat out
-    C* ring;              // [hring][3][nbins]
+    C* ring;              // [hring][3][nbins]; null: Jhat is not kept (L = 1 only)
     const R* ghat;        // [lag][noct][6], lag 1 first
     const C* far[8];      // this step's entries of the far levels ([3][nbins] each)
     const C* tw;
@@ -119,9 +119,10 @@ __device__ __forceinline__ void products(const ZArgs<R>& a, const typename CT<R>
     constexpr int U = sizeof(R) == 4 ? 3 : 2;    // lags whose loads are issued together
     const int g = threadIdx.x & (a.split - 1);     // this lane's share of the lags
     const int items = a.Hw * TB, per = blockDim.x / a.split;
-    // all lanes make every round, the surplus on the last item (their results are dropped):
-    // the shares are added with full-warp shuffles
+    // all lanes of a warp make a round, the surplus on the last item (their results are
+    // dropped): the shares are added with full-warp shuffles
     for (int it0 = 0; it0 < items; it0 += per) {
+        if (it0 + (int)(threadIdx.x & ~31u) / a.split >= items) break;     // a warp without items
         const int it = min(it0 + (int)threadIdx.x / a.split, items - 1);
         const int t = it % TB, kw = it / TB;
         const int f = min(f0 + t, a.plane - 1);
@@ -278,19 +279,20 @@ __global__ void __launch_bounds__(256, 2) k_zmac(const __grid_constant__ ZArgs<R
         cp_async_commit_wait();
     }
     __syncthreads();
-    C* slot = a.ring + (long long)a.slot1 * 3 * a.nbins + f0;
+    const bool keep = a.ring != nullptr;
+    C* slot = keep ? a.ring + (long long)a.slot1 * 3 * a.nbins + f0 : nullptr;
     C* X = b0;
     if (a.fwd) {
         if constexpr (kFourStep) {
             four_step_lines<C, P1, P2, -1, NL>(b0, b1, stw, ld, a.W, [&](int k, int line, C v) {
                 b0[k * ld + line] = v;
                 const int c = line / TB, t = line % TB;
-                if (f0 + t < a.plane) slot[c * a.nbins + (long long)k * a.plane + t] = v;
+                if (keep && f0 + t < a.plane) slot[c * a.nbins + (long long)k * a.plane + t] = v;
             });
             __syncthreads();
         } else {
             X = fft_tile<C, NL>(b0, b1, P, a.rl.r, a.rl.n, ld, stw, -1);
-            for (int it = threadIdx.x; it < P * NL; it += blockDim.x) {
+            for (int it = threadIdx.x; keep && it < P * NL; it += blockDim.x) {
                 const int line = it % NL, k = it / NL;
                 const int c = line / TB, t = line % TB;
                 if (f0 + t < a.plane) slot[c * a.nbins + (long long)k * a.plane + t] = X[k * ld + line];
@@ -338,11 +340,18 @@ void launch(mot_ctx* c, const ZArgs<R>& a, cudaStream_t s) {
         throw MotError{MOT_ERR_ARG, "FFT length too large for one shared-memory tile"};
     MOT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
     MOT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-    // whole rounds of the product step: Hw = P / 2 + 1 is odd, and 33 x 4 pairs on 128 threads
-    // would take a second round for 4 of them (every round holds the FP64 units in full)
+    // Threads: whole rounds of the product step (Hw = P / 2 + 1 is odd, and 33 x 4 pairs on
+    // 128 threads would take a second round for 4 of them); where the transforms are the
+    // larger part (FP32, or few lags), a stage of them in one round too.  More threads than
+    // that leave room for fewer blocks (FP64, 28^3, 7 lags: 64 us with 128, 72 with 256;
+    // 20^3, one lag, Lanczos step: 149 with 96, 132 with 256).
     const int lanes = a.Hw * TB * a.split, rounds = (lanes + 255) / 256;
-    const int threads = ((lanes + rounds - 1) / rounds + 31) / 32 * 32;
-    launch_dependent(mot::dependent_launches(c), kern, (a.plane + TB - 1) / TB, threads, sm, s, a);
+    int threads = (lanes + rounds - 1) / rounds;
+    if (sizeof(R) == 4 || a.L < 4)
+        threads = std::max(threads,
+                           std::min(256, 3 * TB * (P1 * P2 > 1 ? std::max(P1, P2) : a.Pw / 2)));
+    launch_dependent(mot::dependent_launches(c), kern, (a.plane + TB - 1) / TB,
+                     (threads + 31) / 32 * 32, sm, s, a);
     MOT_LAUNCH_CHECK();
 }
 
@@ -356,25 +365,12 @@ void launch_len(mot_ctx* c, const ZArgs<R>& a, cudaStream_t s) {
     }
 }
 
-}  // namespace
-
-namespace mot {
-
 template <typename R>
-void zmac(mot_ctx* c, int n, bool fwd, int L, const typename CT<R>::c* const* far, int nfar,
-          cudaStream_t s) {
-    HistoryBuffers<R>& hb = hbuf<R>(c);
+ZArgs<R> z_args(mot_ctx* c) {
     ZArgs<R> a;
-    a.tmp = hb.tmp2;
-    a.ring = hb.jhat_ring;
-    a.ghat = hb.ghat;
-    for (int k = 0; k < 8; ++k) a.far[k] = k < nfar ? far[k] : nullptr;
+    a.tmp = hbuf<R>(c).tmp2;
+    for (int k = 0; k < 8; ++k) a.far[k] = nullptr;
     a.tw = table<R>(c->ax[2]);
-    a.nfar = nfar;
-    a.fwd = fwd;
-    a.hring = c->hring;
-    a.slot1 = (int)slot_index(n - 1, c->hring);
-    a.L = L;
     a.W = c->W;
     a.Pv = c->ax[1].P; a.Pw = c->ax[2].P;
     a.Hu = c->Hu; a.Hv = c->Hv; a.Hw = c->Hw;
@@ -384,6 +380,11 @@ void zmac(mot_ctx* c, int n, bool fwd, int L, const typename CT<R>::c* const* fa
     a.rl.P = c->ax[2].P;
     a.rl.n = c->ax[2].nrad;
     for (int i = 0; i < 16; ++i) a.rl.r[i] = c->ax[2].rad[i];
+    return a;
+}
+
+template <typename R>
+void run(mot_ctx* c, ZArgs<R>& a, cudaStream_t s) {
     // Lanes that share the lags of a bin: an FP64 instruction holds its sub-partition for 64
     // cycles whatever its lanes do, so a small grid spreads its products over the GPU
     // (8^3, 15 lags, 1,296 bin pairs: 35 us without the split)
@@ -403,6 +404,40 @@ void zmac(mot_ctx* c, int n, bool fwd, int L, const typename CT<R>::c* const* fa
     if (mid) launch_len<R, 4>(c, a, s);
     else if (a.plane >= 2LL * c->nsm) launch_len<R, 2>(c, a, s);
     else launch<R, 1, 1, 1>(c, a, s);
+}
+
+}  // namespace
+
+namespace mot {
+
+template <typename R>
+void zmac(mot_ctx* c, int n, bool fwd, int L, const typename CT<R>::c* const* far, int nfar,
+          cudaStream_t s) {
+    HistoryBuffers<R>& hb = hbuf<R>(c);
+    ZArgs<R> a = z_args<R>(c);
+    a.ring = hb.jhat_ring;
+    a.ghat = hb.ghat;
+    for (int k = 0; k < nfar; ++k) a.far[k] = far[k];
+    a.nfar = nfar;
+    a.fwd = fwd;
+    a.hring = c->hring;
+    a.slot1 = (int)slot_index(n - 1, c->hring);
+    a.L = L;
+    run(c, a, s);
+}
+
+// hb.tmp2 <- z-inverse of (spec [noct][6]) times the z transform of hb.tmp2: the Toeplitz
+// product with one kernel between fft_forward_xy and fft_inverse_yx
+void zproduct(mot_ctx* c, const double* spec, cudaStream_t s) {
+    ZArgs<double> a = z_args<double>(c);
+    a.ring = nullptr;
+    a.ghat = spec;
+    a.nfar = 0;
+    a.fwd = 1;
+    a.hring = 1;
+    a.slot1 = 0;
+    a.L = 1;
+    run(c, a, s);
 }
 
 template void zmac<double>(mot_ctx*, int, bool, int, const double2* const*, int, cudaStream_t);
