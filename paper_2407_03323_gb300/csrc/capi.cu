@@ -643,28 +643,23 @@ struct MarchRun {
         if (ev) MOT_CUDA_TRY(cudaEventRecord(ev[0], s));
         history_for(c, n, s, ev ? ev + 1 : nullptr);
         if (ev) MOT_CUDA_TRY(cudaEventRecord(ev[4], s));
-        mot::solve_step(c, n, En, c->norms + i, s);
+        // J_out: the solve itself writes the AoS copy, into the caller's device buffer or
+        // into slot k of the output ring; a device-to-host copy of a slot runs on the copy
+        // stream, overlapped with the next steps, and the slot is rewritten only after it
+        const bool ring = J_out && !dev_out;
+        const int k = i % kOutSlots;
+        double* dst = J_out ? J_out + (long long)i * step : nullptr;
+        double* out = ring ? c->outbuf + (long long)k * step : dst;
+        if (ring) MOT_CUDA_TRY(cudaStreamWaitEvent(s, c->out_done[k], 0));
+        mot::solve_step(c, n, En, c->norms + i, out, s);
         c->stats.launches += 2;
         if (ev) MOT_CUDA_TRY(cudaEventRecord(ev[5], s));
-        if (J_out) {
-            double* dst = J_out + (long long)i * 3 * c->M;
-            if (dev_out) {
-                mot::write_aos(c, n, dst, s);
-            } else {
-                // AoS copy into ring slot k on s, device-to-host copy on the copy
-                // stream, overlapped with the next steps; slot k is rewritten only
-                // after its previous copy has finished
-                const int k = i % kOutSlots;
-                double* slot = c->outbuf + (long long)k * step;
-                MOT_CUDA_TRY(cudaStreamWaitEvent(s, c->out_done[k], 0));
-                mot::write_aos(c, n, slot, s);
-                MOT_CUDA_TRY(cudaEventRecord(c->out_ready[k], s));
-                MOT_CUDA_TRY(cudaStreamWaitEvent(c->cstream, c->out_ready[k], 0));
-                MOT_CUDA_TRY(cudaMemcpyAsync(dst, slot, sizeof(double) * step,
-                                             cudaMemcpyDeviceToHost, c->cstream));
-                MOT_CUDA_TRY(cudaEventRecord(c->out_done[k], c->cstream));
-            }
-            c->stats.launches += 1;
+        if (ring) {
+            MOT_CUDA_TRY(cudaEventRecord(c->out_ready[k], s));
+            MOT_CUDA_TRY(cudaStreamWaitEvent(c->cstream, c->out_ready[k], 0));
+            MOT_CUDA_TRY(cudaMemcpyAsync(dst, out, sizeof(double) * step, cudaMemcpyDeviceToHost,
+                                         c->cstream));
+            MOT_CUDA_TRY(cudaEventRecord(c->out_done[k], c->cstream));
         }
     }
 

@@ -478,21 +478,6 @@ template <typename R> size_t smem_bytes(int P) {
     return sizeof(C) * ((size_t)tw_entries<C>(P) + 2 * (size_t)P * (Tile<R>::TB + 1));
 }
 
-// Dynamic shared memory of a pass kernel.  The limit is a process-wide attribute of
-// the kernel, and contexts of different sizes may launch it from several threads, so
-// it is set to the device's opt-in maximum (a value that never changes) rather than
-// to one launch's need; the need is checked against it.  The largest shared-memory
-// carveout is preferred so that several tiles are resident per SM.
-template <typename K> void set_smem(K kern, size_t bytes) {
-    int dev = 0, optin = 0;
-    MOT_CUDA_TRY(cudaGetDevice(&dev));
-    MOT_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    if (bytes > (size_t)optin)
-        throw MotError{MOT_ERR_ARG, "FFT length too large for one shared-memory tile"};
-    MOT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-    MOT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-}
-
 template <typename R, int P1, int P2>
 void launch_mid4s(const typename CT<R>::c* in, typename CT<R>::c* out,
                   const typename CT<R>::c* tw, const MidArgs& a, int nblocks, bool dep,
@@ -501,10 +486,10 @@ void launch_mid4s(const typename CT<R>::c* in, typename CT<R>::c* out,
     const size_t sm = sizeof(C) * ((size_t)P1 * P2 * 32 + (size_t)tw_entries<C>(P1 * P2));
     constexpr int threads = 32 * (P1 > P2 ? P1 : P2);
     if (a.dir < 0) {
-        set_smem(k_mid4s<R, P1, P2, -1>, sm);
+        allow_smem<k_mid4s<R, P1, P2, -1>>(sm);
         launch_dependent(dep, k_mid4s<R, P1, P2, -1>, nblocks, threads, sm, s, in, out, tw, a);
     } else {
-        set_smem(k_mid4s<R, P1, P2, +1>, sm);
+        allow_smem<k_mid4s<R, P1, P2, +1>>(sm);
         launch_dependent(dep, k_mid4s<R, P1, P2, +1>, nblocks, threads, sm, s, in, out, tw, a);
     }
     MOT_LAUNCH_CHECK();
@@ -526,7 +511,7 @@ void mid_pass(const typename CT<R>::c* in, typename CT<R>::c* out, const AxisFFT
     }
     constexpr int TB = Tile<R>::TB;
     const size_t sm = smem_bytes<R>(P);
-    set_smem(k_mid<R>, sm);
+    allow_smem<k_mid<R>>(sm);
     launch_dependent(dep, k_mid<R>, (int)((lines + TB - 1) / TB), NT, sm, s, in, out, table<R>(ax),
                                                                     radix_list(ax), a);
     MOT_LAUNCH_CHECK();
@@ -581,11 +566,11 @@ void launch_x4s(bool fwd, mot_ctx* c, const double* Jsoa, typename CT<R>::c* spe
     const long long npairs = 3LL * c->W * ((c->V + 1) / 2);
     const int blocks = (int)((npairs + kXL - 1) / kXL);
     if (fwd) {
-        set_smem(k_fwd_x4s<R, P1, P2>, sm);
+        allow_smem<k_fwd_x4s<R, P1, P2>>(sm);
         launch_dependent(mot::dependent_launches(c), k_fwd_x4s<R, P1, P2>, blocks, threads, sm, s, Jsoa, c->U, c->V, c->W, spec,
                                                          table<R>(c->ax[0]), scale);
     } else {
-        set_smem(k_inv_x4s<R, P1, P2>, sm);
+        allow_smem<k_inv_x4s<R, P1, P2>>(sm);
         launch_dependent(mot::dependent_launches(c), k_inv_x4s<R, P1, P2>, blocks, threads, sm, s, spec, c->U, c->V, c->W, real,
                                                          table<R>(c->ax[0]));
     }
@@ -614,7 +599,7 @@ void fft_forward_xy(mot_ctx* c, const double* Jsoa, cudaStream_t s, const double
     if (!x_pass_codelet<R>(true, c, Jsoa, hb.tmp1, nullptr, scale, s)) {
         const long long npairs = 3LL * W * ((V + 1) / 2);
         const size_t sm = smem_bytes<R>(Pu);
-        set_smem(k_fwd_x<R>, sm);
+        allow_smem<k_fwd_x<R>>(sm);
         launch_dependent(mot::dependent_launches(c), k_fwd_x<R>, (int)((npairs + TB - 1) / TB), NT, sm, s, Jsoa, U, V, W, hb.tmp1,
                                                                  table<R>(c->ax[0]),
                                                                  radix_list(c->ax[0]), scale);
@@ -663,7 +648,7 @@ void fft_inverse_yx(mot_ctx* c, R* out, cudaStream_t s) {
     if (!x_pass_codelet<R>(false, c, nullptr, hb.tmp1, out, nullptr, s)) {
         const long long npairs = 3LL * W * ((V + 1) / 2);
         const size_t sm = smem_bytes<R>(Pu);
-        set_smem(k_inv_x<R>, sm);
+        allow_smem<k_inv_x<R>>(sm);
         launch_dependent(mot::dependent_launches(c), k_inv_x<R>, (int)((npairs + TB - 1) / TB), NT, sm, s, hb.tmp1, U, V, W, out,
                                                                  table<R>(c->ax[0]),
                                                                  radix_list(c->ax[0]));

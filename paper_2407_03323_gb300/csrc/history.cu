@@ -720,10 +720,7 @@ __global__ void __launch_bounds__(96) k_far_reg(FarArgs<R> a) {
 template <typename R, int Q, int T>
 void far_launch_reg(mot_ctx* c, FarArgs<R>& a, cudaStream_t s) {
     typedef FarRegSmem<R, Q, T> SM;
-    MOT_CUDA_TRY(cudaFuncSetAttribute(k_far_reg<R, Q, T>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SM)));
-    MOT_CUDA_TRY(cudaFuncSetAttribute(k_far_reg<R, Q, T>,
-                                      cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+    allow_smem<k_far_reg<R, Q, T>>(sizeof(SM));
     const long long blocks = 4 * ((c->noct + SM::NB - 1) / SM::NB);
     launch_dependent(mot::dependent_launches(c), k_far_reg<R, Q, T>, (int)blocks, 96, sizeof(SM), s, a);
     MOT_LAUNCH_CHECK();
@@ -888,10 +885,7 @@ template <typename R, int P>
 void far_launch_4s(mot_ctx* c, FarArgs<R>& a, cudaStream_t s) {
     typedef Far4<R, P> F;
     const int sm_bytes = (int)sizeof(typename F::Smem);
-    MOT_CUDA_TRY(cudaFuncSetAttribute(k_far_4s<R, P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      sm_bytes));
-    MOT_CUDA_TRY(cudaFuncSetAttribute(k_far_4s<R, P>,
-                                      cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+    allow_smem<k_far_4s<R, P>>(sm_bytes);
     const long long blocks = 4 * ((c->noct + F::NB - 1) / F::NB);
     launch_dependent(mot::dependent_launches(c), k_far_4s<R, P>, (int)blocks, F::NTB, sm_bytes, s, a);
     MOT_LAUNCH_CHECK();
@@ -905,15 +899,7 @@ void far_launch(mot_ctx* c, FarArgs<R>& a, cudaStream_t s) {
     const size_t sm = sizeof(C) * ((size_t)tw_entries<C>(P) + 2 * (size_t)P * (3 * TB + 1));
     if (sm > 220 * 1024 || a.S > kMaxLevel)
         throw MotError{MOT_ERR_ARG, "blocked scheme: level too long for shared memory"};
-    // the limit is process-wide and P varies by level and context: set the device's
-    // opt-in maximum (never lowered by another launch), the need is checked above
-    int dev = 0, optin = 0;
-    MOT_CUDA_TRY(cudaGetDevice(&dev));
-    MOT_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    if (sm > (size_t)optin)
-        throw MotError{MOT_ERR_ARG, "blocked scheme: level too long for shared memory"};
-    MOT_CUDA_TRY(cudaFuncSetAttribute(k_far<R, TB>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-    MOT_CUDA_TRY(cudaFuncSetAttribute(k_far<R, TB>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+    allow_smem<k_far<R, TB>>(sm);
     const long long blocks = (long long)c->Hw * c->Hv * 4 * a.ntile;
     launch_dependent(mot::dependent_launches(c), k_far<R, TB>, (int)blocks, NT, sm, s, a);
     MOT_LAUNCH_CHECK();
@@ -1151,10 +1137,7 @@ template <int P>
 void far_launch_fs(mot_ctx* c, FarArgs<float>& a, cudaStream_t s) {
     typedef FarFS<P> F;
     const int sm_bytes = (int)sizeof(typename F::Smem);
-    MOT_CUDA_TRY(cudaFuncSetAttribute(k_far_fs<P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      sm_bytes));
-    MOT_CUDA_TRY(cudaFuncSetAttribute(k_far_fs<P>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                      100));
+    allow_smem<k_far_fs<P>>(sm_bytes);
     const long long blocks = (c->noct + F::NB - 1) / F::NB;
     launch_dependent(mot::dependent_launches(c), k_far_fs<P>, (int)blocks, F::NTH, sm_bytes, s, a);
     MOT_LAUNCH_CHECK();

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <atomic>
 #include <cstdint>
 #include <cstdio>
 #include <string>
@@ -73,6 +74,26 @@ void launch_dependent(bool dep, void (*kern)(P...), dim3 grid, dim3 block, size_
     cfg.attrs = at;
     cfg.numAttrs = 1;
     MOT_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...));
+}
+
+// Dynamic shared memory of a kernel up to the device's opt-in maximum, with the largest
+// carveout (several tiles per SM).  The limit is a process-wide attribute of the kernel; it
+// is set once per kernel and device, to a value that never changes, and the need of a launch
+// is checked against it.  (Set at every launch it was a third of the host time of a step,
+// which bounds several right-hand sides marched side by side.)
+template <auto Kern> void allow_smem(size_t bytes) {
+    static std::atomic<int> limit[64];      // per device, 0: not set yet
+    int dev = 0;
+    MOT_CUDA_TRY(cudaGetDevice(&dev));
+    int lim = dev < 64 ? limit[dev].load(std::memory_order_relaxed) : 0;
+    if (!lim) {
+        MOT_CUDA_TRY(cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+        MOT_CUDA_TRY(cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+        MOT_CUDA_TRY(cudaFuncSetAttribute(Kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+        if (dev < 64) limit[dev].store(lim, std::memory_order_relaxed);
+    }
+    if (bytes > (size_t)lim)
+        throw MotError{MOT_ERR_ARG, "transform too long for one shared-memory tile"};
 }
 
 // ------------------------------------------------------------------ FFT plan
@@ -296,12 +317,13 @@ template <typename R> void history_step(mot_ctx* c, int n, cudaStream_t s,
 template <typename R> void history_reset(mot_ctx* c, cudaStream_t s);
 template <typename R> void level_spectra(mot_ctx* c);
 // solve.cu
-void solve_step(mot_ctx* c, int n, const double* En, double* norm2_out, cudaStream_t s);
+// out: AoS J_n (device) or null
+void solve_step(mot_ctx* c, int n, const double* En, double* norm2_out, double* out,
+                cudaStream_t s);
 void stencil_setup(mot_ctx* c);
 const std::vector<int>& solve_shape(mot_ctx* c, const std::vector<int> (&tiles)[3]);
 void solve_halo_lists(mot_ctx* c);
 void chebyshev_setup(mot_ctx* c);
-void write_aos(mot_ctx* c, int n, double* out_dev, cudaStream_t s);
 void read_aos(mot_ctx* c, const double* in_dev, double* slot, cudaStream_t s);
 void history_out(mot_ctx* c, int n, double* out_dev, cudaStream_t s);
 void adjoint_step(mot_ctx* c, int tau, int n, const double* g_aos, const double* J_aos,

@@ -106,6 +106,7 @@ struct EpiArgs {
     float* bl;             //   low part of b_n [3][M]
     float4* x0;            //   x0 for the neighbours' reads
     double* rhs;           // adjoint: rhs on vacuum voxels (k_adj_vacuum)
+    double* out;           // AoS J_n (vacuum voxels written here, the others by the solve) or null
     const FitState* fit;
     double* part;          // [kSums][gridDim]
 };
@@ -161,6 +162,7 @@ __global__ void __launch_bounds__(NT) k_epilogue(const __grid_constant__ EpiArgs
             for (int k = 0; k < 3; ++k) {
                 if (ADJ) a.rhs[k * M + m] = (double)hist[k * M + m];
                 Jn[k * M + m] = 0.0;
+                if (!ADJ && a.out) a.out[m * 3 + k] = 0.0;
             }
             continue;
         }
@@ -184,6 +186,7 @@ __global__ void __launch_bounds__(NT) k_epilogue(const __grid_constant__ EpiArgs
                 } else {
                     const double x = t[k] * f2;     // chi = 0: no field term
                     Jn[k * M + m] = x;
+                    if (a.out) a.out[m * 3 + k] = x;
                     xin += x * x;
                 }
             }
@@ -296,6 +299,7 @@ struct CGArgs {
     const int* halo;      // resident tiles: halo voxels (k_halo_list)
     int nw;               // worker blocks; block nw sums the dot products and fits
     double* x;            // J_n slot (in/out), SoA [3][M]
+    double* out;          // AoS J_n or null
     const double* b;      // FP64: rhs / chi, SoA (this step's ring slot)
     const float* diag32;  // A's diagonal (T(0)/eps + delta_0)/chi, FP32 copy
     const double* diag;
@@ -1480,6 +1484,7 @@ __global__ void __launch_bounds__(T::NTH, RES ? 4 : 2) k_cg(const __grid_constan
                 double x = DF && !stored ? (double)a.xb[k * M + m].x : a.x[k * M + m];
                 x += back * (double)ec[k];
                 a.x[k * M + m] = x;
+                if (a.out) a.out[m * 3 + k] = x;
                 if (DF) a.xb[k * M + m].x = (float)x;
                 xx += x * x;
             }
@@ -1521,6 +1526,7 @@ __global__ void __launch_bounds__(T::NTH, RES ? 4 : 2) k_cg(const __grid_constan
                 if (zero) x = 0.0;
                 if (nonfinite) x = __longlong_as_double(0x7ff8000000000000LL);
                 a.x[k * M + m] = x;
+                if (a.out) a.out[m * 3 + k] = x;
                 if (DF) a.xb[k * M + m].x = (float)x;
                 xx += x * x;
             }
@@ -1552,17 +1558,6 @@ __global__ void __launch_bounds__(T::NTH, RES ? 4 : 2) k_cg(const __grid_constan
         a.status[1] |= flag;
         a.status[3] += its;
     }
-}
-
-// SoA slot -> AoS output [m][b]
-__global__ void k_to_aos(const double* __restrict__ x, long long M, double* __restrict__ out) {
-    pdl_trigger();
-    pdl_wait();
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= 3 * M) return;
-    const long long m = i / 3;
-    const int c = (int)(i % 3);
-    out[i] = x[c * M + m];
 }
 
 // AoS [m][b] -> SoA slot
@@ -1913,8 +1908,9 @@ int fit_slot(int n) { return n % kSlots; }
 int fit_pairs(const mot_ctx* c) { return std::min(c->fit_steps, kFit); }
 
 template <typename R, bool ADJ>
-void epilogue(mot_ctx* c, int n, const double* En, cudaStream_t s) {
+void epilogue(mot_ctx* c, int n, const double* En, double* out, cudaStream_t s) {
     EpiArgs a;
+    a.out = out;
     a.M = c->M;
     a.f = c->vfac;
     a.En = En;
@@ -1939,8 +1935,9 @@ void epilogue(mot_ctx* c, int n, const double* En, cudaStream_t s) {
 
 }  // namespace
 
-CGArgs make_cg_args(mot_ctx* c, int n, double* norm2_out) {
+CGArgs make_cg_args(mot_ctx* c, int n, double* norm2_out, double* out) {
     CGArgs a;
+    a.out = out;
     a.M = c->M;
     for (int e = 0; e < 27; ++e) a.noff[e] = c->noff[e];
     a.act = c->active;
@@ -2077,11 +2074,12 @@ void solve_halo_lists(mot_ctx* c) {
     else halo_lists<Tile4>(c);
 }
 
-// rhs + CG for step n; ||J_n||^2 into norm2_out (device), J_n in ring slot n
-void solve_step(mot_ctx* c, int n, const double* En, double* norm2_out, cudaStream_t s) {
-    if (c->precision == MOT_FP64) epilogue<double, false>(c, n, En, s);
-    else epilogue<float, false>(c, n, En, s);
-    CGArgs a = make_cg_args(c, n, norm2_out);
+// rhs + CG for step n; ||J_n||^2 into norm2_out (device), J_n in ring slot n and (AoS) in out
+void solve_step(mot_ctx* c, int n, const double* En, double* norm2_out, double* out,
+                cudaStream_t s) {
+    if (c->precision == MOT_FP64) epilogue<double, false>(c, n, En, out, s);
+    else epilogue<float, false>(c, n, En, out, s);
+    CGArgs a = make_cg_args(c, n, norm2_out, out);
     void* args[] = {&a};
     launch_cg(c, args, s);
 }
@@ -2110,9 +2108,9 @@ void adjoint_step(mot_ctx* c, int tau, int n, const double* g_aos, const double*
                   int j_first, double* grad_chi, double* lam_out, double* norm2_out,
                   cudaStream_t s) {
     const int s0 = (int)slot_index(tau, c->jring);
-    if (c->precision == MOT_FP64) epilogue<double, true>(c, tau, g_aos, s);
-    else epilogue<float, true>(c, tau, g_aos, s);
-    CGArgs a = make_cg_args(c, tau, norm2_out);
+    if (c->precision == MOT_FP64) epilogue<double, true>(c, tau, g_aos, nullptr, s);
+    else epilogue<float, true>(c, tau, g_aos, nullptr, s);
+    CGArgs a = make_cg_args(c, tau, norm2_out, nullptr);
     void* args[] = {&a};
     launch_cg(c, args, s);
     double* mu = c->J + (long long)s0 * 3 * c->M;
@@ -2124,13 +2122,6 @@ void adjoint_step(mot_ctx* c, int tau, int n, const double* g_aos, const double*
                                                          lam_out);
     MOT_LAUNCH_CHECK();
     c->stats.launches += 4;
-}
-
-void write_aos(mot_ctx* c, int n, double* out_dev, cudaStream_t s) {
-    const long long tot = 3 * c->M;
-    launch_dependent(mot::dependent_launches(c), k_to_aos, (int)((tot + NT - 1) / NT), NT, 0, s, c->J + slot_index(n, c->jring) * 3 * c->M,
-                                                       c->M, out_dev);
-    MOT_LAUNCH_CHECK();
 }
 
 }  // namespace mot

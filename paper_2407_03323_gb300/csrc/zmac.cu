@@ -330,16 +330,7 @@ template <typename R> size_t zmac_smem(int P, int TB) {
 template <typename R, int TB, int P1, int P2>
 void launch(mot_ctx* c, const ZArgs<R>& a, cudaStream_t s) {
     const size_t sm = zmac_smem<R>(a.Pw, TB);
-    auto kern = k_zmac<R, TB, P1, P2>;
-    // the limit is process-wide and Pw varies by context: the device's opt-in maximum,
-    // never lowered by another launch; the need was checked against it
-    int dev = 0, optin = 0;
-    MOT_CUDA_TRY(cudaGetDevice(&dev));
-    MOT_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    if (sm > (size_t)optin)
-        throw MotError{MOT_ERR_ARG, "FFT length too large for one shared-memory tile"};
-    MOT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-    MOT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+    allow_smem<k_zmac<R, TB, P1, P2>>(sm);
     // Threads: whole rounds of the product step (Hw = P / 2 + 1 is odd, and 33 x 4 pairs on
     // 128 threads would take a second round for 4 of them); where the transforms are the
     // larger part (FP32, or few lags), a stage of them in one round too.  More threads than
@@ -350,7 +341,7 @@ void launch(mot_ctx* c, const ZArgs<R>& a, cudaStream_t s) {
     if (sizeof(R) == 4 || a.L < 4)
         threads = std::max(threads,
                            std::min(256, 3 * TB * (P1 * P2 > 1 ? std::max(P1, P2) : a.Pw / 2)));
-    launch_dependent(mot::dependent_launches(c), kern, (a.plane + TB - 1) / TB,
+    launch_dependent(mot::dependent_launches(c), k_zmac<R, TB, P1, P2>, (a.plane + TB - 1) / TB,
                      (threads + 31) / 32 * 32, sm, s, a);
     MOT_LAUNCH_CHECK();
 }
