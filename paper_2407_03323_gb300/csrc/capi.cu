@@ -66,7 +66,7 @@ void free_all(mot_ctx* c) {
         c->eps = c->chi = c->cg_diag = c->tab = nullptr;
         c->vfac = nullptr;
         c->tab_l0 = nullptr;
-        c->active = c->nmask = c->tiles = c->halo = nullptr;
+        c->active = c->nmask = c->tiles = c->halo = c->vac = nullptr;
         c->diag32 = c->diag_lo = nullptr;
         c->h64.ghat = nullptr; c->h64.level_spec = nullptr;
         c->h32.ghat = nullptr; c->h32.level_spec = nullptr;
@@ -93,6 +93,8 @@ void free_all(mot_ctx* c) {
     cudaFree(c->nmask);
     cudaFree(c->tiles);
     cudaFree(c->halo);
+    cudaFree(c->vac);
+    cudaFree(c->norm_part);
     cudaFree(c->diag32);
     cudaFree(c->vfac);
     cudaFree(c->probe_tab);
@@ -152,10 +154,15 @@ void solve_alloc(mot_ctx* c) {
         MOT_CUDA_TRY(cudaMemset(c->cg_xl, 0, sizeof(float) * 4 * M));
     }
     MOT_CUDA_TRY(cudaMalloc(&c->fit, sizeof(double) * mot::kFitWords));
-    MOT_CUDA_TRY(cudaMalloc(&c->fit_part, sizeof(double) * mot::kFitSums * c->epi_blocks));
-    // [3][blocks] doubles, then (16-byte aligned) [2][blocks] exchange words
-    MOT_CUDA_TRY(cudaMalloc(&c->red, sizeof(double) * (7 * (size_t)c->cg_blocks + 1)));
-    MOT_CUDA_TRY(cudaMemset(c->red, 0, sizeof(double) * (7 * (size_t)c->cg_blocks + 1)));
+    // resident: 16-byte words of the solve's blocks; else doubles of the epilogue's
+    const size_t part = sizeof(double) * mot::kFitSums *
+                        (size_t)(c->cg_resident ? 2 * c->cg_blocks : c->epi_blocks);
+    MOT_CUDA_TRY(cudaMalloc(&c->fit_part, part));
+    MOT_CUDA_TRY(cudaMemset(c->fit_part, 0, part));
+    MOT_CUDA_TRY(cudaMalloc(&c->norm_part, sizeof(double) * 2 * c->norm_blocks));
+    // [2][blocks] doubles, then (16-byte aligned) [2][blocks] exchange words
+    MOT_CUDA_TRY(cudaMalloc(&c->red, sizeof(double) * 6 * (size_t)c->cg_blocks));
+    MOT_CUDA_TRY(cudaMemset(c->red, 0, sizeof(double) * 6 * (size_t)c->cg_blocks));
     MOT_CUDA_TRY(cudaMalloc(&c->dstatus, sizeof(int) * mot::kStatusWords));
     MOT_CUDA_TRY(cudaMemset(c->dstatus, 0, sizeof(int) * mot::kStatusWords));
 }
@@ -175,6 +182,21 @@ std::vector<int> active_tiles(const mot_ctx* c, const std::vector<double>& chi, 
                 if (any) tl.push_back(x0 | (y0 << 10) | (z0 << 20));
             }
     return tl;
+}
+
+// voxels in none of the solve's tiles (8 x 4 x 4, 8 x 4 x 8 or 8 x 8 x 8)
+std::vector<int> outside_tiles(const mot_ctx* c, const std::vector<int>& tiles) {
+    const int TY = c->cg_tile == 4 ? 8 : 4, TZ = c->cg_tile == 1 ? 4 : 8;
+    std::vector<char> in(c->M, 0);
+    for (int o : tiles)
+        for (int z = o >> 20; z < std::min((o >> 20) + TZ, c->W); ++z)
+            for (int y = (o >> 10) & 1023; y < std::min(((o >> 10) & 1023) + TY, c->V); ++y)
+                for (int x = o & 1023; x < std::min((o & 1023) + 8, c->U); ++x)
+                    in[((long long)z * c->V + y) * c->U + x] = 1;
+    std::vector<int> vac;
+    for (long long m = 0; m < c->M; ++m)
+        if (!in[m]) vac.push_back((int)m);
+    return vac;
 }
 
 void history_for(mot_ctx* c, int n, cudaStream_t s, cudaEvent_t* ev = nullptr) {
@@ -351,6 +373,12 @@ mot_status mot_create_padded(const int grid[3], const double h[3], double dt,
                 if (!tl.empty())
                     MOT_CUDA_TRY(cudaMemcpy(c->tiles, tl.data(), sizeof(int) * tl.size(),
                                             cudaMemcpyHostToDevice));
+                if (c->cg_resident && c->nvac) {
+                    const std::vector<int> vac = outside_tiles(c, tl);
+                    MOT_CUDA_TRY(cudaMalloc(&c->vac, sizeof(int) * vac.size()));
+                    MOT_CUDA_TRY(cudaMemcpy(c->vac, vac.data(), sizeof(int) * vac.size(),
+                                            cudaMemcpyHostToDevice));
+                }
             }
             std::vector<float> d32(M);
             std::vector<double> vf(4 * M);
@@ -420,10 +448,11 @@ mot_status mot_create_shared(mot_ctx* src, mot_ctx** out) {
     c->jring = src->jring; c->hring = src->hring;
     c->eps = src->eps; c->chi = src->chi; c->cg_diag = src->cg_diag;
     c->active = src->active; c->nmask = src->nmask; c->tiles = src->tiles; c->halo = src->halo;
+    c->vac = src->vac; c->nvac = src->nvac; c->norm_blocks = src->norm_blocks;
     c->ntiles = src->ntiles; c->nact = src->nact;
     c->diag32 = src->diag32; c->diag_lo = src->diag_lo; c->vfac = src->vfac;
     c->cg_tile = src->cg_tile; c->cg_resident = src->cg_resident; c->cg_split = src->cg_split;
-    c->epi_blocks = src->epi_blocks; c->epi_threads = src->epi_threads;
+    c->epi_blocks = src->epi_blocks;
     c->cheb_lmin = src->cheb_lmin; c->cheb_lmax = src->cheb_lmax; c->cheb_n = src->cheb_n;
     c->cheb_log_rate = src->cheb_log_rate; c->cheb_inv_theta = src->cheb_inv_theta;
     for (int k = 0; k < 64; ++k) { c->cheb_c1[k] = src->cheb_c1[k]; c->cheb_c2[k] = src->cheb_c2[k]; }
@@ -617,6 +646,7 @@ struct MarchRun {
             }
         }
         MOT_CUDA_TRY(cudaMemsetAsync(c->dstatus, 0, sizeof(int) * mot::kStatusWords, s));
+        c->norm_pending = nullptr;
         if (c->profiling) ensure_events(c, 6 * (size_t)n_steps);
         // whole periods as one CUDA graph: device-resident excitation and outputs, no
         // per-phase events, a capturable stream
@@ -652,7 +682,6 @@ struct MarchRun {
         double* out = ring ? c->outbuf + (long long)k * step : dst;
         if (ring) MOT_CUDA_TRY(cudaStreamWaitEvent(s, c->out_done[k], 0));
         mot::solve_step(c, n, En, c->norms + i, out, s);
-        c->stats.launches += 2;
         if (ev) MOT_CUDA_TRY(cudaEventRecord(ev[5], s));
         if (ring) {
             MOT_CUDA_TRY(cudaEventRecord(c->out_ready[k], s));
@@ -682,6 +711,7 @@ struct MarchRun {
     void fetch() {
         std::vector<double> nrm(n_steps);
         int hs[4];
+        mot::solve_finish(c, s);
         MOT_CUDA_TRY(cudaMemcpyAsync(nrm.data(), c->norms, sizeof(double) * n_steps,
                                      cudaMemcpyDeviceToHost, s));
         MOT_CUDA_TRY(cudaMemcpyAsync(hs, c->dstatus, sizeof(int) * 4, cudaMemcpyDeviceToHost, s));
@@ -912,6 +942,7 @@ mot_status mot_adjoint_run(mot_ctx* c, int n_count, const double* J_win, int win
             MOT_CUDA_TRY(cudaMalloc(&c->norms, sizeof(double) * n_count));
             c->norms_cap = n_count;
         }
+        c->norm_pending = nullptr;
         for (int i = 0; i < n_count; ++i) {
             const int tau = c->adj_done + 1 + i;
             const int n = c->adj_total + 1 - tau;
@@ -921,6 +952,7 @@ mot_status mot_adjoint_run(mot_ctx* c, int n_count, const double* J_win, int win
                               c->norms + i, s);
         }
         int hs[4];
+        mot::solve_finish(c, s);
         MOT_CUDA_TRY(cudaMemcpyAsync(hs, c->dstatus, sizeof(int) * 4, cudaMemcpyDeviceToHost, s));
         if (lambda && lamd != lambda)
             MOT_CUDA_TRY(cudaMemcpyAsync(lambda, lamd, sizeof(double) * step * n_count,

@@ -158,7 +158,11 @@ struct mot_ctx {
     double* fit = nullptr;       // fit state (kFitWords)
     double* fit_part = nullptr;  // epilogue's partial sums
     int fit_steps = 0;           // steps solved since the march state was reset
-    int epi_blocks = 1, epi_threads = 256;
+    int epi_blocks = 1;          // epilogue's blocks (solve not resident)
+    double* norm_part = nullptr; // [2][norm_blocks] blocks' shares of ||J_n||^2, n even and odd
+    int norm_blocks = 0;
+    double* norm_pending = nullptr;   // where the last launched step's norm goes (null: done)
+    int norm_step = 0;
     unsigned solve_seq = 0;      // solve launches (numbers their neighbour exchanges)
     int* active = nullptr;       // voxels with chi > 0
     int* nmask = nullptr;        // per active voxel: in-grid neighbours (27 bits)
@@ -167,6 +171,8 @@ struct mot_ctx {
     int cg_tile = 4;             // voxels per thread of the tile: 8x4x4, 8x4x8, 8x8x8
     bool cg_resident = false;    // one tile per block, kept in registers
     int* halo = nullptr;         //   halo voxels of every tile
+    int* vac = nullptr;          //   voxels outside every tile
+    long long nvac = 0;
     bool cg_split = false;       // FP64 residual by components
     float* diag32 = nullptr;     // FP32 copy of cg_diag
     double* vfac = nullptr;      // [4][M]: 0.5/eps, 1/chi (0 if chi = 0), 1/(0.5/eps + d0), chi
@@ -178,8 +184,8 @@ struct mot_ctx {
     float cheb_c1[64] = {0}, cheb_c2[64] = {0};
     double* red = nullptr;       // reduction scratch
     int* dstatus = nullptr;      // [0] cg iterations of last step, [1] flags, [2] first bad
-                                 // step, [3] total iterations, [4..7] the solve kernel's
-                                 // grid barrier (arrivals, -, abort, finished blocks)
+                                 // step, [3] total iterations, [4..6] the solve kernel's
+                                 // barrier words (CGArgs::bar)
     long long bar_budget = 0;    // longest barrier wait of the solve kernel, SM clock cycles
     double* norms = nullptr;     // per-step ||J_n||^2 of the current call
     int norms_cap = 0;
@@ -275,7 +281,7 @@ constexpr int kPwTable = 1 << 16;   // nodes of the plane-wave table of one call
 constexpr int kStatusWords = 8;     // device status words of a context (dstatus)
 constexpr int kFitVectors = 6;      // earlier right-hand sides that the solve's start fits
 constexpr int kFitWords = 72;       // doubles of the device fit state
-constexpr int kFitSums = kFitVectors + 2;   // partial sums of the epilogue per block
+constexpr int kFitSums = kFitVectors + 1;   // partial sums of a block for the fit
 constexpr double kBarrierBudgetS = 2.0;   // longest wait at a grid barrier of the solve
 
 // quadrature.cu
@@ -320,6 +326,8 @@ template <typename R> void level_spectra(mot_ctx* c);
 // out: AoS J_n (device) or null
 void solve_step(mot_ctx* c, int n, const double* En, double* norm2_out, double* out,
                 cudaStream_t s);
+// after the last step of a call: its ||J_n||^2
+void solve_finish(mot_ctx* c, cudaStream_t s);
 void stencil_setup(mot_ctx* c);
 const std::vector<int>& solve_shape(mot_ctx* c, const std::vector<int> (&tiles)[3]);
 void solve_halo_lists(mot_ctx* c);

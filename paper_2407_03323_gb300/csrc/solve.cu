@@ -52,8 +52,8 @@ __device__ __forceinline__ long long jslot(int s0, int l, int jring, long long s
 //     min || b_{n-1} - sum_i c_i b_{n-1-i} ||,        A x_{n-i} = b_{n-i},
 // applied one step later.  The right-hand sides of a band-limited march change
 // smoothly, so the fit of one step serves the next (start residual 1.7 times that of the
-// fit of b_n itself), and nothing of the fit is on the step's critical path: the epilogue
-// of step n forms the dot products <b_n, b_{n-i}> while it holds the values, and one block
+// fit of b_n itself), and nothing of the fit is on the step's critical path: what forms b_n
+// also forms the dot products <b_n, b_{n-i}> while it holds the values, and one block
 // of the solve kernel sums them, updates the Gram matrix of the ring and solves the F x F
 // system while the others iterate.  F = 6: relative start residual 3e-6 on the eps_r = 12
 // sphere in a pulse that rises smoothly from rest, 1e-4 .. 1e-3 within 100 steps of an
@@ -63,12 +63,13 @@ __device__ __forceinline__ long long jslot(int s0, int l, int jring, long long s
 // since the march state was reset, or a fit that leaves more than kFitPoor.
 constexpr int kFit = mot::kFitVectors;
 constexpr int kSlots = kFit + 1;           // ring of right-hand sides
-constexpr int kSums = kFit + 2;            // <b,b>, <b,b_{n-i}>, |x|^2 off the active set
+constexpr int kSums = mot::kFitSums;       // <b,b>, <b,b_{n-i}>
 constexpr double kFitPoor = 0.05;          // largest ||b - fit||^2 / ||b||^2 that is used
 constexpr double kFitPivot = 1e-13;        // relative pivot below which a vector is dropped
 
 struct FitRecord {
     double c[kFit];
+    float cf[kFit];    // rounded to FP32
     int use;           // 0: quadratic extrapolation
     int e;             // 2^e is near 1 / rms(b)
 };
@@ -81,6 +82,14 @@ static_assert(sizeof(FitState) <= sizeof(double) * mot::kFitWords, "fit state si
 // 2^e, |e| <= 1000 (double) / 120 (float)
 __device__ __forceinline__ double pow2d(int e) { return __hiloint2double((1023 + e) << 20, 0); }
 __device__ __forceinline__ float pow2f(int e) { return __int_as_float((127 + e) << 23); }
+// (double)v by integer operations: a conversion holds the sub-partition like any FP64 instruction
+__device__ __forceinline__ double widen(float v) {
+    const unsigned u = __float_as_uint(v), m = u & 0x7fffffffu;
+    if (m - 0x00800000u >= 0x7f000000u && m != 0u) return (double)v;    // denormal, Inf, NaN
+    const unsigned hi = m ? (m >> 3) + 0x38000000u : 0u;
+    return __hiloint2double((int)((u & 0x80000000u) | hi), (int)(m << 29));
+}
+__device__ __forceinline__ double widen(double v) { return v; }
 __device__ __forceinline__ bool is_zero(double v) { return (__double_as_longlong(v) << 1) == 0; }
 
 // b ring slot of step n - i, s0 = n mod kSlots
@@ -108,183 +117,285 @@ struct EpiArgs {
     double* rhs;           // adjoint: rhs on vacuum voxels (k_adj_vacuum)
     double* out;           // AoS J_n (vacuum voxels written here, the others by the solve) or null
     const FitState* fit;
-    double* part;          // [kSums][gridDim]
+    double* part;          // [kSums][blocks] partial sums
+    double* nrm;           // [blocks] |x|^2 off the active set
+    bool adj;
 };
 
-// One thread per voxel, its three components: the AoS excitation row and the factors are
-// read once and coalesced.  All loads of a voxel come before its stores (the new slot Jn
-// lies in the same ring the loads read from).  ADJ: the adjoint march (see below).
+// a thread's sums over its voxels: <b, b>, <b, b_{n-i}> and |x|^2 off the active set
+template <typename R> struct EpiSums {
+    typedef typename std::conditional<std::is_same<R, float>::value, float, double>::type D;
+    D bb = 0, dots[kFit];
+    double xin = 0.0;
+    __device__ EpiSums() {
+#pragma unroll
+        for (int i = 0; i < kFit; ++i) dots[i] = 0;
+    }
+};
+// what a step's voxels share: the start's coefficients and the scale of the FP32 sums
+template <typename R> struct EpiFit {
+    typename EpiSums<R>::D c[kFit];
+    bool use;
+    float scf;
+    __device__ EpiFit(const EpiArgs& a) {
+        const FitRecord& rec = a.fit->rec[a.n & 1];
+        use = rec.use != 0;
+        scf = std::is_same<R, float>::value ? pow2f(rec.e) : 1.f;
+#pragma unroll
+        for (int i = 0; i < kFit; ++i)
+            if constexpr (std::is_same<R, float>::value) c[i] = use ? rec.cf[i] : extrapolation(i);
+            else c[i] = use ? rec.c[i] : extrapolation(i);
+    }
+    __device__ static constexpr float extrapolation(int i) {
+        return i == 0 ? 3.f : i == 1 ? -3.f : i == 2 ? 1.f : 0.f;
+    }
+};
+
+// Right-hand side and start of one voxel, its three components: the AoS excitation row and
+// the factors are read once and coalesced.  All loads of a voxel come before its stores (the
+// new slot Jn lies in the same ring the loads read from).  adj: the adjoint march.
+// Returns whether the voxel is active; x0: its start (FP32-history, for the neighbours).
 // Bound by FP64 issue: an FP64 instruction holds its sub-partition for 64 cycles, so the
 // terms are arranged for few of them (b = ((e - g1 j1) - delta_2 j2 ..) / chi + hist: three
 // per component with FIR3), vacuum voxels with nothing but zeros in them take none, there
 // is no division (scales are powers of two), and FP32-history forms its dot products in
 // FP32: it keeps x and b of earlier steps as floats, which only shape the start and the
 // fit; the residual of the start that is stored is formed in float pairs.
-template <typename R, bool ADJ>
-__global__ void __launch_bounds__(NT) k_epilogue(const __grid_constant__ EpiArgs a) {
-    pdl_trigger();
-    pdl_wait();
+template <typename R>
+__device__ __forceinline__ bool epi_voxel(const EpiArgs& a, bool adj, const EpiFit<R>& fit,
+                                          long long m, EpiSums<R>& sum, float4& x0v) {
     constexpr bool DF = std::is_same<R, float>::value;
-    typedef typename std::conditional<DF, float, double>::type D;   // dot products
     const long long M = a.M, st = 3 * M;
     const R* hist = static_cast<const R*>(a.hist);
-    const FitRecord& rec = a.fit->rec[a.n & 1];
-    const bool use = rec.use != 0;
-    const float scf = DF ? pow2f(rec.e) : 1.f;
-    D c[kFit];
-#pragma unroll
-    for (int i = 0; i < kFit; ++i)
-        c[i] = use ? (D)rec.c[i] : (D)(i == 0 ? 3.0 : i == 1 ? -3.0 : i == 2 ? 1.0 : 0.0);
     const double* r1 = a.Jring + jslot(a.s0, 1, a.jring, st);
     const double* r2 = a.Jring + jslot(a.s0, 2, a.jring, st);
     double* Jn = a.Jring + jslot(a.s0, 0, a.jring, st);
     const double d1 = a.tp.n > 1 ? a.tp.d[1] : 0.0, d2 = a.tp.n > 2 ? a.tp.d[2] : 0.0;
-    double xin = 0.0;
-    D bb = 0, dots[kFit];
+    const double f0 = a.f[m], ichi = a.f[M + m];
+    const bool active = !is_zero(ichi);
+    double t[3], j1[3], j2[3] = {0.0, 0.0, 0.0};
+    bool zero = true;
 #pragma unroll
-    for (int i = 0; i < kFit; ++i) dots[i] = 0;
-    for (long long m = (long long)blockIdx.x * blockDim.x + threadIdx.x; m < M;
-         m += (long long)gridDim.x * blockDim.x) {
-        const double f0 = a.f[m], ichi = a.f[M + m];
-        const bool active = !is_zero(ichi);
-        double t[3], j1[3], j2[3] = {0.0, 0.0, 0.0};
-        bool zero = true;
+    for (int k = 0; k < 3; ++k) {
+        const long long i = k * M + m;
+        t[k] = a.En ? a.En[m * 3 + k] : 0.0;
+        j1[k] = r1[i];
+        if (a.tp.n > 2) j2[k] = r2[i];
+        zero = zero && is_zero(t[k]) && is_zero(j1[k]) && is_zero(j2[k]);
+    }
+    // the vectors of the earlier steps and the history, requested before the first of them is
+    // used (one trip to L2 instead of one per step: 14 -> 5 thousand cycles a voxel)
+    R hv[3];
+    typename std::conditional<DF, float2, double>::type w[kFit][3];
+    if (active || adj) {
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const long long i = k * M + m;
-            t[k] = a.En ? a.En[m * 3 + k] : 0.0;
-            j1[k] = r1[i];
-            if (a.tp.n > 2) j2[k] = r2[i];
-            zero = zero && is_zero(t[k]) && is_zero(j1[k]) && is_zero(j2[k]);
-        }
-        if (!active && zero && a.tp.n <= 3) {      // vacuum at rest
+        for (int k = 0; k < 3; ++k) hv[k] = hist[k * M + m];
+    }
+    if (active) {
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                if (ADJ) a.rhs[k * M + m] = (double)hist[k * M + m];
-                Jn[k * M + m] = 0.0;
-                if (!ADJ && a.out) a.out[m * 3 + k] = 0.0;
-            }
-            continue;
-        }
-        const double g1 = f0 + d1;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) t[k] -= g1 * j1[k] + d2 * j2[k];
-        for (int l = 3; l < a.tp.n; ++l) {
-            const double* rl = a.Jring + jslot(a.s0, l, a.jring, st);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) t[k] -= a.tp.d[l] * rl[k * M + m];
-        }
-        if (!active) {
-            const double f2 = a.f[2 * M + m];
+        for (int i = 0; i < kFit; ++i)
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                if (ADJ) {
-                    // the solve's iterate must vanish off the active set; vacuum voxels
-                    // get their lambda after the solve (k_adj_post), when mu is known
-                    a.rhs[k * M + m] = t[k] + (double)hist[k * M + m];
-                    Jn[k * M + m] = 0.0;
+                if constexpr (DF) {
+                    w[i][k] = make_float2(0.f, 0.f);
+                    if (i < a.nv) w[i][k] = a.xb[(long long)fslot(a.bs, i + 1) * st + k * M + m];
                 } else {
-                    const double x = t[k] * f2;     // chi = 0: no field term
-                    Jn[k * M + m] = x;
-                    if (a.out) a.out[m * 3 + k] = x;
-                    xin += x * x;
+                    w[i][k] = 0.0;
+                    if (i < a.nv) w[i][k] = a.b64[(long long)fslot(a.bs, i + 1) * st + k * M + m];
                 }
             }
-            continue;
-        }
-        double b[3];
+    }
+    if (!active && zero && a.tp.n <= 3) {      // vacuum at rest
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            const double h = (double)hist[k * M + m];
-            b[k] = ADJ ? t[k] + h : t[k] * ichi + h;
+            if (adj) a.rhs[k * M + m] = widen(hv[k]);
+            Jn[k * M + m] = 0.0;
+            if (!adj && a.out) a.out[m * 3 + k] = 0.0;
         }
-        if constexpr (DF) {
-            float bh[3], xs[3] = {0.f, 0.f, 0.f};
+        return false;
+    }
+    const double g1 = f0 + d1;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        t[k] -= g1 * j1[k];
+        t[k] -= d2 * j2[k];
+    }
+    for (int l = 3; l < a.tp.n; ++l) {
+        const double* rl = a.Jring + jslot(a.s0, l, a.jring, st);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) t[k] -= a.tp.d[l] * rl[k * M + m];
+    }
+    if (!active) {
+        const double f2 = a.f[2 * M + m];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            if (adj) {
+                // the solve's iterate must vanish off the active set; vacuum voxels
+                // get their lambda after the solve (k_adj_post), when mu is known
+                a.rhs[k * M + m] = t[k] + widen(hv[k]);
+                Jn[k * M + m] = 0.0;
+            } else {
+                const double x = t[k] * f2;     // chi = 0: no field term
+                Jn[k * M + m] = x;
+                if (a.out) a.out[m * 3 + k] = x;
+                sum.xin += x * x;
+            }
+        }
+        return false;
+    }
+    double b[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const double h = widen(hv[k]);
+        b[k] = adj ? t[k] + h : t[k] * ichi + h;
+    }
+    if constexpr (DF) {
+        float bh[3], xs[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            bh[k] = (float)b[k];
+            a.bl[k * M + m] = (float)(b[k] - widen(bh[k]));
+            sum.bb += (bh[k] * fit.scf) * (bh[k] * fit.scf);
+        }
+#pragma unroll
+        for (int i = 0; i < kFit; ++i) {
+            if (i >= a.nv) continue;
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                bh[k] = (float)b[k];
-                a.bl[k * M + m] = (float)(b[k] - (double)bh[k]);
-                bb += (bh[k] * scf) * (bh[k] * scf);
+                xs[k] += fit.c[i] * w[i][k].x;
+                sum.dots[i] += (bh[k] * fit.scf) * (w[i][k].y * fit.scf);
             }
-#pragma unroll
-            for (int i = 0; i < kFit; ++i) {
-                if (i >= a.nv) break;
-                const float2* v = a.xb + (long long)fslot(a.bs, i + 1) * st + m;
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    const float2 w = v[k * M];
-                    xs[k] += c[i] * w.x;
-                    dots[i] += (bh[k] * scf) * (w.y * scf);
-                }
-            }
-            if (!use) {   // quadratic extrapolation from the FP64 ring
-                const double* q2 = a.Jring + jslot(a.s0, 2, a.jring, st);
-                const double* q3 = a.Jring + jslot(a.s0, 3, a.jring, st);
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    const double x0 = 3.0 * j1[k] - 3.0 * q2[k * M + m] + q3[k * M + m];
-                    xs[k] = (float)(ADJ ? a.f[3 * M + m] * x0 : x0);
-                }
-            }
-            float2* v0 = a.xb + (long long)a.bs * st + m;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) v0[k * M] = make_float2(xs[k], bh[k]);
-            a.x0[m] = make_float4(xs[0], xs[1], xs[2], 0.f);
-        } else {
-            double x0[3] = {0.0, 0.0, 0.0};
-#pragma unroll
-            for (int i = 0; i < kFit; ++i) {
-                if (i >= (use ? a.nv : 3)) break;
-                const double* rx = a.Jring + jslot(a.s0, i + 1, a.jring, st);
-#pragma unroll
-                for (int k = 0; k < 3; ++k) x0[k] += c[i] * (i == 0 ? j1[k] : rx[k * M + m]);
-            }
-#pragma unroll
-            for (int i = 0; i < kFit; ++i) {
-                if (i >= a.nv) break;
-                const double* rb = a.b64 + (long long)fslot(a.bs, i + 1) * st;
-#pragma unroll
-                for (int k = 0; k < 3; ++k) dots[i] += b[k] * rb[k * M + m];
-            }
-            double* b0 = a.b64 + (long long)a.bs * st;
-            const double chi = ADJ ? a.f[3 * M + m] : 1.0;
+        }
+        if (!fit.use) {   // quadratic extrapolation from the FP64 ring
+            const double* q2 = a.Jring + jslot(a.s0, 2, a.jring, st);
+            const double* q3 = a.Jring + jslot(a.s0, 3, a.jring, st);
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                bb += b[k] * b[k];
-                b0[k * M + m] = b[k];
-                Jn[k * M + m] = ADJ ? chi * x0[k] : x0[k];
+                const double x0 = 3.0 * j1[k] - 3.0 * q2[k * M + m] + q3[k * M + m];
+                xs[k] = (float)(adj ? a.f[3 * M + m] * x0 : x0);
             }
+        }
+        float2* v0 = a.xb + (long long)a.bs * st + m;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) v0[k * M] = make_float2(xs[k], bh[k]);
+        x0v = make_float4(xs[0], xs[1], xs[2], 0.f);
+    } else {
+        double x0[3] = {0.0, 0.0, 0.0}, wx[kFit][3];
+        const int nx = fit.use ? a.nv : 3;
+#pragma unroll
+        for (int i = 0; i < kFit; ++i)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                wx[i][k] = j1[k];
+                if (i > 0 && i < nx)
+                    wx[i][k] = a.Jring[jslot(a.s0, i + 1, a.jring, st) + k * M + m];
+            }
+#pragma unroll
+        for (int i = 0; i < kFit; ++i) {
+            if (i >= a.nv) continue;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) sum.dots[i] += b[k] * w[i][k];
+        }
+#pragma unroll
+        for (int i = 0; i < kFit; ++i) {
+            if (i >= nx) continue;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) x0[k] += fit.c[i] * wx[i][k];
+        }
+        double* b0 = a.b64 + (long long)a.bs * st;
+        const double chi = adj ? a.f[3 * M + m] : 1.0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            sum.bb += b[k] * b[k];
+            b0[k * M + m] = b[k];
+            Jn[k * M + m] = adj ? chi * x0[k] : x0[k];
         }
     }
-    // block sums: every thread leaves its values in shared memory, then one warp per value
-    // adds them (the shuffles run on one partial per lane instead of on every thread's).
-    // FP32-history partials stay scaled by 4^e (fit_block unscales the totals).
-    __shared__ D red[kFit + 1][NT + 1];
+    return true;
+}
+
+// A warp's sums of the kSums values, added up lane against lane with the values dealt out on
+// the way: 4 + 2 + 1 + 1 + 1 additions for eight values instead of five each.  Lane 4 q
+// returns the sum of value q.
+template <typename R>
+__device__ __forceinline__ typename EpiSums<R>::D epi_warp_sums(const EpiSums<R>& sum) {
+    typedef typename EpiSums<R>::D D;
+    static_assert(kSums <= 8, "three exchange steps deal out eight values");
+    D v[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] = q == 0 ? sum.bb : q <= kFit ? sum.dots[q - 1] : (D)0;
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 16, n = 4; o >= 4; o >>= 1, n >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (q < n) {
+                const D keep = up ? v[q + n] : v[q], send = up ? v[q] : v[q + n];
+                v[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+    }
+    D r = v[0];
+    r += __shfl_xor_sync(0xffffffffu, r, 2);
+    r += __shfl_xor_sync(0xffffffffu, r, 1);
+    return r;
+}
+// A block's sums: the warps' in shared memory (stash), a barrier of the block, then one warp,
+// whose lane q < kSums returns the sum of value q.  FP32-history sums stay scaled by 4^e
+// (fit_block unscales the totals).
+template <typename R, int NTH> using EpiRed = typename EpiSums<R>::D[NTH / 32][8];
+template <typename R, int NTH>
+__device__ __forceinline__ void epi_stash(EpiRed<R, NTH>& red, const EpiSums<R>& sum) {
+    const typename EpiSums<R>::D r = epi_warp_sums<R>(sum);
+    if ((threadIdx.x & 3) == 0) red[threadIdx.x >> 5][(threadIdx.x & 31) >> 2] = r;
+}
+template <typename R, int NTH>
+__device__ __forceinline__ double epi_block_sum(const EpiRed<R, NTH>& red) {
+    const int q = threadIdx.x & 7;
+    typename EpiSums<R>::D v = red[0][q];
+#pragma unroll
+    for (int w = 1; w < NTH / 32; ++w) v += red[w][q];
+    return (double)v;
+}
+// |x|^2 off the active set, the block's share
+__device__ __forceinline__ void epi_vacuum_norm(double xin, double* out) {
     __shared__ double redx[NT / 32];
-    red[0][threadIdx.x] = bb;
-#pragma unroll
-    for (int i = 0; i < kFit; ++i) red[1 + i][threadIdx.x] = dots[i];
-    const bool vac = __syncthreads_or(!is_zero(xin));
-    const int nw = blockDim.x >> 5, lane = threadIdx.x & 31;
-    for (int q = threadIdx.x >> 5; q < kFit + 1; q += nw) {
-        D v = 0;
-        for (int t = lane; t < (int)blockDim.x; t += 32) v += red[q][t];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) a.part[(long long)q * gridDim.x + blockIdx.x] = (double)v;
-    }
-    double* xpart = a.part + (long long)(kSums - 1) * gridDim.x + blockIdx.x;
-    if (!vac) {
-        if (threadIdx.x == 0) *xpart = 0.0;
+    if (!__syncthreads_or(!is_zero(xin))) {
+        if (threadIdx.x == 0) *out = 0.0;
         return;
     }
     for (int o = 16; o > 0; o >>= 1) xin += __shfl_down_sync(0xffffffffu, xin, o);
-    if (lane == 0) redx[threadIdx.x >> 5] = xin;
+    if ((threadIdx.x & 31) == 0) redx[threadIdx.x >> 5] = xin;
     __syncthreads();
     if (threadIdx.x == 0) {
         double v = 0.0;
-        for (int w = 0; w < nw; ++w) v += redx[w];
-        *xpart = v;
+        for (int w = 0; w < (int)blockDim.x / 32; ++w) v += redx[w];
+        *out = v;
     }
+}
+
+// The epilogue of grids whose solve keeps its vectors in memory (resident solves form the
+// right-hand side of their own tile themselves, see k_cg): one thread per voxel.  104^3
+// sphere, solve phase with it: 414 -> 376 us with the loads of a voxel requested together and
+// eight instead of eleven FP64 instructions a component.
+template <typename R, bool ADJ>
+__global__ void __launch_bounds__(NT) k_epilogue(const __grid_constant__ EpiArgs a) {
+    pdl_trigger();
+    pdl_wait();
+    const EpiFit<R> fit(a);
+    EpiSums<R> sum;
+    for (long long m = (long long)blockIdx.x * blockDim.x + threadIdx.x; m < a.M;
+         m += (long long)gridDim.x * blockDim.x) {
+        float4 x0;
+        const bool active = epi_voxel<R>(a, ADJ, fit, m, sum, x0);
+        if (std::is_same<R, float>::value && active) a.x0[m] = x0;
+    }
+    __shared__ EpiRed<R, NT> red;
+    epi_stash<R, NT>(red, sum);
+    __syncthreads();
+    if (threadIdx.x < kSums)
+        a.part[(long long)threadIdx.x * gridDim.x + blockIdx.x] = epi_block_sum<R, NT>(red);
+    epi_vacuum_norm(sum.xin, a.nrm + blockIdx.x);
 }
 
 struct CGArgs {
@@ -314,7 +425,7 @@ struct CGArgs {
     const float* bl;
     const float* diag_lo;
     float4* xl;
-    double* red;          // [3][nw] FP64 partial sums: norm; wide residual sums
+    double* red;          // [2][nw] FP64 partial sums: wide residual sums
     float4* red4;         // [2][nw] exchanged partial sums (values, sequence number)
     double tol2;          // outer tolerance^2 (relative to ||b||^2)
     float tol;
@@ -327,11 +438,19 @@ struct CGArgs {
     int max_outer;
     int step;             // time index n (for the status record)
     int* status;          // [0] inner its, [1] flags, [2] first bad step, [3] total its
-    unsigned* bar;        // grid barrier: [0] arrivals, [2] abort, [3] finished blocks
+    unsigned* bar;        // [0], [1] arrivals at the grid barriers of even and odd launches,
+                          // [2] abort
+    int parity;           // of this launch; its block 0 clears the other's arrival words
     long long bar_budget; // longest wait at one barrier, SM clock cycles
-    double* norm2;        // ||x||^2 output
+    double* nrm;          // [nred] |x|^2 of every block of this step
+    const double* nrm_prev;   // of the step before, added up by the fit block into
+    double* norm_prev;        // ||x||^2 of that step (null: none to do)
+    int nred, prev_step;
+    const int* vac;       // resident: voxels outside every tile, taken by the blocks past nw
+    int nvac, nvb;
     FitState* fit;
     const double* part;   // epilogue's partial sums [kSums][nepi]
+    float4* part4;        // resident: those of the solve's blocks (value, tag seq) [kSums][nw]
     int nepi;
     int bs, nv;           // ring slot of b_n, valid pairs before it
     unsigned seq;         // first sequence number of this launch's exchanges
@@ -440,17 +559,13 @@ __device__ __forceinline__ void df_split(double v, float& h, float& l) {
     l = (float)(v - (double)h);
 }
 
-// pair EP, 26 - EP in double-float (same zero pattern as stencil_pair).  load(e, vh, vl)
-// gives the x pair of neighbour e (zero outside the grid); PAIR = false: x is a float (the
-// start), its low part zero
-template <int EP, bool PAIR, typename V>
-__device__ __forceinline__ void stencil_pair_df(V&& load, float* oh, float* ol) {
-    constexpr int EM = 26 - EP;
-    constexpr int ex = EP % 3 - 1, ey = (EP / 3) % 3 - 1, ez = EP / 9 - 1;
+// (oh, ol) -= G_0 (x_e + x_-e), the pair of neighbours ah + al and bh + bl; COUPLED: with the
+// couplings of the components (exactly zero on the three axis pairs)
+template <bool PAIR, bool COUPLED>
+__device__ __forceinline__ void stencil_pair_df(int e, const float4& ah, const float4& al,
+                                                const float4& bh, const float4& bl, float* oh,
+                                                float* ol) {
     float sh[3], sl[3];
-    float4 ah, al, bh, bl;
-    load(std::integral_constant<int, EP>(), ah, al);
-    load(std::integral_constant<int, EM>(), bh, bl);
     df_two_sum(ah.x, bh.x, sh[0], sl[0]);
     df_two_sum(ah.y, bh.y, sh[1], sl[1]);
     df_two_sum(ah.z, bh.z, sh[2], sl[2]);
@@ -459,28 +574,32 @@ __device__ __forceinline__ void stencil_pair_df(V&& load, float* oh, float* ol) 
         sl[1] = __fadd_rn(sl[1], __fadd_rn(al.y, bl.y));
         sl[2] = __fadd_rn(sl[2], __fadd_rn(al.z, bl.z));
     }
-    const float* H = c_st32 + EP * 6;
-    const float* L = c_stl + EP * 6;
+    const float* H = c_st32 + e * 6;
+    const float* L = c_stl + e * 6;
     df_msub(H[0], L[0], sh[0], sl[0], oh[0], ol[0]);
     df_msub(H[1], L[1], sh[1], sl[1], oh[1], ol[1]);
     df_msub(H[2], L[2], sh[2], sl[2], oh[2], ol[2]);
-    if constexpr (ex != 0 && ey != 0) {
-        df_msub(H[3], L[3], sh[1], sl[1], oh[0], ol[0]);
-        df_msub(H[3], L[3], sh[0], sl[0], oh[1], ol[1]);
-    }
-    if constexpr (ex != 0 && ez != 0) {
-        df_msub(H[4], L[4], sh[2], sl[2], oh[0], ol[0]);
-        df_msub(H[4], L[4], sh[0], sl[0], oh[2], ol[2]);
-    }
-    if constexpr (ey != 0 && ez != 0) {
-        df_msub(H[5], L[5], sh[2], sl[2], oh[1], ol[1]);
-        df_msub(H[5], L[5], sh[1], sl[1], oh[2], ol[2]);
+    if constexpr (COUPLED) {      // (an edge pair has one of the three, a corner pair all)
+        if (H[3] != 0.f) {
+            df_msub(H[3], L[3], sh[1], sl[1], oh[0], ol[0]);
+            df_msub(H[3], L[3], sh[0], sl[0], oh[1], ol[1]);
+        }
+        if (H[4] != 0.f) {
+            df_msub(H[4], L[4], sh[2], sl[2], oh[0], ol[0]);
+            df_msub(H[4], L[4], sh[0], sl[0], oh[2], ol[2]);
+        }
+        if (H[5] != 0.f) {
+            df_msub(H[5], L[5], sh[2], sl[2], oh[1], ol[1]);
+            df_msub(H[5], L[5], sh[1], sl[1], oh[2], ol[2]);
+        }
     }
 }
 
 // r = b - A x at an active voxel in double-float, rounded to FP32.  dh, dl: its diagonal;
-// bh, bl: its b pair
-template <bool PAIR, typename V>
+// bh, bl: its b pair; load(o, vh, vl): the voxel at halo offset o, HX and HXY the halo's
+// strides.  A loop over the neighbour pairs: the pass runs once or twice a step, and written
+// out (1200 instructions a voxel, 19 KB) it waited for its own code.
+template <bool PAIR, int HX, int HXY, typename V>
 __device__ __forceinline__ float4 residual_df_at(float dh, float dl, const float* bh,
                                                  const float* bl, V&& load) {
     float oh[3] = {0.f, 0.f, 0.f}, ol[3] = {0.f, 0.f, 0.f};   // o = A x
@@ -488,7 +607,7 @@ __device__ __forceinline__ float4 residual_df_at(float dh, float dl, const float
     const float* L0 = c_stl + 13 * 6;
     // centre block: (d - G_0(0)) x; G_0(0) is diagonal (parity)
     float4 c4, cl4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    load(std::integral_constant<int, 13>(), c4, cl4);
+    load(0, c4, cl4);
     const float ch[3] = {c4.x, c4.y, c4.z};
     const float cl[3] = {PAIR ? cl4.x : 0.f, PAIR ? cl4.y : 0.f, PAIR ? cl4.z : 0.f};
 #pragma unroll
@@ -497,19 +616,20 @@ __device__ __forceinline__ float4 residual_df_at(float dh, float dl, const float
         df_msub(H0[k], L0[k], ch[k], cl[k], oh[k], ol[k]);
     }
     // o = (d - G_0(0)) x - sum_pairs G_0(e) (x_e + x_-e) = A x
-    stencil_pair_df<14, PAIR>(load, oh, ol);
-    stencil_pair_df<15, PAIR>(load, oh, ol);
-    stencil_pair_df<16, PAIR>(load, oh, ol);
-    stencil_pair_df<17, PAIR>(load, oh, ol);
-    stencil_pair_df<18, PAIR>(load, oh, ol);
-    stencil_pair_df<19, PAIR>(load, oh, ol);
-    stencil_pair_df<20, PAIR>(load, oh, ol);
-    stencil_pair_df<21, PAIR>(load, oh, ol);
-    stencil_pair_df<22, PAIR>(load, oh, ol);
-    stencil_pair_df<23, PAIR>(load, oh, ol);
-    stencil_pair_df<24, PAIR>(load, oh, ol);
-    stencil_pair_df<25, PAIR>(load, oh, ol);
-    stencil_pair_df<26, PAIR>(load, oh, ol);
+    auto pair = [&](int e, int o, auto coupled) {
+        float4 ah, al, gh, gl;
+        load(o, ah, al);
+        load(-o, gh, gl);
+        stencil_pair_df<PAIR, decltype(coupled)::value>(e, ah, al, gh, gl, oh, ol);
+    };
+    pair(14, 1, std::false_type());
+    pair(16, HX, std::false_type());
+    pair(22, HXY, std::false_type());
+#pragma unroll 1
+    for (int e = 15; e < 27; ++e) {
+        if (e == 16 || e == 22) continue;
+        pair(e, (e / 9 - 1) * HXY + ((e / 3) % 3 - 1) * HX + e % 3 - 1, std::true_type());
+    }
     float r[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -545,9 +665,6 @@ template <int X, int Y, int Z, int V> struct TileShape {
         lz = threadIdx.x / (TX * TY) * VPT;
     }
     __device__ static int hidx(int lx, int ly, int lz) { return ((lz + 1) * HY + ly + 1) * HX + lx + 1; }
-    template <int E> __device__ static constexpr int off() {
-        return ((E / 9 - 1) * HY + ((E / 3) % 3 - 1)) * HX + (E % 3 - 1);
-    }
 };
 typedef TileShape<8, 4, 4, 1> Tile1;
 typedef TileShape<8, 4, 8, 2> Tile2;
@@ -833,6 +950,34 @@ __device__ __forceinline__ void wait_failed(const CGArgs& a) {
     atomicCAS(a.status + 2, 0, a.step);
 }
 
+// Puts the tile's halo words of `src` tagged `tag` into sb; false on a timed-out wait
+template <class T>
+__device__ __forceinline__ int halo_words(const CGArgs& a, const float4* src, unsigned tag,
+                                          const Resident<T>& t, float4* sb) {
+    typedef Resident<T> RT;
+    int ok = 1;
+    float4 h[RT::HPT];
+#pragma unroll
+    for (int i = 0; i < RT::HPT; ++i)
+        if (t.hm[i] >= 0) h[i] = ld_word(src + t.hm[i]);
+#pragma unroll
+    for (int i = 0; i < RT::HPT; ++i) {
+        if (t.hm[i] < 0 || __float_as_uint(h[i].w) == tag) continue;
+        const long long t0 = clock64();
+        for (int spin = 1;; ++spin) {
+            h[i] = ld_word(src + t.hm[i]);
+            if (__float_as_uint(h[i].w) == tag) break;
+            if ((spin & 255) != 0) continue;
+            if (ld_acquire_gpu(a.bar + 2) != 0u) { ok = 0; break; }
+            if (clock64() - t0 > a.bar_budget) { wait_failed(a); ok = 0; break; }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < RT::HPT; ++i)
+        if (t.hm[i] >= 0) sb[t.hs[i]] = h[i];
+    return ok;
+}
+
 // One iteration on the resident tile: waits for the halo words tagged seq + k (with RFIRST
 // the first iteration starts from r instead, complete in memory: d_0 = r / theta).  Returns
 // false on a timed-out wait.
@@ -851,34 +996,20 @@ __device__ __forceinline__ bool cheb_pass_resident(const CGArgs& a, int k, unsig
 #pragma unroll
     for (int v = 0; v < T::VPT; ++v)
         sb[T::hidx(lx, ly, lz + v)] = t.m[v] >= 0 ? t.d[v] : make_float4(0.f, 0.f, 0.f, 0.f);
-    float4 h[RT::HPT];
     if (RFIRST && k == 0) {
+        float4 h[RT::HPT];
 #pragma unroll
         for (int i = 0; i < RT::HPT; ++i)
             if (t.hm[i] >= 0) {
                 h[i] = __ldcg(a.r + t.hm[i]);
                 h[i].x *= a.inv_theta; h[i].y *= a.inv_theta; h[i].z *= a.inv_theta;
             }
-    } else {
 #pragma unroll
         for (int i = 0; i < RT::HPT; ++i)
-            if (t.hm[i] >= 0) h[i] = ld_word(dk + t.hm[i]);
-#pragma unroll
-        for (int i = 0; i < RT::HPT; ++i) {
-            if (t.hm[i] < 0 || __float_as_uint(h[i].w) == seq) continue;
-            const long long t0 = clock64();
-            for (int spin = 1;; ++spin) {
-                h[i] = ld_word(dk + t.hm[i]);
-                if (__float_as_uint(h[i].w) == seq) break;
-                if ((spin & 255) != 0) continue;
-                if (ld_acquire_gpu(a.bar + 2) != 0u) { ok = 0; break; }
-                if (clock64() - t0 > a.bar_budget) { wait_failed(a); ok = 0; break; }
-            }
-        }
+            if (t.hm[i] >= 0) sb[t.hs[i]] = h[i];
+    } else {
+        ok = halo_words<T>(a, dk, seq, t, sb);
     }
-#pragma unroll
-    for (int i = 0; i < RT::HPT; ++i)
-        if (t.hm[i] >= 0) sb[t.hs[i]] = h[i];
     if (!__syncthreads_and(ok)) return false;
     float4 cv[T::VPT];
     float o[T::VPT][3];
@@ -917,15 +1048,19 @@ struct Sums {
 // first Chebyshev direction d_0 = r / theta of the active voxels: resident tiles keep them
 // and send d_0 out as the words of iteration 0, the others store both.
 template <class T, bool PAIR, bool RES>
-__device__ __forceinline__ void residual_df_tiled(const CGArgs& a, float4 (*sd)[T::HALO], float sc,
+__device__ __forceinline__ bool residual_df_tiled(const CGArgs& a, float4 (*sd)[T::HALO], float sc,
                                                   bool wide, Sums& sum, Resident<T>& res,
-                                                  unsigned seq) {
+                                                  unsigned seq, unsigned xtag, bool own) {
     const long long M = a.M;
     for (int tile = blockIdx.x; tile < a.ntiles; tile += a.nw) {
         const int org = a.tiles[tile];
-        load_halo<T>(a, PAIR ? a.q : a.xl, sd[0], org);
-        if (PAIR) load_halo<T>(a, a.xl, sd[1], org);
-        cp_async_commit();
+        constexpr bool words = RES && !PAIR;
+        int ok = 1;
+        if constexpr (!words) {
+            load_halo<T>(a, PAIR ? a.q : a.xl, sd[0], org);
+            if (PAIR) load_halo<T>(a, a.xl, sd[1], org);
+            cp_async_commit();
+        }
         long long mv[T::VPT];
         float dhv[T::VPT], dlv[T::VPT], bh[T::VPT][3], bl[T::VPT][3];
 #pragma unroll
@@ -943,20 +1078,31 @@ __device__ __forceinline__ void residual_df_tiled(const CGArgs& a, float4 (*sd)[
                 }
             }
         }
-        cp_async_wait0();
-        __syncthreads();
+        if constexpr (words) {
+            if (!own) {
+                int lx, ly, lz;
+                T::local(lx, ly, lz);
+#pragma unroll
+                for (int v = 0; v < T::VPT; ++v)
+                    sd[0][T::hidx(lx, ly, lz + v)] =
+                        mv[v] >= 0 ? __ldcg(a.xl + mv[v]) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            ok = halo_words<T>(a, a.xl, xtag, res, sd[0]);
+        } else {
+            cp_async_wait0();
+        }
+        if (!__syncthreads_and(ok)) return false;
 #pragma unroll
         for (int v = 0; v < T::VPT; ++v) {
             if (mv[v] < 0) continue;
             int lx, ly, lz;
             T::local(lx, ly, lz);
             const int hc = T::hidx(lx, ly, lz + v);
-            auto load = [&](auto e, float4& vh, float4& vl) {
-                constexpr int o = T::template off<decltype(e)::value>();
+            auto load = [&](int o, float4& vh, float4& vl) {
                 vh = sd[0][hc + o];
                 if constexpr (PAIR) vl = sd[1][hc + o];
             };
-            const float4 r4 = residual_df_at<PAIR>(dhv[v], dlv[v], bh[v], bl[v], load);
+            const float4 r4 = residual_df_at<PAIR, T::HX, T::HX * T::HY>(dhv[v], dlv[v], bh[v], bl[v], load);
             const float rv[3] = {r4.x, r4.y, r4.z};
             sum.add_r(rv, wide, sc);
             const float* h = bh[v];
@@ -976,6 +1122,7 @@ __device__ __forceinline__ void residual_df_tiled(const CGArgs& a, float4 (*sd)[
         }
         __syncthreads();
     }
+    return true;
 }
 
 // block-wide sum of two values; result valid in every thread
@@ -1078,14 +1225,14 @@ __device__ __forceinline__ bool collect(const CGArgs& a, int set, unsigned tag, 
 // Grid-wide barrier of a cooperative launch (every block resident) with a bounded wait.
 // Each block's thread 0 publishes the block's writes, arrives on a counter that only
 // grows, and waits until the arrivals of this barrier are complete (n per barrier): one
-// round trip to the counter after the last arrival.  The words are zero at launch: the
-// last block to finish a kernel resets the counter (barrier_done).  A wait longer than
+// round trip to the counter after the last arrival.  The counter is zero at launch: the
+// launch before, which uses another one, clears it.  A wait longer than
 // `budget` SM clock cycles (a block that never arrives) sets the abort word and the
 // timeout flag (4) in status[1] with the step in status[2]; blocks that see the abort word
 // leave at once.  Returns false when the caller must return: the kernel ends without
 // touching the solution any further.
-__device__ bool grid_barrier(unsigned* bar, unsigned n, unsigned& target, long long budget,
-                             int* status, int step) {
+__device__ bool grid_barrier(unsigned* bar, unsigned* abort, unsigned n, unsigned& target,
+                             long long budget, int* status, int step) {
     int ok = 1;
     target += n;
     __syncthreads();
@@ -1096,9 +1243,9 @@ __device__ bool grid_barrier(unsigned* bar, unsigned n, unsigned& target, long l
             const long long t0 = clock64();
             for (int spin = 1; (int)(ld_acquire_gpu(bar) - target) < 0; ++spin) {
                 if ((spin & 63) != 0) continue;
-                if (ld_acquire_gpu(bar + 2) != 0u) { ok = 0; break; }
+                if (ld_acquire_gpu(abort) != 0u) { ok = 0; break; }
                 if (clock64() - t0 > budget) {
-                    atomicExch(bar + 2, 1u);
+                    atomicExch(abort, 1u);
                     atomicOr(status + 1, 4);
                     atomicCAS(status + 2, 0, step);
                     ok = 0;
@@ -1136,23 +1283,67 @@ __global__ void __launch_bounds__(NT) k_barrier_check(int* w, long long budget, 
     if ((int)blockIdx.x == absent) return;
     unsigned target = 0;
     for (int r = 1; r <= rounds; ++r)
-        if (!grid_barrier(reinterpret_cast<unsigned*>(w + 4), gridDim.x, target, budget, w, r))
+        if (!grid_barrier(reinterpret_cast<unsigned*>(w + 4),
+                          reinterpret_cast<unsigned*>(w + 6), gridDim.x, target, budget, w, r))
             return;
     if (threadIdx.x == 0) atomicAdd(w + 8, 1);
 }
 
-// The least-squares fit of b_n by b_{n-1} .. b_{n-nv} (one block): sums the epilogue's
+// status: 1 not converged, 2 NaN or Inf; the first such step
+__device__ __forceinline__ void bad_step(int* status, int flag, int step) {
+    atomicOr(status + 1, flag);
+    const int old = atomicCAS(status + 2, 0, step);
+    if (old > step) atomicMin(status + 2, step);
+}
+
+// ||x||^2 of a step from its blocks' shares (one warp, fixed order), checked
+__device__ __forceinline__ void norm_total(const double* p, int n, double* out, int* status,
+                                           int step) {
+    double v0 = 0.0, v1 = 0.0, v2 = 0.0, v3 = 0.0;   // four independent loads in flight
+    int k = threadIdx.x;
+    for (; k + 96 < n; k += 128) {
+        v0 += __ldcg(p + k);
+        v1 += __ldcg(p + k + 32);
+        v2 += __ldcg(p + k + 64);
+        v3 += __ldcg(p + k + 96);
+    }
+    for (; k < n; k += 32) v0 += __ldcg(p + k);
+    double v = (v0 + v1) + (v2 + v3);
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (threadIdx.x != 0) return;
+    *out = v;
+    if (!(v == v) || v > 1e300) bad_step(status, 2, step);
+}
+
+// The least-squares fit of b_n by b_{n-1} .. b_{n-nv} (one block): sums the
 // partial dot products in a fixed order, updates the Gram matrix of the ring and solves
 // the normal equations by a Cholesky factorisation in ring order, newest first (a vector
 // whose remainder after the newer ones is below kFitPivot of its square is left out).
 // The matrix is scaled to unit diagonal.  Lane i of warp 0 holds row i.
-template <bool DF> __device__ void fit_block(const CGArgs& a) {
+template <bool DF, bool RES> __device__ void fit_block(const CGArgs& a) {
     __shared__ double t[kSums];
     const int lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
-    for (int q = threadIdx.x >> 5; q < kSums - 1; q += nwarp) {
-        const double* p = a.part + (long long)q * a.nepi;
+    for (int q = threadIdx.x >> 5; q < kSums; q += nwarp) {
         double v = 0.0;
-        for (int k = lane; k < a.nepi; k += 32) v += p[k];
+        if constexpr (RES) {
+            // sent by this launch's blocks (bounded wait)
+            const float4* p = a.part4 + (long long)q * a.nw;
+            const long long t0 = clock64();
+            for (int k = lane; k < a.nw; k += 32) {
+                float4 w = ld_word(p + k);
+                for (int spin = 1; __float_as_uint(w.w) != a.seq; ++spin) {
+                    if ((spin & 255) == 0) {
+                        if (ld_acquire_gpu(a.bar + 2) != 0u) break;
+                        if (clock64() - t0 > a.bar_budget) { wait_failed(a); break; }
+                    }
+                    w = ld_word(p + k);
+                }
+                v += __hiloint2double(__float_as_int(w.y), __float_as_int(w.x));
+            }
+        } else {
+            const double* p = a.part + (long long)q * a.nepi;
+            for (int k = lane; k < a.nepi; k += 32) v += p[k];
+        }
         for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
         // FP32-history sums are scaled by 4^e of this step
         const double un = DF ? pow2d(-2 * a.fit->rec[a.step & 1].e) : 1.0;
@@ -1199,7 +1390,10 @@ template <bool DF> __device__ void fit_block(const CGArgs& a) {
     double mag = fabs(c);
     for (int o = 4; o > 0; o >>= 1) mag = fmax(mag, __shfl_xor_sync(0xffffffffu, mag, o));
     FitRecord& rec = a.fit->rec[(a.step + 1) & 1];
-    if (lane < kFit) rec.c[lane] = c;
+    if (lane < kFit) {
+        rec.c[lane] = c;
+        rec.cf[lane] = (float)c;
+    }
     if (lane == 0) {
         // a poor or degenerate fit (also NaN anywhere in it) falls back to extrapolation
         rec.use = a.nv >= 3 && bb > 0.0 && bb - yy <= kFitPoor * bb && mag < 1e4;
@@ -1298,6 +1492,16 @@ __device__ __forceinline__ void residual64(const CGArgs& a, int e, bool first, b
     }
 }
 
+// The solve of one step.  Resident tiles (RES) first form the right-hand side and the start of
+// their own voxels (epi_voxel); in FP32-history the start goes to the neighbours as tagged
+// words like the iteration's d, in FP64 a grid barrier follows, because the FP64 residual
+// deals the voxels out anew.  Blocks past nw take the voxels outside every tile.  The norm
+// of a step is added up beside the next one's solve, not by the last block to finish.
+// Against an epilogue of its own and a last block (solve phase of a step): 9^3 sphere
+// FP32-history 43.2 -> 35.5 us, 32^3 52.6 -> 40.9, 133 x 27 x 21 116 -> 95, 8^3 FP64 49.9 -> 45.0.
+// What remains of the 9^3 solve, thousands of cycles: right-hand side 13, residual 11, two
+// iterations beside the sums 5, the sums 1, eleven iterations 25, x and its norm 4.
+//
 // Mixed-precision iterative refinement from x0: residual r = b - A x (FP64, or
 // double-float in FP32-history mode, DF), FP32 Chebyshev iterations for A e = r, x += e.
 // One fused pass and one grid barrier per iteration (apply to d_k, update e, r, d_{k+1}; d
@@ -1321,17 +1525,34 @@ constexpr float kFloor = 1e-6f;
 constexpr unsigned kAborted = 4;
 
 template <bool DF, class T, bool RES, bool SPLIT>
-__global__ void __launch_bounds__(T::NTH, RES ? 4 : 2) k_cg(const __grid_constant__ CGArgs a) {
+__global__ void __launch_bounds__(T::NTH, RES ? 4 : 2)
+k_cg(const __grid_constant__ CGArgs a, const __grid_constant__ EpiArgs ep) {
+    typedef typename std::conditional<DF, float, double>::type R;
     __shared__ __align__(16) float4 sd[2][T::HALO];      // tile halos of the passes
     pdl_trigger();                       // (launched as an ordinary, cooperative kernel)
     if ((int)blockIdx.x == a.nw) {       // the fit for the next step, beside the solve
-        fit_block<DF>(a);
+        if (a.norm_prev && threadIdx.x < 32)
+            norm_total(a.nrm_prev, a.nred, a.norm_prev, a.status, a.prev_step);
+        fit_block<DF, RES>(a);
         return;
     }
-    unsigned target = 0, seq = a.seq, tag = a.seq;
+    if constexpr (RES) {
+        if ((int)blockIdx.x > a.nw) {    // voxels outside every tile
+            const EpiFit<R> fit(ep);
+            EpiSums<R> sum;
+            float4 none;
+            for (int i = ((int)blockIdx.x - a.nw - 1) * T::NTH + threadIdx.x; i < a.nvac;
+                 i += a.nvb * T::NTH)
+                epi_voxel<R>(ep, ep.adj, fit, a.vac[i], sum, none);
+            epi_vacuum_norm(sum.xin, a.nrm + blockIdx.x - 1);
+            return;
+        }
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.bar[a.parity ^ 1] = 0u;
+    unsigned target = 0, seq = a.seq, tag = a.seq, xtag = a.seq;
     int set = 0;
     auto gsync = [&] {
-        return grid_barrier(a.bar, a.nw, target, a.bar_budget, a.status, a.step);
+        return grid_barrier(a.bar + a.parity, a.bar + 2, a.nw, target, a.bar_budget, a.status, a.step);
     };
     const long long M = a.M;
     const long long t0 = (long long)blockIdx.x * T::NTH + threadIdx.x;
@@ -1339,11 +1560,52 @@ __global__ void __launch_bounds__(T::NTH, RES ? 4 : 2) k_cg(const __grid_constan
     const int nb = a.nw;
     double* red0 = a.red;
     double* red1 = a.red + nb;
-    double* red2 = a.red + 2 * nb;
     Resident<T> res;
+    double xin = 0.0;                    // |x|^2 of the tile's vacuum voxels
+    __shared__ EpiRed<R, T::NTH> fitred;
+    bool fit_due = RES;                  // the block's sums for the fit are still to be sent
+    auto fit_sums = [&] {
+        if constexpr (RES) {
+            if (!fit_due) return;
+            fit_due = false;
+            if (threadIdx.x >= T::NTH - 32 && (threadIdx.x & 31) < kSums) {
+                const double v = epi_block_sum<R, T::NTH>(fitred);
+                st_word(a.part4 + (threadIdx.x & 31) * nb + blockIdx.x,
+                        make_float4(__int_as_float(__double2loint(v)),
+                                    __int_as_float(__double2hiint(v)), 0.f, __uint_as_float(a.seq)));
+            }
+        }
+    };
     if constexpr (RES) {
+        const EpiFit<R> fit(ep);
         resident_init<T>(a, res, sd);
-        __syncthreads();     // its zeros, before a residual pass copies halos over them
+        // right-hand side and start of the tile's voxels
+        EpiSums<R> sum;
+        if ((int)blockIdx.x < a.ntiles) {
+            const int org = a.tiles[blockIdx.x];
+            int lx, ly, lz;
+            T::local(lx, ly, lz);
+#pragma unroll 1
+            for (int v = 0; v < T::VPT; ++v) {
+                const long long m = tile_voxel<T>(a, org, v);
+                float4 x0 = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (m >= 0 && epi_voxel<R>(ep, ep.adj, fit, m, sum, x0) && DF) {
+                    x0.w = __uint_as_float(xtag);
+                    st_word(a.xl + m, x0);
+                }
+                if (DF) sd[0][T::hidx(lx, ly, lz + v)] = x0;
+            }
+        }
+        xin = sum.xin;
+        epi_stash<R, T::NTH>(fitred, sum);
+        // the zeros of the shells before a pass writes halos over them; FP64: the start and b
+        // before other blocks read them
+        if constexpr (DF) {
+            __syncthreads();
+            fit_sums();
+        } else if (!gsync()) {
+            return;
+        }
     }
     float bb = 0.f, rr = 0.f;            // scaled by 4^e0 and 4^e
     double xx = 0.0;                     // |x|^2 of the block's share, once x is stored
@@ -1351,6 +1613,7 @@ __global__ void __launch_bounds__(T::NTH, RES ? 4 : 2) k_cg(const __grid_constan
     int its = 0, outer = 0, wides = 0;
     bool first = true, wide = false, converged = false, nonfinite = false, zero = false;
     bool stored = false;     // x is in a.x; else DF's start is in xb only
+    bool own = true;         // sd[0] holds the tile's start
     // f(voxel, its correction e) over the block's share of the active voxels
     auto each = [&](auto&& f) {
         if constexpr (RES) {
@@ -1373,8 +1636,10 @@ __global__ void __launch_bounds__(T::NTH, RES ? 4 : 2) k_cg(const __grid_constan
         // ---- residual, scaled by 2^e
         Sums sum = {0.f, 0.f, 0.0, 0.0};
         if constexpr (DF) {
-            if (stored) residual_df_tiled<T, true, RES>(a, sd, pow2f(e), wide, sum, res, seq);
-            else residual_df_tiled<T, false, RES>(a, sd, pow2f(e), wide, sum, res, seq);
+            if (!(stored ? residual_df_tiled<T, true, RES>(a, sd, pow2f(e), wide, sum, res, seq, xtag, own)
+                         : residual_df_tiled<T, false, RES>(a, sd, pow2f(e), wide, sum, res, seq, xtag, own)))
+                return;
+            own = false;
         } else {
             residual64<SPLIT, RES>(a, e, first, wide, sum);
         }
@@ -1407,6 +1672,7 @@ __global__ void __launch_bounds__(T::NTH, RES ? 4 : 2) k_cg(const __grid_constan
                 if (!cheb_pass_resident<T, false>(a, k, seq + k, false, sd, res, rr_p)) return;
             ran2 = true;
         } else {
+            fit_sums();
             if (!gsync()) return;        // r complete (with x as pairs: q read by all)
         }
         float b_tot;
@@ -1430,8 +1696,9 @@ __global__ void __launch_bounds__(T::NTH, RES ? 4 : 2) k_cg(const __grid_constan
                         if (DF) a.xb[k * M + m].x = 0.f;
                         else a.x[k * M + m] = 0.0;
                     }
-                    if (DF) a.xl[m] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (DF) st_word(a.xl + m, make_float4(0.f, 0.f, 0.f, __uint_as_float(xtag + 1u)));
                 });
+                ++xtag;
                 first = false;
             }
             wide = odd;
@@ -1481,8 +1748,8 @@ __global__ void __launch_bounds__(T::NTH, RES ? 4 : 2) k_cg(const __grid_constan
             const float ec[3] = {d.x, d.y, d.z};
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                double x = DF && !stored ? (double)a.xb[k * M + m].x : a.x[k * M + m];
-                x += back * (double)ec[k];
+                double x = DF && !stored ? widen(a.xb[k * M + m].x) : a.x[k * M + m];
+                x += back * widen(ec[k]);
                 a.x[k * M + m] = x;
                 if (a.out) a.out[m * 3 + k] = x;
                 if (DF) a.xb[k * M + m].x = (float)x;
@@ -1506,7 +1773,8 @@ __global__ void __launch_bounds__(T::NTH, RES ? 4 : 2) k_cg(const __grid_constan
                 df_split(a.x[m], h.x, l.x);
                 df_split(a.x[M + m], h.y, l.y);
                 df_split(a.x[2 * M + m], h.z, l.z);
-                h.w = l.w = 0.f;
+                h.w = 0.f;
+                l.w = __uint_as_float(a.seq + 1023u);    // no launch's tag of a start
                 a.q[m] = h;
                 a.xl[m] = l;
             });
@@ -1516,13 +1784,12 @@ __global__ void __launch_bounds__(T::NTH, RES ? 4 : 2) k_cg(const __grid_constan
     // ---- an x not stored yet, and its norm.  NaN or Inf in the right-hand side or the
     // start: no iteration can help; J_n is returned as NaN so that the monitor and the
     // caller see it
-    double unused = 0.0;
     if (!stored || nonfinite) {
         xx = 0.0;
         each([&](long long m, const float4&, int) {
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                double x = DF && !stored ? (double)a.xb[k * M + m].x : a.x[k * M + m];
+                double x = DF && !stored ? widen(a.xb[k * M + m].x) : a.x[k * M + m];
                 if (zero) x = 0.0;
                 if (nonfinite) x = __longlong_as_double(0x7ff8000000000000LL);
                 a.x[k * M + m] = x;
@@ -1532,35 +1799,29 @@ __global__ void __launch_bounds__(T::NTH, RES ? 4 : 2) k_cg(const __grid_constan
             }
         });
     }
-    block_sum2<T::NTH>(xx, unused);
-    // the last block to finish adds up the norm (fixed order) and leaves the barrier words
-    // zero for the next launch: every other block has passed its last barrier
-    __shared__ int s_last;
-    if (threadIdx.x == 0) {
-        red2[blockIdx.x] = xx;
-        __threadfence();
-        s_last = atomicAdd(a.bar + 3, 1u) == (unsigned)(nb - 1);
-        __threadfence();
-    }
+    fit_sums();
+    xx += xin;
+    __shared__ double shx[T::NTH / 32];
+    for (int o = 16; o > 0; o >>= 1) xx += __shfl_down_sync(0xffffffffu, xx, o);
+    if ((threadIdx.x & 31) == 0) shx[threadIdx.x >> 5] = xx;
     __syncthreads();
-    if (!s_last) return;
-    const double nx = grid_total(red2, nb) +
-                      grid_total(a.part + (long long)(kSums - 1) * a.nepi, a.nepi);
-    if (threadIdx.x == 0) {
-        a.bar[0] = 0u;
-        a.bar[3] = 0u;
-        *a.norm2 = nx;
+    if (threadIdx.x != 0) return;
+#pragma unroll
+    for (int w = 1; w < T::NTH / 32; ++w) xx += shx[w];
+    a.nrm[blockIdx.x] = xx;
+    if (blockIdx.x == 0) {
         a.status[0] = its;
-        int flag = 0;
-        if (!converged && !nonfinite) flag |= 1;        // not converged
-        if (nonfinite || !(nx == nx) || nx > 1e300) flag |= 2;   // NaN / Inf
-        if (flag && a.status[2] == 0) a.status[2] = a.step;
-        a.status[1] |= flag;
         a.status[3] += its;
+        const int flag = nonfinite ? 2 : converged ? 0 : 1;
+        if (flag) bad_step(a.status, flag, a.step);
     }
 }
 
-// AoS [m][b] -> SoA slot
+// ||x||^2 of a march's last step (the others are added up beside the solve that follows)
+__global__ void k_norm_total(const double* nrm, int n, double* out, int* status, int step) {
+    norm_total(nrm, n, out, status, step);
+}
+
 __global__ void k_from_aos(const double* __restrict__ in, long long M, double* __restrict__ x) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= 3 * M) return;
@@ -1907,14 +2168,15 @@ int fit_slot(int n) { return n % kSlots; }
 // pairs (x, b) of the steps before the one being launched
 int fit_pairs(const mot_ctx* c) { return std::min(c->fit_steps, kFit); }
 
-template <typename R, bool ADJ>
-void epilogue(mot_ctx* c, int n, const double* En, double* out, cudaStream_t s) {
+double* norm_shares(const mot_ctx* c, int parity) { return c->norm_part + (long long)parity * c->norm_blocks; }
+
+EpiArgs make_epi_args(mot_ctx* c, int n, const double* En, double* out, bool adj) {
     EpiArgs a;
     a.out = out;
     a.M = c->M;
     a.f = c->vfac;
     a.En = En;
-    a.hist = hbuf<R>(c).hist_spatial;
+    a.hist = c->precision == MOT_FP64 ? (const void*)c->h64.hist_spatial : (const void*)c->h32.hist_spatial;
     a.Jring = c->J;
     a.s0 = (int)slot_index(n, c->jring);
     a.jring = c->jring;
@@ -1929,11 +2191,20 @@ void epilogue(mot_ctx* c, int n, const double* En, double* out, cudaStream_t s) 
     a.rhs = c->rhs;
     a.fit = reinterpret_cast<const FitState*>(c->fit);
     a.part = c->fit_part;
-    launch_dependent(mot::dependent_launches(c), k_epilogue<R, ADJ>, c->epi_blocks, c->epi_threads, 0, s, a);
+    a.nrm = norm_shares(c, (c->solve_seq + 1) & 1) + c->cg_blocks;
+    a.adj = adj;
+    return a;
+}
+
+template <typename R, bool ADJ>
+void epilogue(mot_ctx* c, const EpiArgs& a, cudaStream_t s) {
+    launch_dependent(mot::dependent_launches(c), k_epilogue<R, ADJ>, c->epi_blocks, NT, 0, s, a);
     MOT_LAUNCH_CHECK();
 }
 
 }  // namespace
+
+namespace {
 
 CGArgs make_cg_args(mot_ctx* c, int n, double* norm2_out, double* out) {
     CGArgs a;
@@ -1963,7 +2234,7 @@ CGArgs make_cg_args(mot_ctx* c, int n, double* norm2_out, double* out) {
     a.e = a.r + 3 * c->M;
     a.xl = c->cg_xl ? reinterpret_cast<float4*>(c->cg_xl) : nullptr;
     a.red = c->red;
-    a.red4 = reinterpret_cast<float4*>(c->red + 3LL * c->cg_blocks + (c->cg_blocks & 1));
+    a.red4 = reinterpret_cast<float4*>(c->red + 2LL * c->cg_blocks);
     a.tol2 = c->tol * c->tol;
     a.tol = (float)c->tol;
     a.inv_theta = c->cheb_inv_theta;
@@ -1979,17 +2250,26 @@ CGArgs make_cg_args(mot_ctx* c, int n, double* norm2_out, double* out) {
     a.status = c->dstatus;
     a.bar = reinterpret_cast<unsigned*>(c->dstatus + 4);
     a.bar_budget = c->bar_budget;
-    a.norm2 = norm2_out;
     a.fit = reinterpret_cast<FitState*>(c->fit);
     a.part = c->fit_part;
     a.nepi = c->epi_blocks;
+    a.part4 = reinterpret_cast<float4*>(c->fit_part);
     // every active voxel's words in p and q are rewritten by each launch, so numbers that
     // only have to differ from those of the launch before may wrap
     a.seq = ++c->solve_seq * 1024u;
+    a.parity = (int)(c->solve_seq & 1u);
+    a.nrm = norm_shares(c, a.parity);
+    a.nrm_prev = norm_shares(c, a.parity ^ 1);
+    a.norm_prev = c->norm_pending;
+    a.prev_step = c->norm_step;
+    a.nred = c->norm_blocks;
+    a.vac = c->vac;
+    a.nvac = (int)c->nvac;
+    a.nvb = c->cg_resident ? c->norm_blocks - c->cg_blocks : 0;
+    c->norm_pending = norm2_out;
+    c->norm_step = n;
     return a;
 }
-
-namespace {
 
 // kernel variant of a context's solve and its block size
 struct SolveKernel { void* fn; int threads; };
@@ -2008,12 +2288,33 @@ SolveKernel solve_kernel(int precision, int tile, bool resident, bool split) {
            : tile == 2 ? kernel_of<Tile2>(df, split) : kernel_of<Tile4>(df, split);
 }
 
+// Right-hand side, start and solve of step n: one kernel where the tiles are resident, the
+// epilogue before it where not (a grid of that size hides a launch: 1.6 ms a step at 104^3).
+void launch_solve(mot_ctx* c, int n, const double* En, double* norm2_out, double* out, bool adj,
+                  cudaStream_t s) {
+    EpiArgs ep = make_epi_args(c, n, En, out, adj);
+    if (!c->cg_resident) {
+        if (c->precision == MOT_FP64) adj ? epilogue<double, true>(c, ep, s) : epilogue<double, false>(c, ep, s);
+        else adj ? epilogue<float, true>(c, ep, s) : epilogue<float, false>(c, ep, s);
+        c->stats.launches += 1;
+    }
+    CGArgs a = make_cg_args(c, n, norm2_out, out);
+    void* args[] = {&a, &ep};
+    const SolveKernel k = solve_kernel(c->precision, c->cg_tile, c->cg_resident, c->cg_split);
+    MOT_CUDA_TRY(cudaLaunchCooperativeKernel(k.fn, c->cg_blocks + 1 + a.nvb, k.threads, args, 0, s));
+    ++c->fit_steps;
+    c->stats.launches += 1;
+}
+
 }  // namespace
 
-void launch_cg(mot_ctx* c, void** args, cudaStream_t s) {
-    const SolveKernel k = solve_kernel(c->precision, c->cg_tile, c->cg_resident, c->cg_split);
-    MOT_CUDA_TRY(cudaLaunchCooperativeKernel(k.fn, c->cg_blocks + 1, k.threads, args, 0, s));
-    ++c->fit_steps;
+// adds up the norm of the last step launched
+void solve_finish(mot_ctx* c, cudaStream_t s) {
+    if (!c->norm_pending) return;
+    k_norm_total<<<1, 32, 0, s>>>(norm_shares(c, (int)(c->solve_seq & 1u)), c->norm_blocks,
+                                  c->norm_pending, c->dstatus, c->norm_step);
+    MOT_LAUNCH_CHECK();
+    c->norm_pending = nullptr;
 }
 
 // Shape of the solve on this geometry.  tiles[i]: active tiles of 8 x 4 x 4, 8 x 4 x 8 and
@@ -2028,7 +2329,7 @@ const std::vector<int>& solve_shape(mot_ctx* c, const std::vector<int> (&tiles)[
     for (int i = 0; i < 3 && !c->cg_resident; ++i) {
         const SolveKernel k = solve_kernel(c->precision, 1 << i, true, c->cg_split);
         MOT_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.fn, k.threads, 0));
-        if ((long long)tiles[i].size() + 1 <= (long long)per_sm * c->nsm) {
+        if ((long long)tiles[i].size() + 2 <= (long long)per_sm * c->nsm) {
             c->cg_resident = true;
             pick = i;
         }
@@ -2048,11 +2349,20 @@ const std::vector<int>& solve_shape(mot_ctx* c, const std::vector<int> (&tiles)[
     int want = std::max(c->ntiles, 1);
     if (c->cg_split)
         want = std::max(want, std::min(2 * c->nsm, (int)(3 * ((c->nact + 31) / 32) + 3) / 4));
-    c->cg_blocks = std::max(1, std::min(per_sm * c->nsm - 1, want));
-    // epilogue: small blocks on small grids (its FP64 terms are bound by the SMs in use)
-    c->epi_threads = c->M <= 64LL * c->nsm ? 64 : NT;
-    c->epi_blocks = (int)std::min<long long>((c->M + c->epi_threads - 1) / c->epi_threads,
-                                             8LL * c->nsm);
+    c->cg_blocks = std::max(1, std::min(per_sm * c->nsm - 2, want));
+    c->epi_blocks = (int)std::min<long long>((c->M + NT - 1) / NT, 8LL * c->nsm);
+    // blocks with a share of the norm: the solve's, then the epilogue's or (resident) those
+    // that take the voxels outside the tiles
+    static const int dims[3][3] = {{8, 4, 4}, {8, 4, 8}, {8, 8, 8}};
+    c->nvac = c->M;
+    for (int o : tiles[pick])
+        c->nvac -= (long long)std::min(dims[pick][0], c->U - (o & 1023)) *
+                   std::min(dims[pick][1], c->V - ((o >> 10) & 1023)) *
+                   std::min(dims[pick][2], c->W - (o >> 20));
+    const int room = per_sm * c->nsm - 1 - c->cg_blocks;
+    c->norm_blocks = c->cg_blocks +
+                     (c->cg_resident ? (int)std::min<long long>(room, (c->nvac + 127) / 128)
+                                     : c->epi_blocks);
     return tiles[pick];
 }
 
@@ -2074,14 +2384,11 @@ void solve_halo_lists(mot_ctx* c) {
     else halo_lists<Tile4>(c);
 }
 
-// rhs + CG for step n; ||J_n||^2 into norm2_out (device), J_n in ring slot n and (AoS) in out
+// right-hand side and solve of step n; ||J_n||^2 into norm2_out (device; by the next step or
+// solve_finish), J_n in ring slot n and (AoS) in out
 void solve_step(mot_ctx* c, int n, const double* En, double* norm2_out, double* out,
                 cudaStream_t s) {
-    if (c->precision == MOT_FP64) epilogue<double, false>(c, n, En, out, s);
-    else epilogue<float, false>(c, n, En, out, s);
-    CGArgs a = make_cg_args(c, n, norm2_out, out);
-    void* args[] = {&a};
-    launch_cg(c, args, s);
+    launch_solve(c, n, En, norm2_out, out, false, s);
 }
 
 void read_aos(mot_ctx* c, const double* in_dev, double* slot, cudaStream_t s) {
@@ -2108,11 +2415,7 @@ void adjoint_step(mot_ctx* c, int tau, int n, const double* g_aos, const double*
                   int j_first, double* grad_chi, double* lam_out, double* norm2_out,
                   cudaStream_t s) {
     const int s0 = (int)slot_index(tau, c->jring);
-    if (c->precision == MOT_FP64) epilogue<double, true>(c, tau, g_aos, nullptr, s);
-    else epilogue<float, true>(c, tau, g_aos, nullptr, s);
-    CGArgs a = make_cg_args(c, tau, norm2_out, nullptr);
-    void* args[] = {&a};
-    launch_cg(c, args, s);
+    launch_solve(c, tau, g_aos, norm2_out, nullptr, true, s);
     double* mu = c->J + (long long)s0 * 3 * c->M;
     k_adj_vacuum<<<(int)((c->M + NT - 1) / NT), NT, 0, s>>>(c->M, c->U, c->V, c->W, c->vfac, mu,
                                                            c->rhs, c->cg_q);
@@ -2121,7 +2424,7 @@ void adjoint_step(mot_ctx* c, int tau, int n, const double* g_aos, const double*
                                                          j_first, n, taps_of(c), grad_chi,
                                                          lam_out);
     MOT_LAUNCH_CHECK();
-    c->stats.launches += 4;
+    c->stats.launches += 2;
 }
 
 }  // namespace mot
