@@ -461,6 +461,192 @@ k_mid4s(const typename CT<R>::c* __restrict__ in, typename CT<R>::c* __restrict_
     }
 }
 
+// ------------------------------------------------------------------ x and y passes in one kernel
+// A CTA takes one plane (component, w): the row pairs along u, then the Hu lines along v,
+// both in shared memory, the Stockham stages of fft_core.cuh with the number of lines at run
+// time.  On small grids the two passes of an axis each are all latency (launch, table, load,
+// store, 6 to 7 us a pass whatever its length); larger planes have enough lines to fill the
+// GPU with a launch of their own (see plane_pass).
+template <typename C, int R, int DIR>
+__device__ __forceinline__ void stage_lines(const C* __restrict__ x, C* __restrict__ y, int P,
+                                            int Ns, int nl, int ld, const C* tw) {
+    const int nb = P / R, items = nb * nl, tstep = P / (Ns * R);
+    const float inv_nl = 1.0f / (float)nl, inv_ns = 1.0f / (float)Ns;
+    for (int it = threadIdx.x; it < items; it += blockDim.x) {
+        // exact for it, j < 2^20, as in stage()
+        const int j = __float2int_rz(((float)it + 0.5f) * inv_nl), t = it - j * nl;
+        const int jq = __float2int_rz(((float)j + 0.5f) * inv_ns), k = j - jq * Ns;
+        C v[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = x[(j + r * nb) * ld + t];
+        if (Ns > 1) {
+            const int kt = k * tstep;
+#pragma unroll
+            for (int r = 1; r < R; ++r) v[r] = twmul_tab(tw, r * kt, P, DIR, v[r]);
+        }
+        dft_small<C, R>(v, tw, P, DIR);
+        const int base = jq * Ns * R + k;
+#pragma unroll
+        for (int r = 0; r < R; ++r) y[(base + r * Ns) * ld + t] = v[r];
+    }
+}
+// transforms of nl lines x[j * ld + t]; returns the buffer that holds the result
+template <typename C, int DIR>
+__device__ __forceinline__ C* fft_lines(C* x, C* y, const RadixList& rl, int nl, int ld,
+                                        const C* tw) {
+    int Ns = 1;
+    for (int s = 0; s < rl.n; ++s) {
+        const int R = rl.r[s];
+        switch (R) {
+            case 2: stage_lines<C, 2, DIR>(x, y, rl.P, Ns, nl, ld, tw); break;
+            case 3: stage_lines<C, 3, DIR>(x, y, rl.P, Ns, nl, ld, tw); break;
+            case 4: stage_lines<C, 4, DIR>(x, y, rl.P, Ns, nl, ld, tw); break;
+            case 5: stage_lines<C, 5, DIR>(x, y, rl.P, Ns, nl, ld, tw); break;
+            case 7: stage_lines<C, 7, DIR>(x, y, rl.P, Ns, nl, ld, tw); break;
+        }
+        __syncthreads();
+        Ns *= R;
+        C* tmp = x; x = y; y = tmp;
+    }
+    return x;
+}
+
+constexpr int kPlaneThreads = 512;
+constexpr size_t kPlaneSmem = 96 << 10;
+// odd line strides: neither the transposed stores nor the line-fastest ones conflict
+__host__ __device__ constexpr int plane_ldx(int V) { return ((V + 1) / 2) | 1; }
+__host__ __device__ constexpr int plane_ldy(int Hu) { return Hu | 1; }
+__host__ __device__ inline int plane_elems(int Pu, int Pv, int V) {
+    const int x = Pu * plane_ldx(V), y = Pv * plane_ldy(Pu / 2 + 1);
+    return x > y ? x : y;
+}
+
+// [3][W][V][U] -> [3][W][Pv][Hu]
+template <typename R>
+__global__ void __launch_bounds__(kPlaneThreads)
+k_plane_fwd(const double* __restrict__ in, int U, int V, int W, typename CT<R>::c* __restrict__ out,
+            const typename CT<R>::c* __restrict__ twx, const typename CT<R>::c* __restrict__ twy,
+            RadixList rx, RadixList ry, const double* __restrict__ scale) {
+    typedef typename CT<R>::c C;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int Pu = rx.P, Pv = ry.P, Hu = Pu / 2 + 1, VP = (V + 1) / 2;
+    const int ldx = plane_ldx(V), ldy = plane_ldy(Hu), ne = plane_elems(Pu, Pv, V);
+    C* sx = reinterpret_cast<C*>(smem_raw);
+    C* sy = sx + tw_entries<C>(Pu);
+    C* b0 = sy + tw_entries<C>(Pv);
+    C* b1 = b0 + ne;
+    const long long cw = blockIdx.x;
+    load_tw(sx, twx, Pu);
+    load_tw(sy, twy, Pv);
+    for (int i = threadIdx.x; i < (Pu - U) * ldx; i += blockDim.x) {   // the padding of the rows
+        b0[U * ldx + i].x = 0;
+        b0[U * ldx + i].y = 0;
+    }
+    pdl_trigger();
+    pdl_wait();
+    const float inv_u = 1.0f / (float)U;
+    for (int it = threadIdx.x; it < VP * U; it += blockDim.x) {
+        const int t = __float2int_rz(((float)it + 0.5f) * inv_u), j = it - t * U, v = 2 * t;
+        const double* row = in + (cw * V + v) * (long long)U;
+        double va = row[j], vb = 0.0;
+        if (v + 1 < V) vb = row[U + j];
+        if (scale) {   // per-voxel factor (the adjoint transforms chi * lambda)
+            const long long m0 = ((cw % W) * V + v) * (long long)U + j;
+            va *= scale[m0];
+            if (v + 1 < V) vb *= scale[m0 + U];
+        }
+        b0[j * ldx + t].x = (R)va;
+        b0[j * ldx + t].y = (R)vb;
+    }
+    __syncthreads();
+    C* X = fft_lines<C, -1>(b0, b1, rx, VP, ldx, sx);
+    C* Y = X == b0 ? b1 : b0;
+    // split: A = (Z[k] + conj Z[P-k]) / 2, B = -i (Z[k] - conj Z[P-k]) / 2
+    const float inv_vp = 1.0f / (float)VP;
+    for (int it = threadIdx.x; it < VP * Hu; it += blockDim.x) {
+        const int k = __float2int_rz(((float)it + 0.5f) * inv_vp), t = it - k * VP;
+        const C zk = X[k * ldx + t], zm = X[(k ? Pu - k : 0) * ldx + t];
+        C A, B;
+        A.x = (R)0.5 * (zk.x + zm.x);
+        A.y = (R)0.5 * (zk.y - zm.y);
+        B.x = (R)0.5 * (zk.y + zm.y);
+        B.y = (R)0.5 * (zm.x - zk.x);
+        Y[2 * t * ldy + k] = A;
+        if (2 * t + 1 < V) Y[(2 * t + 1) * ldy + k] = B;
+    }
+    for (int i = threadIdx.x; i < (Pv - V) * ldy; i += blockDim.x) {
+        Y[V * ldy + i].x = 0;
+        Y[V * ldy + i].y = 0;
+    }
+    __syncthreads();
+    const C* Z = fft_lines<C, -1>(Y, X, ry, Hu, ldy, sy);
+    const float inv_hu = 1.0f / (float)Hu;
+    C* dst = out + cw * Pv * Hu;
+    for (int it = threadIdx.x; it < Pv * Hu; it += blockDim.x) {
+        const int j = __float2int_rz(((float)it + 0.5f) * inv_hu);
+        dst[it] = Z[j * ldy + it - j * Hu];
+    }
+}
+
+// [3][W][Pv][Hu] -> real [3][W][V][U]
+template <typename R>
+__global__ void __launch_bounds__(kPlaneThreads)
+k_plane_inv(const typename CT<R>::c* __restrict__ in, int U, int V, R* __restrict__ out,
+            const typename CT<R>::c* __restrict__ twx, const typename CT<R>::c* __restrict__ twy,
+            RadixList rx, RadixList ry) {
+    typedef typename CT<R>::c C;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int Pu = rx.P, Pv = ry.P, Hu = Pu / 2 + 1, VP = (V + 1) / 2;
+    const int ldx = plane_ldx(V), ldy = plane_ldy(Hu), ne = plane_elems(Pu, Pv, V);
+    C* sx = reinterpret_cast<C*>(smem_raw);
+    C* sy = sx + tw_entries<C>(Pu);
+    C* b0 = sy + tw_entries<C>(Pv);
+    C* b1 = b0 + ne;
+    const long long cw = blockIdx.x;
+    load_tw(sx, twx, Pu);
+    load_tw(sy, twy, Pv);
+    pdl_trigger();
+    pdl_wait();
+    const float inv_hu = 1.0f / (float)Hu;
+    const C* src = in + cw * Pv * Hu;
+    for (int it = threadIdx.x; it < Pv * Hu; it += blockDim.x) {
+        const int j = __float2int_rz(((float)it + 0.5f) * inv_hu);
+        cp_async_c(&b0[j * ldy + it - j * Hu], src + it);
+    }
+    cp_async_commit_wait();
+    __syncthreads();
+    C* Y = fft_lines<C, +1>(b0, b1, ry, Hu, ldy, sy);
+    C* X = Y == b0 ? b1 : b0;
+    // Z[k] = A[k] + i B[k] and Z[P-k] = conj A[k] + i conj B[k] from the two halves
+    const float inv_vp = 1.0f / (float)VP;
+    for (int it = threadIdx.x; it < VP * Hu; it += blockDim.x) {
+        const int k = __float2int_rz(((float)it + 0.5f) * inv_vp), t = it - k * VP;
+        const C A = Y[2 * t * ldy + k];
+        C B;
+        B.x = 0; B.y = 0;
+        if (2 * t + 1 < V) B = Y[(2 * t + 1) * ldy + k];
+        C z;
+        z.x = A.x - B.y;
+        z.y = A.y + B.x;
+        X[k * ldx + t] = z;
+        if (k >= 1 && k < Pu - k) {
+            z.x = A.x + B.y;
+            z.y = B.x - A.y;
+            X[(Pu - k) * ldx + t] = z;
+        }
+    }
+    __syncthreads();
+    const C* Z = fft_lines<C, +1>(X, Y, rx, VP, ldx, sx);
+    const float inv_u = 1.0f / (float)U;
+    for (int it = threadIdx.x; it < VP * U; it += blockDim.x) {
+        const int t = __float2int_rz(((float)it + 0.5f) * inv_u), j = it - t * U;
+        const C z = Z[j * ldx + t];
+        R* row = out + (cw * V + 2 * t) * (long long)U + j;
+        row[0] = z.x;
+        if (2 * t + 1 < V) row[U] = z.y;
+    }
+}
+
 RadixList radix_list(const AxisFFT& ax) {
     RadixList rl;
     rl.P = ax.P;
@@ -495,6 +681,9 @@ void launch_mid4s(const typename CT<R>::c* in, typename CT<R>::c* out,
     MOT_LAUNCH_CHECK();
 }
 
+// lengths with a four-step codelet (mid_pass, x_pass_codelet)
+bool has_codelet(int P) { return P == 64 || P == 96 || P == 210; }
+
 // a strided pass of length ax.P over [3][n_o2] x Hu lines: the four-step kernel for the
 // lengths that have a factor pair below, the generic Stockham tile otherwise
 template <typename R>
@@ -513,7 +702,7 @@ void mid_pass(const typename CT<R>::c* in, typename CT<R>::c* out, const AxisFFT
     const size_t sm = smem_bytes<R>(P);
     allow_smem<k_mid<R>>(sm);
     launch_dependent(dep, k_mid<R>, (int)((lines + TB - 1) / TB), NT, sm, s, in, out, table<R>(ax),
-                                                                    radix_list(ax), a);
+                     radix_list(ax), a);
     MOT_LAUNCH_CHECK();
 }
 
@@ -567,12 +756,12 @@ void launch_x4s(bool fwd, mot_ctx* c, const double* Jsoa, typename CT<R>::c* spe
     const int blocks = (int)((npairs + kXL - 1) / kXL);
     if (fwd) {
         allow_smem<k_fwd_x4s<R, P1, P2>>(sm);
-        launch_dependent(mot::dependent_launches(c), k_fwd_x4s<R, P1, P2>, blocks, threads, sm, s, Jsoa, c->U, c->V, c->W, spec,
-                                                         table<R>(c->ax[0]), scale);
+        launch_dependent(mot::dependent_launches(c), k_fwd_x4s<R, P1, P2>, blocks, threads, sm, s,
+                         Jsoa, c->U, c->V, c->W, spec, table<R>(c->ax[0]), scale);
     } else {
         allow_smem<k_inv_x4s<R, P1, P2>>(sm);
-        launch_dependent(mot::dependent_launches(c), k_inv_x4s<R, P1, P2>, blocks, threads, sm, s, spec, c->U, c->V, c->W, real,
-                                                         table<R>(c->ax[0]));
+        launch_dependent(mot::dependent_launches(c), k_inv_x4s<R, P1, P2>, blocks, threads, sm, s,
+                         spec, c->U, c->V, c->W, real, table<R>(c->ax[0]));
     }
     MOT_LAUNCH_CHECK();
 }
@@ -588,6 +777,35 @@ bool x_pass_codelet(bool fwd, mot_ctx* c, const double* Jsoa, typename CT<R>::c*
     }
 }
 
+// Shared memory of the plane kernels where they are the faster ones, else 0.  Forward +
+// inverse x and y passes of a step, microseconds, two kernels each -> the plane kernels:
+//   FP32  8^3 20.8 -> 16.3, 24^3 27.9 -> 21.0, 40^3 49.4 -> 40.7, 44^3 63.0 -> 53.9,
+//         21 x 27 x 133 46.7 -> 33.3, 64 x 16 x 16 41.7 -> 33.4; but with a codelet for both
+//         lengths 32^3 29.3 -> 29.1 and 48^3 41.4 -> 46.1 (its transforms stay in registers)
+//   FP64  8^3 29.8 -> 24.0, 16^3 32.6 -> 28.6, 20^3 37.3 -> 36.5, 24^3 40.8 -> 41.4, 28^3
+//         52.5 -> 54.2, 16 x 64 x 16 48.1 -> 66.7: a plane is bound by the FP64 units of its
+//         one SM unless it is small
+// A whole step: FP32 8^3 56.9 -> 50.8, 24^3 85.1 -> 78.8, 44^3 244 -> 239; FP64 8^3 85.6 ->
+// 79.4, 16^3 132 -> 123; but 20^3 0.5 us slower, and 16 x 16 x 64 (192 planes, two on some
+// SMs) 326 -> 340; with planes enough to even that out 4 x 100 x 100 (300) 1003 -> 956, 21 x
+// 27 x 133 (399) 1483 -> 1452.
+template <typename R> size_t plane_pass(const mot_ctx* c) {
+    typedef typename CT<R>::c C;
+    const int Pu = c->ax[0].P, Pv = c->ax[1].P;
+    const size_t sm = sizeof(C) * ((size_t)tw_entries<C>(Pu) + tw_entries<C>(Pv) +
+                                   2 * (size_t)plane_elems(Pu, Pv, c->V));
+    if (sm > kPlaneSmem) return 0;
+    if (std::is_same<R, float>::value) return has_codelet(Pu) && has_codelet(Pv) ? 0 : sm;
+    return (Pu * Pv <= 32 * 32 && 3 * c->W <= c->nsm) || 3 * c->W >= 2 * (c->nsm - 2) ? sm : 0;
+}
+int plane_threads(const mot_ctx* c) {
+    const int want = c->ax[1].P * c->Hu / 4;
+    return std::min(kPlaneThreads, std::max(64, (want + 31) / 32 * 32));
+}
+
+// kernels of the x and y passes of a transform
+template <typename R> int fft_xy_launches(const mot_ctx* c) { return plane_pass<R>(c) ? 1 : 2; }
+
 // x and y passes of the forward transform, [3][W][V][U] -> hb.tmp2 [3][W][Pv][Hu]
 template <typename R>
 void fft_forward_xy(mot_ctx* c, const double* Jsoa, cudaStream_t s, const double* scale) {
@@ -595,14 +813,21 @@ void fft_forward_xy(mot_ctx* c, const double* Jsoa, cudaStream_t s, const double
     constexpr int TB = Tile<R>::TB;
     const int U = c->U, V = c->V, W = c->W;
     const int Pu = c->ax[0].P, Pv = c->ax[1].P, Hu = c->Hu;
+    if (const size_t sm = plane_pass<R>(c)) {
+        allow_smem<k_plane_fwd<R>>(sm);
+        launch_dependent(dependent_launches(c), k_plane_fwd<R>, 3 * W, plane_threads(c), sm, s, Jsoa,
+                         U, V, W, hb.tmp2, table<R>(c->ax[0]), table<R>(c->ax[1]),
+                         radix_list(c->ax[0]), radix_list(c->ax[1]), scale);
+        MOT_LAUNCH_CHECK();
+        return;
+    }
     // x
     if (!x_pass_codelet<R>(true, c, Jsoa, hb.tmp1, nullptr, scale, s)) {
         const long long npairs = 3LL * W * ((V + 1) / 2);
         const size_t sm = smem_bytes<R>(Pu);
         allow_smem<k_fwd_x<R>>(sm);
-        launch_dependent(mot::dependent_launches(c), k_fwd_x<R>, (int)((npairs + TB - 1) / TB), NT, sm, s, Jsoa, U, V, W, hb.tmp1,
-                                                                 table<R>(c->ax[0]),
-                                                                 radix_list(c->ax[0]), scale);
+        launch_dependent(dependent_launches(c), k_fwd_x<R>, (int)((npairs + TB - 1) / TB), NT, sm, s,
+                         Jsoa, U, V, W, hb.tmp1, table<R>(c->ax[0]), radix_list(c->ax[0]), scale);
         MOT_LAUNCH_CHECK();
     }
     // y: [3][W][V][Hu] -> [3][W][Pv][Hu]
@@ -635,6 +860,14 @@ void fft_inverse_yx(mot_ctx* c, R* out, cudaStream_t s) {
     constexpr int TB = Tile<R>::TB;
     const int U = c->U, V = c->V, W = c->W;
     const int Pu = c->ax[0].P, Pv = c->ax[1].P, Hu = c->Hu;
+    if (const size_t sm = plane_pass<R>(c)) {
+        allow_smem<k_plane_inv<R>>(sm);
+        launch_dependent(dependent_launches(c), k_plane_inv<R>, 3 * W, plane_threads(c), sm, s, hb.tmp2,
+                         U, V, out, table<R>(c->ax[0]), table<R>(c->ax[1]), radix_list(c->ax[0]),
+                         radix_list(c->ax[1]));
+        MOT_LAUNCH_CHECK();
+        return;
+    }
     // y: [3][W][Pv][Hu] -> [3][W][V][Hu]
     {
         MidArgs a;
@@ -649,9 +882,8 @@ void fft_inverse_yx(mot_ctx* c, R* out, cudaStream_t s) {
         const long long npairs = 3LL * W * ((V + 1) / 2);
         const size_t sm = smem_bytes<R>(Pu);
         allow_smem<k_inv_x<R>>(sm);
-        launch_dependent(mot::dependent_launches(c), k_inv_x<R>, (int)((npairs + TB - 1) / TB), NT, sm, s, hb.tmp1, U, V, W, out,
-                                                                 table<R>(c->ax[0]),
-                                                                 radix_list(c->ax[0]));
+        launch_dependent(dependent_launches(c), k_inv_x<R>, (int)((npairs + TB - 1) / TB), NT, sm, s,
+                         hb.tmp1, U, V, W, out, table<R>(c->ax[0]), radix_list(c->ax[0]));
         MOT_LAUNCH_CHECK();
     }
 }
@@ -669,6 +901,8 @@ void fft_inverse(mot_ctx* c, const typename CT<R>::c* in, R* out, cudaStream_t s
     fft_inverse_yx<R>(c, out, s);
 }
 
+template int fft_xy_launches<double>(const mot_ctx*);
+template int fft_xy_launches<float>(const mot_ctx*);
 template void fft_forward_xy<double>(mot_ctx*, const double*, cudaStream_t, const double*);
 template void fft_forward_xy<float>(mot_ctx*, const double*, cudaStream_t, const double*);
 template void fft_forward_z<double>(mot_ctx*, double2*, cudaStream_t);

@@ -1210,7 +1210,7 @@ void history_step(mot_ctx* c, int n, cudaStream_t s, cudaEvent_t* ev) {
     if (n >= 2) {
         const double* Jprev = c->J + slot_index(n - 1, c->jring) * 3 * c->M;
         fft_forward_xy<R>(c, Jprev, s, c->adjoint ? c->chi : nullptr);
-        c->stats.launches += 2;
+        c->stats.launches += fft_xy_launches<R>(c);
         if (fires || !fused) {     // a firing reads the spectrum of J_{n-1}
             fft_forward_z<R>(c, hb.jhat_ring + slot_index(n - 1, c->hring) * slot, s);
             c->stats.launches += 1;
@@ -1235,9 +1235,8 @@ void history_step(mot_ctx* c, int n, cudaStream_t s, cudaEvent_t* ev) {
         for (int k = 0; k < nfar; ++k) fs.p[k] = far[k];
         const float scale = (float)(1.0 / ((double)c->ax[0].P * c->ax[1].P * c->ax[2].P));
         const long long nblk = (c->noct + 8 * (NT / 32) - 1) / (8 * (NT / 32));
-        launch_dependent(mot::dependent_launches(c), k_mac, (int)nblk, NT, 0, s, hb.ghat, hb.jhat_ring, c->hring,
-                                       (int)slot_index(n - 1, c->hring), L, geom(c), scale,
-                                       hb.phat, fs);
+        launch_dependent(dependent_launches(c), k_mac, (int)nblk, NT, 0, s, hb.ghat, hb.jhat_ring,
+                         c->hring, (int)slot_index(n - 1, c->hring), L, geom(c), scale, hb.phat, fs);
         MOT_LAUNCH_CHECK();
     }
     c->stats.launches += 1;
@@ -1245,7 +1244,7 @@ void history_step(mot_ctx* c, int n, cudaStream_t s, cudaEvent_t* ev) {
     if (ev) MOT_CUDA_TRY(cudaEventRecord(ev[2], s));
     if (fused) fft_inverse_yx<R>(c, hb.hist_spatial, s);
     else fft_inverse<R>(c, hb.phat, hb.hist_spatial, s);
-    c->stats.launches += fused ? 2 : 3;
+    c->stats.launches += fft_xy_launches<R>(c) + (fused ? 0 : 1);
 }
 
 template void history_alloc<double>(mot_ctx*);
