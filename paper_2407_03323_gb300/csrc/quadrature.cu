@@ -116,67 +116,64 @@ __device__ inline Cell make_cell(double dp, double dq, int i, int j, int deriv) 
     return c;
 }
 
-// int_{-h}^{h} (cos t - 1) dt and (cos t - 1)^2 - sin^2 t dt (the difference of the two
-// second moments that the arc needs) without cancellation; ch, sh: cos h, sin h
-__device__ inline void arc_moments(double h, double sh, double ch, double& Ic, double& Id) {
+// int_{-h}^{h} (cos t - 1) dt, sin^2 t dt, (cos t - 1)^2 dt without cancellation
+__device__ inline void arc_moments(double h, double& Ic, double& Iss, double& Icc) {
     if (h < 0.5) {
-        // sum_k (-1)^k h^(2k+1) / (2k+1)! times 2, and times 2^(2k) - 4 + 2^(2k)
-        constexpr double f[10] = {1.0 / 6, 1.0 / 120, 1.0 / 5040, 1.0 / 362880, 1.0 / 39916800,
-                                  1.0 / 6227020800.0, 1.0 / 1307674368000.0,
-                                  1.0 / 355687428096000.0, 1.0 / 121645100408832000.0,
-                                  1.0 / 51090942171709440000.0};
-        const double h2 = h * h;
-        double c = 0.0, d = 0.0, four = 1048576.0;     // 4^10
-#pragma unroll
-        for (int k = 10; k >= 1; --k) {
-            const double t = (k & 1) ? -f[k - 1] : f[k - 1];
-            c = fma(c, h2, 2.0 * t);
-            d = fma(d, h2, (2.0 * four - 4.0) * t);
-            four *= 0.25;
+        double h2 = h * h, pw = h * h2;   // h^(2k+1), k = 1
+        double fact = 6.0;                // (2k+1)!
+        double four = 4.0;                // 2^(2k)
+        Ic = 0.0; Iss = 0.0; Icc = 0.0;
+        double sgn = -1.0;                // (-1)^k
+        for (int k = 1; k <= 10; ++k) {
+            double term = pw / fact;
+            Ic += 2.0 * sgn * term;
+            Iss += -sgn * four * term;
+            Icc += sgn * (four - 4.0) * term;
+            pw *= h2;
+            fact *= (2.0 * k + 2.0) * (2.0 * k + 3.0);
+            four *= 4.0;
+            sgn = -sgn;
         }
-        Ic = c * h2 * h;
-        Id = d * h2 * h;
     } else {
+        double sh, ch;
+        sincos(h, &sh, &ch);
         Ic = 2.0 * sh - 2.0 * h;
-        Id = 2.0 * h + 2.0 * sh * ch - 4.0 * sh;
+        Iss = h - sh * ch;
+        Icc = 3.0 * h + sh * ch - 4.0 * sh;
     }
 }
 
-// Integrals over the circle of radius s of the hats' product on a first-quadrant cell (added
-// to AL) and of their derivatives' product (to AD: constant on the cell, so its value times
-// the arc length; vD).  The two share the arc.  Its half angle comes from the cross and dot
-// product of its ends and its middle from their sum: one arctangent for the pair.
-__device__ inline void arc_cell(double s, const Cell& c, double vD, double& AL, double& AD) {
-    if (!(c.x0 < s && c.y0 < s)) return;
-    const double s2 = s * s;
+// integral over the circle of radius s of the cell weight (first-quadrant cell)
+__device__ inline double arc_cell(double s, const Cell& c) {
+    if (!(c.x0 < s && c.y0 < s)) return 0.0;
+    double s2 = s * s;
     double Xa, Ya, Xb, Yb;
     {   // lower end: larger angle of {leave x <= x1, enter y >= y0}
-        const double xa1 = c.x1 < s ? c.x1 : s;
-        const double ya1 = c.x1 < s ? sqrt(fmax(s2 - c.x1 * c.x1, 0.0)) : 0.0;
-        if (c.y0 > ya1) { Xa = sqrt(fmax(s2 - c.y0 * c.y0, 0.0)); Ya = c.y0; }
-        else { Xa = xa1; Ya = ya1; }
+        double xa1 = c.x1 < s ? c.x1 : s;
+        double ya1 = c.x1 < s ? sqrt(fmax(s2 - c.x1 * c.x1, 0.0)) : 0.0;
+        double xa2 = sqrt(fmax(s2 - c.y0 * c.y0, 0.0));
+        double ya2 = c.y0;
+        if (ya2 > ya1) { Xa = xa2; Ya = ya2; } else { Xa = xa1; Ya = ya1; }
     }
     {   // upper end: smaller angle of {leave x >= x0, leave y <= y1}
-        const double yb1 = sqrt(fmax(s2 - c.x0 * c.x0, 0.0));
-        const double yb2 = c.y1 < s ? c.y1 : s;
-        if (yb2 < yb1) { Xb = c.y1 < s ? sqrt(fmax(s2 - c.y1 * c.y1, 0.0)) : 0.0; Yb = yb2; }
-        else { Xb = c.x0; Yb = yb1; }
+        double xb1 = c.x0, yb1 = sqrt(fmax(s2 - c.x0 * c.x0, 0.0));
+        double xb2 = c.y1 < s ? sqrt(fmax(s2 - c.y1 * c.y1, 0.0)) : 0.0;
+        double yb2 = c.y1 < s ? c.y1 : s;
+        if (yb2 < yb1) { Xb = xb2; Yb = yb2; } else { Xb = xb1; Yb = yb1; }
     }
-    if (!(Yb > Ya)) return;
-    const double cross = Xa * Yb - Ya * Xb, dot = Xa * Xb + Ya * Yb;
-    const double h = 0.5 * atan2(cross, dot);
-    if (h <= 0.0) return;
-    const double mx = Xa + Xb, my = Ya + Yb, im = rsqrt(mx * mx + my * my);
-    const double cm = mx * im, sm = my * im;           // middle direction
-    const double ch = 0.5 * (mx * cm + my * sm) / s;   // |sum| / 2s
-    const double Xm = s * cm, Ym = s * sm;
-    const double Ax = c.wx0 + c.sx * (Xm - c.x0);
-    const double Ay = c.wy0 + c.sy * (Ym - c.y0);
-    double Ic, Id;
-    arc_moments(h, sqrt(fmax(1.0 - ch * ch, 0.0)), ch, Ic, Id);
-    AL += 2.0 * h * Ax * Ay + (Ax * c.sy * Ym + Ay * c.sx * Xm) * Ic +
-          c.sx * c.sy * Xm * Ym * Id;
-    AD += 2.0 * h * vD;
+    if (!(Yb > Ya)) return 0.0;
+    double pa = atan2(Ya, Xa), pb = atan2(Yb, Xb);
+    double h = 0.5 * (pb - pa);
+    if (h <= 0.0) return 0.0;
+    double sm, cm;
+    sincos(0.5 * (pa + pb), &sm, &cm);
+    double Xm = s * cm, Ym = s * sm;
+    double Ax = c.wx0 + c.sx * (Xm - c.x0);
+    double Ay = c.wy0 + c.sy * (Ym - c.y0);
+    double Ic, Iss, Icc;
+    arc_moments(h, Ic, Iss, Icc);
+    return 2.0 * h * Ax * Ay + (Ax * c.sy * Ym + Ay * c.sx * Xm) * Ic +
+           c.sx * c.sy * Xm * Ym * (Icc - Iss);
 }
 
 __device__ inline void add3(double* acc, int idx, double v0, double v1, double v2,
@@ -217,13 +214,11 @@ __global__ void quad_kernel(const int3* __restrict__ triples, int ntriples,
                              fmax(b - 1.0, 0.0) * fmax(b - 1.0, 0.0) +
                              fmax(cc - 1.0, 0.0) * fmax(cc - 1.0, 0.0));
     const int l0 = (int)floor(rmin);
-    Cell cL[4];
-    double vD[4];          // product of the hats' derivatives on each cell
+    Cell cL[4], cD[4];
     for (int i = 0; i < 2; ++i)
         for (int j = 0; j < 2; ++j) {
             cL[2 * i + j] = make_cell(dp, dq, i, j, 0);
-            const Cell d = make_cell(dp, dq, i, j, 1);
-            vD[2 * i + j] = d.wx0 * d.wy0;
+            cD[2 * i + j] = make_cell(dp, dq, i, j, 1);
         }
     // the in-plane weight vanishes for s outside [smin, smax]
     double smax = 0.0, smin = 1e300;
@@ -279,7 +274,7 @@ __global__ void quad_kernel(const int3* __restrict__ triples, int ntriples,
             const double s = sa + (sb - sa) * tt;
             const double Ws = (sb - sa) * ww * s;
             double AL = 0.0, AD = 0.0;
-            for (int i = 0; i < 4; ++i) arc_cell(s, cL[i], vD[i], AL, AD);
+            for (int i = 0; i < 4; ++i) { AL += arc_cell(s, cL[i]); AD += arc_cell(s, cD[i]); }
             const double oL = Ws * AL, oD = Ws * AD;
             if (oL == 0.0 && oD == 0.0) continue;
             // diagonal face term: z-weight delta(z-dz+1) - 2 delta(z-dz) + delta(z-dz-1)
@@ -287,12 +282,12 @@ __global__ void quad_kernel(const int3* __restrict__ triples, int ntriples,
                 const double zks[3] = {zk0, zk1, zk2};
                 const double we[3] = {1.0, -2.0, 1.0};
                 for (int e = 0; e < 3; ++e) {
-                    const double r2 = s * s + zks[e] * zks[e], ri = rsqrt(r2);
-                    const double r = sqrt(r2);      // correctly rounded: floor decides the lag
+                    const double r = sqrt(s * s + zks[e] * zks[e]);
                     const int j = (int)floor(r);
-                    const double sg = r - j, cg = 1.0 - sg;
-                    const double half = (0.5 * we[e] / FOURPI) * oL * ri;
-                    add3(accD, j - l0, half * cg * cg, half * (1.0 + 2.0 * sg * cg), half * sg * sg,
+                    const double sg = r - j;
+                    const double base = we[e] * oL / (FOURPI * r);
+                    add3(accD, j - l0, base * 0.5 * (1.0 - sg) * (1.0 - sg),
+                         base * 0.5 * (1.0 + 2.0 * sg - 2.0 * sg * sg), base * 0.5 * sg * sg,
                          &bad);
                 }
             }
@@ -329,24 +324,20 @@ __global__ void quad_kernel(const int3* __restrict__ triples, int ntriples,
                     add3(accO, -l0, co * (Im1 - 2.0 * I0 + I1), co * (Im1 + 2.0 * I0 - 2.0 * I1),
                          co * I1, &bad);
                 } else {
-                    // sums of q, q sg and q cg with q = wz / (4 pi r), sg = r - j, cg = 1 - sg:
-                    // the spline's three pieces are cg^2 / 2, 1/2 + sg cg and sg^2 / 2
-                    double v0 = 0.0, o0 = 0.0, o2 = 0.0;
-                    const double zr = lower ? zk0 : zk2, sgn = (lower ? 1.0 : -1.0) * hz / FOURPI;
+                    double v0 = 0.0, v1 = 0.0, v2 = 0.0, o0 = 0.0, o1 = 0.0, o2 = 0.0;
                     for (int g = 0; g < NZ; ++g) {
                         const double z = zm + hz * c_gz_x[g];
-                        const double r2 = fma(z, z, s * s), ri = rsqrt(r2);
-                        const double sg = fma(r2, ri, -(double)j), cg = 1.0 - sg;
-                        const double q = c_gz_w[g] * (z - zr) * ri;
+                        const double wz = hz * c_gz_w[g] * (lower ? (z - zk0) : (zk2 - z));
+                        const double r = sqrt(s * s + z * z);
+                        const double sg = r - j;
+                        const double q = wz / (FOURPI * r);
                         v0 += q;
-                        o0 = fma(q * cg, cg, o0);
-                        o2 = fma(q * sg, sg, o2);
+                        o0 += q * 0.5 * (1.0 - sg) * (1.0 - sg);
+                        o1 += q * 0.5 * (1.0 + 2.0 * sg - 2.0 * sg * sg);
+                        o2 += q * 0.5 * sg * sg;
                     }
-                    v0 *= sgn;
-                    o0 *= 0.5 * sgn;
-                    o2 *= 0.5 * sgn;
-                    const double o1 = v0 - o0 - o2;        // the pieces sum to one
-                    const double v1 = -2.0 * v0, v2 = v0;
+                    v1 = -2.0 * v0;
+                    v2 = v0;
                     add3(accV, j - l0, oL * v0, oL * v1, oL * v2, &bad);
                     add3(accO, j - l0, oD * o0, oD * o1, oD * o2, &bad);
                 }
