@@ -101,6 +101,7 @@ void free_all(mot_ctx* c) {
     cudaFree(c->probe_l0);
     cudaFree(c->pdsa_spec);
     cudaFree(c->pdsa_a);
+    cudaFree(c->pdsa_xhat);
     cudaFree(c->pdsa_conv);
     cudaFree(c->pw_tab);
     for (cudaEvent_t e : c->events) cudaEventDestroy(e);

@@ -909,6 +909,7 @@ template void fft_forward_z<double>(mot_ctx*, double2*, cudaStream_t);
 template void fft_forward_z<float>(mot_ctx*, float2*, cudaStream_t);
 template void fft_inverse_yx<double>(mot_ctx*, double*, cudaStream_t);
 template void fft_inverse_yx<float>(mot_ctx*, float*, cudaStream_t);
+template void fft_inverse<double>(mot_ctx*, const double2*, double*, cudaStream_t);
 template void fft_inverse<float>(mot_ctx*, const float2*, float*, cudaStream_t);
 
 }  // namespace mot

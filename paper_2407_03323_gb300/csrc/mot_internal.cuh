@@ -241,6 +241,7 @@ struct mot_ctx {
     // PDSA operator A_n (pdsa.cu): kernel spectrum and diagonal of the last (n, flags)
     double* pdsa_spec = nullptr;   // [noct][6] unnormalised spectrum of sum_i c_i G_i
     double* pdsa_a = nullptr;      // [M] diagonal a_m (0 on voxels with chi = 0)
+    double2* pdsa_xhat = nullptr;  // [3][nbins] spectrum scratch
     double* pdsa_conv = nullptr;   // [3][M] convolution scratch
     int pdsa_n = -1, pdsa_flags = -1;
 
@@ -308,7 +309,6 @@ template <typename R> void fft_inverse_yx(mot_ctx* c, R* out, cudaStream_t s);
 template <typename R>
 void zmac(mot_ctx* c, int n, bool fwd, int L, const typename CT<R>::c* const* far, int nfar,
           cudaStream_t s);
-void zproduct(mot_ctx* c, const double* spec, cudaStream_t s);
 // history.cu
 // far levels of the blocked scheme for block B and ell (host only): level k covers
 // lags [a[k], a[k] + S[k]); returns the number of levels, or -1 if more than 8 are needed

@@ -66,6 +66,38 @@ __global__ void k_pdsa_diag(const double* __restrict__ eps, long long M, double 
     a[m] = e > 1.0 ? (aT + beta * e) / (e - 1.0) : 0.0;
 }
 
+// yhat(k) = scale * Khat(k) xhat(k) over all rfft bins, Khat from its octant
+// ([noct][6]: xx yy zz xy xz yz); mirrored v / w bins flip the components odd there
+__global__ void k_pdsa_mul(const double* __restrict__ spec, double2* __restrict__ xh, int Hu,
+                           int Hv, int Pv, int Pw, long long nbins, double scale) {
+    pdl_trigger();
+    pdl_wait();
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= nbins) return;
+    const int ku = (int)(i % Hu);
+    const int kv = (int)((i / Hu) % Pv);
+    const int kw = (int)(i / ((long long)Hu * Pv));
+    const bool fv = kv >= Hv, fw = 2 * kw > Pw;
+    const int ov = fv ? Pv - kv : kv;
+    const int ow = fw ? Pw - kw : kw;
+    const double* g = spec + (((long long)ow * Hv + ov) * Hu + ku) * 6;
+    const double gxx = g[0], gyy = g[1], gzz = g[2];
+    const double gxy = fv ? -g[3] : g[3];
+    const double gxz = fw ? -g[4] : g[4];
+    const double gyz = (fv != fw) ? -g[5] : g[5];
+    const double2 x = xh[i], y = xh[nbins + i], z = xh[2 * nbins + i];
+    double2 ox, oy, oz;
+    ox.x = scale * (gxx * x.x + gxy * y.x + gxz * z.x);
+    ox.y = scale * (gxx * x.y + gxy * y.y + gxz * z.y);
+    oy.x = scale * (gxy * x.x + gyy * y.x + gyz * z.x);
+    oy.y = scale * (gxy * x.y + gyy * y.y + gyz * z.y);
+    oz.x = scale * (gxz * x.x + gyz * y.x + gzz * z.x);
+    oz.y = scale * (gxz * x.y + gyz * y.y + gzz * z.y);
+    xh[i] = ox;
+    xh[nbins + i] = oy;
+    xh[2 * nbins + i] = oz;
+}
+
 // y = a x - conv on active voxels, 0 elsewhere ([3][M])
 __global__ void k_pdsa_combine(const double* __restrict__ a, const double* __restrict__ eps,
                                const double* __restrict__ x, const double* __restrict__ conv,
@@ -266,9 +298,10 @@ __global__ void k_sub_combo(double* __restrict__ w, const double* __restrict__ V
     acc = warp_sum(acc);
     if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = acc;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        acc = warp_sum(threadIdx.x < NT / 32 ? sm[threadIdx.x] : 0.0);
-        if (threadIdx.x == 0) part[blockIdx.x] = acc;
+    if (threadIdx.x == 0) {      // (in the order of k_dots: the same bits as its w . w)
+        acc = 0.0;
+        for (int k = 0; k < NT / 32; ++k) acc += sm[k];
+        part[blockIdx.x] = acc;
     }
 }
 
@@ -365,6 +398,7 @@ void ensure_operator(mot_ctx* c, int n, int flags) {
     if (!c->pdsa_spec) {
         MOT_CUDA_TRY(cudaMalloc(&c->pdsa_spec, sizeof(double) * 6 * c->noct));
         MOT_CUDA_TRY(cudaMalloc(&c->pdsa_a, sizeof(double) * M));
+        MOT_CUDA_TRY(cudaMalloc(&c->pdsa_xhat, sizeof(double2) * 3 * c->nbins));
         MOT_CUDA_TRY(cudaMalloc(&c->pdsa_conv, sizeof(double) * 3 * M));
     }
     c->pdsa_n = c->pdsa_flags = -1;
@@ -392,9 +426,17 @@ void ensure_operator(mot_ctx* c, int n, int flags) {
 
 // y = A_n x, both [3][M] on the device
 void apply(mot_ctx* c, const double* x, double* y, cudaStream_t s) {
+    // (separate z passes: Lanczos amplifies rounding once a multiple eigenvalue has converged,
+    // and a z transform of another kernel's order changes the low Ritz values of symmetric
+    // bodies by up to 1e-3 after 60 steps or so)
+    const double scale = 1.0 / ((double)c->ax[0].P * c->ax[1].P * c->ax[2].P);
     mot::fft_forward_xy<double>(c, x, s, nullptr);
-    mot::zproduct(c, c->pdsa_spec, s);
-    mot::fft_inverse_yx<double>(c, c->pdsa_conv, s);
+    mot::fft_forward_z<double>(c, c->pdsa_xhat, s);
+    launch_dependent(mot::dependent_launches(c), k_pdsa_mul, nblk(c->nbins, NT), NT, 0, s,
+                     c->pdsa_spec, c->pdsa_xhat, c->Hu, c->Hv, c->ax[1].P, c->ax[2].P, c->nbins,
+                     scale);
+    MOT_LAUNCH_CHECK();
+    mot::fft_inverse<double>(c, c->pdsa_xhat, c->pdsa_conv, s);
     launch_dependent(mot::dependent_launches(c), k_pdsa_combine, nblk(3 * c->M, NT), NT, 0, s,
                      c->pdsa_a, c->eps, x, c->pdsa_conv, c->M, y);
     MOT_LAUNCH_CHECK();

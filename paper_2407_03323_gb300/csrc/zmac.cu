@@ -279,20 +279,19 @@ __global__ void __launch_bounds__(256, 2) k_zmac(const __grid_constant__ ZArgs<R
         cp_async_commit_wait();
     }
     __syncthreads();
-    const bool keep = a.ring != nullptr;
-    C* slot = keep ? a.ring + (long long)a.slot1 * 3 * a.nbins + f0 : nullptr;
+    C* slot = a.ring + (long long)a.slot1 * 3 * a.nbins + f0;
     C* X = b0;
     if (a.fwd) {
         if constexpr (kFourStep) {
             four_step_lines<C, P1, P2, -1, NL>(b0, b1, stw, ld, a.W, [&](int k, int line, C v) {
                 b0[k * ld + line] = v;
                 const int c = line / TB, t = line % TB;
-                if (keep && f0 + t < a.plane) slot[c * a.nbins + (long long)k * a.plane + t] = v;
+                if (f0 + t < a.plane) slot[c * a.nbins + (long long)k * a.plane + t] = v;
             });
             __syncthreads();
         } else {
             X = fft_tile<C, NL>(b0, b1, P, a.rl.r, a.rl.n, ld, stw, -1);
-            for (int it = threadIdx.x; keep && it < P * NL; it += blockDim.x) {
+            for (int it = threadIdx.x; it < P * NL; it += blockDim.x) {
                 const int line = it % NL, k = it / NL;
                 const int c = line / TB, t = line % TB;
                 if (f0 + t < a.plane) slot[c * a.nbins + (long long)k * a.plane + t] = X[k * ld + line];
@@ -414,20 +413,6 @@ void zmac(mot_ctx* c, int n, bool fwd, int L, const typename CT<R>::c* const* fa
     a.hring = c->hring;
     a.slot1 = (int)slot_index(n - 1, c->hring);
     a.L = L;
-    run(c, a, s);
-}
-
-// hb.tmp2 <- z-inverse of (spec [noct][6]) times the z transform of hb.tmp2: the Toeplitz
-// product with one kernel between fft_forward_xy and fft_inverse_yx
-void zproduct(mot_ctx* c, const double* spec, cudaStream_t s) {
-    ZArgs<double> a = z_args<double>(c);
-    a.ring = nullptr;
-    a.ghat = spec;
-    a.nfar = 0;
-    a.fwd = 1;
-    a.hring = 1;
-    a.slot1 = 0;
-    a.L = 1;
     run(c, a, s);
 }
 
