@@ -397,7 +397,9 @@ def run_variant(args, cfg, prec, scheme, block, dev, world, steps, warmup, want_
     out["fft_comparison"] = {
         "ours_forward_fft_ms": st["ms_fft_fwd"] / max(st["steps"], 1),
         "cufft_rfftn_full_padded_ms": cufft_comparison(info["P"], U_, V_, W_, prec),
-        "note": "timing comparison only; cuFFT transforms the full padded grid"}
+        "note": "timing comparison only; cuFFT transforms the full padded grid"
+                + ("; ours: x and y passes, z runs in the lag-product kernel (phase mac)"
+                   if prec == "fp64" else "")}
     e2e = None
     if want_e2e:
         k = per                                  # one bench step through host buffers

@@ -448,7 +448,9 @@ mot_status mot_set_solver(mot_ctx* ctx, double tol, int max_iter, double growth_
  *  ms_*          summed CUDA-event durations of the phases, recorded on the stream
  *                mot_march ran on, only while profiling is enabled: forward FFT of
  *                J_{n-1}, far-lag block products (blocked scheme), near-lag MAC,
- *                inverse FFT, rhs + solve                                          */
+ *                inverse FFT, rhs + solve.  In FP64 and on small FP32 grids one kernel
+ *                takes both z passes with the lag products: its time is in ms_mac, and
+ *                ms_fft_* hold the x and y passes (with z on steps where a level fires) */
 typedef struct {
     long long launches;
     long long mac_launches;

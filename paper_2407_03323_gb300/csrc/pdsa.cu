@@ -702,9 +702,11 @@ mot_status mot_pdsa_lanczos(mot_ctx* c, int n, int flags, int k, unsigned long l
             }
             k_rand_vec<<<g1, NT, 0, s>>>(seed, c->eps, M, w);
             MOT_LAUNCH_CHECK();
-            launch_dependent(mot::dependent_launches(c), k_dots, dim3(nb, 1), NT, 0, s, w, 1, L, w, part);
+            launch_dependent(mot::dependent_launches(c), k_dots, dim3(nb, 1), NT, 0, s, w, 1, L, w,
+                             part);
             MOT_LAUNCH_CHECK();
-            launch_dependent(mot::dependent_launches(c), k_normalise, g1, NT, 0, s, w, part, nb, L, V, coef + 3LL * k);
+            launch_dependent(mot::dependent_launches(c), k_normalise, g1, NT, 0, s, w, part, nb, L,
+                             V, coef + 3LL * k);
             MOT_LAUNCH_CHECK();
             // the scalars of a step stay on the device and are read every BATCH steps (a
             // host read per orthogonalisation left the GPU idle for a third of a step);
@@ -718,12 +720,13 @@ mot_status mot_pdsa_lanczos(mot_ctx* c, int n, int flags, int k, unsigned long l
                     apply(c, V + (long long)j * L, w, s);
                     for (int pass = 0; pass < 2; ++pass) {   // w -= V_{0..j} (V_{0..j}^T w), twice
                         dots(c, V, j + 1, L, w, part, h, s);
-                        launch_dependent(mot::dependent_launches(c), k_sub_combo, nb, NT, shm, s, w, V, h, j + 1, L, coef + 3LL * j + pass,
-                                                        pass ? part : nullptr);
+                        launch_dependent(mot::dependent_launches(c), k_sub_combo, nb, NT, shm, s, w,
+                                         V, h, j + 1, L, coef + 3LL * j + pass,
+                                         pass ? part : nullptr);
                         MOT_LAUNCH_CHECK();
                     }
-                    launch_dependent(mot::dependent_launches(c), k_normalise, g1, NT, 0, s, w, part, nb, L, V + (long long)(j + 1) * L,
-                                                  coef + 3LL * j + 2);
+                    launch_dependent(mot::dependent_launches(c), k_normalise, g1, NT, 0, s, w, part,
+                                     nb, L, V + (long long)(j + 1) * L, coef + 3LL * j + 2);
                     MOT_LAUNCH_CHECK();
                 }
                 MOT_CUDA_TRY(cudaMemcpyAsync(hc.data(), coef + 3LL * done, sizeof(double) * 3 * cnt,
@@ -752,7 +755,8 @@ mot_status mot_pdsa_lanczos(mot_ctx* c, int n, int flags, int k, unsigned long l
             k_rand_vec<<<g1, NT, 0, s>>>(seed, c->eps, M, w);
             MOT_LAUNCH_CHECK();
             dots(c, w, 1, L, w, part, b2d + k, s);               // ||w||^2 of the start
-            launch_dependent(mot::dependent_launches(c), k_lz_c, g1, NT, 0, s, w, b2d + k, L, vbuf[1]);   // v_0
+            launch_dependent(mot::dependent_launches(c), k_lz_c, g1, NT, 0, s, w, b2d + k, L,
+                             vbuf[1]);   // v_0
             MOT_LAUNCH_CHECK();
             constexpr int BATCH = 256;
             std::vector<double> ha(BATCH), hb(BATCH);
@@ -766,15 +770,20 @@ mot_status mot_pdsa_lanczos(mot_ctx* c, int n, int flags, int k, unsigned long l
                     double* v = vbuf[(j + 1) % 3];
                     double* vnext = vbuf[(j + 2) % 3];
                     apply(c, v, w, s);
-                    launch_dependent(mot::dependent_launches(c), k_lz_a, nb, NT, 0, s, w, vprev, j ? b2d + j - 1 : nullptr, v, L, part);
+                    launch_dependent(mot::dependent_launches(c), k_lz_a, nb, NT, 0, s, w, vprev,
+                                     j ? b2d + j - 1 : nullptr, v, L, part);
                     MOT_LAUNCH_CHECK();
-                    launch_dependent(mot::dependent_launches(c), k_sum_parts, 1, NT, 0, s, part, nb, ad + j);
+                    launch_dependent(mot::dependent_launches(c), k_sum_parts, 1, NT, 0, s, part, nb,
+                                     ad + j);
                     MOT_LAUNCH_CHECK();
-                    launch_dependent(mot::dependent_launches(c), k_lz_b, nb, NT, 0, s, w, ad + j, v, L, part);
+                    launch_dependent(mot::dependent_launches(c), k_lz_b, nb, NT, 0, s, w, ad + j, v,
+                                     L, part);
                     MOT_LAUNCH_CHECK();
-                    launch_dependent(mot::dependent_launches(c), k_sum_parts, 1, NT, 0, s, part, nb, b2d + j);
+                    launch_dependent(mot::dependent_launches(c), k_sum_parts, 1, NT, 0, s, part, nb,
+                                     b2d + j);
                     MOT_LAUNCH_CHECK();
-                    launch_dependent(mot::dependent_launches(c), k_lz_c, g1, NT, 0, s, w, b2d + j, L, vnext);
+                    launch_dependent(mot::dependent_launches(c), k_lz_c, g1, NT, 0, s, w, b2d + j,
+                                     L, vnext);
                     MOT_LAUNCH_CHECK();
                 }
                 MOT_CUDA_TRY(cudaMemcpyAsync(ha.data(), ad + done, sizeof(double) * cnt,

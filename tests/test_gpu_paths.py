@@ -133,3 +133,18 @@ def test_plane_wave_in_pieces(mot, n0):
             at += k
     assert np.abs(whole).max() > 0
     assert np.abs(np.concatenate(parts) - whole).max() <= 1e-14 * np.abs(whole).max()
+
+
+def test_lanczos_across_reads(mot):
+    """The scalars of the reorthogonalised Lanczos are read every 32 steps: with more steps the
+    extreme Ritz values move outwards only (interlacing, to 1e-12 of the largest), on both
+    sides of a read."""
+    with mot.Context(_noise((4, 5, 6))) as c:
+        last = None
+        for k in (1, 2, 31, 32, 33, 64, 65):
+            r = c.pdsa_lanczos(c.ell, k, seed=2, reorth=True, n_out=1)
+            assert r["steps"] == k
+            low, high = r["ritz"][0], r["theta_max"]
+            if last:
+                assert low <= last[0] + 1e-12 * high and high >= last[1] - 1e-12 * high
+            last = (low, high)
