@@ -323,7 +323,10 @@ def run_variant(args, cfg, prec, scheme, block, dev, world, steps, warmup, want_
     # a bench step: one time step (direct); 128 time steps, whole periods of the block
     # schedule (every level fires in each), for the blocked scheme
     per = ctx.period * max(1, 128 // ctx.period) if scheme.startswith("blocked") else 1
-    n_warm, n_time = warmup * per, steps * per
+    # the first ell steps have shorter lag sums (no currents before step 1): the timed steps
+    # come after them
+    n_warm = max(warmup, -(-(ctx.ell + 1) // per)) * per
+    n_time = steps * per
     # warm-up marches the pulse's leading edge; the timed steps get the pulse itself
     Ew = torch.zeros((min(n_warm, per), M, 3), dtype=torch.float64, device="cuda")
     done = 0
