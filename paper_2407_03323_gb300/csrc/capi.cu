@@ -145,27 +145,27 @@ void solve_alloc(mot_ctx* c) {
     MOT_CUDA_TRY(cudaMalloc(&c->rhs, sizeof(double) * 3 * M));
     MOT_CUDA_TRY(cudaMalloc(&c->cg_q, sizeof(double) * 3 * M));
     MOT_CUDA_TRY(cudaMalloc(&c->cg32, sizeof(float) * 16 * M));
-    MOT_CUDA_TRY(cudaMemset(c->cg32, 0, sizeof(float) * 16 * M));
+    clear(c->cg32, 16 * M, c->stream);
     if (c->precision == MOT_FP64) {
         MOT_CUDA_TRY(cudaMalloc(&c->b_ring, sizeof(double) * 3 * M * slots));
     } else {
         MOT_CUDA_TRY(cudaMalloc(&c->xb_ring, sizeof(float2) * 3 * M * slots));
         MOT_CUDA_TRY(cudaMalloc(&c->b_lo, sizeof(float) * 3 * M));
         MOT_CUDA_TRY(cudaMalloc(&c->cg_xl, sizeof(float) * 4 * M));
-        MOT_CUDA_TRY(cudaMemset(c->cg_xl, 0, sizeof(float) * 4 * M));
+        clear(c->cg_xl, 4 * M, c->stream);
     }
     MOT_CUDA_TRY(cudaMalloc(&c->fit, sizeof(double) * mot::kFitWords));
     // resident: 16-byte words of the solve's blocks; else doubles of the epilogue's
     const size_t part = sizeof(double) * mot::kFitSums *
                         (size_t)(c->cg_resident ? 2 * c->cg_blocks : c->epi_blocks);
     MOT_CUDA_TRY(cudaMalloc(&c->fit_part, part));
-    MOT_CUDA_TRY(cudaMemset(c->fit_part, 0, part));
+    MOT_CUDA_TRY(cudaMemsetAsync(c->fit_part, 0, part, c->stream));
     MOT_CUDA_TRY(cudaMalloc(&c->norm_part, sizeof(double) * 2 * c->norm_blocks));
     // [2][blocks] doubles, then (16-byte aligned) [2][blocks] exchange words
     MOT_CUDA_TRY(cudaMalloc(&c->red, sizeof(double) * 6 * (size_t)c->cg_blocks));
-    MOT_CUDA_TRY(cudaMemset(c->red, 0, sizeof(double) * 6 * (size_t)c->cg_blocks));
+    clear(c->red, 6 * (size_t)c->cg_blocks, c->stream);
     MOT_CUDA_TRY(cudaMalloc(&c->dstatus, sizeof(int) * mot::kStatusWords));
-    MOT_CUDA_TRY(cudaMemset(c->dstatus, 0, sizeof(int) * mot::kStatusWords));
+    clear(c->dstatus, mot::kStatusWords, c->stream);
 }
 
 // origins (x | y << 10 | z << 20) of the tiles of TX x TY x TZ voxels with chi > 0 somewhere
@@ -323,9 +323,9 @@ mot_status mot_create_padded(const int grid[3], const double h[3], double dt,
         MOT_CUDA_TRY(cudaMalloc(&c->eps, sizeof(double) * M));
         MOT_CUDA_TRY(cudaMalloc(&c->chi, sizeof(double) * M));
         MOT_CUDA_TRY(cudaMalloc(&c->cg_diag, sizeof(double) * M));
-        MOT_CUDA_TRY(cudaMemcpy(c->eps, e.data(), sizeof(double) * M, cudaMemcpyHostToDevice));
-        MOT_CUDA_TRY(cudaMemcpy(c->chi, chi.data(), sizeof(double) * M, cudaMemcpyHostToDevice));
-        MOT_CUDA_TRY(cudaMemcpy(c->cg_diag, dg.data(), sizeof(double) * M, cudaMemcpyHostToDevice));
+        upload(c->eps, e.data(), M, c->stream);
+        upload(c->chi, chi.data(), M, c->stream);
+        upload(c->cg_diag, dg.data(), M, c->stream);
         // elements, stencil, spectra
         mot::compute_table(c);
         mot::stencil_setup(c);
@@ -360,10 +360,8 @@ mot_status mot_create_padded(const int grid[3], const double h[3], double dt,
             MOT_CUDA_TRY(cudaMalloc(&c->active, sizeof(int) * na));
             MOT_CUDA_TRY(cudaMalloc(&c->nmask, sizeof(int) * na));
             if (c->nact) {
-                MOT_CUDA_TRY(cudaMemcpy(c->active, act.data(), sizeof(int) * c->nact,
-                                        cudaMemcpyHostToDevice));
-                MOT_CUDA_TRY(cudaMemcpy(c->nmask, nm.data(), sizeof(int) * c->nact,
-                                        cudaMemcpyHostToDevice));
+                upload(c->active, act.data(), c->nact, c->stream);
+                upload(c->nmask, nm.data(), c->nact, c->stream);
             }
             {
                 const std::vector<int> lists[3] = {active_tiles(c, chi, 8, 4, 4),
@@ -371,14 +369,11 @@ mot_status mot_create_padded(const int grid[3], const double h[3], double dt,
                                                    active_tiles(c, chi, 8, 8, 8)};
                 const std::vector<int>& tl = mot::solve_shape(c, lists);
                 MOT_CUDA_TRY(cudaMalloc(&c->tiles, sizeof(int) * std::max<size_t>(tl.size(), 1)));
-                if (!tl.empty())
-                    MOT_CUDA_TRY(cudaMemcpy(c->tiles, tl.data(), sizeof(int) * tl.size(),
-                                            cudaMemcpyHostToDevice));
+                if (!tl.empty()) upload(c->tiles, tl.data(), tl.size(), c->stream);
                 if (c->cg_resident && c->nvac) {
                     const std::vector<int> vac = outside_tiles(c, tl);
                     MOT_CUDA_TRY(cudaMalloc(&c->vac, sizeof(int) * vac.size()));
-                    MOT_CUDA_TRY(cudaMemcpy(c->vac, vac.data(), sizeof(int) * vac.size(),
-                                            cudaMemcpyHostToDevice));
+                    upload(c->vac, vac.data(), vac.size(), c->stream);
                 }
             }
             std::vector<float> d32(M);
@@ -392,15 +387,14 @@ mot_status mot_create_padded(const int grid[3], const double h[3], double dt,
             }
             MOT_CUDA_TRY(cudaMalloc(&c->diag32, sizeof(float) * M));
             MOT_CUDA_TRY(cudaMalloc(&c->vfac, sizeof(double) * 4 * M));
-            MOT_CUDA_TRY(cudaMemcpy(c->diag32, d32.data(), sizeof(float) * M, cudaMemcpyHostToDevice));
+            upload(c->diag32, d32.data(), M, c->stream);
             if (precision == MOT_FP32_HISTORY) {
                 std::vector<float> dlo(M);
                 for (long long m = 0; m < M; ++m) dlo[m] = (float)(dg[m] - (double)d32[m]);
                 MOT_CUDA_TRY(cudaMalloc(&c->diag_lo, sizeof(float) * M));
-                MOT_CUDA_TRY(cudaMemcpy(c->diag_lo, dlo.data(), sizeof(float) * M,
-                                        cudaMemcpyHostToDevice));
+                upload(c->diag_lo, dlo.data(), M, c->stream);
             }
-            MOT_CUDA_TRY(cudaMemcpy(c->vfac, vf.data(), sizeof(double) * 4 * M, cudaMemcpyHostToDevice));
+            upload(c->vfac, vf.data(), 4 * M, c->stream);
         }
         mot::solve_halo_lists(c);
         if (c->nact) mot::chebyshev_setup(c);

@@ -46,6 +46,21 @@ struct MotError {
 
 #define MOT_LAUNCH_CHECK() MOT_CUDA_TRY(cudaGetLastError())
 
+// Uploads and clears of a context's setup, in the order of its own stream, which every kernel
+// of the setup and of the marches uses.  That stream does not wait for the legacy one: a plain
+// cudaMemcpy of a small pageable buffer returns once the buffer is staged, and a plain
+// cudaMemset returns at once, so either could land behind the kernels that need it while the
+// program keeps the legacy stream busy.  The host buffer may be freed on return.
+template <typename T> void upload(T* dst, const T* src, size_t n, cudaStream_t s) {
+    MOT_CUDA_TRY(cudaMemcpyAsync(dst, src, sizeof(T) * n, cudaMemcpyHostToDevice, s));
+}
+template <typename T> void clear(T* dst, size_t n, cudaStream_t s) {
+    MOT_CUDA_TRY(cudaMemsetAsync(dst, 0, sizeof(T) * n, s));
+}
+template <typename S> void upload_symbol(const S& sym, const void* src, size_t bytes, cudaStream_t s) {
+    MOT_CUDA_TRY(cudaMemcpyToSymbolAsync(sym, src, bytes, 0, cudaMemcpyHostToDevice, s));
+}
+
 // ------------------------------------------------------------------ dependent launches
 // The kernels of a step are short on small grids (5 to 15 us) and each needs the one before
 // it.  Launched as programmatic dependents, the blocks of a kernel are placed while the

@@ -555,14 +555,14 @@ void compute_table(mot_ctx* c) {
     {
         std::vector<double> t, w;
         sigmoid_rule(NS_MAIN, 2, t, w);
-        MOT_CUDA_TRY(cudaMemcpyToSymbol(c_sm_t, t.data(), sizeof(double) * NS_MAIN));
-        MOT_CUDA_TRY(cudaMemcpyToSymbol(c_sm_w, w.data(), sizeof(double) * NS_MAIN));
+        upload_symbol(c_sm_t, t.data(), sizeof(double) * NS_MAIN, c->stream);
+        upload_symbol(c_sm_w, w.data(), sizeof(double) * NS_MAIN, c->stream);
         sigmoid_rule(NS_ORIG, 3, t, w);
-        MOT_CUDA_TRY(cudaMemcpyToSymbol(c_so_t, t.data(), sizeof(double) * NS_ORIG));
-        MOT_CUDA_TRY(cudaMemcpyToSymbol(c_so_w, w.data(), sizeof(double) * NS_ORIG));
+        upload_symbol(c_so_t, t.data(), sizeof(double) * NS_ORIG, c->stream);
+        upload_symbol(c_so_w, w.data(), sizeof(double) * NS_ORIG, c->stream);
         gauss_legendre(NZ, t, w);
-        MOT_CUDA_TRY(cudaMemcpyToSymbol(c_gz_x, t.data(), sizeof(double) * NZ));
-        MOT_CUDA_TRY(cudaMemcpyToSymbol(c_gz_w, w.data(), sizeof(double) * NZ));
+        upload_symbol(c_gz_x, t.data(), sizeof(double) * NZ, c->stream);
+        upload_symbol(c_gz_w, w.data(), sizeof(double) * NZ, c->stream);
     }
     // the sorted offsets a >= b >= c that occur in this grid (see tri_before_b)
     int L[3] = {c->U, c->V, c->W};

@@ -2013,15 +2013,17 @@ void stencil_setup(mot_ctx* c) {
     MOT_CUDA_TRY(cudaGetDevice(&dev));
     static bool have_complete[64] = {};
     if (complete || dev >= 64 || !have_complete[dev]) {
-        MOT_CUDA_TRY(cudaMemcpyToSymbol(c_stencil, c->stencil, sizeof(double) * 27 * 6));
+        upload_symbol(c_stencil, c->stencil, sizeof(double) * 27 * 6, c->stream);
         float st32[27 * 6];
         float stl[27 * 6];
         for (int k = 0; k < 27 * 6; ++k) {
             st32[k] = (float)c->stencil[k];
             stl[k] = (float)(c->stencil[k] - (double)st32[k]);
         }
-        MOT_CUDA_TRY(cudaMemcpyToSymbol(c_st32, st32, sizeof st32));
-        MOT_CUDA_TRY(cudaMemcpyToSymbol(c_stl, stl, sizeof stl));
+        upload_symbol(c_st32, st32, sizeof st32, c->stream);
+        upload_symbol(c_stl, stl, sizeof stl, c->stream);
+        // (another context's stream may read them next)
+        MOT_CUDA_TRY(cudaStreamSynchronize(c->stream));
         if (complete && dev < 64) have_complete[dev] = true;
     }
     int noff[27];
@@ -2080,7 +2082,9 @@ void chebyshev_setup(mot_ctx* c) {
     try {
         std::vector<double> h(n3, 0.0), act(c->nact);
         std::vector<int> ai(c->nact);
-        MOT_CUDA_TRY(cudaMemcpy(ai.data(), c->active, sizeof(int) * c->nact, cudaMemcpyDeviceToHost));
+        MOT_CUDA_TRY(cudaMemcpyAsync(ai.data(), c->active, sizeof(int) * c->nact,
+                                     cudaMemcpyDeviceToHost, c->stream));
+        MOT_CUDA_TRY(cudaStreamSynchronize(c->stream));
         unsigned long long st = 240703323ULL;
         double nrm = 0.0;
         for (long long i = 0; i < c->nact; ++i)
@@ -2092,8 +2096,8 @@ void chebyshev_setup(mot_ctx* c) {
             }
         nrm = std::sqrt(nrm);
         for (double& x : h) x /= nrm;
-        MOT_CUDA_TRY(cudaMemcpy(v1, h.data(), sizeof(double) * n3, cudaMemcpyHostToDevice));
-        MOT_CUDA_TRY(cudaMemset(v0, 0, sizeof(double) * n3));
+        upload(v1, h.data(), n3, c->stream);
+        clear(v0, n3, c->stream);
         CGArgs a{};
         a.M = c->M; a.act = c->active; a.nmask = c->nmask; a.nact = c->nact; a.diag = c->cg_diag;
         for (int e = 0; e < 27; ++e) a.noff[e] = c->noff[e];
