@@ -85,7 +85,7 @@ constexpr int kStepsPerThread = 16;
 // SM): about 13 operations for each active voxel and step.
 __global__ void __launch_bounds__(256) k_plane_wave_tab(
     long long M, int U, int V, const double* __restrict__ chi, double kx, double ky, double kz,
-    double px, double py, double pz, double t0, int n_first, int n_steps, long long j0, int K,
+    double px, double py, double pz, double phase, int n_steps, long long jr, int K,
     const double* __restrict__ A, double* __restrict__ E) {
     const long long m0 = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31);
     const int lane = threadIdx.x & 31;
@@ -96,13 +96,12 @@ __global__ void __launch_bounds__(256) k_plane_wave_tab(
     const double* Ai = A;
     if (ch != 0.0) {
         const int u = (int)(m % U), v = (int)((m / U) % V), w = (int)(m / ((long long)U * V));
-        // position on the node lattice of the step floor(t0), the same for every call; step n
-        // lies (n - floor(t0)) K nodes further (whole numbers: a late pulse loses no digits)
-        const double t0i = floor(t0);
-        const double y = ((t0i - t0) - ((u + 0.5) * kx + (v + 0.5) * ky + (w + 0.5) * kz)) * (double)K;
+        // position on the node lattice, counted from the whole part of the call's first
+        // n - t0, with phase = floor(t0) - t0: the same for every call, and no digits are lost
+        // to a late pulse; step s lies s K nodes further
+        const double y = (phase - ((u + 0.5) * kx + (v + 0.5) * ky + (w + 0.5) * kz)) * (double)K;
         const double fl = floor(y), t = y - fl;
-        Ai = A + ((long long)fl - (kInterp / 2 - 1) +
-                  (n_first + s_lo - (long long)t0i) * K - j0);
+        Ai = A + ((long long)fl - (kInterp / 2 - 1) + s_lo * K - jr);
         // 1 / prod_{i != j} (j - i) = (-1)^(9 - j) C(9, j) / 9!
         constexpr double f9 = 362880.0;
         constexpr double cj[kInterp] = {-1 / f9, 9 / f9, -36 / f9, 84 / f9, -126 / f9,
@@ -211,10 +210,14 @@ void plane_wave(mot_ctx* c, const double k[3], const double p[3], double fc, dou
         rk_hi += std::max(e0, e1);
     }
     // steps per sub-call so that its tau range fits the table with 6 spare nodes a side
-    const double span_rk = rk_hi - rk_lo;
-    const int cap = (int)std::floor((kPwTable - 40) * hstep - span_rk);
-    const int per = std::max(1, std::min(n_steps, cap));
-    if (cap < 1) {      // a grid too large for one table even for one step
+    const double cap = std::floor((kPwTable - 40) * hstep - (rk_hi - rk_lo));
+    // Node numbers are whole numbers near (n - t0 - r . k_hat) K.  Below 2^44 FP64 leaves them
+    // 2^-7 of a node: the kernel's and the host's differ by less than the spare nodes.  Past that
+    // (|t0| of 1e11 steps and more, or a number that is not finite) there is no table.
+    const double t0i = std::floor(t0), phase = t0i - t0;
+    const bool exact = (std::fabs(t0i) + std::fabs((double)n_first) + n_steps +
+                        std::fabs(rk_lo) + std::fabs(rk_hi)) * K < 0x1p44;
+    if (!(cap >= 1.0) || !exact) {   // nor for a grid too large for one table at one step
         const long long tot = c->M * n_steps;
         k_plane_wave<<<(int)((tot + 255) / 256), 256, 0, s>>>(c->M, c->U, c->V, c->chi, k[0], k[1],
                                                               k[2], p[0], p[1], p[2], fc, st, t0,
@@ -222,19 +225,22 @@ void plane_wave(mot_ctx* c, const double k[3], const double p[3], double fc, dou
         MOT_LAUNCH_CHECK();
         return;
     }
+    const int per = (int)std::min((double)n_steps, cap);
     for (int s0 = 0; s0 < n_steps; s0 += per) {
         const int cnt = std::min(per, n_steps - s0);
         const int nf = n_first + s0;
-        const double tlo = (double)nf - t0 - rk_hi, thi = (double)(nf + cnt - 1) - t0 - rk_lo;
-        const long long j0 = (long long)std::floor(tlo * K) - 6;
-        const int J = std::min(kPwTable, (int)((long long)std::ceil(thi * K) + 7 - j0));
+        // the table's nodes relative to (nf - floor(t0)) K, from the same sums as the kernel's
+        const long long jr = (long long)std::floor((phase - rk_hi) * K) - 6;
+        const int J = (int)std::min((long long)kPwTable,
+                                    (long long)std::ceil((phase - rk_lo + (cnt - 1)) * K) + 7 - jr);
+        const long long j0 = (long long)((double)nf - t0i) * K + jr;
         k_pw_table<<<(J + 7) / 8, 256, 0, s>>>(J, j0, (double)K, k[0], k[1], k[2], fc, st,
                                                c->pw_tab);
         MOT_LAUNCH_CHECK();
         const dim3 grid((unsigned)((c->M + 255) / 256),
                         (unsigned)((cnt + kStepsPerThread - 1) / kStepsPerThread));
         k_plane_wave_tab<<<grid, 256, 0, s>>>(
-            c->M, c->U, c->V, c->chi, k[0], k[1], k[2], p[0], p[1], p[2], t0, nf, cnt, j0, K,
+            c->M, c->U, c->V, c->chi, k[0], k[1], k[2], p[0], p[1], p[2], phase, cnt, jr, K,
             c->pw_tab, Edev + (long long)s0 * 3 * c->M);
         MOT_LAUNCH_CHECK();
     }
