@@ -93,8 +93,9 @@ void launch_dependent(bool dep, void (*kern)(P...), dim3 grid, dim3 block, size_
 
 // Dynamic shared memory of a kernel up to the device's opt-in maximum, with the largest
 // carveout (several tiles per SM).  The limit is a process-wide attribute of the kernel; it
-// is set once per kernel and device, to a value that never changes, and the need of a launch
-// is checked against it.  (Set at every launch it was a third of the host time of a step,
+// is set once per kernel and device, to a value that never changes (the device's maximum less
+// the kernel's static arrays: the two together must fit), and the need of a launch is checked
+// against it.  (Set at every launch it was a third of the host time of a step,
 // which bounds several right-hand sides marched side by side.)
 template <auto Kern> void allow_smem(size_t bytes) {
     static std::atomic<int> limit[64];      // per device, 0: not set yet
@@ -103,6 +104,9 @@ template <auto Kern> void allow_smem(size_t bytes) {
     int lim = dev < 64 ? limit[dev].load(std::memory_order_relaxed) : 0;
     if (!lim) {
         MOT_CUDA_TRY(cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+        cudaFuncAttributes fa;
+        MOT_CUDA_TRY(cudaFuncGetAttributes(&fa, Kern));
+        lim -= (int)fa.sharedSizeBytes;
         MOT_CUDA_TRY(cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
         MOT_CUDA_TRY(cudaFuncSetAttribute(Kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
         if (dev < 64) limit[dev].store(lim, std::memory_order_relaxed);

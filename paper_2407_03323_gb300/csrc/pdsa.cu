@@ -281,8 +281,9 @@ __global__ void k_sub_combo(double* __restrict__ w, const double* __restrict__ V
                             double* __restrict__ coef, double* __restrict__ part) {
     pdl_trigger();
     pdl_wait();
+    // the nvec coefficients, later the warps' sums: all of the shared memory is dynamic, so that
+    // k may grow to the opt-in maximum
     extern __shared__ double sh[];
-    __shared__ double sm[NT / 32];
     for (int j = threadIdx.x; j < nvec; j += blockDim.x) sh[j] = h[j];
     __syncthreads();
     if (blockIdx.x == 0 && threadIdx.x == 0) *coef = sh[nvec - 1];
@@ -296,11 +297,12 @@ __global__ void k_sub_combo(double* __restrict__ w, const double* __restrict__ V
     }
     if (!part) return;
     acc = warp_sum(acc);
-    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
     __syncthreads();
     if (threadIdx.x == 0) {      // (in the order of k_dots: the same bits as its w . w)
         acc = 0.0;
-        for (int k = 0; k < NT / 32; ++k) acc += sm[k];
+        for (int k = 0; k < NT / 32; ++k) acc += sh[k];
         part[blockIdx.x] = acc;
     }
 }
@@ -688,7 +690,7 @@ mot_status mot_pdsa_lanczos(mot_ctx* c, int n, int flags, int k, unsigned long l
             double* h = sc.get<double>(k + 2);
             double* part = sc.get<double>((long long)(k + 2) * nb);
             double* coef = sc.get<double>(3LL * (k + 1));   // per step: two coefficients, ||w||^2
-            const size_t shm = sizeof(double) * (k + 1);
+            const size_t shm = sizeof(double) * std::max(k + 1, NT / 32);
             if (shm > 48 * 1024) {   // raise to the opt-in maximum (process-wide attribute)
                 int dev = 0, optin = 0;
                 MOT_CUDA_TRY(cudaGetDevice(&dev));
