@@ -803,12 +803,21 @@ int plane_threads(const mot_ctx* c) {
     return std::min(kPlaneThreads, std::max(64, (want + 31) / 32 * 32));
 }
 
+// Every length needs a codelet or a tile of the general kernel (P <= 764 in FP64, 807 in FP32),
+// also where another kernel takes the axis: which one does depends on the grid and the step, so a
+// longer axis would fail in the middle of a march, and with it the z pass of only some steps.
+template <typename R> void fft_require(const mot_ctx* c) {
+    for (const AxisFFT& ax : c->ax)
+        if (!has_codelet(ax.P)) allow_smem<k_mid<R>>(smem_bytes<R>(ax.P));
+}
+
 // kernels of the x and y passes of a transform
 template <typename R> int fft_xy_launches(const mot_ctx* c) { return plane_pass<R>(c) ? 1 : 2; }
 
 // x and y passes of the forward transform, [3][W][V][U] -> hb.tmp2 [3][W][Pv][Hu]
 template <typename R>
 void fft_forward_xy(mot_ctx* c, const double* Jsoa, cudaStream_t s, const double* scale) {
+    fft_require<R>(c);
     HistoryBuffers<R>& hb = hbuf<R>(c);
     constexpr int TB = Tile<R>::TB;
     const int U = c->U, V = c->V, W = c->W;
@@ -901,6 +910,8 @@ void fft_inverse(mot_ctx* c, const typename CT<R>::c* in, R* out, cudaStream_t s
     fft_inverse_yx<R>(c, out, s);
 }
 
+template void fft_require<double>(const mot_ctx*);
+template void fft_require<float>(const mot_ctx*);
 template int fft_xy_launches<double>(const mot_ctx*);
 template int fft_xy_launches<float>(const mot_ctx*);
 template void fft_forward_xy<double>(mot_ctx*, const double*, cudaStream_t, const double*);

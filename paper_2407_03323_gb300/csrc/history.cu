@@ -1207,6 +1207,7 @@ void history_step(mot_ctx* c, int n, cudaStream_t s, cudaEvent_t* ev) {
     const bool fused = fused_z<R>(c);
     bool fires = false;
     for (int k = 0; blocked && k < c->nlev; ++k) fires = fires || (n - 1) % c->lev_S[k] == 0;
+    if (n == 1) fft_require<R>(c);      // no forward transform, which would check it
     if (n >= 2) {
         const double* Jprev = c->J + slot_index(n - 1, c->jring) * 3 * c->M;
         fft_forward_xy<R>(c, Jprev, s, c->adjoint ? c->chi : nullptr);

@@ -321,6 +321,7 @@ template <typename R>
 void fft_inverse(mot_ctx* c, const typename CT<R>::c* in, R* out, cudaStream_t s);
 template <typename R>
 void fft_forward_xy(mot_ctx* c, const double* Jsoa, cudaStream_t s, const double* scale);
+template <typename R> void fft_require(const mot_ctx* c);     // throws for a length no tile takes
 template <typename R> int fft_xy_launches(const mot_ctx* c);   // kernels of the x and y passes
 template <typename R> void fft_forward_z(mot_ctx* c, typename CT<R>::c* out, cudaStream_t s);
 template <typename R> void fft_inverse_yx(mot_ctx* c, R* out, cudaStream_t s);

@@ -44,3 +44,33 @@ def test_level_of_256_lags(mot, precision, tol):
             c.set_excitation(E)
             out.append(c.march(n))
     assert np.linalg.norm(out[1] - out[0]) <= tol * np.linalg.norm(out[0])
+
+
+# longest lengths that the general FFT tile takes (756 in FP64, 800 in FP32) and the next ones
+@pytest.mark.parametrize("axis", [0, 1, 2])
+@pytest.mark.parametrize("precision,side,ok", [("fp64", 378, True), ("fp64", 383, False),
+                                               ("fp32_history", 400, True),
+                                               ("fp32_history", 404, False)])
+def test_longest_transforms(mot, precision, side, ok, axis):
+    """A length without a tile is refused at the first step of a march, on any axis and whichever
+    kernels the other steps would take; the longest one marches (against a longer padding of the
+    short axes, 1e-12 / 1e-5)."""
+    grid = [2, 2, 2]
+    grid[axis] = side
+    eps = 2.0 + np.random.default_rng(2).random(grid)
+    E = np.random.default_rng(3).normal(size=(5, eps.size, 3))
+
+    def march(**kw):
+        with mot.Context(eps, wl.fir_taps("fir3", 1e-3), precision=precision, **kw) as c:
+            c.set_excitation(E)
+            return c.march(5), tuple(c.P)
+
+    for kw in (dict(scheme="direct"), dict(scheme="blocked", block=8)):
+        if not ok:
+            with pytest.raises(mot.MotError, match="MOT_ERR_ARG"):
+                march(**kw)
+            continue
+        J, P = march(**kw)
+        other, _ = march(fft_len=tuple(2 * p if p < 8 else p for p in P), **kw)
+        tol = 1e-12 if precision == "fp64" else 1e-5
+        assert np.linalg.norm(J - other) <= tol * np.linalg.norm(J)
