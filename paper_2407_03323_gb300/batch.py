@@ -37,9 +37,9 @@ from .mot import Context, codelet_size, pad_size
 
 
 def _state_bytes(N, precision, block, P=None):
-    """Device bytes of one excitation's march state on an N^3 grid with FFT length P
-    (default: the library's padding) (spectral ring and far-level accumulators
-    dominate; the accumulators counted for the doubling level plan, an upper bound)."""
+    """Device bytes of one excitation's rings on an N^3 grid with FFT length P (default: the
+    library's padding): spectral ring and far-level accumulators, the accumulators counted for
+    the doubling level plan, an upper bound; with 200 bytes a voxel beside them."""
     P = P or pad_size(N)
     c = 8 if precision == "fp32_history" else 16
     slot = 3 * P * P * (P // 2 + 1) * c
@@ -49,6 +49,20 @@ def _state_bytes(N, precision, block, P=None):
         acc += S
         S *= 2
     return slot * (ell + acc) + 200 * N ** 3
+
+
+def march_bytes(N, precision, block, P=None, n_taps=3):
+    """Device bytes of one excitation's whole march state: _state_bytes with what it leaves out,
+    the product's spectrum, the transforms' intermediates and the rest of the solve's state.  Per
+    voxel that is the J ring (24 a slot), the six fitted right-hand sides and the current one
+    (168), rhs and lambda (48), the inner vectors (64) and the history (24, or 12 with 28 for the
+    low parts of b and x)."""
+    P = P or pad_size(N)
+    f32 = precision == "fp32_history"
+    c, Hu = 8 if f32 else 16, P // 2 + 1
+    voxel = 24 * (max(n_taps, 6) + 1) + 168 + 48 + 64 + (40 if f32 else 24)
+    planes = 3 * P * P * Hu * c + 3 * N * (N + P) * Hu * c
+    return _state_bytes(N, precision, block, P) + planes + (voxel - 200) * N ** 3 + (1 << 20)
 
 
 def fft_lengths(N, strategy):
@@ -165,8 +179,9 @@ def run_batched(instances, n_steps, precision="fp32_history", tuner=None, chunk=
     order = sorted(range(len(instances)), key=lambda i: -instances[i]["N"])
     waves, cur, used = [], [], 0.0
     for i in order:
-        need = len(instances[i]["waves"]) * _state_bytes(instances[i]["N"], precision, blocks[i],
-                                                          tuner.fft_len(instances[i]["N"])[0])
+        need = len(instances[i]["waves"]) * march_bytes(instances[i]["N"], precision, blocks[i],
+                                                         tuner.fft_len(instances[i]["N"])[0],
+                                                         len(instances[i]["taps"]))
         if cur and used + need > memory_budget:
             waves.append(cur)
             cur, used = [], 0.0
