@@ -1519,8 +1519,16 @@ __device__ __forceinline__ void residual64(const CGArgs& a, int e, bool first, b
 // square root, logarithm and division for every warp cost 4 to 7 us of a 45 us solve).  Sums
 // that leave FP32's range at the scale of the step before (wide) are formed again in FP64,
 // which gives the new scale.
+// kDrift: the carried residual was at most 2.9e-7 of the start residual away from that of
+// x + e in 32,000 refinements of 3 to 64 iterations (cubes, cores, films and noise, eps_r 1.001
+// to 1000, spectral intervals 3 to 10,000 wide, rough and smooth residuals): the width comes from
+// the diagonal, which scales a voxel's error with its own residual, not from G_0.
 constexpr float kDrift = 1e-6f;
 constexpr float kFloor = 1e-6f;
+// A refinement aims at a tenth of the tolerance but may fall short of it by kFloor; what it then
+// leaves just below the tolerance (half of the FP64 steps of a field that the fit follows to 1e-7)
+// would be 5 times the usual error.  One more refinement of three iterations or so follows.
+constexpr float kNear = 0.2f;
 // sequence numbers that a residual and two iterations whose results are dropped may have used
 constexpr unsigned kAborted = 4;
 
@@ -1614,6 +1622,7 @@ k_cg(const __grid_constant__ CGArgs a, const __grid_constant__ EpiArgs ep) {
     bool first = true, wide = false, converged = false, nonfinite = false, zero = false;
     bool stored = false;     // x is in a.x; else DF's start is in xb only
     bool own = true;         // sd[0] holds the tile's start
+    bool polished = false;   // a residual that met the tolerance is being refined (kNear)
     // f(voxel, its correction e) over the block's share of the active voxels
     auto each = [&](auto&& f) {
         if constexpr (RES) {
@@ -1686,7 +1695,14 @@ k_cg(const __grid_constant__ CGArgs a, const __grid_constant__ EpiArgs ep) {
                          (!first && have > goal && rr < 1e-30f);
         const bool odd = off && ++wides <= 3;      // (the FP64 sums settle it the first time)
         if (!odd && !(rr <= 1e30f)) { nonfinite = true; break; }
-        if (!odd && have <= goal) { converged = true; break; }
+        if (!odd && have <= goal) {
+            // a residual formed anew that lies near the tolerance is refined once more
+            if (polished || have <= kNear * goal || outer >= a.max_outer || its >= a.max_iter) {
+                converged = true;
+                break;
+            }
+            polished = true;
+        }
         if (odd || (first && rr > bb)) {
             if (!odd) {
                 // a start worse than none (an abrupt change of the excitation): from zero
@@ -1709,11 +1725,13 @@ k_cg(const __grid_constant__ CGArgs a, const __grid_constant__ EpiArgs ep) {
         first = false;
         if (outer >= a.max_outer || its >= a.max_iter) break;
         // ---- Chebyshev: iterations for the reduction still needed, never asking for more
-        // than FP32 can deliver in one refinement (kFloor).  FP64 aims a factor 10 below the
-        // tolerance (the march's error is then the history's rounding, 1e-14 on the 8^3
-        // cube, not the solve's 2e-13); the FP32 history's own error is far above its
-        // tolerance already
-        const float need = fmaxf((DF ? 0.8f : 0.1f) * (goal - kDrift * have) / have, kFloor);
+        // than FP32 can deliver in one refinement (kFloor), and below the tolerance: what a step
+        // leaves adds up along smooth modes.  FP64 at a hundredth instead of a tenth: 7 x 8 x 9
+        // cube, eps_r 30, 1.1e-13 -> 3.3e-14 from the exact march, 9^3 sphere 4.7e-14 -> 1.8e-14, 8^3
+        // cube 2.0e-14 -> 6.5e-15, for two iterations of 30.  FP32-history at a tenth instead of 0.8: 24^3
+        // cube 9.6e-7 -> 9.1e-7 from FP64, 66 x 27 x 21 noise 1.35e-6 -> 1.29e-6, the errors of
+        // 10 and 100 times smaller tolerances, for two iterations of 15
+        const float need = fmaxf((DF ? 0.1f : 0.01f) * (goal - kDrift * have) / have, kFloor);
         const int n_it = min(a.n_cheb, max(3, (int)ceilf(log2f(0.5f * need) * a.inv_log2_rate)));
         if constexpr (RES) {
             if constexpr (!DF) {
