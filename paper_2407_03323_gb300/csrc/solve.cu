@@ -76,7 +76,17 @@ struct FitRecord {
 struct FitState {      // device, zeroed with the march state
     FitRecord rec[2];                  // step n reads rec[n & 1]; its solve writes the other
     double gram[kSlots * kSlots];      // <b_i, b_j> by ring slot
+    // the scale that a solve had to find by FP64 sums (an excitation beyond FP32's range at the
+    // scale before it: 1e19 times larger or 1e-23), kWide + e, for the step after it; else 0.  The
+    // epilogue's own sums overflowed, so that the record alone would never find it, and every step
+    // of such a march would start from the extrapolation and form its sums twice
+    int wide[2];
 };
+constexpr int kWide = 1 << 16;
+__device__ __forceinline__ int scale_of(const FitState& f, int step) {
+    const int w = f.wide[step & 1];
+    return w ? w - kWide : f.rec[step & 1].e;
+}
 static_assert(sizeof(FitState) <= sizeof(double) * mot::kFitWords, "fit state size");
 
 // 2^e, |e| <= 1000 (double) / 120 (float)
@@ -140,7 +150,7 @@ template <typename R> struct EpiFit {
     __device__ EpiFit(const EpiArgs& a) {
         const FitRecord& rec = a.fit->rec[a.n & 1];
         use = rec.use != 0;
-        scf = std::is_same<R, float>::value ? pow2f(rec.e) : 1.f;
+        scf = std::is_same<R, float>::value ? pow2f(scale_of(*a.fit, a.n)) : 1.f;
 #pragma unroll
         for (int i = 0; i < kFit; ++i)
             if constexpr (std::is_same<R, float>::value) c[i] = use ? rec.cf[i] : extrapolation(i);
@@ -1033,7 +1043,9 @@ __device__ __forceinline__ bool cheb_pass_resident(const CGArgs& a, int k, unsig
     return true;
 }
 
-// Partial sums of a thread: |r|^2 and |b|^2 scaled by 4^e in FP32, or (wide) unscaled in FP64
+// Partial sums of a thread: |r|^2 and |b|^2 scaled by 4^e in FP32, or (wide) unscaled in FP64.
+// They only steer the iteration; in FP32 they are at most 40 roundings, 1.2e-6 of a norm, off
+// (thread, warp, block and grid sums in turn), less than the allowance kDrift and kNear make.
 struct Sums {
     float rr, bb;
     double rrw, bbw;
@@ -1346,7 +1358,7 @@ template <bool DF, bool RES> __device__ void fit_block(const CGArgs& a) {
         }
         for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
         // FP32-history sums are scaled by 4^e of this step
-        const double un = DF ? pow2d(-2 * a.fit->rec[a.step & 1].e) : 1.0;
+        const double un = DF ? pow2d(-2 * scale_of(*a.fit, a.step)) : 1.0;
         if (lane == 0) t[q] = v * un;
     }
     __syncthreads();
@@ -1617,11 +1629,12 @@ k_cg(const __grid_constant__ CGArgs a, const __grid_constant__ EpiArgs ep) {
     }
     float bb = 0.f, rr = 0.f;            // scaled by 4^e0 and 4^e
     double xx = 0.0;                     // |x|^2 of the block's share, once x is stored
-    int e = a.fit->rec[a.step & 1].e, e0 = e;
+    int e = scale_of(*a.fit, a.step), e0 = e;
     int its = 0, outer = 0, wides = 0;
     bool first = true, wide = false, converged = false, nonfinite = false, zero = false;
     bool stored = false;     // x is in a.x; else DF's start is in xb only
     bool own = true;         // sd[0] holds the tile's start
+    bool rescaled = false;   // e0 comes from FP64 sums
     bool polished = false;   // a residual that met the tolerance is being refined (kNear)
     // f(voxel, its correction e) over the block's share of the active voxels
     auto each = [&](auto&& f) {
@@ -1662,7 +1675,10 @@ k_cg(const __grid_constant__ CGArgs a, const __grid_constant__ EpiArgs ep) {
             int ex = 0;
             frexp(sqrt(first ? bw : rw), &ex);
             e = max(-(DF ? 120 : 500), min(DF ? 120 : 500, -ex));
-            if (first) e0 = e;
+            if (first) {
+                e0 = e;
+                rescaled = true;
+            }
             wide = false;
             seq += kAborted;
             if (!gsync()) return;
@@ -1828,6 +1844,7 @@ k_cg(const __grid_constant__ CGArgs a, const __grid_constant__ EpiArgs ep) {
     for (int w = 1; w < T::NTH / 32; ++w) xx += shx[w];
     a.nrm[blockIdx.x] = xx;
     if (blockIdx.x == 0) {
+        a.fit->wide[(a.step + 1) & 1] = rescaled ? kWide + e0 : 0;
         a.status[0] = its;
         a.status[3] += its;
         const int flag = nonfinite ? 2 : converged ? 0 : 1;

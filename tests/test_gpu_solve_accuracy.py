@@ -83,3 +83,30 @@ def test_residuals(mot, eps_r, kind, precision):
             got.append(np.linalg.norm(r) / np.linalg.norm(b) / tol)
     assert max(got) <= 1.01
     assert np.median(got) <= 0.2
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32_history"])
+@pytest.mark.parametrize("grid", [(9, 10, 12), (60, 58, 61)])
+@pytest.mark.parametrize("power", [83, -83])
+def test_units_of_the_excitation(mot, power, grid, precision):
+    """An excitation scaled by 2^83 or 2^-83 (1e25, 1e-25: beyond FP32's squares) marches with the
+    iterations of the unscaled one, and in FP64 to its currents (1e-12).  The first 16 steps may
+    differ (a fit without the first right-hand sides); the next 32 take the same iterations to 5 %."""
+    eps = np.full(grid, 6.0)
+    w = wl.pulse(max(grid), 6.0)
+    n = 48
+    got = []
+    for scale in (1.0, 2.0 ** power):
+        with mot.Context(eps, wl.fir_taps("fir3", 1e-3), precision=precision, scheme="blocked",
+                         block=4) as c:
+            E = scale * np.asarray(c.plane_wave(w["k_hat"], w["p_hat"], w["f_c"], w["sigma_t"],
+                                                w["t0"] - 60, 1, n))
+            c.set_excitation(E)
+            first = c.march(16)
+            before = c.stats()["cg_iters"]
+            J = np.concatenate([first, c.march(n - 16)])
+            got.append((J / scale, c.stats()["cg_iters"] - before))
+    (J0, its0), (J1, its1) = got
+    assert abs(its1 - its0) <= 0.05 * its0
+    if precision == "fp64":
+        assert np.linalg.norm(J1 - J0) <= 1e-12 * np.linalg.norm(J0)
