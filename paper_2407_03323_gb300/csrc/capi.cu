@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <deque>
 #include <new>
 
 namespace {
@@ -781,6 +782,8 @@ mot_status mot_march(mot_ctx* c, int n_steps, double* J_out, void* stream) {
     if (n_steps < 1) { c->err = "n_steps must be >= 1"; return MOT_ERR_ARG; }
     MarchRun run{c, n_steps, J_out, stream ? (cudaStream_t)stream : c->stream};
     mot_status st = guarded(c, [&] {
+        // a graph of a period is updated in place only while its launches stay of one kind
+        const mot::MarchScope scope(c, c->graph_steps > 0 ? !c->shared_src && !c->n_shared : -1);
         run.begin();
         run.launch_all();
         run.fetch();
@@ -938,6 +941,7 @@ mot_status mot_adjoint_run(mot_ctx* c, int n_count, const double* J_win, int win
             c->norms_cap = n_count;
         }
         c->norm_pending = nullptr;
+        const mot::MarchScope scope(c);
         for (int i = 0; i < n_count; ++i) {
             const int tau = c->adj_done + 1 + i;
             const int n = c->adj_total + 1 - tau;
@@ -1198,7 +1202,9 @@ mot_status mot_march_rhs(mot_ctx* c, int n_steps, double* J_out, void* stream) {
                                 stream ? (cudaStream_t)stream : all[k]->stream});
     // the steps of all right-hand sides interleaved, each on its own stream
     mot_status st = guarded(c, [&] {
+        std::deque<mot::MarchScope> scopes;
         for (MarchRun& r : runs) {
+            scopes.emplace_back(r.c, runs.size() > 1 ? 0 : -1);
             r.graphs_allowed = false;
             r.begin();
         }

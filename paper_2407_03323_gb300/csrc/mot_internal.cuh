@@ -68,10 +68,10 @@ template <typename S> void upload_symbol(const S& sym, const void* src, size_t b
 // finished and its writes are visible) instead of being launched only then.  Each of them
 // waits before it touches anything that another kernel writes, and allows its own dependent
 // at once (pdl_trigger).  Before pdl_wait a kernel may read setup constants only.
-// `dep` false: an ordinary launch.  Contexts that march side by side on their own streams
-// (several right-hand sides, borrowers of one setup: dependent_launches) use it, because
-// blocks that wait hold SM resources another stream could use: 9^3 alone 11.4 -> 9.8 ms a
-// pass, 32^3 FP32-history 23.4 -> 21.9, but eight right-hand sides of 24^3 17.4 -> 18.6.
+// `dep` false: an ordinary launch.  Marches that run side by side on their own streams use it
+// (dependent_launches), because blocks that wait hold SM resources another stream could use: 9^3
+// alone 11.4 -> 9.8 ms a pass, 32^3 FP32-history 23.4 -> 21.9, but eight right-hand sides of 24^3
+// 17.4 -> 18.6.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
 
@@ -281,6 +281,8 @@ struct mot_ctx {
     // shared_src, which must outlive this context; n_shared counts the borrowers
     mot_ctx* shared_src = nullptr;
     int n_shared = 0;
+    std::atomic<int> marching{0};   // of the setup's owner: marches of the setup under way
+    int dep_fixed = -1;          // dependent launches of this call: 0 no, 1 yes, -1 as marching says
     int nsm = 0;
     int cg_blocks = 0;
     bool broken = false;
@@ -294,7 +296,26 @@ template <> inline HistoryBuffers<float>& hbuf<float>(mot_ctx* c) { return c->h3
 // ------------------------------------------------------------------ internals
 namespace mot {
 
-inline bool dependent_launches(const mot_ctx* c) { return !c->shared_src && c->rhs_ctx.empty(); }
+// Whether a launch of this context is a programmatic dependent: not while another march of the
+// same setup is under way, nor in a call that marches several right-hand sides.
+inline bool dependent_launches(const mot_ctx* c) {
+    if (c->dep_fixed >= 0) return c->dep_fixed != 0;
+    return (c->shared_src ? c->shared_src : c)->marching.load(std::memory_order_relaxed) <= 1;
+}
+// A march call of c, counted with its setup.  fixed: see dep_fixed.
+struct MarchScope {
+    mot_ctx* c;
+    MarchScope(mot_ctx* ctx, int fixed = -1) : c(ctx) {
+        c->dep_fixed = fixed;
+        (c->shared_src ? c->shared_src : c)->marching.fetch_add(1, std::memory_order_relaxed);
+    }
+    ~MarchScope() {
+        (c->shared_src ? c->shared_src : c)->marching.fetch_sub(1, std::memory_order_relaxed);
+        c->dep_fixed = -1;
+    }
+    MarchScope(const MarchScope&) = delete;
+    MarchScope& operator=(const MarchScope&) = delete;
+};
 
 constexpr int WIN = 8;  // lag window per octant offset of the interaction table
 constexpr int kPwTable = 1 << 16;   // nodes of the plane-wave table of one call
