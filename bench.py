@@ -350,7 +350,9 @@ def run_variant(args, cfg, prec, scheme, block, dev, world, steps, warmup, want_
     mac_b = mac_bytes_per_launch(ctx, prec, mac_lags,
                                  len(ctx.levels) if scheme.startswith("blocked") else 0)
     mac_ms = st["ms_mac"] / max(st["mac_launches"], 1)
-    cands = [("k_mac", mac_b, mac_ms, st["ms_mac"])]
+    # (FP64 takes the lag products together with both z passes)
+    mac = "k_zmac" if prec == "fp64" else "k_mac"
+    cands = [(mac, mac_b, mac_ms, st["ms_mac"])]
     if scheme.startswith("blocked") and st["far_launches"]:
         fb, fl = far_bytes_per_period(ctx, prec)
         periods = st["far_launches"] / max(fl, 1)

@@ -8,7 +8,7 @@
  *
  * on a uniform voxel grid, with the history P evaluated by zero-padded 3D FFTs
  * (Sec. 3, Eq. PnFFTMOT, App. A), the FIR regularisation Z_n + delta_n I (Sec. 6.1)
- * and a conjugate-gradient solve of the near-field operator Z_0 each step.
+ * and an iterative solve of the near-field operator Z_0 each step.
  *
  * Conventions for every call:
  *  - Units: c0 = 1, eps0 = 1.  Voxels are cubes of edge h with c0 dt = h (the
@@ -41,7 +41,7 @@ typedef enum {
     MOT_ERR_ARG = 1,            /* invalid argument (message says which)            */
     MOT_ERR_OOM = 2,            /* device allocation failed                         */
     MOT_ERR_CUDA = 3,           /* CUDA runtime error                               */
-    MOT_ERR_NOT_CONVERGED = 4,  /* CG did not reach its tolerance within max_iter    */
+    MOT_ERR_NOT_CONVERGED = 4,  /* the solve missed its tolerance within max_iter    */
     MOT_ERR_UNSTABLE = 5,       /* NaN/Inf or runaway growth of ||J_n|| (Sec. 5.2)   */
     MOT_ERR_TIMEOUT = 6,        /* a device-side wait ran out of its budget          */
     MOT_ERR_STATE = 7           /* context unusable (earlier device fault)           */
@@ -51,7 +51,7 @@ typedef enum {
     MOT_FP64 = 0,          /* every stage in FP64                                    */
     MOT_FP32_HISTORY = 1   /* FFTs, spectra and lag MAC in FP32 with compensated
                               accumulation; element quadrature, Z_0, FIR state and
-                              the solution J stay FP64; the CG residual is formed in
+                              the solution J stay FP64; the solve's residual is in
                               double-float (float pairs, ~48 bits)                  */
 } mot_precision;
 
@@ -190,7 +190,7 @@ mot_status mot_plane_wave_static(mot_ctx* ctx, const double k_hat[3], const doub
  *            run on a copy stream while the next steps compute, and is complete when
  *            the call returns
  *  stream    cudaStream_t or NULL
- * Errors: MOT_ERR_NOT_CONVERGED (CG exceeded max_iter; J of that step is the last
+ * Errors: MOT_ERR_NOT_CONVERGED (solve exceeded max_iter; J of that step is the last
  * iterate), MOT_ERR_UNSTABLE (NaN/Inf or ||J_n|| above the growth limit; see
  * mot_get_info for the step), MOT_ERR_CUDA.
  */
@@ -398,7 +398,7 @@ mot_status mot_frequency_response(int n_steps, int n_probe, const double* J, dou
  *  n_done               steps marched so far
  *  last_norm            ||J_{n_done}||_2
  *  fail_step            step index of the first UNSTABLE/NOT_CONVERGED event, or 0
- *  last_cg_iters        CG iterations of the last step                             */
+ *  last_cg_iters        solve iterations of the last step                          */
 mot_status mot_get_info(const mot_ctx* ctx, int* ell, int P[3], int* n_done,
                         double* last_norm, int* fail_step, int* last_cg_iters);
 
@@ -443,7 +443,7 @@ mot_status mot_set_solver(mot_ctx* ctx, double tol, int max_iter, double growth_
  *  launches      kernels launched by mot_march
  *  mac_launches  of which lag multiply-accumulate kernels
  *  steps         time steps marched
- *  cg_iters      total CG iterations
+ *  cg_iters      total iterations of the solves
  *  far_launches  of which block Toeplitz (temporal FFT) kernels, blocked scheme
  *  ms_*          summed CUDA-event durations of the phases, recorded on the stream
  *                mot_march ran on, only while profiling is enabled: forward FFT of
@@ -564,7 +564,7 @@ mot_status mot_fma_peak(int fp64, int iters, float* ms, double* flops);
 
 /*
  * mot_barrier_check - exercise the bounded wait of the grid barrier that the solve
- * kernel (the CG of Eq. MOTInversion) uses between its passes (no counterpart in the
+ * kernel (Eq. MOTInversion) uses between its passes (no counterpart in the
  * paper: a failure guard).  One cooperative launch of n_blocks blocks on the current
  * device passes `rounds` barriers; block `absent` (0 <= absent < n_blocks; -1: none)
  * returns without arriving, so the other blocks' wait runs out after budget_s seconds

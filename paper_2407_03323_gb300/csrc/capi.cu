@@ -2,7 +2,7 @@
 // loop (Eqs. MOTInversion, PnMOT).  Per step n:
 //   1. forward FFT of J_{n-1} into the spectral ring        (Sec. 3)
 //   2. lag MAC over the ring, inverse FFT -> (G * J)_hist    (Eq. PnFFTMOT)
-//   3. FIR epilogue -> rhs, CG solve of Z_0 J_n = rhs        (Eq. MOTInversion, Sec. 6.1)
+//   3. FIR epilogue -> rhs, solve of Z_0 J_n = rhs           (Eq. MOTInversion, Sec. 6.1)
 //   4. ||J_n|| monitor, optional AoS write-out
 #include "mot_internal.cuh"
 

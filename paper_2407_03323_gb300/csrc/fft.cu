@@ -788,7 +788,10 @@ bool x_pass_codelet(bool fwd, mot_ctx* c, const double* Jsoa, typename CT<R>::c*
 // A whole step: FP32 8^3 56.9 -> 50.8, 24^3 85.1 -> 78.8, 44^3 244 -> 239; FP64 8^3 85.6 ->
 // 79.4, 16^3 132 -> 123; but 20^3 0.5 us slower, and 16 x 16 x 64 (192 planes, two on some
 // SMs) 326 -> 340; with planes enough to even that out 4 x 100 x 100 (300) 1003 -> 956, 21 x
-// 27 x 133 (399) 1483 -> 1452.
+// 27 x 133 (399) 1483 -> 1452.  Between 152 and 300 planes the line is cautious, forward +
+// inverse of FP64 grids U x V x W, two kernels -> plane kernels: 27 x 21 153 planes 69.6 -> 80.9,
+// 210 81.0 -> 83.3, 228 104 -> 83.2, 294 115 -> 84.9; 20 x 20 153 51.3 -> 53.0, 240 65.3 -> 58.0, 294
+// 84.5 -> 60.3; 16 x 16 153 42.7 -> 37.2, 294 57.1 -> 44.6.
 template <typename R> size_t plane_pass(const mot_ctx* c) {
     typedef typename CT<R>::c C;
     const int Pu = c->ax[0].P, Pv = c->ax[1].P;

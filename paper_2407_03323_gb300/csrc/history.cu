@@ -26,6 +26,7 @@
 // computed currents); levels double in length so a step costs O(log ell) block work on
 // average, the temporal counterpart of Eq. ComplexityHierarchicalDivisionInTime.
 #include "mot_internal.cuh"
+#include "accumulate.cuh"
 #include "fft_core.cuh"
 
 #include <algorithm>
@@ -35,23 +36,6 @@ using namespace mot_fft;
 namespace {
 
 constexpr int NT = 256;
-
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-    s = a + b;
-    const float bp = s - a;
-    const float ap = s - bp;
-    e = (a - ap) + (b - bp);
-}
-struct Acc {
-    float2 s, c;
-    __device__ void zero() { s = make_float2(0.f, 0.f); c = make_float2(0.f, 0.f); }
-    __device__ void add(float2 v) {
-        float e;
-        two_sum(s.x, v.x, s.x, e); c.x += e;
-        two_sum(s.y, v.y, s.y, e); c.y += e;
-    }
-    __device__ float2 get() const { return make_float2(s.x + c.x, s.y + c.y); }
-};
 
 struct MacGeom {
     int Hu, Hv, Hw, Pv, Pw;
@@ -100,7 +84,7 @@ __global__ void __launch_bounds__(NT) k_mac(const float* __restrict__ ghat,
     const R sxy = fv ? (R)-1 : (R)1;
     const R sxz = fw ? (R)-1 : (R)1;
     const R syz = (fv != fw) ? (R)-1 : (R)1;
-    Acc ax, ay, az;
+    Acc<float> ax, ay, az;
     ax.zero(); ay.zero(); az.zero();
     for (int k = 0; k < far.n; ++k) {   // far-lag contributions of this step
         const C* f = far.p[k];
@@ -424,7 +408,7 @@ template <> const float2* twtab<float>(const AxisFFT& a) { return a.tw32; }
 
 // ---------------------------------------------------------------- register variant
 // For 2S <= 64: one thread per (bin, component) line.  A block is three warps (warp =
-// component) over 32 consecutive bins of one rfft row.  Each thread loads its 2S window
+// component) over 32 consecutive octant bins.  Each thread loads its 2S window
 // samples (coalesced across the warp), runs an unrolled radix-2 DIF FFT in registers
 // (output in bit-reversed order), the three spectra are exchanged through shared memory
 // for the 3x3 product (frequency of slot i is bitrev(i)), and an unrolled radix-2 DIT
@@ -632,7 +616,8 @@ template <typename R, int Q, int T> struct FarRegSmem {
 };
 
 // One level firing at step n0: y(n0 + j), j < S, written to the level's accumulator
-// ring.  Block = three warps (warp = component) over 32 / T bins of one rfft row.
+// ring.  Block = three warps (warp = component) over 32 / T consecutive octant bins, which run
+// across rfft rows (a lane's rfft row comes from mirror_bin; o0 + l < noct bounds the last block).
 // The block's kernel spectra are copied to shared memory asynchronously while the
 // window is loaded and transformed.  Mirror signs: the off-diagonal spectra of the
 // mirrored rows flip as s_ab = sigma_a sigma_b (sigma_x = 1, sigma_y = -1 if v is
@@ -727,7 +712,7 @@ void far_launch_reg(mot_ctx* c, FarArgs<R>& a, cudaStream_t s) {
 }
 
 // ---------------------------------------------------------------- four-step variant
-// Levels with 2S = P > 32 (FP32) / 16 (FP64): the temporal transform of length
+// FP64 levels with 2S = P = 32, 64 and 128: the temporal transform of length
 // P = T Q1 is split as n = t + T n2, k = k2 + Q1 k1 (Bailey's four-step form):
 //   X[k2 + Q1 k1] = sum_t W_T^{t k1} W_P^{t k2} sum_{n2} x[t + T n2] W_Q1^{n2 k2}.
 // Phase A: a thread per (component, bin, t) loads its time-strided subsequence and
@@ -740,11 +725,11 @@ void far_launch_reg(mot_ctx* c, FarArgs<R>& a, cudaStream_t s) {
 // Phase C: the thread of phase A runs the inverse Q1-point transform and stores its
 //   outputs in the second half of the window (times n0 .. n0 + S - 1).
 // A block is 256 threads: phases A and C use 3 NB T = 192 of them, phase B all.
-template <typename R, int P> struct Far4 {
-    typedef typename CT<R>::c C;
-    static constexpr int Q1 = sizeof(R) == 4 ? 32 : 16;
+template <int P> struct Far4 {
+    typedef double2 C;
+    static constexpr int Q1 = 16;
     static constexpr int T = P / Q1;
-    static constexpr int NB = (sizeof(R) == 4 ? 2048 : 1024) / P;
+    static constexpr int NB = 1024 / P;
     static constexpr int S = P / 2;
     static constexpr int NA = 3 * NB * T;
     static constexpr int NI = NB * Q1;
@@ -763,10 +748,8 @@ template <typename R, int P> struct Far4 {
     __device__ static int col(int k2, int a) { return k2 ^ (a & (Q1 - 1)); }
 };
 
-template <typename R, int P>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k_far_4s(FarArgs<R> a) {
-    static_assert(std::is_same<R, double>::value, "FP32 far levels run k_far_fs");
-    typedef Far4<R, P> F;
+template <int P> __global__ void __launch_bounds__(256, 1) k_far_4s(FarArgs<double> a) {
+    typedef Far4<P> F;
     typedef typename F::C C;
     constexpr int Q1 = F::Q1, T = F::T, NB = F::NB, S = F::S;
     pdl_trigger();
@@ -881,13 +864,12 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k_far_4s(FarArgs<
     });
 }
 
-template <typename R, int P>
-void far_launch_4s(mot_ctx* c, FarArgs<R>& a, cudaStream_t s) {
-    typedef Far4<R, P> F;
+template <int P> void far_launch_4s(mot_ctx* c, FarArgs<double>& a, cudaStream_t s) {
+    typedef Far4<P> F;
     const int sm_bytes = (int)sizeof(typename F::Smem);
-    allow_smem<k_far_4s<R, P>>(sm_bytes);
+    allow_smem<k_far_4s<P>>(sm_bytes);
     const long long blocks = 4 * ((c->noct + F::NB - 1) / F::NB);
-    launch_dependent(mot::dependent_launches(c), k_far_4s<R, P>, (int)blocks, F::NTB, sm_bytes, s, a);
+    launch_dependent(mot::dependent_launches(c), k_far_4s<P>, (int)blocks, F::NTB, sm_bytes, s, a);
     MOT_LAUNCH_CHECK();
 }
 
@@ -1186,9 +1168,9 @@ void far_level(mot_ctx* c, int k, int n0, cudaStream_t s) {
             case 2: far_launch_reg<R, 4, 1>(c, a, s); break;
             case 4: far_launch_reg<R, 8, 1>(c, a, s); break;
             case 8: far_launch_reg<R, 16, 1>(c, a, s); break;
-            case 16: far_launch_4s<R, 32>(c, a, s); break;
-            case 32: far_launch_4s<R, 64>(c, a, s); break;
-            case 64: far_launch_4s<R, 128>(c, a, s); break;
+            case 16: far_launch_4s<32>(c, a, s); break;
+            case 32: far_launch_4s<64>(c, a, s); break;
+            case 64: far_launch_4s<128>(c, a, s); break;
             case 128: far_launch_reg<R, 32, 8>(c, a, s); break;
             default: far_launch<R, 2>(c, a, s);
         }

@@ -167,12 +167,12 @@ struct mot_ctx {
     double* J = nullptr;         // spatial J ring [jring][3][M] (SoA per slot)
     double* rhs = nullptr;       // [3][M] adjoint: right-hand side on vacuum voxels
     double* cg_q = nullptr;      // [3][M] adjoint: lambda on vacuum voxels
-    float* cg32 = nullptr;       // FP32 inner CG vectors r, p, q, e ([4][M] float4)
+    float* cg32 = nullptr;       // FP32 inner vectors r, p and q (d_k of even and odd k), e ([4][M] float4)
     // start of the solve (solve.cu): right-hand sides of the last steps and the fit
     double* b_ring = nullptr;    // FP64: [kFitVectors + 1][3][M]
     float* xb_ring = nullptr;    // FP32-history: (x, b) float2, [kFitVectors + 1][3][M]
     float* b_lo = nullptr;       //   low part of b_n [3][M]
-    float* cg_xl = nullptr;      //   low part of x, [M] float4 (later refinements)
+    float* cg_xl = nullptr;      //   [M] float4: the start, for the neighbours; later the low parts of x
     float* diag_lo = nullptr;    //   low part of cg_diag [M]
     double* fit = nullptr;       // fit state (kFitWords)
     double* fit_part = nullptr;  // epilogue's partial sums

@@ -6,12 +6,14 @@
 //
 // Z_0^delta = diag(T(0)/eps + delta_0) - diag(chi) G_0 couples each voxel to its 26
 // neighbours when c dt = h (Sec. 5.2).  Scaled by diag(1/chi) it is symmetric positive
-// definite on the voxels with chi > 0 (D_0 = Z_0 in the PDSA, Eq. Dn), so it is solved
-// with conjugate gradients on A = diag((T(0)/eps + delta_0)/chi) - G_0 and b = rhs/chi.
-// Voxels with eps = 1 (chi = 0) carry J = rhs / (T(0) + delta_0), which is zero for
-// the zero initial state.  The CG runs as one cooperative kernel with grid-wide
-// barriers (bounded waits: a barrier that is not reached in time ends the kernel with
-// a timeout flag); it stops at ||r|| <= tol ||b|| or after max_iter iterations.
+// definite on the voxels with chi > 0 (D_0 = Z_0 in the PDSA, Eq. Dn): the system is A x = b,
+// A = diag((T(0)/eps + delta_0)/chi) - G_0 and b = rhs/chi, solved by iterative refinement with
+// Chebyshev iterations in FP32 (k_cg) from a fit of the earlier solutions.  Voxels with eps = 1
+// (chi = 0) carry J = rhs / (T(0) + delta_0), which is zero for the zero initial state.  The
+// solve is one cooperative kernel: on grids whose tiles all fit the GPU its blocks exchange words
+// with their neighbours, on larger ones they meet at grid barriers (bounded waits either way: one
+// that runs out ends the kernel with a timeout flag).  It stops at ||b - A x|| <= tol ||b|| or
+// after max_iter iterations.
 #include "mot_internal.cuh"
 
 #include <type_traits>
@@ -437,8 +439,7 @@ struct CGArgs {
     float4* xl;
     double* red;          // [2][nw] FP64 partial sums: wide residual sums
     float4* red4;         // [2][nw] exchanged partial sums (values, sequence number)
-    double tol2;          // outer tolerance^2 (relative to ||b||^2)
-    float tol;
+    float tol;            // outer tolerance, relative to ||b||
     float inv_theta;      // Chebyshev: 1 / theta, theta = (lmin + lmax) / 2
     int n_cheb;           // most Chebyshev iterations per refinement (<= MAXCHEB)
     float inv_log2_rate;  // 1 / log2 of the Chebyshev convergence rate (< 0)
@@ -2274,7 +2275,6 @@ CGArgs make_cg_args(mot_ctx* c, int n, double* norm2_out, double* out) {
     a.xl = c->cg_xl ? reinterpret_cast<float4*>(c->cg_xl) : nullptr;
     a.red = c->red;
     a.red4 = reinterpret_cast<float4*>(c->red + 2LL * c->cg_blocks);
-    a.tol2 = c->tol * c->tol;
     a.tol = (float)c->tol;
     a.inv_theta = c->cheb_inv_theta;
     a.n_cheb = c->cheb_n;
