@@ -297,12 +297,15 @@ void launch(mot_ctx* c, const ZArgs<R>& a, cudaStream_t s) {
     allow_smem<k_zmac<R, TB, P1, P2>>(sm);
     // Threads: whole rounds of the product step (Hw = P / 2 + 1 is odd, and 33 x 4 pairs on
     // 128 threads would take a second round for 4 of them); where the transforms are the
-    // larger part (FP32, or few lags), a stage of them in one round too.  More threads than
-    // that leave room for fewer blocks (FP64, 28^3, 7 lags: 64 us with 128, 72 with 256;
-    // 20^3, one lag, Lanczos step: 149 with 96, 132 with 256).
+    // larger part (FP32, or up to three lags on a small plane), a stage of them in one round
+    // too.  More threads than that leave room for fewer blocks: FP64, 28^3, 7 lags 64 us with
+    // 128, 72 with 256.  FP64 with the lags of block 2 (one) and 4 (three), without -> with the
+    // stage's threads: 12^3 18.9 -> 15.7 and 19.1 -> 18.3, 20^3 24.3 -> 23.4 and 30.9 -> 31.7,
+    // 24^3 28.6 -> 26.5 and 34.4 -> 32.8; but past eight positions an SM 28^3 40.9 -> 46.9 and
+    // 49.6 -> 57.1, 64 x 16 x 16 31.0 -> 37.7 and 39.5 -> 46.3.
     const int lanes = a.Hw * TB * a.split, rounds = (lanes + 255) / 256;
     int threads = (lanes + rounds - 1) / rounds;
-    if (sizeof(R) == 4 || a.L < 4)
+    if (sizeof(R) == 4 || (a.L < 4 && a.plane <= 8 * c->nsm))
         threads = std::max(threads,
                            std::min(256, 3 * TB * (P1 * P2 > 1 ? std::max(P1, P2) : a.Pw / 2)));
     launch_dependent(mot::dependent_launches(c), k_zmac<R, TB, P1, P2>, (a.plane + TB - 1) / TB,
