@@ -50,15 +50,19 @@ struct MotError {
 // of the setup and of the marches uses.  That stream does not wait for the legacy one: a plain
 // cudaMemcpy of a small pageable buffer returns once the buffer is staged, and a plain
 // cudaMemset returns at once, so either could land behind the kernels that need it while the
-// program keeps the legacy stream busy.  The host buffer may be freed on return.
+// program keeps the legacy stream busy.  An upload is complete on return: where the device reads
+// pageable memory in place (Grace), an asynchronous copy of it is not staged, and the buffer must
+// outlive it.
 template <typename T> void upload(T* dst, const T* src, size_t n, cudaStream_t s) {
     MOT_CUDA_TRY(cudaMemcpyAsync(dst, src, sizeof(T) * n, cudaMemcpyHostToDevice, s));
+    MOT_CUDA_TRY(cudaStreamSynchronize(s));
 }
 template <typename T> void clear(T* dst, size_t n, cudaStream_t s) {
     MOT_CUDA_TRY(cudaMemsetAsync(dst, 0, sizeof(T) * n, s));
 }
 template <typename S> void upload_symbol(const S& sym, const void* src, size_t bytes, cudaStream_t s) {
     MOT_CUDA_TRY(cudaMemcpyToSymbolAsync(sym, src, bytes, 0, cudaMemcpyHostToDevice, s));
+    MOT_CUDA_TRY(cudaStreamSynchronize(s));
 }
 
 // ------------------------------------------------------------------ dependent launches

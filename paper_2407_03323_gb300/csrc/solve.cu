@@ -2058,8 +2058,6 @@ void stencil_setup(mot_ctx* c) {
         }
         upload_symbol(c_st32, st32, sizeof st32, c->stream);
         upload_symbol(c_stl, stl, sizeof stl, c->stream);
-        // (another context's stream may read them next)
-        MOT_CUDA_TRY(cudaStreamSynchronize(c->stream));
         if (complete && dev < 64) have_complete[dev] = true;
     }
     int noff[27];
