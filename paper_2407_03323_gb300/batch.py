@@ -7,8 +7,8 @@ driven from its own host thread (the library calls release the GIL), so the kern
 different contexts run concurrently on their own streams.  With rhs=True a scatterer's
 excitations are instead the right-hand sides of its one context
 (mot_set_excitation_rhs / mot_march_rhs: one call interleaves their steps on their
-streams) and the pool drives scatterers; measured slower (3.9e8 against 4.2e8
-voxel-timesteps/s on the 24 x 8 workload), so it is off by default.  Scatterers are processed in
+streams) and the pool drives scatterers; measured slower when it was written (3.9e8 against 4.2e8
+voxel-timesteps/s on the 24 x 8 workload, 5.4e8 now without it), so it is off by default.  Scatterers are processed in
 waves whose march state fits a device-memory budget.  Each round first stages every
 march's excitation chunk on the device (the tested plane wave, generated by the
 library), then times the marches of the round; setup, tuning and excitation staging

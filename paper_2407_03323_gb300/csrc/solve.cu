@@ -1511,7 +1511,8 @@ __device__ __forceinline__ void residual64(const CGArgs& a, int e, bool first, b
 // deals the voxels out anew.  Blocks past nw take the voxels outside every tile.  The norm
 // of a step is added up beside the next one's solve, not by the last block to finish.
 // Against an epilogue of its own and a last block (solve phase of a step): 9^3 sphere
-// FP32-history 43.2 -> 35.5 us, 32^3 52.6 -> 40.9, 133 x 27 x 21 116 -> 95, 8^3 FP64 49.9 -> 45.0.
+// FP32-history 43.2 -> 35.5 us, 32^3 52.6 -> 40.9, 133 x 27 x 21 116 -> 95, 8^3 FP64 49.9 -> 45.0
+// (36.9, 44.4, 102 and 46.8 with the aims of `need` below, two iterations more).
 // What remains of the 9^3 solve, thousands of cycles: right-hand side 13, residual 11, two
 // iterations beside the sums 5, the sums 1, eleven iterations 25, x and its norm 4.
 //
